@@ -208,33 +208,38 @@ __device__ __forceinline__ Cx<double> g_expm1_over(Cx<double> z) {
     return cdiv(one_minus, z);
 }
 
+
+// point q of edge ed: the radius rho and the angular weight w
+__device__ __forceinline__ void slp_self_point(const GeomD& g, int e, int ed, int q, double& rho, double& w) {
+    double x[3], A[3], B[3];
+    for (int k = 0; k < 3; ++k) {
+        x[k] = g.c[k * g.E + e];
+        A[k] = g.v[(ed * 3 + k) * g.E + e];
+        B[k] = g.v[((ed + 1) % 3 * 3 + k) * g.E + e];
+    }
+    double t[3] = {B[0] - A[0], B[1] - A[1], B[2] - A[2]};
+    const double L = sqrt(t[0] * t[0] + t[1] * t[1] + t[2] * t[2]);
+    for (int k = 0; k < 3; ++k) t[k] /= L;
+    const double t1 = (A[0] - x[0]) * t[0] + (A[1] - x[1]) * t[1] + (A[2] - x[2]) * t[2];
+    const double t2 = (B[0] - x[0]) * t[0] + (B[1] - x[1]) * t[1] + (B[2] - x[2]) * t[2];
+    const double f[3] = {A[0] - x[0] - t1 * t[0], A[1] - x[1] - t1 * t[1], A[2] - x[2] - t1 * t[2]};
+    const double dd = sqrt(f[0] * f[0] + f[1] * f[1] + f[2] * f[2]);
+    const double p1 = atan2(t1, dd), p2 = atan2(t2, dd);
+    const double hm = 0.5 * (p2 - p1), hp = 0.5 * (p2 + p1);
+    w = hm * g.gl[24 + q];
+    rho = dd / cos(hm * g.gl[q] + hp);
+}
+
 __device__ inline Cx<double> slp_self_f64(const GeomD& g, int e, double sre, double sim) {
-    double x[3], v[3][3];
-    for (int k = 0; k < 3; ++k) x[k] = g.c[k * g.E + e];
-    for (int a = 0; a < 3; ++a)
-        for (int k = 0; k < 3; ++k) v[a][k] = g.v[(a * 3 + k) * g.E + e];
     Cx<double> tot{0.0, 0.0};
-    for (int ed = 0; ed < 3; ++ed) {
-        const double* A = v[ed];
-        const double* B = v[(ed + 1) % 3];
-        double t[3] = {B[0] - A[0], B[1] - A[1], B[2] - A[2]};
-        double L = sqrt(t[0] * t[0] + t[1] * t[1] + t[2] * t[2]);
-        for (int k = 0; k < 3; ++k) t[k] /= L;
-        double t1 = (A[0] - x[0]) * t[0] + (A[1] - x[1]) * t[1] + (A[2] - x[2]) * t[2];
-        double t2 = (B[0] - x[0]) * t[0] + (B[1] - x[1]) * t[1] + (B[2] - x[2]) * t[2];
-        double f[3] = {A[0] - x[0] - t1 * t[0], A[1] - x[1] - t1 * t[1], A[2] - x[2] - t1 * t[2]};
-        double dd = sqrt(f[0] * f[0] + f[1] * f[1] + f[2] * f[2]);
-        double p1 = atan2(t1, dd), p2 = atan2(t2, dd);
-        double hm = 0.5 * (p2 - p1), hp = 0.5 * (p2 + p1);
+    for (int ed = 0; ed < 3; ++ed)
         for (int q = 0; q < 24; ++q) {
-            double ph = hm * g.gl[q] + hp;
-            double w = hm * g.gl[24 + q];
-            double rho = dd / cos(ph);
-            Cx<double> gz = g_expm1_over(Cx<double>{sre * rho, sim * rho});
+            double rho, w;
+            slp_self_point(g, e, ed, q, rho, w);
+            const Cx<double> gz = g_expm1_over(Cx<double>{sre * rho, sim * rho});
             tot.x += w * rho * gz.x;
             tot.y += w * rho * gz.y;
         }
-    }
     tot.x *= G3_INV4PI;
     tot.y *= G3_INV4PI;
     return tot;

@@ -414,9 +414,25 @@ g3_status launch_entries(g3_ctx* ctx, const g3_tree* t, const g3_freqs* f, int k
 // geometry once and evaluates it at the KCH frequencies.  Layout of a block:
 // [k][j][i] (frequency-major, column-major per frequency: the apply reads a
 // column of rows with one coalesced load), complex, starting at offs[b].
-// Self entries (i == j) are left to k_near_self.
+//
+// The frequencies come in the working precision (FreqT): a float64 pair per
+// (entry, frequency) costs two float64-to-float32 conversions, which this part
+// issues at its float64 rate.  Entries of the double layer with i == j are 0
+// (x_i lies in the element's plane); those of the single layer are left to
+// k_near_self.
+template <class T>
+struct FreqOf {
+    using type = double2;
+};
+template <>
+struct FreqOf<float> {
+    using type = float2;
+};
+template <class T>
+using FreqT = typename FreqOf<T>::type;
+
 template <int KER, class T, int KCH>
-__global__ void __launch_bounds__(256) k_near(GeomF gf, GeomD gd, const double2* __restrict__ sd,
+__global__ void __launch_bounds__(256) k_near(GeomF gf, GeomD gd, const FreqT<T>* __restrict__ sk,
                                               const BlockRange* __restrict__ ranges,
                                               const long long* __restrict__ offs, int Ku, Cx<T>* __restrict__ out) {
     const int b = blockIdx.x;
@@ -428,7 +444,11 @@ __global__ void __launch_bounds__(256) k_near(GeomF gf, GeomD gd, const double2*
     const int kn = min(KCH, Ku - k0);
     for (int e = threadIdx.x; e < MN; e += blockDim.x) {
         int i = br.rb + e % M, j = br.cb + e / M;
-        if (i == j) continue;
+        if (i == j) {
+            if constexpr (KER == G3_DLP)
+                for (int kk = 0; kk < kn; ++kk) out[base + (long long)(k0 + kk) * MN + e] = Cx<T>{0, 0};
+            continue;
+        }
         if constexpr (KER == G3_GAL_SLP) {
             // regular rule for every off-diagonal pair; pairs with a common
             // vertex are overwritten by k_near_ss
@@ -438,8 +458,8 @@ __global__ void __launch_bounds__(256) k_near(GeomF gf, GeomD gd, const double2*
             else
                 gal_setup(gd, i, j, p);
             for (int kk = 0; kk < kn; ++kk) {
-                double2 s = sd[k0 + kk];
-                out[base + (long long)(k0 + kk) * MN + e] = gal_eval<T>(p, (T)s.x, (T)s.y);
+                const FreqT<T> s = sk[k0 + kk];
+                out[base + (long long)(k0 + kk) * MN + e] = gal_eval<T>(p, s.x, s.y);
             }
         } else {
             Pair7<T> p;
@@ -448,8 +468,8 @@ __global__ void __launch_bounds__(256) k_near(GeomF gf, GeomD gd, const double2*
             else
                 pair_setup<KER>(gd, i, j, p);
             for (int kk = 0; kk < kn; ++kk) {
-                double2 s = sd[k0 + kk];
-                out[base + (long long)(k0 + kk) * MN + e] = pair_eval<KER, T>(p, (T)s.x, (T)s.y);
+                const FreqT<T> s = sk[k0 + kk];
+                out[base + (long long)(k0 + kk) * MN + e] = pair_eval<KER, T>(p, s.x, s.y);
             }
         }
     }
@@ -516,7 +536,7 @@ __global__ void __launch_bounds__(NT) k_near_ss(GeomD gd, SsRule gr, const SsPai
 // block, chunk of KCH unique frequencies), layout [k][j][i] as k_near.
 template <int OP, class T, int KCH>
 __global__ void __launch_bounds__(256) k_near_p1(GeomF gf, GeomD gd, const int* __restrict__ tv,
-                                                 const double2* __restrict__ sd, const BlockRange* __restrict__ ranges,
+                                                 const FreqT<T>* __restrict__ sk, const BlockRange* __restrict__ ranges,
                                                  const long long* __restrict__ offs, int Ku, Cx<T>* __restrict__ out) {
     const int b = blockIdx.x;
     const int k0 = blockIdx.y * KCH;
@@ -539,9 +559,9 @@ __global__ void __launch_bounds__(256) k_near_p1(GeomF gf, GeomD gd, const int* 
             p1_pair_setup<OP>(gd, pe, qe, r, m, gz, cab, nn);
         const long long e0 = base + (long long)(3 * (qe - br.cb / 3)) * M + 3 * (pe - br.rb / 3);
         for (int kk = 0; kk < kn; ++kk) {
-            const double2 s = sd[k0 + kk];
+            const FreqT<T> s = sk[k0 + kk];
             Cx<T> v[9];
-            p1_pair_eval<OP, T>(r, m, gz, cab, nn, (T)s.x, (T)s.y, v);
+            p1_pair_eval<OP, T>(r, m, gz, cab, nn, s.x, s.y, v);
             Cx<T>* o = out + (long long)(k0 + kk) * M * N + e0;
 #pragma unroll
             for (int a = 0; a < 3; ++a)
@@ -668,13 +688,20 @@ __global__ void __launch_bounds__(NT) k_near_ss_p1(GeomD gd, SsRule gr, const Ss
     }
 }
 
+// the unique frequencies in the working precision
+template <class T>
+static const FreqT<T>* freqs_of(const g3_freqs* f) {
+    if constexpr (sizeof(T) == 4) return f->d_sf.as<float2>();
+    else return f->d_sd.as<double2>();
+}
+
 template <int OP, class T>
 static g3_status launch_near_p1_t(g3_ctx* ctx, const g3_tree* t, const g3_freqs* f, g3_near* nf) {
     const int nb = (int)nf->order.size();
     constexpr int KCH = 16;
     dim3 grid(nb, (f->Ku + KCH - 1) / KCH);
     Cx<T>* o = reinterpret_cast<Cx<T>*>(nf->data.p);
-    k_near_p1<OP, T, KCH><<<grid, 256, 0, ctx->stream>>>(t->gf, t->gd, t->d_tv.as<int>(), f->d_sd.as<double2>(),
+    k_near_p1<OP, T, KCH><<<grid, 256, 0, ctx->stream>>>(t->gf, t->gd, t->d_tv.as<int>(), freqs_of<T>(f),
                                                           nf->d_ranges.as<BlockRange>(), nf->d_offs.as<long long>(),
                                                           f->Ku, o);
     ctx->count("k_near_p1");
@@ -695,24 +722,136 @@ static g3_status launch_near_p1_t(g3_ctx* ctx, const g3_tree* t, const g3_freqs*
     return G3_OK;
 }
 
-// Self entries of the near field, float64: one thread per (element p, unique
-// frequency k); the entry (p, p) of the diagonal leaf block sits at
-// diag_base[p] + k * diag_mn[p] (diag_base[p] < 0: not in this tree's blocks).
-template <int KER, class T>
-__global__ void k_near_self(GeomD gd, const double2* __restrict__ sd, int E, int Ku,
-                            const long long* __restrict__ diag_base, const int* __restrict__ diag_mn,
-                            Cx<T>* __restrict__ out) {
-    long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (idx >= (long long)E * Ku) return;
-    const int p = (int)(idx % E), k = (int)(idx / E);
-    if (diag_base[p] < 0) return;  // the diagonal block belongs to another rank's subset
-    Cx<T> v{0, 0};
-    if (KER == G3_SLP) {
-        double2 s = sd[k];
-        Cx<double> d = slp_self_f64(gd, p, s.x, s.y);
-        v = Cx<T>{(T)d.x, (T)d.y};
+// Self entries of the single layer in the near field, float64: one warp per
+// element p; the entry (p, p) of the diagonal leaf block sits at diag_base[p] +
+// k * diag_mn[p] (diag_base[p] < 0: not in this tree's blocks).
+//
+// In polar coordinates about the centroid (slp_self_f64) the entry is
+//   V(s) = (1 / 4 pi) sum_q w_q (1 - exp(-s rho_q)) / s
+// over the 72 angular points (24 per edge), whose rho_q and w_q do not depend
+// on the frequency.  Evaluated as it stands it takes an exponential, a sine
+// and a cosine in float64 per point and frequency, on a part with two float64
+// lanes per SM.  So the warp forms the points once and their moments
+//   m0_n = sum_q w_q rho_q (rho_q / rmax)^n          (about 0)
+//   m1_n = sum_q w_q ((rho_q - rc) / rh)^n           (about the middle rc of
+//                                                     [rmin, rmax], rh its half width)
+// for n < 32, and every lane (one frequency each) sums one of
+//   |s| rmax <= 4:  V = (1/4 pi) sum_n (-z)^n / (n+1)! m0_n,            z = s rmax
+//   |s| rh <= 4:    V = (1/4 pi s) (m1_0 - e^{-s rc} sum_n (-x)^n / n! m1_n),  x = s rh
+// whose first omitted terms are below 4^32 / 32! = 7e-17 and whose largest
+// terms exceed the sum by at most e^4, so both hold ~1e-14 relative; larger
+// |s| rh sums the points directly.
+// Bound by the float64 pipe (the moments and the series).  12,288 elements x 65
+// frequencies on a GB300: 14.0 -> 1.1 ms.
+__constant__ double SELF_INV[34] = {0.0,      1.0,      1.0 / 2,  1.0 / 3,  1.0 / 4,  1.0 / 5,  1.0 / 6,  1.0 / 7,  1.0 / 8,
+                                    1.0 / 9,  1.0 / 10, 1.0 / 11, 1.0 / 12, 1.0 / 13, 1.0 / 14, 1.0 / 15, 1.0 / 16, 1.0 / 17,
+                                    1.0 / 18, 1.0 / 19, 1.0 / 20, 1.0 / 21, 1.0 / 22, 1.0 / 23, 1.0 / 24, 1.0 / 25, 1.0 / 26,
+                                    1.0 / 27, 1.0 / 28, 1.0 / 29, 1.0 / 30, 1.0 / 31, 1.0 / 32, 1.0 / 33};
+constexpr int SELF_NM = 32;   // moments of each kind (one per lane)
+constexpr int SELF_NW = 4;    // elements (warps) per CTA
+template <class T>
+__global__ void __launch_bounds__(SELF_NW * 32) k_near_self(GeomD gd, const double2* __restrict__ sd, int E, int Ku,
+                                                            const long long* __restrict__ diag_base,
+                                                            const int* __restrict__ diag_mn, Cx<T>* __restrict__ out) {
+    __shared__ double pts[SELF_NW][2][72];           // rho_q, w_q
+    __shared__ double mom[SELF_NW][2][SELF_NM];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int p = blockIdx.x * SELF_NW + warp;
+    if (p >= E || diag_base[p] < 0) return;  // the whole warp (only warp-level synchronisation below)
+    double* rho = pts[warp][0];
+    double* wq = pts[warp][1];
+    double rmin = 1e300, rmax = 0.0;
+    for (int q = lane; q < 72; q += 32) {
+        slp_self_point(gd, p, q / 24, q % 24, rho[q], wq[q]);
+        rmin = fmin(rmin, rho[q]);
+        rmax = fmax(rmax, rho[q]);
     }
-    out[diag_base[p] + (long long)k * diag_mn[p]] = v;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        rmin = fmin(rmin, __shfl_xor_sync(0xffffffffu, rmin, o));
+        rmax = fmax(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
+    }
+    __syncwarp();
+    const double rc = 0.5 * (rmin + rmax), rh = fmax(0.5 * (rmax - rmin), 1e-9 * rmax);
+    {
+        // lane = point (up to three per lane), running powers; 32 moments of a
+        // kind are summed over the warp by halving exchanges, which leave
+        // moment n in lane n
+        for (int kind = 0; kind < 2; ++kind) {
+            double b[3], t[3], v[SELF_NM];
+#pragma unroll
+            for (int u = 0; u < 3; ++u) {
+                const int q = lane + 32 * u;
+                const bool in = q < 72;
+                const double r = in ? rho[q] : 0.0, w = in ? wq[q] : 0.0;
+                b[u] = kind == 0 ? r / rmax : (in ? (r - rc) / rh : 0.0);
+                t[u] = kind == 0 ? w * r : w;
+            }
+#pragma unroll
+            for (int n = 0; n < SELF_NM; ++n) {
+                v[n] = t[0] + t[1] + t[2];
+#pragma unroll
+                for (int u = 0; u < 3; ++u) t[u] *= b[u];
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const bool hi = (lane & o) != 0;
+#pragma unroll
+                for (int n = 0; n < o; ++n) {
+                    const double send = hi ? v[n] : v[n + o], keep = hi ? v[n + o] : v[n];
+                    v[n] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
+            }
+            mom[warp][kind][lane] = v[0];
+        }
+    }
+    __syncwarp();
+    const double* m0 = mom[warp][0];
+    const double* m1 = mom[warp][1];
+    for (int k = lane; k < Ku; k += 32) {
+        const double2 s = sd[k];
+        const double as = sqrt(s.x * s.x + s.y * s.y);
+        Cx<double> v;
+        if (as * rmax <= 4.0) {
+            const Cx<double> mz{-s.x * rmax, -s.y * rmax};
+            Cx<double> term{1.0, 0.0};
+            v = Cx<double>{m0[0], 0.0};
+#pragma unroll 4
+            for (int n = 1; n < SELF_NM; ++n) {
+                const double inv = SELF_INV[n + 1];
+                term = cmul(term, Cx<double>{mz.x * inv, mz.y * inv});
+                v.x = fma(term.x, m0[n], v.x);
+                v.y = fma(term.y, m0[n], v.y);
+            }
+        } else {
+            Cx<double> sum{0.0, 0.0};  // sum_q w_q exp(-s rho_q)
+            if (as * rh <= 4.0) {
+                const Cx<double> mx{-s.x * rh, -s.y * rh};
+                Cx<double> term{1.0, 0.0}, acc{m1[0], 0.0};
+#pragma unroll 4
+                for (int n = 1; n < SELF_NM; ++n) {
+                    const double inv = SELF_INV[n];
+                    term = cmul(term, Cx<double>{mx.x * inv, mx.y * inv});
+                    acc.x = fma(term.x, m1[n], acc.x);
+                    acc.y = fma(term.y, m1[n], acc.y);
+                }
+                double sn, cs;
+                sincos(s.y * rc, &sn, &cs);
+                const double e = exp(-s.x * rc);
+                sum = cmul(acc, Cx<double>{e * cs, -e * sn});
+            } else {
+                for (int q = 0; q < 72; ++q) {
+                    double sn, cs;
+                    sincos(s.y * rho[q], &sn, &cs);
+                    const double e = wq[q] * exp(-s.x * rho[q]);
+                    sum.x += e * cs;
+                    sum.y -= e * sn;
+                }
+            }
+            v = cdiv(Cx<double>{m1[0] - sum.x, -sum.y}, Cx<double>{s.x, s.y});
+        }
+        out[diag_base[p] + (long long)k * diag_mn[p]] = Cx<T>{(T)(v.x * G3_INV4PI), (T)(v.y * G3_INV4PI)};
+    }
 }
 
 // Galerkin: near-field pairs with a common vertex (the list of SsPair records
@@ -723,7 +862,7 @@ static g3_status launch_near_galerkin(g3_ctx* ctx, const g3_tree* t, const g3_fr
     constexpr int KCH = 16;
     dim3 grid(nb, (f->Ku + KCH - 1) / KCH);
     Cx<T>* o = reinterpret_cast<Cx<T>*>(nf->data.p);
-    k_near<G3_GAL_SLP, T, KCH><<<grid, 256, 0, ctx->stream>>>(t->gf, t->gd, f->d_sd.as<double2>(),
+    k_near<G3_GAL_SLP, T, KCH><<<grid, 256, 0, ctx->stream>>>(t->gf, t->gd, freqs_of<T>(f),
                                                                nf->d_ranges.as<BlockRange>(),
                                                                nf->d_offs.as<long long>(), f->Ku, o);
     ctx->count("k_near");
@@ -759,33 +898,26 @@ g3_status launch_near(g3_ctx* ctx, const g3_tree* t, const g3_freqs* f, g3_near*
     }
     constexpr int KCH = 16;
     dim3 grid(nb, (f->Ku + KCH - 1) / KCH);
-    const double2* sd = f->d_sd.as<double2>();
     const BlockRange* rg = nf->d_ranges.as<BlockRange>();
     const long long* of = nf->d_offs.as<long long>();
     const long long* db = nf->d_diag_base.as<long long>();
     const int* dm = nf->d_diag_mn.as<int>();
-    const int sgrid = (int)(((long long)t->ne * f->Ku + 255) / 256);
-    if (nf->prec == G3_MIXED) {
-        Cx<float>* o = nf->data.as<Cx<float>>();
+    auto go = [&](auto zero) -> g3_status {
+        using T = decltype(zero);
+        Cx<T>* o = nf->data.as<Cx<T>>();
         if (kernel == G3_SLP) {
-            k_near<G3_SLP, float, KCH><<<grid, 256, 0, ctx->stream>>>(t->gf, t->gd, sd, rg, of, f->Ku, o);
-            k_near_self<G3_SLP, float><<<sgrid, 256, 0, ctx->stream>>>(t->gd, sd, t->ne, f->Ku, db, dm, o);
+            k_near<G3_SLP, T, KCH><<<grid, 256, 0, ctx->stream>>>(t->gf, t->gd, freqs_of<T>(f), rg, of, f->Ku, o);
+            k_near_self<T><<<(t->ne + SELF_NW - 1) / SELF_NW, SELF_NW * 32, 0, ctx->stream>>>(
+                t->gd, f->d_sd.as<double2>(), t->ne, f->Ku, db, dm, o);
+            ctx->count("k_near_self");
         } else {
-            k_near<G3_DLP, float, KCH><<<grid, 256, 0, ctx->stream>>>(t->gf, t->gd, sd, rg, of, f->Ku, o);
-            k_near_self<G3_DLP, float><<<sgrid, 256, 0, ctx->stream>>>(t->gd, sd, t->ne, f->Ku, db, dm, o);
+            k_near<G3_DLP, T, KCH><<<grid, 256, 0, ctx->stream>>>(t->gf, t->gd, freqs_of<T>(f), rg, of, f->Ku, o);
         }
-    } else {
-        Cx<double>* o = nf->data.as<Cx<double>>();
-        if (kernel == G3_SLP) {
-            k_near<G3_SLP, double, KCH><<<grid, 256, 0, ctx->stream>>>(t->gf, t->gd, sd, rg, of, f->Ku, o);
-            k_near_self<G3_SLP, double><<<sgrid, 256, 0, ctx->stream>>>(t->gd, sd, t->ne, f->Ku, db, dm, o);
-        } else {
-            k_near<G3_DLP, double, KCH><<<grid, 256, 0, ctx->stream>>>(t->gf, t->gd, sd, rg, of, f->Ku, o);
-            k_near_self<G3_DLP, double><<<sgrid, 256, 0, ctx->stream>>>(t->gd, sd, t->ne, f->Ku, db, dm, o);
-        }
-    }
+        return G3_OK;
+    };
+    const g3_status st = nf->prec == G3_MIXED ? go(0.0f) : go(0.0);
+    if (st != G3_OK) return st;
     ctx->count("k_near");
-    ctx->count("k_near_self");
     G3_CUDA(cudaGetLastError());
     return G3_OK;
 }
