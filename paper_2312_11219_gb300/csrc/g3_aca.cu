@@ -132,6 +132,30 @@ static void take(DevBuf& dst, DevBuf& src) {
     src.bytes = 0;
 }
 
+// float64: four RS x RS float64 matrices, or two of them and the Gram staging
+template <class T>
+static size_t recomp_arena_bytes(int RF) {
+    if (sizeof(T) == 4) return 0;
+    return 2 * (size_t)RS * RS * sizeof(Cx<double>) +
+           std::max(2 * (size_t)RS * RS * sizeof(Cx<T>), 33 * (size_t)RF * sizeof(Cx<T>));
+}
+
+// float32: the arena that holds all RF columns of an M x N face and the two
+// matrices of its recompression (after the row buffer, or after the tables of
+// the on-demand lines), as far as two CTAs per SM leave room (one at 512
+// threads): 28 columns of a 192 x 192 face, all 48 of a 96 x 96 one.  Columns
+// beyond it live in the workspace.
+static size_t arena_grow(const g3_ctx* ctx, int M, int N, int RF, int drf, int nt, size_t base) {
+    const bool dres = drf > 0 && (long long)M * N <= drf;
+    const size_t off = dres ? (N <= ROWMAX ? (size_t)N * sizeof(Cx<float>) + 16 : 0) : facetab_smem_bytes<float>() + 256;
+    const int cap = std::min(std::min(M, N), RF);
+    const size_t want = off + (size_t)cap * cs_ld(M, N) * sizeof(Cx<float>) + 2 * (size_t)cap * (cap + 4) * sizeof(Cx<float>);
+    const size_t fixed = 1024 + ((sizeof(BlockSh<float>) + sizeof(AcaArgs<float>) + 256 + 127) & ~size_t(127));
+    const size_t room = (ctx->smem_optin + 1024) / (nt >= 512 ? 1 : 2);
+    const size_t most = room > fixed ? (room - fixed) & ~size_t(127) : 0;
+    return std::max(base, std::min(want, most));
+}
+
 template <class T>
 static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, double eps3, const g3_opts& o,
                            const void* sep_a, const void* sep_b, const void* sep_c, int sep_R) {
@@ -305,14 +329,12 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
         sv = SepView<T>{sep_R, fa->M_sep, fa->N_sep, Ku, d_sa.as<T>(), d_sb.as<T>(), d_sc.as<T>()};
     }
     constexpr int NT = 256;
-    // dynamic shared memory arena, reused phase by phase: the four RS x RS
-    // matrices of the recompression (+ Gram staging; float32: + the working-
-    // precision copies of the two Cholesky factors), the pivot-search
+    // dynamic shared memory arena, reused phase by phase: float64 the four RS x RS
+    // matrices of the recompression or its Gram staging (float32: the face's
+    // columns and two matrices, arena_grow below), the pivot-search
     // tiles (2 RF TM complex T, TM = 64 float / 32 double) and the eq. (norm)
     // staging ((NORM_RC + 1) (32 + RF) + 32 RF complex T, then 64 column pointers)
-    const size_t recomp_bytes = 2 * (size_t)RS * RS * sizeof(Cx<double>) +
-                                std::max(2 * (size_t)RS * RS * sizeof(Cx<T>), 33 * (size_t)RF * sizeof(Cx<T>)) +
-                                (sizeof(T) == 4 ? 2 * (size_t)RS * RS * sizeof(Cx<T>) : 0);
+    const size_t recomp_bytes = recomp_arena_bytes<T>(RF);
     const size_t tile_bytes = 2 * (size_t)RF * (sizeof(T) == 4 ? 64 : 32) * sizeof(Cx<T>);
     const size_t gram_bytes = ((NORM_RC<T> + 1) * (size_t)(32 + RF) + 32 * (size_t)RF) * sizeof(Cx<T>) + 64 * sizeof(void*);
     const size_t tab_bytes = 2 * TABMAX * sizeof(long long) + TABMAX * sizeof(short) +
@@ -333,13 +355,19 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
     }
     const size_t drf_smem =
         drf > 0 ? drf_stage_offset<T>() + std::max(drf_stage_bytes<T, 256>(), drf_stage_bytes<T, 512>()) : 0;
-    const size_t smem =
+    const size_t smem_base =
         std::max(std::max(std::max(std::max(recomp_bytes, tile_bytes), gram_bytes), tab_bytes), drf_smem);
     // low-rank class: 128, 256, 384 or 512 threads per CTA (float32 path); more
     // threads shorten each block, which matters for the largest blocks at the
     // end, fewer keep more blocks in flight per SM
     const int nt_low = (sizeof(T) == 4 && (o.threads == 128 || o.threads == 384 || o.threads == 512)) ? o.threads
                                                                                                          : NT;
+    size_t smem = smem_base;
+    if constexpr (sizeof(T) == 4)
+        for (int q = 0; q < n_run; ++q) {
+            const BlockRange& r = ranges[queue[q]];
+            if (!is_dense(r)) smem = std::max(smem, arena_grow(ctx, r.re - r.rb, r.ce - r.cb, RF, drf, nt_low, smem));
+        }
     int per_low = o.ctas_per_sm;
     if (per_low <= 0) {
         if constexpr (sizeof(T) == 4)
@@ -350,7 +378,7 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
         else
             per_low = occupancy_kind<T, NT, false>(kernel, smem);
     }
-    const int per_dense = o.ctas_per_sm > 0 ? o.ctas_per_sm : occupancy_kind<T, NT, true>(kernel, smem);
+    const int per_dense = o.ctas_per_sm > 0 ? o.ctas_per_sm : occupancy_kind<T, NT, true>(kernel, smem_base);
     const int grid_low = o.unbatched ? 1 : std::max(1, std::min(n_low, ctx->n_sm * per_low));
     const int grid_dense = o.unbatched ? 1 : std::max(1, std::min(n_dense, ctx->n_sm * per_dense));
     const int grid = std::max(grid_low, grid_dense);
@@ -483,6 +511,7 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
         A.Nmax = Nmax;
         A.drf_max = drf > 0 ? drf : 0;
         A.drf_off = drf > 0 ? drf_off : 0;
+        A.arena_bytes = (int)smem;
         if (!graph) G3_CUDA(cudaEventRecord(e0, ctx->stream));
         g3_status st = G3_OK;
         for (int cls = 0; cls < 2 && st == G3_OK; ++cls) {
@@ -498,7 +527,7 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
             for (int l = 0; l < launches && st == G3_OK; ++l) {
                 if (o.unbatched) B.single = l;
                 if (cls == 1)
-                    st = launch_kind<T, NT, true>(ctx, kernel, B, g, smem);
+                    st = launch_kind<T, NT, true>(ctx, kernel, B, g, smem_base);
                 else if constexpr (sizeof(T) == 4)
                     st = nt_low == 512   ? launch_kind<T, 512, false>(ctx, kernel, B, g, smem)
                          : nt_low == 384 ? launch_kind<T, 384, false>(ctx, kernel, B, g, smem)
@@ -772,13 +801,13 @@ static g3_status run_aca_whole_t(g3_ctx* ctx, const g3_tree* t, const g3_freqs* 
         return (long long)(ranges[a].re - ranges[a].rb) * (ranges[a].ce - ranges[a].cb) >
                (long long)(ranges[b].re - ranges[b].rb) * (ranges[b].ce - ranges[b].cb);
     });
-    const size_t recomp_bytes = 2 * (size_t)RS * RS * sizeof(Cx<double>) +
-                                std::max(2 * (size_t)RS * RS * sizeof(Cx<T>), 33 * (size_t)RF * sizeof(Cx<T>)) +
-                                (sizeof(T) == 4 ? 2 * (size_t)RS * RS * sizeof(Cx<T>) : 0);
+    const size_t recomp_bytes = recomp_arena_bytes<T>(RF);
     const size_t gram_bytes = ((NORM_RC<T> + 1) * (size_t)(32 + RF) + 32 * (size_t)RF) * sizeof(Cx<T>) + 64 * sizeof(void*);
     const size_t tab_bytes = 2 * TABMAX * sizeof(long long) + TABMAX * sizeof(short) +
                              (TABMAX + RF_MAX) * sizeof(Cx<T>) + ROWMAX * sizeof(Cx<T>) + 64;
-    const size_t smem = std::max(std::max(recomp_bytes, gram_bytes), tab_bytes);
+    size_t smem = std::max(std::max(recomp_bytes, gram_bytes), tab_bytes);
+    if constexpr (sizeof(T) == 4)
+        for (auto& r : ranges) smem = std::max(smem, arena_grow(ctx, r.re - r.rb, r.ce - r.cb, RF, -1, 256, smem));
     const int grid = std::max(1, std::min(n_far, 2 * ctx->n_sm));
     const size_t stride = al256(ws_bytes<T>(RF, Mmax, Nmax, Cmax, Ku));
     DevBuf d_ws, d_ranges, d_queue, d_head, d_counters, d_ctr, d_rec, d_r3, d_normb, d_cand, d_hh, d_hself, d_fib,
@@ -809,6 +838,7 @@ static g3_status run_aca_whole_t(g3_ctx* ctx, const g3_tree* t, const g3_freqs* 
     long long cap = 4 * worst;
     G3_CUDA(pool->alloc((size_t)cap * sizeof(Cx<T>)));
     AcaArgs<T> A{};
+    A.arena_bytes = (int)smem;
     A.gf = t->gf;
     A.gd = t->gd;
     A.sd = f->d_sd.as<double2>();

@@ -6,12 +6,12 @@
 // Algorithm 1 on the block restricted to the unique frequencies:
 //   face    partial-pivot ACA of the residual face at k_l (eps_face), with the
 //           residual of earlier crosses subtracted row/column-wise;
-//   recomp  Cholesky-QR of both ACA factors (float64 Cholesky of column-scaled
-//           Gram matrices), then the r x r core R_U R_V^H is factored: float64
-//           (T = double) by a one-sided Jacobi SVD truncated at
-//           sigma_i < eps_face sigma_1, float32 (T = float) by a column-pivoted
-//           QR stopped when the largest remaining column norm falls below the
-//           same threshold (Section 4, second implementation remark);
+//   recomp  (Section 4, second implementation remark) float64: Cholesky-QR of
+//           both ACA factors (column-scaled Gram matrices), then a one-sided
+//           Jacobi SVD of the r x r core R_U R_V^H truncated at sigma_i <
+//           eps_face sigma_1; float32: QR of V by modified Gram-Schmidt, then a
+//           column-pivoted QR of W = U R^H stopped when the largest remaining
+//           column norm falls below the same threshold (g3_face32.cuh);
 //   pivot   argmax |H_l[i, j]| over the dense expansion of U' V'^H, tiled
 //           through shared memory, ties to the smallest row-major index
 //           (Section 4, last remark), or optionally (single layer) the
@@ -28,10 +28,10 @@
 //
 // Precision: T = float (mixed) evaluates entries and face arithmetic in
 // float32 and stores complex64 factors; T = double does everything in float64.
-// In both, the fiber residuals, the Cholesky factors of the recompression,
-// the sums over crosses of eq. (norm) and ||C^(l)|| are float64; with
-// T = float the Gram products, the core factorisation and the back
-// substitution of the recompression are float32.
+// In both, the fiber residuals, the sums over crosses of eq. (norm) and
+// ||C^(l)|| are float64; with T = float the recompression is float32
+// throughout (it forms no Gram matrices) and the face test's sum over crosses
+// float-float.
 //
 // No CTA waits on another: the only inter-CTA communication is the atomic
 // queue counter and the atomic pool allocator.
@@ -70,6 +70,7 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
 }
 
 constexpr int RF_MAX = 64;    // largest face rank cap
+constexpr int CS_PAD = 16;    // padding of a float32 face column (ColStore)
 
 // geometry and frequencies of one mesh of a batched compression
 struct GeoDesc {
@@ -123,12 +124,15 @@ struct AcaArgs {
     int drf_max;             // float32 low-rank faces of blocks with M N <= drf_max are evaluated
                              // densely into a working buffer before their ACA (0 = never)
     size_t drf_off;          // byte offset of that buffer in each CTA's workspace slice
+    int arena_bytes;         // dynamic shared memory of the launch
 };
 
 template <class T>
 struct Ws {
-    Cx<T>* uw;            // [RF][Mmax]
-    Cx<T>* vw;            // [RF][Nmax]
+    // face columns: float64 uw [RF][Mmax] and vw [RF][Nmax]; float32: uw and vw
+    // together are one array [RF][ld], ld <= Mmax + Nmax + CS_PAD (ColStore)
+    Cx<T>* uw;
+    Cx<T>* vw;
     Cx<T>* row;           // [Nmax]
     unsigned char* used;  // [Mmax]
     Cx<T>* pre;           // [Cmax * RF]
@@ -151,7 +155,7 @@ template <class T>
 __host__ __device__ inline size_t ws_bytes(int RF, int Mmax, int Nmax, int Cmax, int Ku) {
     size_t b = 0;
     auto add = [&](size_t n) { b += (n + 255) & ~size_t(255); };
-    add((size_t)RF * Mmax * sizeof(Cx<T>));
+    add((size_t)RF * (Mmax + CS_PAD) * sizeof(Cx<T>));
     add((size_t)RF * Nmax * sizeof(Cx<T>));
     add((size_t)Nmax * sizeof(Cx<T>));
     add((size_t)Mmax);
@@ -176,7 +180,7 @@ __device__ inline Ws<T> ws_carve(char* base, int RF, int Mmax, int Nmax, int Cma
         o += (n + 255) & ~size_t(255);
         return p;
     };
-    w.uw = (Cx<T>*)take((size_t)RF * Mmax * sizeof(Cx<T>));
+    w.uw = (Cx<T>*)take((size_t)RF * (Mmax + CS_PAD) * sizeof(Cx<T>));
     w.vw = (Cx<T>*)take((size_t)RF * Nmax * sizeof(Cx<T>));
     w.row = (Cx<T>*)take((size_t)Nmax * sizeof(Cx<T>));
     w.used = (unsigned char*)take((size_t)Mmax);
@@ -214,14 +218,19 @@ struct BlockSh {
     double dU[RF_MAX], dV[RF_MAX];
     double rdU[RF_MAX], rdV[RF_MAX];  // 1 / diagonal of the Cholesky factors
     T cnV[RF_MAX];                    // column norms of V' (pivot of eq. (index))
-    T tdU[RF_MAX], tdV[RF_MAX];       // dU, dV and rdU, rdV in the working precision
-    T trdU[RF_MAX], trdV[RF_MAX];
+    // float32 faces: warp candidates of the row and column argmax, the warps'
+    // terms of ||S_m||_F^2 (float-float) and the newest cross's own term
+    uint2 key[2][32];
+    float2 nrm[32];
+    float2 own;
+    // float32 recompression: squared norms, norms and their reciprocals of the
+    // orthogonalised V columns; squared norms of W's columns (double-buffered);
+    // norms of the pivot columns
+    float n2[RF_MAX], nv[RF_MAX], rnv[RF_MAX], cn[2][RF_MAX], rk32[RF_MAX];
     double fsn2;             // ||S_m||_F^2 of the face approximant (recursive)
     int fconv;               // face test passed (written by warp 0)
     int fbs;                 // sample of the largest residual
     int sel[RF_MAX];
-    int piv;                 // pivoted QR of the core: pivot column of the step
-    float rkk;               // and its norm
     ArgMaxT<T> am[32];
     double red[64];
     double norm2;
@@ -494,6 +503,61 @@ __device__ void line_coeffs(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, 
     }
 }
 
+constexpr int LIF = 16;  // loads in flight per thread in the residual lines' sums
+
+// the part of a gang in a residual line's sum over the earlier crosses (element
+// v of the line), in four independent partial sums
+template <class T, bool ROW>
+__device__ __forceinline__ void cross_sum(const AcaArgs<T>& A, const FaceTab<T>& F, int v, int part, int G, Cx<T>& s0,
+                                          Cx<T>& s1, Cx<T>& s2, Cx<T>& s3) {
+    const long long* col = ROW ? F.colV : F.colU;
+    const int nt = F.ncol;
+                int c = part;
+                // LIF loads in flight per thread (the sums wait on memory, not on arithmetic)
+                for (; c + (LIF - 1) * G < nt; c += LIF * G) {
+                    Cx<T> x[LIF];
+    #pragma unroll
+                    for (int u = 0; u < LIF; ++u) x[u] = ldcx(A.pool + col[c + u * G] + v);
+    #pragma unroll
+                    for (int u = 0; u < LIF; ++u) {
+                        Cx<T>& acc_u = (u & 3) == 0 ? s0 : (u & 3) == 1 ? s1 : (u & 3) == 2 ? s2 : s3;
+                        if (ROW) cfmac(acc_u, F.coef[c + u * G], x[u]);
+                        else cfma(acc_u, x[u], F.coef[c + u * G]);
+                    }
+                }
+                for (; c + 7 * G < nt; c += 8 * G) {
+                    Cx<T> x[8];
+    #pragma unroll
+                    for (int u = 0; u < 8; ++u) x[u] = ldcx(A.pool + col[c + u * G] + v);
+    #pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        Cx<T>& acc_u = (u & 3) == 0 ? s0 : (u & 3) == 1 ? s1 : (u & 3) == 2 ? s2 : s3;
+                        if (ROW) cfmac(acc_u, F.coef[c + u * G], x[u]);
+                        else cfma(acc_u, x[u], F.coef[c + u * G]);
+                    }
+                }
+                for (; c + 3 * G < nt; c += 4 * G) {
+                    const Cx<T> x0 = ldcx(A.pool + col[c] + v), x1 = ldcx(A.pool + col[c + G] + v);
+                    const Cx<T> x2 = ldcx(A.pool + col[c + 2 * G] + v), x3 = ldcx(A.pool + col[c + 3 * G] + v);
+                    if (ROW) {
+                        cfmac(s0, F.coef[c], x0);
+                        cfmac(s1, F.coef[c + G], x1);
+                        cfmac(s2, F.coef[c + 2 * G], x2);
+                        cfmac(s3, F.coef[c + 3 * G], x3);
+                    } else {
+                        cfma(s0, x0, F.coef[c]);
+                        cfma(s1, x1, F.coef[c + G]);
+                        cfma(s2, x2, F.coef[c + 2 * G]);
+                        cfma(s3, x3, F.coef[c + 3 * G]);
+                    }
+                }
+                for (; c < nt; c += G) {
+                    const Cx<T> x0 = ldcx(A.pool + col[c] + v);
+                    if (ROW) cfmac(s0, F.coef[c], x0);
+                    else cfma(s0, x0, F.coef[c]);
+                }
+}
+
 // Residual of one row (ROW: fixed row `fix`, all columns) or one column (!ROW:
 // fixed column `fix`, all rows) of the face at kf:
 //   ENTRY - sum_p f_p[kf] (U_p V_p^H) - sum_{t<m} u_t v_t^H
@@ -503,18 +567,15 @@ __device__ void line_coeffs(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, 
 // independent partial sums) and the quadrature points.  Returns the
 // block-wide argmax of |out|^2 (ROW: over all columns; !ROW: over the rows
 // not yet used).
-constexpr int LIF = 16;  // loads in flight per thread in the residual lines' sums
-
 template <int KER, class T, int NT, bool ROW>
 __device__ ArgMaxT<T> residual_line(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, const FaceTab<T>& F,
-                                    int fix, int kf, int m, Cx<T>* out, const Cx<T>* D) {
+                                    int fix, int kf, int m, Cx<T>* out) {
     const int tid = threadIdx.x;
     const int M = S.M, N = S.N;
     const int L = ROW ? N : M;
     const int G = gang_size<NT>(L);
     const int per = NT / G;
     const int part = tid % G;
-    const long long* col = ROW ? F.colV : F.colU;
     const Cx<T>* cur = ROW ? w.vw : w.uw;
     const size_t ldc = ROW ? A.Nmax : A.Mmax;
     const int nt = F.ncol;
@@ -523,60 +584,12 @@ __device__ ArgMaxT<T> residual_line(const AcaArgs<T>& A, const Ws<T>& w, BlockSh
         const int v = base + tid / G;
         Cx<T> acc{0, 0};
         if (v < L) {
-            if (D) {
-                // the dense residual working face holds ENTRY minus the earlier crosses
-                if (part == 0) acc = ldcx(D + (ROW ? (size_t)fix * N + v : (size_t)v * N + fix));
-            } else {
-                const int gi = S.rb + (ROW ? fix : v), gj = S.cb + (ROW ? v : fix);
-                const long long te = tid == 0 ? clock64() : 0;
-                acc = ent_part<KER, T>(A, gi, gj, kf, part, G);
-                if (tid == 0) S.sub[10] += clock64() - te;
-            }
+            const int gi = S.rb + (ROW ? fix : v), gj = S.cb + (ROW ? v : fix);
+            const long long te = tid == 0 ? clock64() : 0;
+            acc = ent_part<KER, T>(A, gi, gj, kf, part, G);
+            if (tid == 0) S.sub[10] += clock64() - te;
             Cx<T> s0{0, 0}, s1{0, 0}, s2{0, 0}, s3{0, 0};
-            int c = part;
-            // LIF loads in flight per thread (the sums wait on memory, not on arithmetic)
-            for (; c + (LIF - 1) * G < nt; c += LIF * G) {
-                Cx<T> x[LIF];
-#pragma unroll
-                for (int u = 0; u < LIF; ++u) x[u] = ldcx(A.pool + col[c + u * G] + v);
-#pragma unroll
-                for (int u = 0; u < LIF; ++u) {
-                    Cx<T>& acc_u = (u & 3) == 0 ? s0 : (u & 3) == 1 ? s1 : (u & 3) == 2 ? s2 : s3;
-                    if (ROW) cfmac(acc_u, F.coef[c + u * G], x[u]);
-                    else cfma(acc_u, x[u], F.coef[c + u * G]);
-                }
-            }
-            for (; c + 7 * G < nt; c += 8 * G) {
-                Cx<T> x[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) x[u] = ldcx(A.pool + col[c + u * G] + v);
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    Cx<T>& acc_u = (u & 3) == 0 ? s0 : (u & 3) == 1 ? s1 : (u & 3) == 2 ? s2 : s3;
-                    if (ROW) cfmac(acc_u, F.coef[c + u * G], x[u]);
-                    else cfma(acc_u, x[u], F.coef[c + u * G]);
-                }
-            }
-            for (; c + 3 * G < nt; c += 4 * G) {
-                const Cx<T> x0 = ldcx(A.pool + col[c] + v), x1 = ldcx(A.pool + col[c + G] + v);
-                const Cx<T> x2 = ldcx(A.pool + col[c + 2 * G] + v), x3 = ldcx(A.pool + col[c + 3 * G] + v);
-                if (ROW) {
-                    cfmac(s0, F.coef[c], x0);
-                    cfmac(s1, F.coef[c + G], x1);
-                    cfmac(s2, F.coef[c + 2 * G], x2);
-                    cfmac(s3, F.coef[c + 3 * G], x3);
-                } else {
-                    cfma(s0, x0, F.coef[c]);
-                    cfma(s1, x1, F.coef[c + G]);
-                    cfma(s2, x2, F.coef[c + 2 * G]);
-                    cfma(s3, x3, F.coef[c + 3 * G]);
-                }
-            }
-            for (; c < nt; c += G) {
-                const Cx<T> x0 = ldcx(A.pool + col[c] + v);
-                if (ROW) cfmac(s0, F.coef[c], x0);
-                else cfma(s0, x0, F.coef[c]);
-            }
+            cross_sum<T, ROW>(A, F, v, part, G, s0, s1, s2, s3);
             int t = part;
             for (; t + G < m; t += 2 * G) {
                 const Cx<T> x0 = ldcx(cur + (size_t)t * ldc + v), x1 = ldcx(cur + (size_t)(t + G) * ldc + v);
@@ -616,7 +629,7 @@ __device__ ArgMaxT<T> residual_line(const AcaArgs<T>& A, const Ws<T>& w, BlockSh
 // columns of the earlier crosses.  Writes |R_s|^2 to S.samp.
 template <int KER, class T, int NT>
 __device__ void face_samples(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, const FaceTab<T>& F, int kf,
-                             int m, const Cx<T>* D) {
+                             int m) {
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int M = S.M, N = S.N;
     for (int sm = wid; sm < SAMPLES; sm += NT / 32) {
@@ -630,7 +643,7 @@ __device__ void face_samples(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S,
         acc.x = warp_sum(acc.x);
         acc.y = warp_sum(acc.y);
         if (lane == 0) {
-            const Cx<T> e = D ? D[(size_t)i * N + j] : ent<KER, T>(A, S.rb + i, S.cb + j, kf);
+            const Cx<T> e = ent<KER, T>(A, S.rb + i, S.cb + j, kf);
             S.samp[sm] = cabs2d(Cx<T>{e.x - acc.x, e.y - acc.y});
         }
     }
@@ -870,18 +883,6 @@ __device__ int face_aca(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, int 
     FaceTab<T> F = facetab_build<T, NT>(A, w, S, arena);
     for (int i = tid; i < M; i += NT) w.used[i] = 0;
     __syncthreads();
-    // dense residual working face (float32, blocks up to drf_max entries): ENTRY
-    // minus the earlier crosses evaluated for the whole face at once; the lines
-    // below then subtract only the current face's crosses
-    const Cx<T>* D = nullptr;
-    if constexpr (sizeof(T) == 4 && KER != G3_SEPARABLE) {
-        if (w.dres && (long long)M * N <= A.drf_max) {
-            face_dense_residual<KER, T, NT>(A, w, S, F, kf, arena);
-            D = w.dres;
-            F.ncol = 0;
-            sublap(S, 11, tf);
-        }
-    }
     if (tid == 0) S.fsn2 = 0.0;
     int m = 0;
     int irow = 0;
@@ -897,7 +898,7 @@ __device__ int face_aca(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, int 
             sublap(S, 5, tf);
             line_coeffs<T, NT, true>(A, w, S, F, irow, m);
             __syncthreads();
-            ArgMaxT<T> am = residual_line<KER, T, NT, true>(A, w, S, F, irow, kf, m, F.row, D);
+            ArgMaxT<T> am = residual_line<KER, T, NT, true>(A, w, S, F, irow, kf, m, F.row);
             if (tid == 0) w.used[irow] = 1;
             // a row counts as nonzero when |delta|^2 is a normal number of the
             // working precision (below that the entries are far under any tolerance)
@@ -935,7 +936,7 @@ __device__ int face_aca(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, int 
         // residual column jp = u_m; the argmax over unused rows of |u_m| is the next row
         Cx<T>* um = w.uw + (size_t)m * A.Mmax;
         sublap(S, 6, tf);
-        ArgMaxT<T> nx = residual_line<KER, T, NT, false>(A, w, S, F, jp, kf, m, um, D);
+        ArgMaxT<T> nx = residual_line<KER, T, NT, false>(A, w, S, F, jp, kf, m, um);
         sublap(S, 7, tf);
         // recursive Frobenius norm of the face approximant:
         // ||S_m||^2 = ||S_{m-1}||^2 + 2 Re sum_t (u_t^H u_m)(v_m^H v_t) + ||u_m||^2 ||v_m||^2
@@ -982,7 +983,7 @@ __device__ int face_aca(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, int 
             }
             // confirm on the sample entries: partial pivoting can miss a block
             // of the face that no visited row or column reaches
-            face_samples<KER, T, NT>(A, w, S, F, kf, m, D);
+            face_samples<KER, T, NT>(A, w, S, F, kf, m);
             sublap(S, 9, tf);
             static_assert(SAMPLES == 32, "one sample per lane");
             if (wid == 0) {
@@ -1084,7 +1085,7 @@ __device__ __forceinline__ double rsqrt_pivot(double x) {
     return y * (1.5 - 0.5 * x * y * y);
 }
 
-// ---- recompression: Cholesky-QR + one-sided Jacobi SVD ---------------------------------
+// ---- recompression (float64): Cholesky-QR + one-sided Jacobi SVD -------------------------
 // Input uw, vw (r columns).  Output: the rank r' and the transforms T_U, T_V
 // (r x r', complex T, row-major with stride *ldT) such that U' = uw T_U,
 // V' = vw T_V.  For any invertible triangular R used consistently,
@@ -1100,8 +1101,6 @@ constexpr int RS = 32;
 
 template <class T>
 __device__ __forceinline__ T jacobi_tol();
-template <>
-__device__ __forceinline__ float jacobi_tol<float>() { return 1e-3f; }
 template <>
 __device__ __forceinline__ double jacobi_tol<double>() { return 1e-12; }
 
@@ -1215,86 +1214,6 @@ __device__ int jacobi_core(const AcaArgs<T>& A, BlockSh<T>& S, Cx<T>* shB, Cx<T>
     return rn;
 }
 
-// Column-pivoted QR of the r x r core C (columns of B) by modified
-// Gram-Schmidt (see the caller).  On return B[:, sel[k]] = q_k and
-// J[:, sel[k]] = (Pi R^H)[:, k] in the original column order, k < rank.
-template <class T, int NT>
-__device__ int cpqr_core(const AcaArgs<T>& A, BlockSh<T>& S, Cx<T>* shB, Cx<T>* shJ, int ld, int r) {
-    const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
-    constexpr int NW = NT / 32;
-    T* cn = reinterpret_cast<T*>(S.sig);     // squared column norms, -1 once used
-    for (int c = wid; c < r; c += NW) {
-        T s2 = 0;
-        for (int i = lane; i < r; i += 32) s2 += cabs2(shB[c * ld + i]);
-        s2 = warp_sum(s2);
-        if (lane == 0) cn[c] = s2;
-    }
-    for (int e = tid; e < r * r; e += NT) shJ[(e / r) * ld + (e % r)] = Cx<T>{0, 0};
-    __syncthreads();
-    const double sfloor = A.trunc_floor * sqrt(S.norm2 / (double)A.Ku);
-    float r00 = 0.f;
-    int k = 0;
-    for (; k < r; ++k) {
-        if (wid == 0) {
-            ArgMaxT<T> best = amax_none<T>();
-            for (int c = lane; c < r; c += 32)
-                if (cn[c] >= (T)0) best = amax_better(best, ArgMaxT<T>{cn[c], c});
-            best = warp_argmax(best);
-            const int pv = best.i;
-            T s2 = 0;
-            if (best.v >= (T)0 && pv >= 0 && pv < r)
-                for (int i = lane; i < r; i += 32) s2 += cabs2(shB[pv * ld + i]);
-            s2 = warp_sum(s2);
-            if (lane == 0) {
-                S.piv = (best.v >= (T)0 && pv >= 0 && pv < r) ? pv : -1;
-                S.rkk = sqrt(s2);
-                if (S.piv >= 0) cn[pv] = (T)-1;
-            }
-        }
-        __syncthreads();
-        const int pv = S.piv;
-        const float rkk = S.rkk;
-        if (k == 0) r00 = rkk;
-        if (pv < 0 || !(rkk > 0.f) || !isfinite(rkk) || rkk < (float)A.eps_face * r00 ||
-            (k > 0 && (double)rkk < sfloor))
-            break;
-        const T inv = (T)1 / (T)rkk;
-        const Cx<T>* q = shB + pv * ld;
-        if (tid == 0) {
-            S.sel[k] = pv;
-            shJ[pv * ld + pv] = Cx<T>{(T)rkk, (T)0};
-        }
-        for (int j = wid; j < r; j += NW) {
-            if (!(cn[j] >= (T)0)) continue;  // used (or the pivot)
-            Cx<T>* cj = shB + j * ld;
-            Cx<T> g{0, 0};
-            for (int i = lane; i < r; i += 32) cfmac(g, cj[i], q[i]);  // conj(q) c_j, q unscaled
-            g.x = warp_sum(g.x) * inv;
-            g.y = warp_sum(g.y) * inv;
-            for (int i = lane; i < r; i += 32) {
-                const Cx<T> qi{q[i].x * inv, q[i].y * inv};
-                cj[i].x -= qi.x * g.x - qi.y * g.y;
-                cj[i].y -= qi.x * g.y + qi.y * g.x;
-            }
-            if (lane == 0) {
-                shJ[pv * ld + j] = Cx<T>{g.x, -g.y};  // conj(R[k][j])
-                cn[j] = fmax(cn[j] - cabs2(g), (T)0);
-            }
-        }
-        __syncthreads();
-    }
-    // scale the pivot columns to q (their norms rkk sit on J's diagonal)
-    for (int e = tid; e < k * r; e += NT) {
-        const int b = e / r, i = e - b * r;
-        const int pv = S.sel[b];
-        const T inv = (T)1 / shJ[pv * ld + pv].x;
-        shB[pv * ld + i].x *= inv;
-        shB[pv * ld + i].y *= inv;
-    }
-    __syncthreads();
-    return k;
-}
-
 template <class T, int NT>
 __device__ int recompress(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, int r, Cx<double>* smem,
                           const Cx<T>** tUo, const Cx<T>** tVo, int* ldTo) {
@@ -1374,28 +1293,6 @@ __device__ int recompress(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, in
     }
     sublap(S, 1, tc);
     if (S.flag) return -1;
-    // working-precision copies of Rhat_U, Rhat_V (upper triangles) and of the
-    // scalings for the back substitution (float32: after the two r x r float64
-    // matrices and B, J in shared memory, or in the workspace's T_V block)
-    Cx<T>* RUf = small ? reinterpret_cast<Cx<T>*>(smem + 2 * RS * RS) + 2 * RS * RS : reinterpret_cast<Cx<T>*>(w.TV);
-    Cx<T>* RVf = RUf + (small ? RS * RS : A.RF * A.RF);
-    if constexpr (sizeof(T) == 4) {
-        for (int e = tid; e < 2 * r * r; e += NT) {
-            const int mtx = e / (r * r), q = e - mtx * r * r, a = q / r, c = q - a * r;
-            if (c < a) continue;
-            (mtx == 0 ? RUf : RVf)[a * ld + c] = ccast<T>((mtx == 0 ? RU : RV)[a * ld + c]);
-        }
-        for (int e = tid; e < 2 * r; e += NT) {
-            const int a = e < r ? e : e - r;
-            if (e < r) {
-                S.tdU[a] = (T)S.dU[a];
-                S.trdU[a] = (T)S.rdU[a];
-            } else {
-                S.tdV[a] = (T)S.dV[a];
-                S.trdV[a] = (T)S.rdV[a];
-            }
-        }
-    }
     // core C = R_U R_V^H with R_U = Rhat_U diag(1/dU): C[a][b] = sum_{c >= max(a,b)}
     //   RhatU[a][c] conj(RhatV[b][c]) / (dU[c] dV[c]); stored column-major in B, J = I
     double* isc = S.sig;  // 1 / (dU[c] dV[c]); S.sig is free until the core is factored
@@ -1415,53 +1312,11 @@ __device__ int recompress(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, in
     }
     __syncthreads();
     sublap(S, 2, tc);
-    int rn = 0;
-    if constexpr (sizeof(T) == 4) {
-        // float32: column-pivoted QR of C by modified Gram-Schmidt, C Pi = Q R,
-        // stopped when the largest remaining column norm falls below the
-        // truncation threshold; dropping the remaining columns removes exactly
-        // their norms (||R_22||_F), as truncating the SVD removes its dropped
-        // singular values.  Step k (two barriers): warp 0 picks the unused
-        // column of largest (downdated) norm and recomputes its norm exactly;
-        // then every other unused column j is orthogonalised against it by a
-        // warp (g = q^H c_j, c_j -= q g) and J[:, pivot][j] = conj(g), which
-        // builds Pi R^H column by column.  The pivot columns are scaled to q
-        // at the end; sel[k] = pivot of step k.
-        rn = cpqr_core<T, NT>(A, S, shB, shJ, ld, r);
-        if (rn < 0) return -1;
-    } else {
-        rn = jacobi_core<T, NT>(A, S, shB, shJ, ld, r);
-        if (rn < 0) return -1;
-    }
+    const int rn = jacobi_core<T, NT>(A, S, shB, shJ, ld, r);
+    if (rn < 0) return -1;
     sublap(S, 3, tc);
     // T_U[:, b] = diag(dU) RhatU^{-1} B[:, sel[b]],  T_V[:, b] = diag(dV) RhatV^{-1} J[:, sel[b]]
-    // in place on the selected columns.  float32: in the working precision (the
-    // columns of B and J are held in it already, so the solve's forward error
-    // is of the order cond(Rhat) u either way); float64: in float64.
-    if constexpr (sizeof(T) == 4) {
-        for (int item = tid; item < 2 * rn; item += NT) {
-            const bool isU = item < rn;
-            const int b = isU ? item : item - rn;
-            const Cx<T>* R = isU ? RUf : RVf;
-            Cx<T>* z = (isU ? shB : shJ) + S.sel[b] * ld;
-            const T* dsc = isU ? S.tdU : S.tdV;
-            const T* rdg = isU ? S.trdU : S.trdV;
-            for (int a = r - 1; a >= 0; --a) {
-                Cx<T> acc = z[a];
-                for (int c = a + 1; c < r; ++c) {
-                    const Cx<T> rr = R[a * ld + c], zc = z[c];
-                    acc.x -= rr.x * zc.x - rr.y * zc.y;
-                    acc.y -= rr.x * zc.y + rr.y * zc.x;
-                }
-                const T rd = rdg[a];
-                z[a] = Cx<T>{acc.x * rd, acc.y * rd};
-            }
-            for (int a = 0; a < r; ++a) {
-                z[a].x *= dsc[a];
-                z[a].y *= dsc[a];
-            }
-        }
-    } else
+    // in place on the selected columns
     for (int item = tid; item < 2 * rn; item += NT) {
         const bool isU = item < rn;
         const int b = isU ? item : item - rn;
@@ -1500,6 +1355,99 @@ __device__ int recompress(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, in
     *tVo = tV;
     *ldTo = ld;
     return rn;
+}
+
+}  // namespace g3
+
+#include "g3_face32.cuh"
+
+namespace g3 {
+
+// ---- face, recompression and formation of U', V' by working precision --------------------
+// float32: columns and recompression in shared memory (g3_face32.cuh); float64:
+// columns in the workspace, Cholesky-QR and Jacobi SVD.
+struct NoCols {};
+template <class T>
+struct FaceForm {
+    const Cx<T>* tU = nullptr;
+    const Cx<T>* tV = nullptr;
+    int ldT = 0;
+};
+template <>
+struct FaceForm<float> {
+    Recomp32 p;
+};
+template <class T>
+struct FaceColsOf {
+    using type = NoCols;
+};
+template <>
+struct FaceColsOf<float> {
+    using type = ColStore;
+};
+template <class T>
+using FaceCols = typename FaceColsOf<T>::type;
+
+template <int KER, class T, int NT>
+__device__ __forceinline__ int face_of(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, int kf,
+                                       unsigned char* arena, FaceCols<T>& cs) {
+    if constexpr (sizeof(T) == 4) return face32<KER, NT>(A, w, S, kf, arena, cs);
+    else return face_aca<KER, T, NT>(A, w, S, kf, arena);
+}
+
+// the kept rank, or -1 (raw factors: recompression off or broken down)
+template <class T, int NT>
+__device__ __forceinline__ int recompress_of(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, int r,
+                                             const FaceCols<T>& cs, FaceForm<T>& ff, unsigned char* arena) {
+    if (A.no_recompress) return -1;
+    if constexpr (sizeof(T) == 4) {
+        ff.p = recomp32_place(A, w, cs, r, arena);
+        return recompress32<NT>(A, S, cs, r, ff.p, arena);
+    } else {
+        const int rn = recompress<T, NT>(A, w, S, r, reinterpret_cast<Cx<double>*>(arena), &ff.tU, &ff.tV, &ff.ldT);
+        if (rn < 0 && threadIdx.x == 0) {
+            atomicOr(A.status, ST_CHOL_FALLBACK);
+            atomicAdd(&A.counters[4], 1ull);
+        }
+        return rn;
+    }
+}
+
+template <class T, int NT>
+__device__ __forceinline__ void form_of(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, int r, int rn, bool raw,
+                                        const FaceCols<T>& cs, const FaceForm<T>& ff, Cx<T>* Un, Cx<T>* Vn) {
+    if constexpr (sizeof(T) == 4) {
+        form32<NT>(S, cs, r, rn, raw, ff.p, Un, Vn);
+    } else {
+        const int tid = threadIdx.x, M = S.M, N = S.N;
+        if (raw) {
+            for (int e = tid; e < rn * M; e += NT) Un[e] = w.uw[(size_t)(e / M) * A.Mmax + e % M];
+            for (int e = tid; e < rn * N; e += NT) Vn[e] = w.vw[(size_t)(e / N) * A.Nmax + e % N];
+            return;
+        }
+        // U' = uw T_U, V' = vw T_V in the working precision, 8 output columns per pass
+        for (int e = tid; e < (M + N) * ((rn + 7) / 8); e += NT) {
+            const int row = e % (M + N), b0 = (e / (M + N)) * 8;
+            const bool isU = row < M;
+            const int i = isU ? row : row - M;
+            const Cx<T>* src = isU ? w.uw + i : w.vw + i;
+            const size_t ld = isU ? A.Mmax : A.Nmax;
+            const Cx<T>* Tm = isU ? ff.tU : ff.tV;
+            Cx<T> acc[8];
+#pragma unroll
+            for (int bb = 0; bb < 8; ++bb) acc[bb] = Cx<T>{0, 0};
+            for (int a = 0; a < r; ++a) {
+                const Cx<T> u = src[(size_t)a * ld];
+#pragma unroll
+                for (int bb = 0; bb < 8; ++bb) cfma(acc[bb], u, Tm[a * ff.ldT + min(b0 + bb, rn - 1)]);
+            }
+            Cx<T>* dst = isU ? Un + i : Vn + i;
+            const long long L = isU ? M : N;
+#pragma unroll
+            for (int bb = 0; bb < 8; ++bb)
+                if (b0 + bb < rn) dst[(long long)(b0 + bb) * L] = acc[bb];
+        }
+    }
 }
 
 // ---- eq. (norm) inner products ------------------------------------------------------------
@@ -1916,7 +1864,6 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3(const AcaArgs<T
     __shared__ AcaArgs<T> Ash;
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
     const int RF = P.RF;
-    Cx<double>* shB = reinterpret_cast<Cx<double>*>(smem_raw);  // arena base
     const Ws<T> w = ws_carve<T>(P.ws + (size_t)blockIdx.x * P.ws_stride, RF, P.Mmax, P.Nmax, P.Cmax, P.Ku,
                                 P.drf_max > 0 ? P.drf_off : 0);
     __shared__ int s_q;
@@ -1991,7 +1938,8 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3(const AcaArgs<T
         while (!overflow) {
             // ---------------- face at S.k ----------------
             int kf = S.k;
-            int r = face_aca<KER, T, NT>(A, w, S, kf, smem_raw);
+            FaceCols<T> cs;
+            int r = face_of<KER, T, NT>(A, w, S, kf, smem_raw, cs);
             if (tid == 0) S.used_k[kf >> 5] |= 1u << (kf & 31);
             __syncthreads();
             if (r == 0) {
@@ -2008,7 +1956,7 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3(const AcaArgs<T
                     __syncthreads();
                     if (tid == 0) S.used_k[kk >> 5] |= 1u << (kk & 31);
                     __syncthreads();
-                    r = face_aca<KER, T, NT>(A, w, S, kk, smem_raw);
+                    r = face_of<KER, T, NT>(A, w, S, kk, smem_raw, cs);
                     if (r > 0) {
                         found = true;
                         kf = kk;
@@ -2024,17 +1972,8 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3(const AcaArgs<T
             ++computed;
             lap(0);
             // ---------------- recompression ----------------
-            int rn = -1;
-            const Cx<T>* tU = nullptr;
-            const Cx<T>* tV = nullptr;
-            int ldT = 0;
-            if (!A.no_recompress) {
-                rn = recompress<T, NT>(A, w, S, r, shB, &tU, &tV, &ldT);
-                if (rn < 0 && tid == 0) {
-                    atomicOr(A.status, ST_CHOL_FALLBACK);
-                    atomicAdd(&A.counters[4], 1ull);
-                }
-            }
+            FaceForm<T> ff;
+            int rn = recompress_of<T, NT>(A, w, S, r, cs, ff, smem_raw);
             const bool raw = rn < 0;
             if (raw) rn = r;
             lap(1);
@@ -2059,33 +1998,7 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3(const AcaArgs<T
             Cx<T>* Un = A.pool + off;
             Cx<T>* Vn = A.pool + off + (long long)rn * M;
             Cx<T>* Fn = A.pool + off + (long long)rn * (M + N);
-            if (raw) {
-                for (int e = tid; e < rn * M; e += NT) Un[e] = w.uw[(size_t)(e / M) * A.Mmax + e % M];
-                for (int e = tid; e < rn * N; e += NT) Vn[e] = w.vw[(size_t)(e / N) * A.Nmax + e % N];
-            } else {
-                // U' = uw T_U, V' = vw T_V in the working precision, 8 output columns per pass
-                for (int e = tid; e < (M + N) * ((rn + 7) / 8); e += NT) {
-                    const int row = e % (M + N), b0 = (e / (M + N)) * 8;
-                    const bool isU = row < M;
-                    const int i = isU ? row : row - M;
-                    const Cx<T>* src = isU ? w.uw + i : w.vw + i;
-                    const size_t ld = isU ? A.Mmax : A.Nmax;
-                    const Cx<T>* Tm = isU ? tU : tV;
-                    Cx<T> acc[8];
-#pragma unroll
-                    for (int bb = 0; bb < 8; ++bb) acc[bb] = Cx<T>{0, 0};
-                    for (int a = 0; a < r; ++a) {
-                        const Cx<T> u = src[(size_t)a * ld];
-#pragma unroll
-                        for (int bb = 0; bb < 8; ++bb) cfma(acc[bb], u, Tm[a * ldT + min(b0 + bb, rn - 1)]);
-                    }
-                    Cx<T>* dst = isU ? Un + i : Vn + i;
-                    const long long L = isU ? M : N;
-#pragma unroll
-                    for (int bb = 0; bb < 8; ++bb)
-                        if (b0 + bb < rn) dst[(long long)(b0 + bb) * L] = acc[bb];
-                }
-            }
+            form_of<T, NT>(A, w, S, r, rn, raw, cs, ff, Un, Vn);
             __syncthreads();
             lap(2);
             // ---------------- pivot: argmax |U' V'^H| ----------------
@@ -2372,7 +2285,6 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3_face(const AcaA
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
     const AcaArgs<T>& A = P;
     const int RF = A.RF;
-    Cx<double>* shB = reinterpret_cast<Cx<double>*>(smem_raw);
     const Ws<T> w = ws_carve<T>(A.ws + (size_t)blockIdx.x * A.ws_stride, RF, A.Mmax, A.Nmax, A.Cmax, A.Ku);
     for (;;) {
         if (tid == 0) {
@@ -2408,14 +2320,13 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3_face(const AcaA
         __syncthreads();
         const int M = S.M, N = S.N;
         bool ok = M <= A.Mmax && N <= A.Nmax;
-        int r = ok ? face_aca<KER, T, NT>(A, w, S, kf, smem_raw) : 0;
+        FaceCols<T> cs;
+        FaceForm<T> ff;
+        int r = ok ? face_of<KER, T, NT>(A, w, S, kf, smem_raw, cs) : 0;
         int rn = 0;
-        const Cx<T>* tU = nullptr;
-        const Cx<T>* tV = nullptr;
-        int ldT = 0;
         bool raw = false;
         if (r > 0) {
-            rn = A.no_recompress ? -1 : recompress<T, NT>(A, w, S, r, shB, &tU, &tV, &ldT);
+            rn = recompress_of<T, NT>(A, w, S, r, cs, ff, smem_raw);
             raw = rn < 0;
             if (raw) rn = r;
         }
@@ -2444,24 +2355,7 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3_face(const AcaA
         }
         Cx<T>* Un = A.pool + off;
         Cx<T>* Vn = A.pool + off + (long long)rn * M;
-        if (rn > 0) {
-            if (raw) {
-                for (int e = tid; e < rn * M; e += NT) Un[e] = w.uw[(size_t)(e / M) * A.Mmax + e % M];
-                for (int e = tid; e < rn * N; e += NT) Vn[e] = w.vw[(size_t)(e / N) * A.Nmax + e % N];
-            } else {
-                for (int e = tid; e < (M + N) * rn; e += NT) {
-                    const int row = e % (M + N), b = e / (M + N);
-                    const bool isU = row < M;
-                    const int i = isU ? row : row - M;
-                    const Cx<T>* src = isU ? w.uw + i : w.vw + i;
-                    const size_t ld = isU ? A.Mmax : A.Nmax;
-                    const Cx<T>* Tm = isU ? tU : tV;
-                    Cx<T> acc{0, 0};
-                    for (int a = 0; a < r; ++a) cfma(acc, src[(size_t)a * ld], Tm[a * ldT + b]);
-                    (isU ? Un + i : Vn + i)[(long long)b * (isU ? M : N)] = acc;
-                }
-            }
-        }
+        if (rn > 0) form_of<T, NT>(A, w, S, r, rn, raw, cs, ff, Un, Vn);
         __syncthreads();
         // the block's largest face entry: dense expansion of U' V'^H, one
         // entry per thread and pass (ties to the smallest row-major index)

@@ -1,0 +1,699 @@
+#pragma once
+// Float32 faces of the three-way ACA: the partial-pivot ACA of one residual
+// face and its recompression, with the face's columns in shared memory.
+//
+// Included by g3_aca_dev.cuh (which defines the block state, the line helpers
+// and the dense residual working face) and used by the float32 kernels only.
+//
+// A face of a 192 x 192 block takes 20 to 40 ACA steps, and every step walks
+// all earlier columns three times (row, column, norm).  With the columns in
+// the global workspace each of those walks is a chain of L2 round trips
+// (~25,000 SM cycles per step, measured); in shared memory it is a few hundred
+// cycles of multiply-adds, so a step costs two barriers and the latency of one
+// row and one column of the dense residual working face.
+
+namespace g3 {
+
+// Columns of the face: column t holds u_t (M values) and then v_t (N values).
+// The first ncs columns live in shared memory, the others (faces of higher
+// rank than the arena holds) in the CTA's workspace.  ld is 4 modulo 16, so
+// that the parts of a gang, which read columns t, t + 1, .. at the same
+// element, fall in different banks.
+struct ColStore {
+    Cx<float>* sm;
+    Cx<float>* gm;
+    int ncs, ld, M;
+};
+template <bool SM>
+__device__ __forceinline__ Cx<float>* cs_u(const ColStore& c, int t) {
+    if constexpr (SM) return c.sm + t * c.ld;
+    else return t < c.ncs ? c.sm + t * c.ld : c.gm + (size_t)t * c.ld;
+}
+template <bool SM>
+__device__ __forceinline__ Cx<float>* cs_v(const ColStore& c, int t) {
+    return cs_u<SM>(c, t) + c.M;
+}
+__host__ __device__ inline int cs_ld(int M, int N) {
+    const int l = M + N;
+    return l + ((4 - l) & 15);   // <= M + N + CS_PAD - 1
+}
+
+// float-float accumulation (two-sum): the squared norms of the face test keep
+// about 48 bits without the float64 pipe
+__device__ __forceinline__ void ff_add(float2& a, float hi, float lo) {
+    const float s = a.x + hi, bb = s - a.x;
+    const float e = (a.x - (s - bb)) + (hi - bb);
+    const float l = a.y + lo + e;
+    a.x = s + l;
+    a.y = l - (a.x - s);
+}
+__device__ __forceinline__ void ff_add_prod(float2& a, float x, float y) {
+    const float p = x * y;
+    ff_add(a, p, fmaf(x, y, -p));
+}
+
+// warp argmax of non-negative float32 values, ties to the smallest index:
+// {value bits + 1 (0: no candidate), index}
+__device__ __forceinline__ uint2 warp_key(ArgMaxT<float> a) {
+    const unsigned enc = a.v >= 0.f ? __float_as_uint(a.v + 0.f) + 1u : 0u;
+    const unsigned mx = __reduce_max_sync(0xffffffffu, enc);
+    const unsigned ix = __reduce_min_sync(0xffffffffu, enc == mx ? (unsigned)a.i : 0xffffffffu);
+    return make_uint2(mx, ix);
+}
+// the block's candidate from its warps' (after a barrier)
+template <int NT>
+__device__ __forceinline__ ArgMaxT<float> block_key(const uint2* k) {
+    uint2 b = k[0];
+#pragma unroll
+    for (int w = 1; w < NT / 32; ++w) {
+        const uint2 y = k[w];
+        if (y.x > b.x || (y.x == b.x && y.y < b.y)) b = y;
+    }
+    if (b.x == 0u) return amax_none<float>();
+    return ArgMaxT<float>{__uint_as_float(b.x - 1u), (int)b.y};
+}
+
+// the part of a gang in sum_t u_t[fix] conj(v_t[v]) (ROW) or
+// sum_t u_t[v] conj(v_t[fix]) over the face's columns t < m
+template <bool ROW>
+__device__ __forceinline__ Cx<float> cur_sum(const ColStore& c, int fix, int v, int m, int part, int G) {
+    Cx<float> s0{0, 0}, s1{0, 0}, s2{0, 0}, s3{0, 0};
+    const int ou = ROW ? fix : v, ov = c.M + (ROW ? v : fix);
+    const int ms = min(m, c.ncs);
+    int t = part;
+    for (; t + 3 * G < ms; t += 4 * G) {
+        const Cx<float>* p = c.sm + t * c.ld;
+        const int st = G * c.ld;
+        const Cx<float> a0 = ldcx(p + ou), a1 = ldcx(p + st + ou), a2 = ldcx(p + 2 * st + ou), a3 = ldcx(p + 3 * st + ou);
+        const Cx<float> b0 = ldcx(p + ov), b1 = ldcx(p + st + ov), b2 = ldcx(p + 2 * st + ov), b3 = ldcx(p + 3 * st + ov);
+        cfmac(s0, a0, b0);
+        cfmac(s1, a1, b1);
+        cfmac(s2, a2, b2);
+        cfmac(s3, a3, b3);
+    }
+    for (; t < ms; t += G) {
+        const Cx<float>* p = c.sm + t * c.ld;
+        cfmac(s0, ldcx(p + ou), ldcx(p + ov));
+    }
+    for (; t < m; t += G) {  // columns beyond the arena
+        const Cx<float>* p = c.gm + (size_t)t * c.ld;
+        cfmac(s1, ldcx(p + ou), ldcx(p + ov));
+    }
+    return Cx<float>{(s0.x + s1.x) + (s2.x + s3.x), (s0.y + s1.y) + (s2.y + s3.y)};
+}
+
+// One residual row (ROW: fixed row `fix`) or column of the face:
+//   ENTRY - sum_p f_p[kf] (U_p V_p^H) - sum_{t<m} u_t v_t^H
+// read from the dense residual working face D (which holds the first two
+// terms), or evaluated with the earlier crosses' tables.  G threads share an
+// element.  Writes the line to out and returns the thread's largest |.|^2
+// (columns: over the rows not yet used, `skip` being used too).
+template <int KER, int NT, bool ROW>
+__device__ __forceinline__ ArgMaxT<float> line32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float>& S,
+                                                 const FaceTab<float>& F, const ColStore& c, int fix, int skip, int kf,
+                                                 int m, Cx<float>* out, const Cx<float>* D) {
+    const int tid = threadIdx.x;
+    const int M = S.M, N = S.N;
+    const int L = ROW ? N : M;
+    // D: one pass over the line where it fits; else as many passes as the
+    // entries and tables want (gang_size)
+    const int G = D ? (L * 4 <= NT ? 4 : (L * 2 <= NT ? 2 : 1)) : gang_size<NT>(L);
+    const int per = NT / G, part = tid % G;
+    ArgMaxT<float> am = amax_none<float>();
+    for (int base = 0; base < L; base += per) {
+        const int v = base + tid / G;
+        Cx<float> acc{0, 0};
+        bool cand = false;
+        if (v < L) {
+            if (D) {
+                if (part == 0) acc = ldcx(D + (ROW ? (size_t)fix * N + v : (size_t)v * N + fix));
+            } else {
+                const long long te = tid == 0 ? clock64() : 0;
+                acc = ent_part<KER, float>(A, S.rb + (ROW ? fix : v), S.cb + (ROW ? v : fix), kf, part, G);
+                if (tid == 0) S.sub[10] += clock64() - te;
+                Cx<float> s0{0, 0}, s1{0, 0}, s2{0, 0}, s3{0, 0};
+                cross_sum<float, ROW>(A, F, v, part, G, s0, s1, s2, s3);
+                acc.x -= (s0.x + s1.x) + (s2.x + s3.x);
+                acc.y -= (s0.y + s1.y) + (s2.y + s3.y);
+            }
+            cand = part == 0 && (ROW || (v != skip && !w.used[v]));
+            const Cx<float> q = cur_sum<ROW>(c, fix, v, m, part, G);
+            acc.x -= q.x;
+            acc.y -= q.y;
+        }
+        for (int o = G >> 1; o > 0; o >>= 1) {
+            const Cx<float> y = shfl_xor_c(acc, o);
+            acc.x += y.x;
+            acc.y += y.y;
+        }
+        if (part == 0 && v < L) {
+            out[v] = acc;
+            if (cand) am = amax_better(am, ArgMaxT<float>{cabs2(acc), v});
+        }
+    }
+    if (tid == 0) S.entries += L;
+    return am;
+}
+
+// The residual of the face approximant (m columns) at the 32 fixed samples,
+// one warp per sample; |R_s|^2 to S.samp.
+template <int KER, int NT>
+__device__ void samples32(const AcaArgs<float>& A, BlockSh<float>& S, const FaceTab<float>& F, const ColStore& c,
+                          int kf, int m, const Cx<float>* D) {
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int M = S.M, N = S.N;
+    for (int sm = wid; sm < SAMPLES; sm += NT / 32) {
+        const int i = (2 * sm + 1) * M / (2 * SAMPLES), j = (2 * ((11 * sm) % SAMPLES) + 1) * N / (2 * SAMPLES);
+        Cx<float> e{0, 0};
+        if (lane == 0) e = D ? ldcx(D + (size_t)i * N + j) : ent<KER, float>(A, S.rb + i, S.cb + j, kf);
+        Cx<float> acc{0, 0};
+        for (int q = lane; q < F.ncol; q += 32)
+            cfma(acc, S.fk[F.colP[q]], cmulc(A.pool[F.colU[q] + i], A.pool[F.colV[q] + j]));
+        for (int t = lane; t < m; t += 32) cfmac(acc, ldcx(cs_u<false>(c, t) + i), ldcx(cs_v<false>(c, t) + j));
+        acc.x = warp_sum(acc.x);
+        acc.y = warp_sum(acc.y);
+        if (lane == 0) S.samp[sm] = cabs2d(Cx<float>{e.x - acc.x, e.y - acc.y});
+    }
+    if (threadIdx.x == 0) S.entries += SAMPLES;
+    __syncthreads();
+}
+
+// Partial-pivot ACA of the residual face at frequency kf.  Returns the rank m;
+// c holds the crosses.  Same rows, columns and tests as the float64 face_aca.
+//
+// Two barriers per step.  Between them run (1) the residual row of the next
+// pivot row together with the newest cross's terms of the recursive Frobenius
+// norm
+//   ||S_m||^2 = ||S_{m-1}||^2 + 2 Re sum_t (u_t^H u_m)(v_m^H v_t) + ||u_m||^2 ||v_m||^2,
+// and (2) the column of the row's pivot.  The test of cross m - 1 is thus
+// evaluated with the row of cross m in hand; when it passes, that row is
+// dropped.
+template <int KER, int NT>
+__device__ int face32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float>& S, int kf, unsigned char* arena,
+                      ColStore& c) {
+    constexpr int NW = NT / 32;
+    const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
+    const int M = S.M, N = S.N, nc = S.ncross;
+    const int cap = min(min(M, N), A.RF);
+    c = ColStore{nullptr, w.uw, 0, cs_ld(M, N), M};
+    if (kf < 0 || kf >= A.Ku) {  // cannot happen: every caller passes a checked index
+        if (tid == 0) atomicOr(A.status, ST_BAD_INDEX);
+        return 0;
+    }
+    for (int p = tid; p < nc; p += NT) S.fk[p] = Fp(A, S, p)[kf];
+    long long tf = clock64();
+    FaceTab<float> F = facetab_build<float, NT>(A, w, S, arena);
+    for (int i = tid; i < M; i += NT) w.used[i] = 0;
+    __syncthreads();
+    const Cx<float>* D = nullptr;
+    size_t off = (facetab_smem_bytes<float>() + 255) & ~size_t(255);
+    if constexpr (KER != G3_SEPARABLE) {
+        if (w.dres && (long long)M * N <= A.drf_max) {
+            face_dense_residual<KER, float, NT>(A, w, S, F, kf, arena);
+            D = w.dres;
+            // the tables are not needed any more: only the row buffer stays
+            F.ncol = 0;
+            F.row = N <= ROWMAX ? reinterpret_cast<Cx<float>*>(arena) : w.row;
+            off = N <= ROWMAX ? ((size_t)N * sizeof(Cx<float>) + 15) & ~size_t(15) : 0;
+            sublap(S, 11, tf);
+        }
+    }
+    c.sm = reinterpret_cast<Cx<float>*>(arena + off);
+    c.ncs = (size_t)A.arena_bytes > off ? (int)(((size_t)A.arena_bytes - off) / ((size_t)c.ld * sizeof(Cx<float>))) : 0;
+    c.ncs = min(c.ncs, A.RF);
+    int m = 0, irow = 0;
+    bool converged = false, pending = false, last = false;
+    float2 fsn2 = make_float2(0.f, 0.f);  // ||S_m||^2 (the same in every thread)
+    // own <= max(eps^2 ||S||^2, floor^2), divided by eps^2 (eps^2 alone can take
+    // the norms of strongly damped faces below the float32 range)
+    const float e1 = (float)A.eps_face, inv_e2 = 1.f / (e1 * e1);
+    const float fl = (float)A.face_floor / e1, floor_s = fl * fl * ((float)S.norm2 / (float)A.Ku);
+    for (;;) {
+        // ---- (1) residual row, and the norm terms of the newest cross ----
+        ArgMaxT<float> am = amax_none<float>();
+        if (m < cap && !last) {
+            if (F.ncol > 0) {
+                // (the current columns' coefficients are read from c directly)
+                for (int q = tid; q < F.ncol; q += NT) F.coef[q] = cmul(S.fk[F.colP[q]], A.pool[F.colU[q] + irow]);
+                __syncthreads();
+            }
+            am = line32<KER, NT, true>(A, w, S, F, c, irow, -1, kf, m, F.row, D);
+        }
+        if (pending) {
+            const int mm = m - 1;
+            const Cx<float>* um = cs_u<false>(c, mm);
+            const Cx<float>* vm = um + M;
+            float2 part = make_float2(0.f, 0.f);
+            for (int t = wid; t <= mm; t += NW) {
+                const Cx<float>* ut = cs_u<false>(c, t);
+                const Cx<float>* vt = ut + M;
+                Cx<float> gu{0, 0}, gv{0, 0};
+#pragma unroll 4
+                for (int i = lane; i < M; i += 32) cfmac(gu, ldcx(um + i), ldcx(ut + i));  // conj(u_t) u_m
+#pragma unroll 4
+                for (int i = lane; i < N; i += 32) cfmac(gv, ldcx(vt + i), ldcx(vm + i));  // conj(v_m) v_t
+                gu.x = warp_sum(gu.x);
+                gu.y = warp_sum(gu.y);
+                gv.x = warp_sum(gv.x);
+                gv.y = warp_sum(gv.y);
+                if (t < mm) {
+                    ff_add_prod(part, 2.f * gu.x, gv.x);
+                    ff_add_prod(part, -2.f * gu.y, gv.y);
+                } else {
+                    float2 own = make_float2(0.f, 0.f);
+                    ff_add_prod(own, gu.x, gv.x);
+                    if (lane == 0) S.own = own;
+                }
+            }
+            if (lane == 0) S.nrm[wid] = part;
+        }
+        {
+            const uint2 k = warp_key(am);
+            if (lane == 0) S.key[0][wid] = k;
+        }
+        __syncthreads();
+        if (pending) {
+            pending = false;
+            const float2 own = S.own;
+#pragma unroll
+            for (int q = 0; q < NW; ++q) {
+                const float2 p = S.nrm[q];
+                ff_add(fsn2, p.x, p.y);
+            }
+            ff_add(fsn2, own.x, own.y);
+            if (own.x * inv_e2 <= fmaxf(fmaxf(fsn2.x, 0.f), floor_s)) {
+                if (!A.sample_check) {
+                    converged = true;
+                    break;
+                }
+                // confirm on the sample entries: partial pivoting can miss a block
+                // of the face that no visited row or column reaches
+                sublap(S, 6, tf);
+                samples32<KER, NT>(A, S, F, c, kf, m, D);
+                static_assert(SAMPLES == 32, "one sample per lane");
+                if (wid == 0) {
+                    const double sv = S.samp[lane];
+                    const double tot = warp_sum(sv);
+                    ArgMaxT<float> b{(float)sv, lane};
+                    b = warp_argmax(b);
+                    if (lane == 0) {
+                        const double e2 = A.eps_face * A.eps_face;
+                        S.fconv = (double)M * (double)N / SAMPLES * tot <=
+                                  fmax(e2 * fmax((double)fsn2.x + (double)fsn2.y, 0.0),
+                                       A.face_floor * A.face_floor * S.norm2 / (double)A.Ku);
+                        S.fbs = b.i;
+                    }
+                }
+                __syncthreads();
+                const bool ok = S.fconv;
+                const int bs = S.fbs;
+                __syncthreads();  // both are rewritten by the next test
+                sublap(S, 9, tf);
+                if (ok) {
+                    converged = true;
+                    break;
+                }
+                if (tid == 0) atomicAdd(&A.counters[5], 1ull);
+                irow = (2 * bs + 1) * M / (2 * SAMPLES);
+                last = false;
+                if (m < cap) continue;
+            }
+        }
+        if (m >= cap || last) break;  // the cap, or every row used
+        am = block_key<NT>(S.key[0]);
+        if (tid == 0) w.used[irow] = 1;
+        // a row counts as nonzero when |delta|^2 is a normal number of the
+        // working precision (below that the entries are far under any tolerance)
+        if (!(am.v > tiny_norm2<float>())) {
+            // zero residual row: next unused row in index order
+            ArgMaxT<float> un = amax_none<float>();
+            for (int i = tid; i < M; i += NT)
+                if (i != irow && !w.used[i]) un = amax_better(un, ArgMaxT<float>{0.f, i});
+            un = block_argmax<NT>(un, S.am);
+            if (un.v < 0.f) break;  // no row with a nonzero residual left
+            irow = un.i;
+            continue;
+        }
+        const int jp = am.i;
+        sublap(S, 6, tf);
+        // ---- (2) v = conj(row / delta), the column of the pivot ----
+        // delta is scaled to magnitude ~1 first, so that a tiny pivot of a strongly
+        // damped face cannot overflow 1 / |delta|^2 (|row[j]| <= |delta|)
+        const Cx<float> delta = F.row[jp];
+        const float sc = 1.f / fmaxf(fabsf(delta.x), fabsf(delta.y));
+        const Cx<float> ds{delta.x * sc, delta.y * sc};
+        const float dn = 1.f / cabs2(ds);
+        if (F.ncol > 0) {
+            for (int q = tid; q < F.ncol; q += NT) F.coef[q] = cmul(S.fk[F.colP[q]], cconj(A.pool[F.colV[q] + jp]));
+            __syncthreads();
+        }
+        Cx<float>* um = cs_u<false>(c, m);
+        Cx<float>* vm = um + M;
+        for (int j = tid; j < N; j += NT) {
+            const Cx<float> rj = F.row[j];
+            const Cx<float> q = cmulc(Cx<float>{rj.x * sc, rj.y * sc}, ds);  // (row / s) conj(delta / s)
+            vm[j] = Cx<float>{q.x * dn, -q.y * dn};                          // conj(row / delta)
+        }
+        ArgMaxT<float> nx = line32<KER, NT, false>(A, w, S, F, c, jp, irow, kf, m, um, D);
+        {
+            const uint2 k = warp_key(nx);
+            if (lane == 0) S.key[1][wid] = k;
+        }
+        __syncthreads();
+        nx = block_key<NT>(S.key[1]);
+        ++m;
+        pending = true;
+        last = nx.v < 0.f;  // every row used: one more test, then the end
+        if (!last) irow = nx.i;
+        sublap(S, 7, tf);
+    }
+    if (tid == 0) S.raw += m;
+    if (!converged && m == A.RF && m < min(M, N)) {
+        if (tid == 0) {
+            atomicOr(A.status, ST_FACE_CAPPED);
+            atomicAdd(&A.counters[3], 1ull);
+        }
+    }
+    __syncthreads();
+    return m;
+}
+
+// ---- recompression ----------------------------------------------------------------------
+// The r crosses of c are replaced in place by the factors of a truncated
+// H = U V^H (Section 4, second implementation remark), all in float32 and in
+// shared memory when the columns and two r x r matrices fit:
+//   1. V = Q R by modified Gram-Schmidt (R unit upper triangular, Q's columns
+//      orthogonal with norms n_b), one barrier per column.  v_t = conj(row /
+//      pivot) vanishes at the earlier pivot columns, so V is well conditioned;
+//   2. W = U R^H diag(n), row by row in place: H = W (Q diag(1/n))^H, and W has
+//      the column norms of the core R_U R_V^H without a QR of U;
+//   3. column-pivoted QR of W by modified Gram-Schmidt, stopped when the
+//      largest remaining column norm falls below eps_face times the first one:
+//      dropping the remaining columns removes exactly their norms, as a
+//      truncated SVD removes its dropped singular values.  One barrier per step:
+//      every warp picks the pivot from the column norms (double-buffered) and
+//      forms its norm itself.
+// U' = W's pivot columns (normalised), V' = Q diag(1/n) J, J = Pi R_W^H.
+// Modified Gram-Schmidt keeps A = Q R to rounding whatever the orthogonality
+// of Q, so U' V'^H + (the dropped columns) is H to float32 rounding; a Gram
+// (Cholesky) QR squares the condition number and needed float64, at 4x the
+// cycles (12,288-triangle single layer, 192 x 192 blocks: 310,000 -> see
+// k_aca3's table).
+// RT [r][ldr]: conj(R) transposed; JT [r][ldr].  Returns the kept rank;
+// S.sel, S.rk32: pivot columns and their norms.
+template <int NT, bool SM>
+__device__ int recompress32_t(const AcaArgs<float>& A, BlockSh<float>& S, const ColStore& c, int r, Cx<float>* RT,
+                              Cx<float>* JT, int ldr) {
+    constexpr int NW = NT / 32;
+    const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
+    const int M = S.M, N = S.N;
+    long long tc = clock64();
+    for (int e = tid; e < r * ldr; e += NT) RT[e] = JT[e] = Cx<float>{0, 0};
+    if (wid == 0) {
+        const Cx<float>* v = cs_v<SM>(c, 0);
+        float s2 = 0;
+        for (int i = lane; i < N; i += 32) s2 += cabs2(ldcx(v + i));
+        s2 = warp_sum(s2);
+        if (lane == 0) S.n2[0] = s2;
+    }
+    __syncthreads();
+    // ---- 1. V = Q R ----
+    for (int k = 0; k < r; ++k) {
+        const float n2 = S.n2[k];
+        const float inv = n2 > 0.f ? 1.f / n2 : 0.f;
+        const Cx<float>* vk = cs_v<SM>(c, k);
+        if (tid == 0) RT[k * ldr + k] = Cx<float>{1.f, 0.f};
+        // two columns per warp and pass
+        for (int j = k + 1 + wid; j < r; j += 2 * NW) {
+            const bool two = j + NW < r;
+            Cx<float>* va = cs_v<SM>(c, j);
+            Cx<float>* vb = two ? cs_v<SM>(c, j + NW) : va;
+            Cx<float> ga{0, 0}, gb{0, 0};
+#pragma unroll 2
+            for (int i = lane; i < N; i += 32) {
+                const Cx<float> q = ldcx(vk + i);
+                cfmac(ga, ldcx(va + i), q);  // conj(v_k) v_j
+                cfmac(gb, ldcx(vb + i), q);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                ga.x += __shfl_xor_sync(0xffffffffu, ga.x, o);
+                ga.y += __shfl_xor_sync(0xffffffffu, ga.y, o);
+                gb.x += __shfl_xor_sync(0xffffffffu, gb.x, o);
+                gb.y += __shfl_xor_sync(0xffffffffu, gb.y, o);
+            }
+            ga.x *= inv;
+            ga.y *= inv;
+            gb.x *= inv;
+            gb.y *= inv;
+            float s2 = 0;
+#pragma unroll 2
+            for (int i = lane; i < N; i += 32) {
+                const Cx<float> q = ldcx(vk + i);
+                Cx<float> x = ldcx(va + i);
+                x.x -= q.x * ga.x - q.y * ga.y;
+                x.y -= q.x * ga.y + q.y * ga.x;
+                va[i] = x;
+                s2 += cabs2(x);
+                if (two) {
+                    Cx<float> y = ldcx(vb + i);
+                    y.x -= q.x * gb.x - q.y * gb.y;
+                    y.y -= q.x * gb.y + q.y * gb.x;
+                    vb[i] = y;
+                }
+            }
+            if (j == k + 1) {  // the next step's column
+                s2 = warp_sum(s2);
+                if (lane == 0) S.n2[j] = s2;
+            }
+            if (lane == 0) {
+                RT[j * ldr + k] = cconj(ga);
+                if (two) RT[(j + NW) * ldr + k] = cconj(gb);
+            }
+        }
+        __syncthreads();
+    }
+    for (int b = tid; b < r; b += NT) {
+        const float n = sqrtf(S.n2[b]);
+        S.nv[b] = n;
+        S.rnv[b] = n > 0.f ? 1.f / n : 0.f;
+    }
+    __syncthreads();
+    sublap(S, 0, tc);
+    // ---- 2. W = U R^H diag(n) in place: W[i][b] = n_b sum_{c >= b} U[i][c] conj(R[b][c]) ----
+    {
+        // G threads (one warp's neighbours) per row, four columns b each per pass; a
+        // pass overwrites columns that no later pass reads
+        const int G = M * 4 <= NT ? 4 : (M * 2 <= NT ? 2 : 1);
+        const int per = NT / G, part = tid % G;
+        for (int base = 0; base < M; base += per) {
+            const int i = base + tid / G;
+            for (int b0 = 0; b0 < r; b0 += 4 * G) {
+                const int b = b0 + 4 * part;
+                Cx<float> acc[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[q] = Cx<float>{0, 0};
+                if (i < M && b < r) {
+                    for (int cc = b; cc < r; ++cc) {
+                        const Cx<float> u = ldcx(cs_u<SM>(c, cc) + i);
+                        const float4 r0 = *reinterpret_cast<const float4*>(RT + cc * ldr + b);
+                        const float4 r1 = *reinterpret_cast<const float4*>(RT + cc * ldr + b + 2);
+                        cfma(acc[0], u, Cx<float>{r0.x, r0.y});
+                        cfma(acc[1], u, Cx<float>{r0.z, r0.w});
+                        cfma(acc[2], u, Cx<float>{r1.x, r1.y});
+                        cfma(acc[3], u, Cx<float>{r1.z, r1.w});
+                    }
+                }
+                __syncwarp();
+                if (i < M) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (b + q < r) {
+                            const float n = S.nv[b + q];
+                            cs_u<SM>(c, b + q)[i] = Cx<float>{acc[q].x * n, acc[q].y * n};
+                        }
+                }
+                __syncwarp();
+            }
+        }
+    }
+    __syncthreads();
+    sublap(S, 1, tc);
+    // ---- 3. column-pivoted QR of W ----
+    for (int j = wid; j < r; j += NW) {
+        const Cx<float>* x = cs_u<SM>(c, j);
+        float s2 = 0;
+        for (int i = lane; i < M; i += 32) s2 += cabs2(ldcx(x + i));
+        s2 = warp_sum(s2);
+        if (lane == 0) S.cn[0][j] = s2;
+    }
+    __syncthreads();
+    const float sfloor = (float)A.trunc_floor * sqrtf((float)S.norm2 / (float)A.Ku);
+    float r00 = 0.f;
+    int k = 0;
+    for (; k < r; ++k) {
+        const float* cn = S.cn[k & 1];
+        float* cx = S.cn[(k & 1) ^ 1];
+        ArgMaxT<float> best = amax_none<float>();
+        for (int q = lane; q < r; q += 32) best = amax_better(best, ArgMaxT<float>{cn[q], q});
+        const uint2 key = warp_key(best);
+        if (key.x == 0u) break;
+        const int pv = (int)key.y;
+        const Cx<float>* qv = cs_u<SM>(c, pv);
+        float s2 = 0;
+        for (int i = lane; i < M; i += 32) s2 += cabs2(ldcx(qv + i));
+        s2 = warp_sum(s2);
+        const float rkk = sqrtf(s2);
+        if (k == 0) r00 = rkk;
+        if (!(rkk > 0.f) || !isfinite(rkk) || rkk < (float)A.eps_face * r00 || (k > 0 && rkk < sfloor)) break;
+        const float inv = 1.f / rkk;
+        if (tid == 0) {
+            S.sel[k] = pv;
+            S.rk32[k] = rkk;
+            JT[pv * ldr + k] = Cx<float>{rkk, 0.f};
+        }
+        for (int j = wid; j < r; j += 2 * NW) {
+            const int j2 = j + NW;
+            const float c1 = cn[j], c2 = j2 < r ? cn[j2] : -1.f;
+            const bool o1 = c1 >= 0.f && j != pv, o2 = c2 >= 0.f && j2 != pv;
+            Cx<float>* xa = cs_u<SM>(c, j);
+            Cx<float>* xb = o2 ? cs_u<SM>(c, j2) : xa;
+            Cx<float> ga{0, 0}, gb{0, 0};
+            if (o1 || o2) {
+#pragma unroll 2
+                for (int i = lane; i < M; i += 32) {
+                    const Cx<float> q = ldcx(qv + i);
+                    cfmac(ga, ldcx(xa + i), q);
+                    cfmac(gb, ldcx(xb + i), q);
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    ga.x += __shfl_xor_sync(0xffffffffu, ga.x, o);
+                    ga.y += __shfl_xor_sync(0xffffffffu, ga.y, o);
+                    gb.x += __shfl_xor_sync(0xffffffffu, gb.x, o);
+                    gb.y += __shfl_xor_sync(0xffffffffu, gb.y, o);
+                }
+                ga.x *= inv;
+                ga.y *= inv;
+                gb.x *= inv;
+                gb.y *= inv;
+#pragma unroll 2
+                for (int i = lane; i < M; i += 32) {
+                    Cx<float> q = ldcx(qv + i);
+                    q.x *= inv;
+                    q.y *= inv;
+                    if (o1) {
+                        Cx<float> x = ldcx(xa + i);
+                        x.x -= q.x * ga.x - q.y * ga.y;
+                        x.y -= q.x * ga.y + q.y * ga.x;
+                        xa[i] = x;
+                    }
+                    if (o2) {
+                        Cx<float> y = ldcx(xb + i);
+                        y.x -= q.x * gb.x - q.y * gb.y;
+                        y.y -= q.x * gb.y + q.y * gb.x;
+                        xb[i] = y;
+                    }
+                }
+            }
+            if (lane == 0) {
+                cx[j] = o1 ? fmaxf(c1 - cabs2(ga), 0.f) : -1.f;
+                if (o1) JT[j * ldr + k] = cconj(ga);
+                if (j2 < r) {
+                    cx[j2] = o2 ? fmaxf(c2 - cabs2(gb), 0.f) : -1.f;
+                    if (o2) JT[j2 * ldr + k] = cconj(gb);
+                }
+            }
+        }
+        __syncthreads();
+    }
+    __syncthreads();
+    sublap(S, 3, tc);
+    // fold Q's normalisation into J
+    for (int e = tid; e < r * ldr; e += NT) {
+        const float n = S.rnv[e / ldr];
+        JT[e].x *= n;
+        JT[e].y *= n;
+    }
+    __syncthreads();
+    return k;
+}
+
+// U' and V' of the recompressed face into the pool (M x rn, N x rn, column-major)
+template <int NT, bool SM>
+__device__ void form32_t(BlockSh<float>& S, const ColStore& c, int r, int rn, const Cx<float>* JT, int ldr,
+                         Cx<float>* Un, Cx<float>* Vn) {
+    const int tid = threadIdx.x;
+    const int M = S.M, N = S.N;
+    for (int e = tid; e < rn * M; e += NT) {
+        const int b = e / M, i = e - b * M;
+        const float inv = 1.f / S.rk32[b];
+        const Cx<float> x = ldcx(cs_u<SM>(c, S.sel[b]) + i);
+        Un[e] = Cx<float>{x.x * inv, x.y * inv};
+    }
+    const int nb = (rn + 3) / 4;
+    for (int e = tid; e < N * nb; e += NT) {
+        const int b = (e / N) * 4, j = e % N;
+        Cx<float> acc[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] = Cx<float>{0, 0};
+#pragma unroll 2
+        for (int a = 0; a < r; ++a) {
+            const Cx<float> v = ldcx(cs_v<SM>(c, a) + j);
+            const float4 r0 = *reinterpret_cast<const float4*>(JT + a * ldr + b);
+            const float4 r1 = *reinterpret_cast<const float4*>(JT + a * ldr + b + 2);
+            cfma(acc[0], v, Cx<float>{r0.x, r0.y});
+            cfma(acc[1], v, Cx<float>{r0.z, r0.w});
+            cfma(acc[2], v, Cx<float>{r1.x, r1.y});
+            cfma(acc[3], v, Cx<float>{r1.z, r1.w});
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (b + q < rn) Vn[(long long)(b + q) * N + j] = acc[q];
+    }
+}
+
+// where the recompression's two r x r matrices go, and whether everything is
+// in shared memory
+struct Recomp32 {
+    Cx<float>* RT;
+    Cx<float>* JT;
+    int ldr;
+    bool sm;
+};
+__device__ __forceinline__ Recomp32 recomp32_place(const AcaArgs<float>& A, const Ws<float>& w, const ColStore& c, int r,
+                                                   unsigned char* arena) {
+    Recomp32 p;
+    p.ldr = (r + 3) & ~3;
+    const size_t one = (size_t)r * p.ldr;
+    unsigned char* end = reinterpret_cast<unsigned char*>(c.sm + (size_t)r * c.ld);
+    p.sm = r <= c.ncs && (size_t)(end - arena) + 2 * one * sizeof(Cx<float>) <= (size_t)A.arena_bytes;
+    p.RT = p.sm ? reinterpret_cast<Cx<float>*>(end) : reinterpret_cast<Cx<float>*>(w.RU);
+    p.JT = p.sm ? p.RT + one : reinterpret_cast<Cx<float>*>(w.RV);
+    return p;
+}
+template <int NT>
+__device__ int recompress32(const AcaArgs<float>& A, BlockSh<float>& S, const ColStore& c, int r, const Recomp32& p,
+                            unsigned char* arena) {
+    // (addresses formed from the arena, so that they stay shared-memory accesses)
+    if (p.sm) {
+        Cx<float>* RT = reinterpret_cast<Cx<float>*>(arena + (reinterpret_cast<unsigned char*>(p.RT) - arena));
+        return recompress32_t<NT, true>(A, S, c, r, RT, RT + (size_t)r * p.ldr, p.ldr);
+    }
+    return recompress32_t<NT, false>(A, S, c, r, p.RT, p.JT, p.ldr);
+}
+template <int NT>
+__device__ void form32(BlockSh<float>& S, const ColStore& c, int r, int rn, bool raw, const Recomp32& p, Cx<float>* Un,
+                       Cx<float>* Vn) {
+    if (raw) {
+        const int M = S.M, N = S.N;
+        for (int e = threadIdx.x; e < rn * M; e += NT) Un[e] = cs_u<false>(c, e / M)[e % M];
+        for (int e = threadIdx.x; e < rn * N; e += NT) Vn[e] = cs_v<false>(c, e / N)[e % N];
+    } else if (p.sm) {
+        form32_t<NT, true>(S, c, r, rn, p.JT, p.ldr, Un, Vn);
+    } else {
+        form32_t<NT, false>(S, c, r, rn, p.JT, p.ldr, Un, Vn);
+    }
+}
+
+}  // namespace g3
