@@ -378,7 +378,7 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
         else
             per_low = occupancy_kind<T, NT, false>(kernel, smem);
     }
-    const int per_dense = o.ctas_per_sm > 0 ? o.ctas_per_sm : occupancy_kind<T, NT, true>(kernel, smem_base);
+    const int per_dense = o.ctas_per_sm > 0 ? o.ctas_per_sm : occupancy_kind<T, NT, true>(kernel, 0);
     const int grid_low = o.unbatched ? 1 : std::max(1, std::min(n_low, ctx->n_sm * per_low));
     const int grid_dense = o.unbatched ? 1 : std::max(1, std::min(n_dense, ctx->n_sm * per_dense));
     const int grid = std::max(grid_low, grid_dense);
@@ -527,7 +527,7 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
             for (int l = 0; l < launches && st == G3_OK; ++l) {
                 if (o.unbatched) B.single = l;
                 if (cls == 1)
-                    st = launch_kind<T, NT, true>(ctx, kernel, B, g, smem_base);
+                    st = launch_kind<T, NT, true>(ctx, kernel, B, g, 0);
                 else if constexpr (sizeof(T) == 4)
                     st = nt_low == 512   ? launch_kind<T, 512, false>(ctx, kernel, B, g, smem)
                          : nt_low == 384 ? launch_kind<T, 384, false>(ctx, kernel, B, g, smem)

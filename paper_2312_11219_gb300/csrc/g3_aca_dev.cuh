@@ -70,6 +70,7 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
 }
 
 constexpr int RF_MAX = 64;    // largest face rank cap
+constexpr int USED_W = 24;    // words of the float32 face ACA's mask of used rows
 constexpr int CS_PAD = 16;    // padding of a float32 face column (ColStore)
 
 // geometry and frequencies of one mesh of a batched compression
@@ -218,11 +219,13 @@ struct BlockSh {
     double dU[RF_MAX], dV[RF_MAX];
     double rdU[RF_MAX], rdV[RF_MAX];  // 1 / diagonal of the Cholesky factors
     T cnV[RF_MAX];                    // column norms of V' (pivot of eq. (index))
-    // float32 faces: warp candidates of the row and column argmax, the warps'
-    // terms of ||S_m||_F^2 (float-float) and the newest cross's own term
+    // float32 faces: warp candidates of the row and column argmax; the warps'
+    // parts of ||u_m||^2 and ||v_m||^2 (of ||D||_F^2 before the first step) and of
+    // the recursive norm's cross terms (float-float)
     uint2 key[2][32];
+    unsigned usedm[USED_W];  // rows taken by the face ACA
     float2 nrm[32];
-    float2 own;
+    float2 crs[32];
     // float32 recompression: squared norms, norms and their reciprocals of the
     // orthogonalised V columns; squared norms of W's columns (double-buffered);
     // norms of the pivot columns
@@ -656,41 +659,116 @@ __device__ void face_samples(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S,
 // i < M, j < N, in one parallel pass before the face ACA: the ACA then reads its rows
 // and columns from D and sums only the current face's crosses.  The partial-pivot
 // ACA takes the same rows and columns as with on-demand lines; only the order of
-// the float32 sums over the earlier crosses differs.  Tiles of 64 x (NT / 4)
+// the float32 sums over the earlier crosses differs.  The warps' parts of
+// ||D||_F^2 are left in S.nrm.  Tiles of 64 x (NT / 4)
 // outputs; the earlier crosses' columns (scaled by f_p[kf]) staged DRF_KC at a
 // time in shared memory.  The sum over them is a dense complex product, on the
 // tensor cores at 256 threads (the TF32 three-term split, float32 accuracy),
 // else on the CUDA cores (a 4 x 4 micro-tile per thread).  Float32 only.
-constexpr int DRF_KC = 16;     // columns per staged chunk, CUDA-core path
-constexpr int DRF_KC_TC = 16;  // columns per staged chunk, tensor-core path (256 threads, two buffers)
+constexpr int DRF_KC = 16;     // columns per staged chunk
+constexpr int DRF_ST = 3;      // staging buffers of the tensor-core path (256 threads)
 // shared-memory staging of the dense residual face, placed after the face's
-// column tables (the coefficient and row buffers that follow them are not in
-// use while the dense face is formed)
+// column tables and coefficients (the row buffer that follows them is not in use
+// while the dense face is formed)
 template <class T>
 constexpr size_t drf_stage_offset() {
-    return (2 * TABMAX * sizeof(long long) + TABMAX * sizeof(short) + 255) & ~size_t(255);
+    return (2 * TABMAX * sizeof(long long) + TABMAX * sizeof(short) + (TABMAX + RF_MAX) * sizeof(Cx<T>) + 255) &
+           ~size_t(255);
 }
 template <class T, int NT>
 constexpr size_t drf_stage_bytes() {
-    return (size_t)(NT == 256 ? 2 * DRF_KC_TC : DRF_KC) * (64 + NT / 4) * sizeof(Cx<T>);
+    return (size_t)(NT == 256 ? DRF_ST : 1) * DRF_KC * (64 + NT / 4) * sizeof(Cx<T>);
 }
 
+constexpr int DRF_RB = 24;     // rows per warp and pass of the entries
+
+// A column element's geometry in registers, evaluated against row elements at
+// one frequency (the arithmetic of pair_setup / pair_eval, gal_setup / gal_eval).
+template <int KER>
+struct ColGeo {
+    static constexpr bool GAL = KER == G3_GAL_SLP;
+    static constexpr int NQ = GAL ? 4 : 7;
+    float h[3], l[3], q[NQ][3], w[NQ], n[3];
+    __device__ __forceinline__ void load(const GeomF& g, int j) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            h[k] = g.ch[k * g.E + j];
+            l[k] = g.cl[k * g.E + j];
+            if (KER == G3_DLP) n[k] = nrm(g, k, j);
+        }
+#pragma unroll
+        for (int a = 0; a < NQ; ++a) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) q[a][k] = GAL ? q4off(g, a, k, j) : qoff(g, a, k, j);
+            w[a] = GAL ? q4wt(g, a, j) : qwt(g, a, j) * (float)G3_INV4PI;
+        }
+    }
+    __device__ __forceinline__ Cx<float> eval(const GeomF& g, int i, float sre, float sim) const {
+        float d[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) d[k] = (g.ch[k * g.E + i] - h[k]) + (g.cl[k * g.E + i] - l[k]);
+        Cx<float> acc{0, 0};
+        if constexpr (GAL) {
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const float x0 = d[0] + q4off(g, a, 0, i), x1 = d[1] + q4off(g, a, 1, i), x2 = d[2] + q4off(g, a, 2, i);
+                const float wa = q4wt(g, a, i) * (float)G3_INV4PI;
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    const float rx = x0 - q[b][0], ry = x1 - q[b][1], rz = x2 - q[b][2];
+                    const float r2 = rx * rx + ry * ry + rz * rz;
+                    const float ri = krsqrt(r2), r = r2 * ri;
+                    const float m = wa * w[b] * ri * kexp(-sre * r);
+                    float sn, cs;
+                    ksincos(sim * r, &sn, &cs);
+                    acc.x += m * cs;
+                    acc.y -= m * sn;
+                }
+            }
+        } else {
+            float pd = 0;
+            if (KER == G3_DLP) pd = d[0] * n[0] + d[1] * n[1] + d[2] * n[2];
+#pragma unroll
+            for (int a = 0; a < 7; ++a) {
+                const float rx = d[0] - q[a][0], ry = d[1] - q[a][1], rz = d[2] - q[a][2];
+                const float r2 = rx * rx + ry * ry + rz * rz;
+                const float ri = krsqrt(r2), r = r2 * ri;
+                const float amp = KER == G3_DLP ? w[a] * pd * ri * ri * ri : w[a] * ri;
+                const float m = amp * kexp(-sre * r);
+                float sn, cs;
+                ksincos(sim * r, &sn, &cs);
+                if (KER == G3_DLP) {
+                    const float fr = 1.f + sre * r, fi = sim * r;
+                    acc.x += m * (fr * cs + fi * sn);
+                    acc.y += m * (fi * cs - fr * sn);
+                } else {
+                    acc.x += m * cs;
+                    acc.y -= m * sn;
+                }
+            }
+        }
+        return acc;
+    }
+};
+
+// (not inlined: its tiles need most of the 128 registers; the staging buffers are
+// addressed from the arena's own symbol so that they stay shared-memory accesses)
 template <int KER, class T, int NT>
-__device__ void face_dense_residual(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, const FaceTab<T>& F,
-                                    int kf, unsigned char* arena) {
+__device__ __noinline__ void face_dense_residual(const AcaArgs<T>& A, Cx<T>* __restrict__ D, BlockSh<T>& S,
+                                                 const FaceTab<T> F, int kf) {
     static_assert(sizeof(T) == 4, "dense residual faces are a float32 path");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    unsigned char* arena = smem_raw;
     constexpr int TI = 64, TJ = NT / 4, TXN = TJ / 4;
     const int tid = threadIdx.x;
     const int M = S.M, N = S.N, nc = F.ncol;
     const int tx = tid % TXN, ty = tid / TXN;  // ty < 16
     Cx<T>* su = reinterpret_cast<Cx<T>*>(arena + drf_stage_offset<T>());  // [DRF_KC][TI]
     Cx<T>* sv = su + DRF_KC * TI;                                          // [DRF_KC][TJ]
-    Cx<T>* D = w.dres;
-    // the entries, one thread per entry (consecutive threads take consecutive
-    // columns); linear elements: one thread per element pair, whose nine local
+    // the entries; linear elements: one thread per element pair, whose nine local
     // entries share the pair's quadrature points
-    const int MN = M * N;
     long long te = clock64();
+    float dn = 0;   // this thread's part of ||D||_F^2 (of the entries, then of the residual)
     if constexpr (KER == G3_GAL_P1D || KER == G3_GAL_P1KP) {
         const float2 s = A.sf[kf];
         const int Me = M / 3, Ne = N / 3;
@@ -703,14 +781,38 @@ __device__ void face_dense_residual(const AcaArgs<T>& A, const Ws<T>& w, BlockSh
 #pragma unroll
             for (int a = 0; a < 3; ++a)
 #pragma unroll
-                for (int b = 0; b < 3; ++b) D[(size_t)(3 * pe + a) * N + 3 * qe + b] = v[a * 3 + b];
+                for (int b = 0; b < 3; ++b) {
+                    D[(size_t)(3 * pe + a) * N + 3 * qe + b] = v[a * 3 + b];
+                    dn += cabs2(v[a * 3 + b]);
+                }
         }
     } else {
-        for (int e = tid; e < MN; e += NT) {
-            const int i = e / N, j = e - i * N;
-            D[e] = ent<KER, T>(A, S.rb + i, S.cb + j, kf);
+        // one warp per 32 columns and DRF_RB rows: a lane keeps the geometry of its
+        // column's element in registers and walks the rows, whose centroids are
+        // uniform loads (34 loads per entry otherwise, as many issue slots as the
+        // exponentials).  A last group of at most 16 columns takes two or more
+        // rows at a time.
+        const float2 s = A.sf[kf];
+        const int wid = tid >> 5, lane = tid & 31;
+        const int ncg = (N + 31) / 32, nrg = (M + DRF_RB - 1) / DRF_RB;
+        for (int u = wid; u < ncg * nrg; u += NT / 32) {
+            const int j0 = (u % ncg) * 32, r0 = (u / ncg) * DRF_RB, r1 = min(M, r0 + DRF_RB);
+            const int nj = min(32, N - j0);
+            const int lw = nj > 16 ? 32 : (nj > 8 ? 16 : 8);   // lanes per row
+            const int j = j0 + lane % lw;
+            if (j < N) {
+                ColGeo<KER> g;
+                g.load(A.gf, S.cb + j);
+                for (int i = r0 + lane / lw; i < r1; i += 32 / lw) {
+                    const Cx<T> v = g.eval(A.gf, S.rb + i, s.x, s.y);
+                    D[(size_t)i * N + j] = v;
+                    dn += cabs2(v);
+                }
+            }
         }
     }
+    // f_p[kf] of every earlier column
+    for (int c = tid; c < nc; c += NT) F.coef[c] = S.fk[F.colP[c]];
     __syncthreads();
     sublap(S, 10, te);  // the residual lines evaluate no entries when this runs
     if constexpr (NT == 256) {
@@ -719,101 +821,129 @@ __device__ void face_dense_residual(const AcaArgs<T>& A, const Ws<T>& w, BlockSh
         // products Re = ur vr + ui vi, Im = ui vr - ur vi (mma_tf32x3 each)
         const int warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
         const int rw = (warp & 3) * 16, cw = (warp >> 2) * 32;
-        constexpr int KC = DRF_KC_TC;
-        // two staging buffers of KC columns each, filled by cp.async (8 bytes per
-        // element, zero-filled outside the face and past the last column) while the
-        // tensor cores work on the other; f_p[kf] is applied to the A fragments
-        Cx<T>* bu[2] = {su, su + KC * (TI + TJ)};
-        auto issue = [&](int buf, int i0, int j0, int c0) {
-            Cx<T>* du = bu[buf];
-            Cx<T>* dv = du + KC * TI;
-            for (int e = tid; e < KC * TI; e += NT) {
-                const int kk = e / TI, ii = e - kk * TI, c = c0 + kk;
-                const bool in = c < nc && i0 + ii < M;
-                cp_async8(du + e, in ? A.pool + F.colU[c] + i0 + ii : A.pool, in);
+        constexpr int KC = DRF_KC, ST = DRF_ST;
+        // ST staging buffers of KC columns each, filled by cp.async (8 bytes per
+        // element, zero-filled outside the face and past the last column) ST - 1
+        // chunks ahead of the tensor cores, over the chunks of all tiles in one
+        // sequence: the L2 latency is two to three chunks of work (with one chunk
+        // ahead the product waited on it: 2,100 SM cycles per 64 x 64 x 8 against
+        // ~450 issued).  f_p[kf] is applied to the A fragments.
+        const int nch = (nc + KC - 1) / KC, ntj = (N + TJ - 1) / TJ, nti = (M + TI - 1) / TI;
+        const int total = nch * ntj * nti;
+        const int sc = tid % 64, sk = tid / 64;   // staged element: column part and offset
+        static_assert(TI == 64 && TJ == 64 && NT == 256, "staging map");
+        auto issue = [&](int q) {
+            if (q < total) {
+                const int tile = q / nch, c0 = (q - tile * nch) * KC;
+                const int i0 = (tile / ntj) * TI, j0 = (tile % ntj) * TJ;
+                Cx<T>* du = su + (q % ST) * KC * (TI + TJ);
+                Cx<T>* dv = du + KC * TI;
+                const bool iu = i0 + sc < M, iv = j0 + sc < N;
+#pragma unroll
+                for (int x = 0; x < KC; x += 4) {
+                    const int kk = x + sk, c = c0 + kk;
+                    const bool in = c < nc;
+                    cp_async8(du + kk * TI + sc, in && iu ? A.pool + F.colU[c] + i0 + sc : A.pool, in && iu);
+                    cp_async8(dv + kk * TJ + sc, in && iv ? A.pool + F.colV[c] + j0 + sc : A.pool, in && iv);
+                }
             }
-            for (int e = tid; e < KC * TJ; e += NT) {
-                const int kk = e / TJ, jj = e - kk * TJ, c = c0 + kk;
-                const bool in = c < nc && j0 + jj < N;
-                cp_async8(dv + e, in ? A.pool + F.colV[c] + j0 + jj : A.pool, in);
-            }
-            cp_async_commit();
+            cp_async_commit();   // (an empty group past the end keeps the count)
         };
-        for (int i0 = 0; i0 < M; i0 += TI) {
-            for (int j0 = 0; j0 < N; j0 += TJ) {
-                float are[4][4], aim[4][4];
+#pragma unroll 1
+        for (int q = 0; q < ST - 1; ++q) issue(q);
+        float are[4][4], aim[4][4];
+        if (total > 0) dn = 0;
+        for (int q = 0; q < total; ++q) {
+            const int tile = q / nch, ch = q - tile * nch, c0 = ch * KC;
+            if (ch == 0) {
 #pragma unroll
                 for (int n8 = 0; n8 < 4; ++n8)
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) are[n8][q] = aim[n8][q] = 0.f;
-                __syncthreads();  // the previous tile's buffers are consumed
-                if (nc > 0) issue(0, i0, j0, 0);
-                for (int c0 = 0, b = 0; c0 < nc; c0 += KC, b ^= 1) {
-                    if (c0 + KC < nc) {
-                        issue(b ^ 1, i0, j0, c0 + KC);
-                        cp_async_wait<1>();
-                    } else {
-                        cp_async_wait<0>();
+                    for (int x = 0; x < 4; ++x) are[n8][x] = aim[n8][x] = 0.f;
+            }
+            cp_async_wait<ST - 2>();
+            __syncthreads();   // chunk q has landed for every thread, chunk q - 1 is consumed
+            issue(q + ST - 1);
+            const Cx<T>* cu = su + (q % ST) * KC * (TI + TJ);
+            const Cx<T>* cv = cu + KC * TI;
+#pragma unroll 1
+            for (int ks = 0; ks < min(KC, nc - c0); ks += 8) {
+                // A fragment (row i, column c): (g, t), (g + 8, t), (g, t + 4), (g + 8, t + 4)
+                unsigned urh[4], url[4], uih[4], uil[4], nrh[4], nrl[4];
+#pragma unroll
+                for (int y = 0; y < 2; ++y) {
+                    const int c = c0 + ks + t + y * 4;
+                    const Cx<T> fc = c < nc ? F.coef[c] : Cx<T>{0, 0};
+#pragma unroll
+                    for (int x = 2 * y; x < 2 * y + 2; ++x) {
+                        const Cx<T> u = cmul(fc, cu[(ks + t + y * 4) * TI + rw + g + (x & 1) * 8]);
+                        const Tf32Pair pr = tf32_split(u.x), pi = tf32_split(u.y);
+                        urh[x] = pr.hi;
+                        url[x] = pr.lo;
+                        uih[x] = pi.hi;
+                        uil[x] = pi.lo;
                     }
-                    __syncthreads();  // chunk c0 is in buffer b for every thread
-                    const Cx<T>* cu = bu[b];
-                    const Cx<T>* cv = cu + KC * TI;
-#pragma unroll
-                    for (int ks = 0; ks < KC; ks += 8) {
-                        // A fragment (row i, column c): (g, t), (g + 8, t), (g, t + 4), (g + 8, t + 4)
-                        unsigned urh[4], url[4], uih[4], uil[4], nrh[4], nrl[4];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const int c = c0 + ks + t + (q >> 1) * 4;
-                            const Cx<T> u = c < nc ? cmul(S.fk[F.colP[c]], cu[(ks + t + (q >> 1) * 4) * TI + rw + g + (q & 1) * 8])
-                                                   : Cx<T>{0, 0};
-                            const Tf32Pair pr = tf32_split(u.x), pi = tf32_split(u.y);
-                            urh[q] = pr.hi;
-                            url[q] = pr.lo;
-                            uih[q] = pi.hi;
-                            uil[q] = pi.lo;
-                        }
-                        tf32_neg4(urh, nrh);
-                        tf32_neg4(url, nrl);
-#pragma unroll
-                        for (int n8 = 0; n8 < 4; ++n8) {
-                            // B fragment (row c, column j): (t, g), (t + 4, g)
-                            unsigned vrh[2], vrl[2], vih[2], vil[2];
-#pragma unroll
-                            for (int q = 0; q < 2; ++q) {
-                                const Cx<T> v = cv[(ks + t + q * 4) * TJ + cw + n8 * 8 + g];
-                                const Tf32Pair pr = tf32_split(v.x), pi = tf32_split(v.y);
-                                vrh[q] = pr.hi;
-                                vrl[q] = pr.lo;
-                                vih[q] = pi.hi;
-                                vil[q] = pi.lo;
-                            }
-                            mma_tf32x3(are[n8], urh, url, vrh, vrl);
-                            mma_tf32x3(are[n8], uih, uil, vih, vil);
-                            mma_tf32x3(aim[n8], uih, uil, vrh, vrl);
-                            mma_tf32x3(aim[n8], nrh, nrl, vih, vil);
-                        }
-                    }
-                    __syncthreads();  // buffer b is consumed before the next chunk refills it
                 }
+                tf32_neg4(urh, nrh);
+                tf32_neg4(url, nrl);
+                // B fragments (row c, column j): (t, g), (t + 4, g), of the warp's four tiles
+                unsigned vrh[4][2], vrl[4][2], vih[4][2], vil[4][2];
+#pragma unroll
+                for (int n8 = 0; n8 < 4; ++n8)
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) {
+                        const Cx<T> v = cv[(ks + t + x * 4) * TJ + cw + n8 * 8 + g];
+                        const Tf32Pair pr = tf32_split(v.x), pi = tf32_split(v.y);
+                        vrh[n8][x] = pr.hi;
+                        vrl[n8][x] = pr.lo;
+                        vih[n8][x] = pi.hi;
+                        vil[n8][x] = pi.lo;
+                    }
+                // Re += ur vr + ui vi, Im += ui vr - ur vi, three products each (small
+                // terms first), ordered so that the eight products between two into the
+                // same accumulator are independent
+#define G3_MMA4(ACC, X, Y) \
+    _Pragma("unroll") for (int n8 = 0; n8 < 4; ++n8) mma_tf32(ACC[n8], X, Y[n8])
+                G3_MMA4(are, urh, vrl);
+                G3_MMA4(aim, uih, vrl);
+                G3_MMA4(are, url, vrh);
+                G3_MMA4(aim, uil, vrh);
+                G3_MMA4(are, uih, vil);
+                G3_MMA4(aim, nrh, vil);
+                G3_MMA4(are, uil, vih);
+                G3_MMA4(aim, nrl, vih);
+                G3_MMA4(are, urh, vrh);
+                G3_MMA4(aim, uih, vrh);
+                G3_MMA4(are, uih, vih);
+                G3_MMA4(aim, nrh, vih);
+#undef G3_MMA4
+            }
+            if (ch == nch - 1) {
+                const int i0 = (tile / ntj) * TI, j0 = (tile % ntj) * TJ;
                 // C fragment (row, column): (g, 2t), (g, 2t + 1), (g + 8, 2t), (g + 8, 2t + 1)
 #pragma unroll
-                for (int n8 = 0; n8 < 4; ++n8)
+                for (int hx = 0; hx < 16; hx += 8) {   // eight loads in flight
+                    Cx<T> e[8];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int gi = i0 + rw + g + (q >> 1) * 8, gj = j0 + cw + n8 * 8 + 2 * t + (q & 1);
+                    for (int x = 0; x < 8; ++x) {
+                        const int gi = i0 + rw + g + ((x >> 1) & 1) * 8, gj = j0 + cw + ((x + hx) >> 2) * 8 + 2 * t + (x & 1);
+                        e[x] = gi < M && gj < N ? ldcx(D + (size_t)gi * N + gj) : Cx<T>{0, 0};
+                    }
+#pragma unroll
+                    for (int x = 0; x < 8; ++x) {
+                        const int gi = i0 + rw + g + ((x >> 1) & 1) * 8, gj = j0 + cw + ((x + hx) >> 2) * 8 + 2 * t + (x & 1);
                         if (gi < M && gj < N) {
-                            Cx<T>* dp = D + (size_t)gi * N + gj;
-                            const Cx<T> e = *dp;
-                            *dp = Cx<T>{e.x - are[n8][q], e.y - aim[n8][q]};
+                            const Cx<T> v{e[x].x - are[(x + hx) >> 2][x & 3], e[x].y - aim[(x + hx) >> 2][x & 3]};
+                            D[(size_t)gi * N + gj] = v;
+                            dn += cabs2(v);
                         }
                     }
+                }
             }
         }
-        if (tid == 0) atomicAdd(&A.counters[7], (unsigned long long)M * N);
-        __syncthreads();
-        return;
-    }
+        cp_async_wait<0>();
+    } else if (nc > 0) {
+    dn = 0;
     for (int i0 = 0; i0 < M; i0 += TI) {
         for (int j0 = 0; j0 < N; j0 += TJ) {
             Cx<T> acc[4][4];
@@ -828,7 +958,7 @@ __device__ void face_dense_residual(const AcaArgs<T>& A, const Ws<T>& w, BlockSh
                 __syncthreads();  // the previous chunk is consumed
                 for (int e = tid; e < DRF_KC * TI; e += NT) {
                     const int kk = e / TI, ii = e - kk * TI, c = c0 + kk;
-                    su[e] = (c < nc && i0 + ii < M) ? cmul(S.fk[F.colP[c]], ldcx(A.pool + F.colU[c] + i0 + ii))
+                    su[e] = (c < nc && i0 + ii < M) ? cmul(F.coef[c], ldcx(A.pool + F.colU[c] + i0 + ii))
                                                     : Cx<T>{0, 0};
                 }
                 for (int e = tid; e < DRF_KC * TJ; e += NT) {
@@ -858,10 +988,16 @@ __device__ void face_dense_residual(const AcaArgs<T>& A, const Ws<T>& w, BlockSh
 #pragma unroll
                 for (int b = 0; b < 4; ++b) {
                     const int gi = i0 + ty * 4 + a, gj = j0 + tx * 4 + b;
-                    if (gi < M && gj < N) D[(size_t)gi * N + gj] = acc[a][b];
+                    if (gi < M && gj < N) {
+                        D[(size_t)gi * N + gj] = acc[a][b];
+                        dn += cabs2(acc[a][b]);
+                    }
                 }
         }
     }
+    }
+    dn = warp_sum(dn);
+    if ((tid & 31) == 0) S.nrm[tid >> 5] = make_float2(dn, 0.f);
     if (tid == 0) atomicAdd(&A.counters[7], (unsigned long long)M * N);
     __syncthreads();
 }

@@ -582,11 +582,9 @@ __device__ inline void ss_point(const SsPanels& S, int cas, int m, const double 
 // accumulation, in the three-term split a b ~ a_hi b_hi + a_hi b_lo + a_lo b_hi (a_hi =
 // a rounded to TF32, a_lo = the rounded remainder), which keeps float32 accuracy (about
 // 2^-21 relative per product instead of TF32's 2^-11).
-__device__ __forceinline__ unsigned tf32_rna(float x) {
-    unsigned r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return r;
-}
+// (rounding to TF32, nearest with ties away from zero, in two integer operations:
+// the conversion instruction issues at the special-function rate)
+__device__ __forceinline__ unsigned tf32_rna(float x) { return (__float_as_uint(x) + 0x1000u) & 0xffffe000u; }
 struct Tf32Pair {
     unsigned hi, lo;
 };

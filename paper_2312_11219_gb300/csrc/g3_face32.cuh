@@ -52,6 +52,33 @@ __device__ __forceinline__ void ff_add_prod(float2& a, float x, float y) {
     ff_add(a, p, fmaf(x, y, -p));
 }
 
+// four sums over a warp with six exchanges instead of twenty: the halves of
+// the warp first split the values between them, then the lanes below.
+// Lanes 0-15 get (sum a, sum b), lanes 16-31 (sum c, sum d).
+__device__ __forceinline__ float2 warp_sum4(float a, float b, float c, float d) {
+    const int lane = threadIdx.x & 31;
+    const bool h16 = (lane & 16) != 0, h8 = (lane & 8) != 0;
+    float x = h16 ? c : a, y = h16 ? d : b;
+    x += __shfl_xor_sync(0xffffffffu, h16 ? a : c, 16);
+    y += __shfl_xor_sync(0xffffffffu, h16 ? b : d, 16);
+    float z = (h8 ? y : x) + __shfl_xor_sync(0xffffffffu, h8 ? x : y, 8);
+    z += __shfl_xor_sync(0xffffffffu, z, 4);
+    z += __shfl_xor_sync(0xffffffffu, z, 2);
+    z += __shfl_xor_sync(0xffffffffu, z, 1);
+    // every lane of a half holds its x sum (lanes 0-7, 16-23) or its y sum
+    const float w = __shfl_xor_sync(0xffffffffu, z, 8);
+    return h8 ? make_float2(w, z) : make_float2(z, w);
+}
+
+// two complex sums over a warp, known to every lane
+__device__ __forceinline__ void warp_sum_pair(Cx<float>& p, Cx<float>& q) {
+    const float2 v = warp_sum4(p.x, p.y, q.x, q.y);
+    const bool hi = (threadIdx.x & 16) != 0;
+    const float ox = __shfl_xor_sync(0xffffffffu, v.x, 16), oy = __shfl_xor_sync(0xffffffffu, v.y, 16);
+    p = hi ? Cx<float>{ox, oy} : Cx<float>{v.x, v.y};
+    q = hi ? Cx<float>{v.x, v.y} : Cx<float>{ox, oy};
+}
+
 // warp argmax of non-negative float32 values, ties to the smallest index:
 // {value bits + 1 (0: no candidate), index}
 __device__ __forceinline__ uint2 warp_key(ArgMaxT<float> a) {
@@ -71,6 +98,12 @@ __device__ __forceinline__ ArgMaxT<float> block_key(const uint2* k) {
     }
     if (b.x == 0u) return amax_none<float>();
     return ArgMaxT<float>{__uint_as_float(b.x - 1u), (int)b.y};
+}
+
+// rows already taken by the face ACA: a bit mask in shared memory (blocks of
+// more than 32 USED_W rows: bytes in the workspace)
+__device__ __forceinline__ bool row_used(const BlockSh<float>& S, const Ws<float>& w, int i) {
+    return S.M <= 32 * USED_W ? (S.usedm[i >> 5] >> (i & 31)) & 1u : w.used[i] != 0;
 }
 
 // the part of a gang in sum_t u_t[fix] conj(v_t[v]) (ROW) or
@@ -111,7 +144,7 @@ __device__ __forceinline__ Cx<float> cur_sum(const ColStore& c, int fix, int v, 
 template <int KER, int NT, bool ROW>
 __device__ __forceinline__ ArgMaxT<float> line32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float>& S,
                                                  const FaceTab<float>& F, const ColStore& c, int fix, int skip, int kf,
-                                                 int m, Cx<float>* out, const Cx<float>* D) {
+                                                 int m, Cx<float>* out, const Cx<float>* D, float* n2 = nullptr) {
     const int tid = threadIdx.x;
     const int M = S.M, N = S.N;
     const int L = ROW ? N : M;
@@ -136,7 +169,7 @@ __device__ __forceinline__ ArgMaxT<float> line32(const AcaArgs<float>& A, const 
                 acc.x -= (s0.x + s1.x) + (s2.x + s3.x);
                 acc.y -= (s0.y + s1.y) + (s2.y + s3.y);
             }
-            cand = part == 0 && (ROW || (v != skip && !w.used[v]));
+            cand = part == 0 && (ROW || (v != skip && !row_used(S, w, v)));
             const Cx<float> q = cur_sum<ROW>(c, fix, v, m, part, G);
             acc.x -= q.x;
             acc.y -= q.y;
@@ -148,6 +181,7 @@ __device__ __forceinline__ ArgMaxT<float> line32(const AcaArgs<float>& A, const 
         }
         if (part == 0 && v < L) {
             out[v] = acc;
+            if (n2) *n2 += cabs2(acc);
             if (cand) am = amax_better(am, ArgMaxT<float>{cabs2(acc), v});
         }
     }
@@ -179,15 +213,16 @@ __device__ void samples32(const AcaArgs<float>& A, BlockSh<float>& S, const Face
 }
 
 // Partial-pivot ACA of the residual face at frequency kf.  Returns the rank m;
-// c holds the crosses.  Same rows, columns and tests as the float64 face_aca.
-//
-// Two barriers per step.  Between them run (1) the residual row of the next
-// pivot row together with the newest cross's terms of the recursive Frobenius
-// norm
-//   ||S_m||^2 = ||S_{m-1}||^2 + 2 Re sum_t (u_t^H u_m)(v_m^H v_t) + ||u_m||^2 ||v_m||^2,
-// and (2) the column of the row's pivot.  The test of cross m - 1 is thus
-// evaluated with the row of cross m in hand; when it passes, that row is
-// dropped.
+// c holds the crosses.  Rows, columns and tests as in the float64 face_aca:
+//   ||u_m|| ||v_m|| <= eps_face ||S_m||_F  (or the absolute floor), confirmed on
+//   the sample entries.
+// Two barriers per step: the residual row and its largest entry; then the
+// column of that entry, the norms of both and the test.  With the dense
+// residual working face D, ||D||_F stands for ||S_m||_F: the two agree to
+// eps_face where the test can pass, and D's norm is a by-product of forming it.
+// Without D, ||S_m||_F is the recursive
+//   ||S_m||^2 = ||S_{m-1}||^2 + 2 Re sum_t (u_t^H u_m)(v_m^H v_t) + ||u_m||^2 ||v_m||^2
+// (a third barrier; the sum over t took a third of the step's instructions).
 template <int KER, int NT>
 __device__ int face32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float>& S, int kf, unsigned char* arena,
                       ColStore& c) {
@@ -203,13 +238,17 @@ __device__ int face32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float
     for (int p = tid; p < nc; p += NT) S.fk[p] = Fp(A, S, p)[kf];
     long long tf = clock64();
     FaceTab<float> F = facetab_build<float, NT>(A, w, S, arena);
-    for (int i = tid; i < M; i += NT) w.used[i] = 0;
+    if (M <= 32 * USED_W) {
+        if (tid < USED_W) S.usedm[tid] = 0u;
+    } else {
+        for (int i = tid; i < M; i += NT) w.used[i] = 0;
+    }
     __syncthreads();
     const Cx<float>* D = nullptr;
     size_t off = (facetab_smem_bytes<float>() + 255) & ~size_t(255);
     if constexpr (KER != G3_SEPARABLE) {
         if (w.dres && (long long)M * N <= A.drf_max) {
-            face_dense_residual<KER, float, NT>(A, w, S, F, kf, arena);
+            face_dense_residual<KER, float, NT>(A, w.dres, S, F, kf);
             D = w.dres;
             // the tables are not needed any more: only the row buffer stays
             F.ncol = 0;
@@ -222,113 +261,42 @@ __device__ int face32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float
     c.ncs = (size_t)A.arena_bytes > off ? (int)(((size_t)A.arena_bytes - off) / ((size_t)c.ld * sizeof(Cx<float>))) : 0;
     c.ncs = min(c.ncs, A.RF);
     int m = 0, irow = 0;
-    bool converged = false, pending = false, last = false;
-    float2 fsn2 = make_float2(0.f, 0.f);  // ||S_m||^2 (the same in every thread)
+    bool converged = false;
+    // ||S_m||_F^2 (the same in every thread)
+    float2 fsn2 = make_float2(0.f, 0.f);
+    if (D) {
+        for (int q = 0; q < NW; ++q) ff_add(fsn2, S.nrm[q].x, 0.f);
+        __syncthreads();   // S.nrm is rewritten by the first step
+    }
     // own <= max(eps^2 ||S||^2, floor^2), divided by eps^2 (eps^2 alone can take
     // the norms of strongly damped faces below the float32 range)
     const float e1 = (float)A.eps_face, inv_e2 = 1.f / (e1 * e1);
     const float fl = (float)A.face_floor / e1, floor_s = fl * fl * ((float)S.norm2 / (float)A.Ku);
-    for (;;) {
-        // ---- (1) residual row, and the norm terms of the newest cross ----
-        ArgMaxT<float> am = amax_none<float>();
-        if (m < cap && !last) {
-            if (F.ncol > 0) {
-                // (the current columns' coefficients are read from c directly)
-                for (int q = tid; q < F.ncol; q += NT) F.coef[q] = cmul(S.fk[F.colP[q]], A.pool[F.colU[q] + irow]);
-                __syncthreads();
-            }
-            am = line32<KER, NT, true>(A, w, S, F, c, irow, -1, kf, m, F.row, D);
+    while (m < cap) {
+        // ---- the residual row ----
+        if (F.ncol > 0) {
+            // (the current columns' coefficients are read from c directly)
+            for (int q = tid; q < F.ncol; q += NT) F.coef[q] = cmul(S.fk[F.colP[q]], A.pool[F.colU[q] + irow]);
+            __syncthreads();
         }
-        if (pending) {
-            const int mm = m - 1;
-            const Cx<float>* um = cs_u<false>(c, mm);
-            const Cx<float>* vm = um + M;
-            float2 part = make_float2(0.f, 0.f);
-            for (int t = wid; t <= mm; t += NW) {
-                const Cx<float>* ut = cs_u<false>(c, t);
-                const Cx<float>* vt = ut + M;
-                Cx<float> gu{0, 0}, gv{0, 0};
-#pragma unroll 4
-                for (int i = lane; i < M; i += 32) cfmac(gu, ldcx(um + i), ldcx(ut + i));  // conj(u_t) u_m
-#pragma unroll 4
-                for (int i = lane; i < N; i += 32) cfmac(gv, ldcx(vt + i), ldcx(vm + i));  // conj(v_m) v_t
-                gu.x = warp_sum(gu.x);
-                gu.y = warp_sum(gu.y);
-                gv.x = warp_sum(gv.x);
-                gv.y = warp_sum(gv.y);
-                if (t < mm) {
-                    ff_add_prod(part, 2.f * gu.x, gv.x);
-                    ff_add_prod(part, -2.f * gu.y, gv.y);
-                } else {
-                    float2 own = make_float2(0.f, 0.f);
-                    ff_add_prod(own, gu.x, gv.x);
-                    if (lane == 0) S.own = own;
-                }
-            }
-            if (lane == 0) S.nrm[wid] = part;
-        }
+        ArgMaxT<float> am = line32<KER, NT, true>(A, w, S, F, c, irow, -1, kf, m, F.row, D);
         {
             const uint2 k = warp_key(am);
             if (lane == 0) S.key[0][wid] = k;
         }
-        __syncthreads();
-        if (pending) {
-            pending = false;
-            const float2 own = S.own;
-#pragma unroll
-            for (int q = 0; q < NW; ++q) {
-                const float2 p = S.nrm[q];
-                ff_add(fsn2, p.x, p.y);
-            }
-            ff_add(fsn2, own.x, own.y);
-            if (own.x * inv_e2 <= fmaxf(fmaxf(fsn2.x, 0.f), floor_s)) {
-                if (!A.sample_check) {
-                    converged = true;
-                    break;
-                }
-                // confirm on the sample entries: partial pivoting can miss a block
-                // of the face that no visited row or column reaches
-                sublap(S, 6, tf);
-                samples32<KER, NT>(A, S, F, c, kf, m, D);
-                static_assert(SAMPLES == 32, "one sample per lane");
-                if (wid == 0) {
-                    const double sv = S.samp[lane];
-                    const double tot = warp_sum(sv);
-                    ArgMaxT<float> b{(float)sv, lane};
-                    b = warp_argmax(b);
-                    if (lane == 0) {
-                        const double e2 = A.eps_face * A.eps_face;
-                        S.fconv = (double)M * (double)N / SAMPLES * tot <=
-                                  fmax(e2 * fmax((double)fsn2.x + (double)fsn2.y, 0.0),
-                                       A.face_floor * A.face_floor * S.norm2 / (double)A.Ku);
-                        S.fbs = b.i;
-                    }
-                }
-                __syncthreads();
-                const bool ok = S.fconv;
-                const int bs = S.fbs;
-                __syncthreads();  // both are rewritten by the next test
-                sublap(S, 9, tf);
-                if (ok) {
-                    converged = true;
-                    break;
-                }
-                if (tid == 0) atomicAdd(&A.counters[5], 1ull);
-                irow = (2 * bs + 1) * M / (2 * SAMPLES);
-                last = false;
-                if (m < cap) continue;
-            }
+        if (tid == 0) {
+            if (M <= 32 * USED_W) S.usedm[irow >> 5] |= 1u << (irow & 31);
+            else w.used[irow] = 1;
         }
-        if (m >= cap || last) break;  // the cap, or every row used
+        __syncthreads();
         am = block_key<NT>(S.key[0]);
-        if (tid == 0) w.used[irow] = 1;
         // a row counts as nonzero when |delta|^2 is a normal number of the
         // working precision (below that the entries are far under any tolerance)
         if (!(am.v > tiny_norm2<float>())) {
             // zero residual row: next unused row in index order
             ArgMaxT<float> un = amax_none<float>();
             for (int i = tid; i < M; i += NT)
-                if (i != irow && !w.used[i]) un = amax_better(un, ArgMaxT<float>{0.f, i});
+                if (!row_used(S, w, i)) un = amax_better(un, ArgMaxT<float>{0.f, i});
             un = block_argmax<NT>(un, S.am);
             if (un.v < 0.f) break;  // no row with a nonzero residual left
             irow = un.i;
@@ -336,7 +304,7 @@ __device__ int face32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float
         }
         const int jp = am.i;
         sublap(S, 6, tf);
-        // ---- (2) v = conj(row / delta), the column of the pivot ----
+        // ---- v = conj(row / delta), the column of the pivot ----
         // delta is scaled to magnitude ~1 first, so that a tiny pivot of a strongly
         // damped face cannot overflow 1 / |delta|^2 (|row[j]| <= |delta|)
         const Cx<float> delta = F.row[jp];
@@ -349,23 +317,95 @@ __device__ int face32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float
         }
         Cx<float>* um = cs_u<false>(c, m);
         Cx<float>* vm = um + M;
+        float nv2 = 0, nu2 = 0;
         for (int j = tid; j < N; j += NT) {
             const Cx<float> rj = F.row[j];
             const Cx<float> q = cmulc(Cx<float>{rj.x * sc, rj.y * sc}, ds);  // (row / s) conj(delta / s)
-            vm[j] = Cx<float>{q.x * dn, -q.y * dn};                          // conj(row / delta)
+            const Cx<float> v{q.x * dn, -q.y * dn};                          // conj(row / delta)
+            vm[j] = v;
+            nv2 += cabs2(v);
         }
-        ArgMaxT<float> nx = line32<KER, NT, false>(A, w, S, F, c, jp, irow, kf, m, um, D);
+        ArgMaxT<float> nx = line32<KER, NT, false>(A, w, S, F, c, jp, irow, kf, m, um, D, &nu2);
         {
             const uint2 k = warp_key(nx);
-            if (lane == 0) S.key[1][wid] = k;
+            nu2 = warp_sum(nu2);
+            nv2 = warp_sum(nv2);
+            if (lane == 0) {
+                S.key[1][wid] = k;
+                S.nrm[wid] = make_float2(nu2, nv2);
+            }
         }
         __syncthreads();
         nx = block_key<NT>(S.key[1]);
-        ++m;
-        pending = true;
-        last = nx.v < 0.f;  // every row used: one more test, then the end
-        if (!last) irow = nx.i;
+        nu2 = nv2 = 0;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+            const float2 x = S.nrm[q];
+            nu2 += x.x;
+            nv2 += x.y;
+        }
         sublap(S, 7, tf);
+        if (!D) {
+            // the recursive norm's cross terms, in float-float
+            float2 part = make_float2(0.f, 0.f);
+            for (int t = wid; t < m; t += NW) {
+                const Cx<float>* ut = cs_u<false>(c, t);
+                const Cx<float>* vt = ut + M;
+                Cx<float> gu{0, 0}, gv{0, 0};
+#pragma unroll 4
+                for (int i = lane; i < M; i += 32) cfmac(gu, ldcx(um + i), ldcx(ut + i));  // conj(u_t) u_m
+#pragma unroll 4
+                for (int i = lane; i < N; i += 32) cfmac(gv, ldcx(vt + i), ldcx(vm + i));  // conj(v_m) v_t
+                // lanes 0-15: Re gu, Re gv; lanes 16-31: Im gu, Im gv
+                const float2 g = warp_sum4(gu.x, gv.x, gu.y, gv.y);
+                ff_add_prod(part, (lane & 16) ? -2.f * g.x : 2.f * g.x, g.y);
+            }
+            const float px = __shfl_xor_sync(0xffffffffu, part.x, 16), py = __shfl_xor_sync(0xffffffffu, part.y, 16);
+            ff_add(part, px, py);
+            if (lane == 0) S.crs[wid] = part;
+            __syncthreads();
+            for (int q = 0; q < NW; ++q) ff_add(fsn2, S.crs[q].x, S.crs[q].y);
+            ff_add_prod(fsn2, nu2, nv2);
+            sublap(S, 8, tf);
+        }
+        ++m;
+        if (nu2 * nv2 * inv_e2 <= fmaxf(fmaxf(fsn2.x, 0.f), floor_s)) {
+            if (!A.sample_check) {
+                converged = true;
+                break;
+            }
+            // confirm on the sample entries: partial pivoting can miss a block
+            // of the face that no visited row or column reaches
+            samples32<KER, NT>(A, S, F, c, kf, m, D);
+            static_assert(SAMPLES == 32, "one sample per lane");
+            if (wid == 0) {
+                const double sv = S.samp[lane];
+                const double tot = warp_sum(sv);
+                ArgMaxT<float> b{(float)sv, lane};
+                b = warp_argmax(b);
+                if (lane == 0) {
+                    const double e2 = A.eps_face * A.eps_face;
+                    S.fconv = (double)M * (double)N / SAMPLES * tot <=
+                              fmax(e2 * fmax((double)fsn2.x + (double)fsn2.y, 0.0),
+                                   A.face_floor * A.face_floor * S.norm2 / (double)A.Ku);
+                    S.fbs = b.i;
+                }
+            }
+            __syncthreads();
+            const bool ok = S.fconv;
+            const int bs = S.fbs;
+            __syncthreads();  // both are rewritten by the next test
+            sublap(S, 9, tf);
+            if (ok) {
+                converged = true;
+                break;
+            }
+            if (tid == 0) atomicAdd(&A.counters[5], 1ull);
+            irow = (2 * bs + 1) * M / (2 * SAMPLES);
+            continue;
+        }
+        if (nx.v < 0.f) break;  // every row used
+        irow = nx.i;
     }
     if (tid == 0) S.raw += m;
     if (!converged && m == A.RF && m < min(M, N)) {
@@ -435,13 +475,7 @@ __device__ int recompress32_t(const AcaArgs<float>& A, BlockSh<float>& S, const 
                 cfmac(ga, ldcx(va + i), q);  // conj(v_k) v_j
                 cfmac(gb, ldcx(vb + i), q);
             }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                ga.x += __shfl_xor_sync(0xffffffffu, ga.x, o);
-                ga.y += __shfl_xor_sync(0xffffffffu, ga.y, o);
-                gb.x += __shfl_xor_sync(0xffffffffu, gb.x, o);
-                gb.y += __shfl_xor_sync(0xffffffffu, gb.y, o);
-            }
+            warp_sum_pair(ga, gb);
             ga.x *= inv;
             ga.y *= inv;
             gb.x *= inv;
@@ -566,13 +600,7 @@ __device__ int recompress32_t(const AcaArgs<float>& A, BlockSh<float>& S, const 
                     cfmac(ga, ldcx(xa + i), q);
                     cfmac(gb, ldcx(xb + i), q);
                 }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    ga.x += __shfl_xor_sync(0xffffffffu, ga.x, o);
-                    ga.y += __shfl_xor_sync(0xffffffffu, ga.y, o);
-                    gb.x += __shfl_xor_sync(0xffffffffu, gb.x, o);
-                    gb.y += __shfl_xor_sync(0xffffffffu, gb.y, o);
-                }
+                warp_sum_pair(ga, gb);
                 ga.x *= inv;
                 ga.y *= inv;
                 gb.x *= inv;
