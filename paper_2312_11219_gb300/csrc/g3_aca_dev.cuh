@@ -666,6 +666,7 @@ __device__ void face_samples(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S,
 // tensor cores at 256 threads (the TF32 three-term split, float32 accuracy),
 // else on the CUDA cores (a 4 x 4 micro-tile per thread).  Float32 only.
 constexpr int DRF_KC = 16;     // columns per staged chunk
+constexpr int DRF_PAD = 4;     // padding of a staged column: the four columns of a fragment fall in different banks
 constexpr int DRF_ST = 3;      // staging buffers of the tensor-core path (256 threads)
 // shared-memory staging of the dense residual face, placed after the face's
 // column tables and coefficients (the row buffer that follows them is not in use
@@ -677,7 +678,7 @@ constexpr size_t drf_stage_offset() {
 }
 template <class T, int NT>
 constexpr size_t drf_stage_bytes() {
-    return (size_t)(NT == 256 ? DRF_ST : 1) * DRF_KC * (64 + NT / 4) * sizeof(Cx<T>);
+    return (size_t)(NT == 256 ? DRF_ST : 1) * DRF_KC * (64 + NT / 4 + 2 * DRF_PAD) * sizeof(Cx<T>);
 }
 
 constexpr int DRF_RB = 24;     // rows per warp and pass of the entries
@@ -825,47 +826,56 @@ __device__ __noinline__ void face_dense_residual(const AcaArgs<T>& A, Cx<T>* __r
         // ST staging buffers of KC columns each, filled by cp.async (8 bytes per
         // element, zero-filled outside the face and past the last column) ST - 1
         // chunks ahead of the tensor cores, over the chunks of all tiles in one
-        // sequence: the L2 latency is two to three chunks of work (with one chunk
-        // ahead the product waited on it: 2,100 SM cycles per 64 x 64 x 8 against
-        // ~450 issued).  f_p[kf] is applied to the A fragments.
-        const int nch = (nc + KC - 1) / KC, ntj = (N + TJ - 1) / TJ, nti = (M + TI - 1) / TI;
-        const int total = nch * ntj * nti;
+        // sequence.  f_p[kf] is applied to the A fragments.
+        constexpr int SU = TI + DRF_PAD, SV = TJ + DRF_PAD, BUF = KC * (SU + SV);
         const int sc = tid % 64, sk = tid / 64;   // staged element: column part and offset
         static_assert(TI == 64 && TJ == 64 && NT == 256, "staging map");
-        auto issue = [&](int q) {
-            if (q < total) {
-                const int tile = q / nch, c0 = (q - tile * nch) * KC;
-                const int i0 = (tile / ntj) * TI, j0 = (tile % ntj) * TJ;
-                Cx<T>* du = su + (q % ST) * KC * (TI + TJ);
-                Cx<T>* dv = du + KC * TI;
-                const bool iu = i0 + sc < M, iv = j0 + sc < N;
+        int qi = 0, qj = 0, qc = 0, qb = 0;       // next chunk to stage: tile, first column, buffer
+        auto issue = [&]() {
+            if (nc > 0 && qi < M) {
+                Cx<T>* du = su + qb * BUF;
+                Cx<T>* dv = du + KC * SU;
+                const bool iu = qi + sc < M, iv = qj + sc < N;
 #pragma unroll
                 for (int x = 0; x < KC; x += 4) {
-                    const int kk = x + sk, c = c0 + kk;
+                    const int kk = x + sk, c = qc + kk;
                     const bool in = c < nc;
-                    cp_async8(du + kk * TI + sc, in && iu ? A.pool + F.colU[c] + i0 + sc : A.pool, in && iu);
-                    cp_async8(dv + kk * TJ + sc, in && iv ? A.pool + F.colV[c] + j0 + sc : A.pool, in && iv);
+                    cp_async8(du + kk * SU + sc, in && iu ? A.pool + F.colU[c] + qi + sc : A.pool, in && iu);
+                    cp_async8(dv + kk * SV + sc, in && iv ? A.pool + F.colV[c] + qj + sc : A.pool, in && iv);
+                }
+                qb = qb + 1 == ST ? 0 : qb + 1;
+                qc += KC;
+                if (qc >= nc) {
+                    qc = 0;
+                    qj += TJ;
+                    if (qj >= N) {
+                        qj = 0;
+                        qi += TI;
+                    }
                 }
             }
             cp_async_commit();   // (an empty group past the end keeps the count)
         };
 #pragma unroll 1
-        for (int q = 0; q < ST - 1; ++q) issue(q);
+        for (int q = 0; q < ST - 1; ++q) issue();
         float are[4][4], aim[4][4];
-        if (total > 0) dn = 0;
-        for (int q = 0; q < total; ++q) {
-            const int tile = q / nch, ch = q - tile * nch, c0 = ch * KC;
-            if (ch == 0) {
+        if (nc > 0) dn = 0;
+        int buf = 0;
+        const bool pairs = (N & 1) == 0;   // 16-byte accesses of D
+        for (int i0 = 0; nc > 0 && i0 < M; i0 += TI)
+        for (int j0 = 0; j0 < N; j0 += TJ) {
 #pragma unroll
-                for (int n8 = 0; n8 < 4; ++n8)
+            for (int n8 = 0; n8 < 4; ++n8)
 #pragma unroll
-                    for (int x = 0; x < 4; ++x) are[n8][x] = aim[n8][x] = 0.f;
-            }
+                for (int x = 0; x < 4; ++x) are[n8][x] = aim[n8][x] = 0.f;
+#pragma unroll 1
+        for (int c0 = 0; c0 < nc; c0 += KC) {
             cp_async_wait<ST - 2>();
-            __syncthreads();   // chunk q has landed for every thread, chunk q - 1 is consumed
-            issue(q + ST - 1);
-            const Cx<T>* cu = su + (q % ST) * KC * (TI + TJ);
-            const Cx<T>* cv = cu + KC * TI;
+            __syncthreads();   // this chunk has landed for every thread, the last one is consumed
+            issue();
+            const Cx<T>* cu = su + buf * BUF;
+            const Cx<T>* cv = cu + KC * SU;
+            buf = buf + 1 == ST ? 0 : buf + 1;
 #pragma unroll 1
             for (int ks = 0; ks < min(KC, nc - c0); ks += 8) {
                 // A fragment (row i, column c): (g, t), (g + 8, t), (g, t + 4), (g + 8, t + 4)
@@ -876,7 +886,7 @@ __device__ __noinline__ void face_dense_residual(const AcaArgs<T>& A, Cx<T>* __r
                     const Cx<T> fc = c < nc ? F.coef[c] : Cx<T>{0, 0};
 #pragma unroll
                     for (int x = 2 * y; x < 2 * y + 2; ++x) {
-                        const Cx<T> u = cmul(fc, cu[(ks + t + y * 4) * TI + rw + g + (x & 1) * 8]);
+                        const Cx<T> u = cmul(fc, cu[(ks + t + y * 4) * SU + rw + g + (x & 1) * 8]);
                         const Tf32Pair pr = tf32_split(u.x), pi = tf32_split(u.y);
                         urh[x] = pr.hi;
                         url[x] = pr.lo;
@@ -892,7 +902,7 @@ __device__ __noinline__ void face_dense_residual(const AcaArgs<T>& A, Cx<T>* __r
                 for (int n8 = 0; n8 < 4; ++n8)
 #pragma unroll
                     for (int x = 0; x < 2; ++x) {
-                        const Cx<T> v = cv[(ks + t + x * 4) * TJ + cw + n8 * 8 + g];
+                        const Cx<T> v = cv[(ks + t + x * 4) * SV + cw + n8 * 8 + g];
                         const Tf32Pair pr = tf32_split(v.x), pi = tf32_split(v.y);
                         vrh[n8][x] = pr.hi;
                         vrl[n8][x] = pr.lo;
@@ -918,26 +928,42 @@ __device__ __noinline__ void face_dense_residual(const AcaArgs<T>& A, Cx<T>* __r
                 G3_MMA4(aim, nrh, vih);
 #undef G3_MMA4
             }
-            if (ch == nch - 1) {
-                const int i0 = (tile / ntj) * TI, j0 = (tile % ntj) * TJ;
-                // C fragment (row, column): (g, 2t), (g, 2t + 1), (g + 8, 2t), (g + 8, 2t + 1)
+        }
+            // C fragment (row, column): (g, 2t), (g, 2t + 1), (g + 8, 2t), (g + 8, 2t + 1)
 #pragma unroll
-                for (int hx = 0; hx < 16; hx += 8) {   // eight loads in flight
-                    Cx<T> e[8];
+            for (int h = 0; h < 2; ++h) {
+                const int gi = i0 + rw + g + h * 8;
+                float4 e[4];
 #pragma unroll
-                    for (int x = 0; x < 8; ++x) {
-                        const int gi = i0 + rw + g + ((x >> 1) & 1) * 8, gj = j0 + cw + ((x + hx) >> 2) * 8 + 2 * t + (x & 1);
-                        e[x] = gi < M && gj < N ? ldcx(D + (size_t)gi * N + gj) : Cx<T>{0, 0};
-                    }
-#pragma unroll
-                    for (int x = 0; x < 8; ++x) {
-                        const int gi = i0 + rw + g + ((x >> 1) & 1) * 8, gj = j0 + cw + ((x + hx) >> 2) * 8 + 2 * t + (x & 1);
-                        if (gi < M && gj < N) {
-                            const Cx<T> v{e[x].x - are[(x + hx) >> 2][x & 3], e[x].y - aim[(x + hx) >> 2][x & 3]};
-                            D[(size_t)gi * N + gj] = v;
-                            dn += cabs2(v);
+                for (int n8 = 0; n8 < 4; ++n8) {
+                    const int gj = j0 + cw + n8 * 8 + 2 * t;
+                    const Cx<T>* dp = D + (size_t)gi * N + gj;
+                    e[n8] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (gi < M && gj + 1 < N && pairs) {
+                        e[n8] = *reinterpret_cast<const float4*>(dp);
+                    } else if (gi < M && gj < N) {
+                        e[n8].x = dp[0].x;
+                        e[n8].y = dp[0].y;
+                        if (gj + 1 < N) {
+                            e[n8].z = dp[1].x;
+                            e[n8].w = dp[1].y;
                         }
                     }
+                }
+#pragma unroll
+                for (int n8 = 0; n8 < 4; ++n8) {
+                    const int gj = j0 + cw + n8 * 8 + 2 * t;
+                    Cx<T>* dp = D + (size_t)gi * N + gj;
+                    // (outside the face both operands are zero)
+                    const float4 v = make_float4(e[n8].x - are[n8][2 * h], e[n8].y - aim[n8][2 * h],
+                                                 e[n8].z - are[n8][2 * h + 1], e[n8].w - aim[n8][2 * h + 1]);
+                    if (gi < M && gj + 1 < N && pairs) {
+                        *reinterpret_cast<float4*>(dp) = v;
+                    } else if (gi < M && gj < N) {
+                        dp[0] = Cx<T>{v.x, v.y};
+                        if (gj + 1 < N) dp[1] = Cx<T>{v.z, v.w};
+                    }
+                    dn += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
                 }
             }
         }
@@ -1722,6 +1748,29 @@ __device__ void norm_grams(const AcaArgs<T>& A, BlockSh<T>& S, const Cx<T>* Un, 
     }
 }
 
+// ||C^(l)||^2 and Algorithm 1's stopping test from the inner products (warp 0;
+// visible to the others after the next barrier).  S.flag: every frequency used.
+template <class T>
+__device__ __forceinline__ bool all_used(const AcaArgs<T>& A, const BlockSh<T>& S) {
+    int n = 0;
+    for (int i = 0; i < KU_MAX / 32; ++i) n += __popc(S.used_k[i]);
+    return n >= A.Ku;
+}
+template <class T>
+__device__ __forceinline__ void norm_test(const AcaArgs<T>& A, BlockSh<T>& S, int nc) {
+    if (threadIdx.x < 32) {
+        double add = 0.0;
+        for (int d = threadIdx.x; d < nc; d += 32) add += 2.0 * (S.hh[d].x * S.ff[d].x - S.hh[d].y * S.ff[d].y);
+        add = warp_sum(add);
+        if (threadIdx.x == 0) {
+            const double own = S.hself * S.fself;
+            S.norm2 += add + own;
+            S.stop = sqrt(fmax(own, 0.0)) <= A.eps3 * sqrt(fmax(S.norm2, 0.0));
+            S.flag = all_used(A, S);
+        }
+    }
+}
+
 // ---- confirmed stop --------------------------------------------------------------------
 // Algorithm 1's test measures only the newest cross.  When it passes, the
 // residual of the approximant with crosses 0..ncl-1 (the newest one included,
@@ -1762,24 +1811,27 @@ __device__ __noinline__ bool confirm_stop(const AcaArgs<T>& A, const Ws<T>& w, B
         S.entries += (long long)SAMPLES * Ku;
     }
     __syncthreads();
+    // items (sample, frequency), frequencies fastest; the residual energy per
+    // frequency is summed in shared memory (S.hh is not in use here)
+    double* rk = reinterpret_cast<double*>(S.hh);
+    for (int k = tid; k < Ku; k += NT) rk[k] = 0.0;
+    __syncthreads();
     double rr_t = 0.0, aa_t = 0.0;
-    for (int k = tid; k < Ku; k += NT) {
-        double rr = 0.0, aa = 0.0;
-        for (int sm = 0; sm < SAMPLES; ++sm) {
-            const int i = (2 * sm + 1) * M / (2 * SAMPLES), j = (2 * ((11 * sm) % SAMPLES) + 1) * N / (2 * SAMPLES);
-            const Cx<T> a = ent<KER, T>(A, S.rb + i, S.cb + j, k);
-            Cx<T> r = a;
-            for (int p = 0; p < ncl; ++p) {
-                const Cx<T> c = cmul(hs[sm * A.Cmax + p], f_of(A, S, p)[k]);
-                r.x -= c.x;
-                r.y -= c.y;
-            }
-            rr += cabs2d(r);
-            aa += cabs2d(a);
+    for (int e = tid; e < SAMPLES * Ku; e += NT) {
+        const int sm = e / Ku, k = e - sm * Ku;
+        const int i = (2 * sm + 1) * M / (2 * SAMPLES), j = (2 * ((11 * sm) % SAMPLES) + 1) * N / (2 * SAMPLES);
+        const Cx<T> a = ent<KER, T>(A, S.rb + i, S.cb + j, k);
+        Cx<T> r = a;
+#pragma unroll 4
+        for (int p = 0; p < ncl; ++p) {
+            const Cx<T> c = cmul(hs[sm * A.Cmax + p], ldcx(f_of(A, S, p) + k));
+            r.x -= c.x;
+            r.y -= c.y;
         }
-        w.rk[k] = rr;
+        const double rr = cabs2d(r);
+        atomicAdd(&rk[k], rr);
         rr_t += rr;
-        aa_t += aa;
+        aa_t += cabs2d(a);
     }
     rr_t = warp_sum(rr_t);
     aa_t = warp_sum(aa_t);
@@ -1788,6 +1840,7 @@ __device__ __noinline__ bool confirm_stop(const AcaArgs<T>& A, const Ws<T>& w, B
         atomicAdd(&S.red2[1], aa_t);
     }
     __syncthreads();
+    for (int k = tid; k < Ku; k += NT) w.rk[k] = rk[k];
     const bool ok = S.red2[0] <= A.eps3 * A.eps3 * S.red2[1];
     __syncthreads();
     return ok;
@@ -1928,15 +1981,8 @@ __device__ void dense_block(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, 
             }
         }
         __syncthreads();
+        norm_test(A, S, nc);
         if (tid == 0) {
-            double add = 0.0;
-            for (int d = 0; d < nc; ++d) add += 2.0 * (S.hh[d].x * S.ff[d].x - S.hh[d].y * S.ff[d].y);
-            double own = S.hself * S.fself;
-            S.norm2 += add + own;
-            S.stop = sqrt(fmax(own, 0.0)) <= A.eps3 * sqrt(fmax(S.norm2, 0.0));
-            bool all_used = true;
-            for (int k = 0; k < Ku; ++k) all_used &= (S.used_k[k >> 5] >> (k & 31)) & 1u;
-            S.flag = all_used;
             S.off[nc] = off;  // staged for the stop check
             S.r[nc] = -1;
         }
@@ -1960,9 +2006,7 @@ __device__ void dense_block(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, 
                 S.off[nc] = off;
                 S.r[nc] = -1;
                 S.ncross = nc + 1;
-                bool all_used = true;
-                for (int k = 0; k < Ku; ++k) all_used &= (S.used_k[k >> 5] >> (k & 31)) & 1u;
-                if (S.ncross >= A.Cmax || all_used) S.flag = 1;
+                if (S.ncross >= A.Cmax || all_used(A, S)) S.flag = 1;
             } else {
                 S.flag = 1;
             }
@@ -2136,6 +2180,11 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3(const AcaArgs<T
             Cx<T>* Fn = A.pool + off + (long long)rn * (M + N);
             form_of<T, NT>(A, w, S, r, rn, raw, cs, ff, Un, Vn);
             __syncthreads();
+            NewFac nf{};
+            if constexpr (sizeof(T) == 4) {
+                nf = stage_new<NT>(A, S, Un, Vn, rn, smem_raw);
+                __syncthreads();
+            }
             lap(2);
             // ---------------- pivot: argmax |U' V'^H| ----------------
             if (KER != G3_DLP && A.pivot_index) {
@@ -2188,70 +2237,76 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3(const AcaArgs<T
                     }
                 }
             } else {
-                constexpr int TM = sizeof(T) == 4 ? 64 : 32;
-                constexpr int TN = TM;
-                constexpr int RM = TM * TN / NT >= 16 ? 4 : 2;  // micro-tile edge
-                constexpr int TX = TN / RM;                     // micro-tiles along j
-                constexpr int NMT = (TM / RM) * TX;             // micro-tiles per tile
-                Cx<T>* tu = reinterpret_cast<Cx<T>*>(smem_raw);  // [rn][TM]
-                Cx<T>* tv = tu + (size_t)RF * TM;                // [rn][TN]
                 ArgMaxT<T> best = amax_none<T>();
-                for (int i0 = 0; i0 < M; i0 += TM) {
-                    for (int j0 = 0; j0 < N; j0 += TN) {
-                        for (int e = tid; e < rn * TM; e += NT) {
-                            int b = e / TM, ii = e % TM;
-                            tu[b * TM + ii] = (i0 + ii < M) ? ldcx(Un + (long long)b * M + i0 + ii) : Cx<T>{0, 0};
-                        }
-                        for (int e = tid; e < rn * TN; e += NT) {
-                            int b = e / TN, jj = e % TN;
-                            tv[b * TN + jj] = (j0 + jj < N) ? ldcx(Vn + (long long)b * N + j0 + jj) : Cx<T>{0, 0};
-                        }
-                        __syncthreads();
-                        for (int mt = tid; mt < NMT; mt += NT) {
-                            const int tx = mt % TX, ty = mt / TX;
-                            Cx<T> acc[RM][RM];
-#pragma unroll
-                            for (int a = 0; a < RM; ++a)
-#pragma unroll
-                                for (int c = 0; c < RM; ++c) acc[a][c] = Cx<T>{0, 0};
-                            for (int b = 0; b < rn; ++b) {
-                                Cx<T> uu[RM], vv[RM];
-#pragma unroll
-                                for (int a = 0; a < RM; ++a) uu[a] = tu[b * TM + ty * RM + a];
-#pragma unroll
-                                for (int c = 0; c < RM; ++c) vv[c] = tv[b * TN + tx * RM + c];
+                if constexpr (sizeof(T) == 4)
+                    if (nf.sm) best = pivot32<NT>(S, nf, rn);
+                if (!nf.sm) {
+                    constexpr int TM = sizeof(T) == 4 ? 64 : 32;
+                    constexpr int TN = TM;
+                    constexpr int RM = TM * TN / NT >= 16 ? 4 : 2;  // micro-tile edge
+                    constexpr int TX = TN / RM;                     // micro-tiles along j
+                    constexpr int NMT = (TM / RM) * TX;             // micro-tiles per tile
+                    Cx<T>* tu = reinterpret_cast<Cx<T>*>(smem_raw);  // [rn][TM]
+                    Cx<T>* tv = tu + (size_t)RF * TM;                // [rn][TN]
+                    for (int i0 = 0; i0 < M; i0 += TM) {
+                        for (int j0 = 0; j0 < N; j0 += TN) {
+                            for (int e = tid; e < rn * TM; e += NT) {
+                                int b = e / TM, ii = e % TM;
+                                tu[b * TM + ii] = (i0 + ii < M) ? ldcx(Un + (long long)b * M + i0 + ii) : Cx<T>{0, 0};
+                            }
+                            for (int e = tid; e < rn * TN; e += NT) {
+                                int b = e / TN, jj = e % TN;
+                                tv[b * TN + jj] = (j0 + jj < N) ? ldcx(Vn + (long long)b * N + j0 + jj) : Cx<T>{0, 0};
+                            }
+                            __syncthreads();
+                            for (int mt = tid; mt < NMT; mt += NT) {
+                                const int tx = mt % TX, ty = mt / TX;
+                                Cx<T> acc[RM][RM];
 #pragma unroll
                                 for (int a = 0; a < RM; ++a)
 #pragma unroll
-                                    for (int c = 0; c < RM; ++c) cfmac(acc[a][c], uu[a], vv[c]);
-                            }
+                                    for (int c = 0; c < RM; ++c) acc[a][c] = Cx<T>{0, 0};
+                                for (int b = 0; b < rn; ++b) {
+                                    Cx<T> uu[RM], vv[RM];
 #pragma unroll
-                            for (int a = 0; a < RM; ++a)
+                                    for (int a = 0; a < RM; ++a) uu[a] = tu[b * TM + ty * RM + a];
 #pragma unroll
-                                for (int c = 0; c < RM; ++c) {
-                                    int gi = i0 + ty * RM + a, gj = j0 + tx * RM + c;
-                                    if (gi < M && gj < N)
-                                        best = amax_better(best, ArgMaxT<T>{cabs2(acc[a][c]), gi * N + gj});
+                                    for (int c = 0; c < RM; ++c) vv[c] = tv[b * TN + tx * RM + c];
+#pragma unroll
+                                    for (int a = 0; a < RM; ++a)
+#pragma unroll
+                                        for (int c = 0; c < RM; ++c) cfmac(acc[a][c], uu[a], vv[c]);
                                 }
+#pragma unroll
+                                for (int a = 0; a < RM; ++a)
+#pragma unroll
+                                    for (int c = 0; c < RM; ++c) {
+                                        int gi = i0 + ty * RM + a, gj = j0 + tx * RM + c;
+                                        if (gi < M && gj < N)
+                                            best = amax_better(best, ArgMaxT<T>{cabs2(acc[a][c]), gi * N + gj});
+                                    }
+                            }
+                            __syncthreads();
                         }
-                        __syncthreads();
                     }
                 }
                 best = block_argmax<NT>(best, S.am);
-                if (tid == 0) {
-                    // no finite candidate (a non-finite face): report a vanishing pivot
-                    if (best.v < 0 || best.i < 0 || best.i >= M * N) {
-                        S.ip = 0;
-                        S.jp = 0;
-                        S.hpiv = Cx<double>{0.0, 0.0};
-                        if (best.v >= 0) atomicOr(A.status, ST_BAD_INDEX);
-                    } else {
-                        S.ip = (int)(best.i / N);
-                        S.jp = (int)(best.i % N);
-                        Cx<T> hw{0, 0};
-                        for (int b = 0; b < rn; ++b) cfmac(hw, Un[(long long)b * M + S.ip], Vn[(long long)b * N + S.jp]);
+                // no finite candidate (a non-finite face): report a vanishing pivot
+                const bool have = best.v >= 0 && best.i >= 0 && best.i < M * N;
+                if (wid == 0) {
+                    const int bi = have ? best.i / N : 0, bj = have ? best.i % N : 0;
+                    Cx<T> hw{0, 0};
+                    if (have)
+                        for (int b = lane; b < rn; b += 32)
+                            cfmac(hw, ldcx(Un + (long long)b * M + bi), ldcx(Vn + (long long)b * N + bj));
+                    hw.x = warp_sum(hw.x);
+                    hw.y = warp_sum(hw.y);
+                    if (lane == 0) {
+                        S.ip = bi;
+                        S.jp = bj;
+                        if (!have && best.v >= 0) atomicOr(A.status, ST_BAD_INDEX);
                         Cx<double> h = ccast<double>(hw);
-                        if (!isfinite(h.x) || !isfinite(h.y)) h = Cx<double>{0.0, 0.0};
+                        if (!have || !isfinite(h.x) || !isfinite(h.y)) h = Cx<double>{0.0, 0.0};
                         S.hpiv = h;
                     }
                 }
@@ -2259,13 +2314,17 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3(const AcaArgs<T
             __syncthreads();
             lap(3);
             if (S.hpiv.x == 0.0 && S.hpiv.y == 0.0) break;  // vanishing face: nothing to divide by
-            // H_p[i_l, j_l] of earlier crosses (values of the face's scale: working precision)
-            for (int p = tid; p < S.ncross; p += NT) {
+            // H_p[i_l, j_l] of earlier crosses (values of the face's scale: working
+            // precision), one warp per cross, lanes over its columns
+            for (int p = wid; p < S.ncross; p += NT / 32) {
                 const Cx<T>* U = Up(A, S, p);
                 const Cx<T>* V = Vp(A, S, p);
                 Cx<T> h{0, 0};
-                for (int t = 0; t < S.r[p]; ++t) cfmac(h, U[(long long)t * M + S.ip], V[(long long)t * N + S.jp]);
-                S.hp[p] = ccast<double>(h);
+                for (int t = lane; t < S.r[p]; t += 32)
+                    cfmac(h, ldcx(U + (long long)t * M + S.ip), ldcx(V + (long long)t * N + S.jp));
+                h.x = warp_sum(h.x);
+                h.y = warp_sum(h.y);
+                if (lane == 0) S.hp[p] = ccast<double>(h);
             }
             __syncthreads();
             // ---------------- fiber (float64 residual) ----------------
@@ -2304,20 +2363,18 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3(const AcaArgs<T
                     else S.fself = (double)acc.x;
                 }
             }
-            for (int d = tid; d < nc; d += NT) S.hh[d] = Cx<double>{0, 0};
-            if (tid == 0) S.hself = 0.0;
-            __syncthreads();
-            // <H_l, H_d> and ||H_l||^2 through tiled Gram products
-            norm_grams<T, NT>(A, S, Un, Vn, rn, reinterpret_cast<Cx<T>*>(smem_raw));
+            // <H_l, H_d> and ||H_l||^2 through Gram products
+            if constexpr (sizeof(T) == 4) {
+                if (nf.sm) norm32_t<NT, true>(A, S, Un, Vn, rn, nf, w.pre);
+                else norm32_t<NT, false>(A, S, Un, Vn, rn, nf, w.pre);
+            } else {
+                for (int d = tid; d < nc; d += NT) S.hh[d] = Cx<double>{0, 0};
+                if (tid == 0) S.hself = 0.0;
+                __syncthreads();
+                norm_grams<T, NT>(A, S, Un, Vn, rn, reinterpret_cast<Cx<T>*>(smem_raw));
+            }
+            norm_test(A, S, nc);
             if (tid == 0) {
-                double add = 0.0;
-                for (int d = 0; d < nc; ++d) add += 2.0 * (S.hh[d].x * S.ff[d].x - S.hh[d].y * S.ff[d].y);
-                double own = S.hself * S.fself;
-                S.norm2 += add + own;
-                S.stop = sqrt(fmax(own, 0.0)) <= A.eps3 * sqrt(fmax(S.norm2, 0.0));
-                bool all_used = true;
-                for (int k = 0; k < Ku; ++k) all_used &= (S.used_k[k >> 5] >> (k & 31)) & 1u;
-                S.flag = all_used;
                 S.off[nc] = off;  // staged for the stop check
                 S.r[nc] = rn;
             }
@@ -2342,9 +2399,7 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3(const AcaArgs<T
                     S.r[nc] = rn;
                     S.pre[nc + 1] = S.pre[nc] + rn;
                     S.ncross = nc + 1;
-                    bool all_used = true;
-                    for (int k = 0; k < Ku; ++k) all_used &= (S.used_k[k >> 5] >> (k & 31)) & 1u;
-                    if (S.ncross >= A.Cmax || all_used) S.flag = 1;
+                    if (S.ncross >= A.Cmax || all_used(A, S)) S.flag = 1;
                 } else {
                     S.flag = 1;
                 }

@@ -724,4 +724,237 @@ __device__ void form32(BlockSh<float>& S, const ColStore& c, int r, int rn, bool
     }
 }
 
+// ---- the new cross's factors in shared memory --------------------------------------------
+// U' and V' (just written to the pool) staged once for the pivot search and
+// eq. (norm): column b at su + b ldu (ldu is 8 modulo 16 and at least M + 8, zero
+// beyond M; sv likewise), when the arena holds them.
+struct NewFac {
+    Cx<float>* su;
+    Cx<float>* sv;
+    int ldu, ldv;
+    bool sm;
+};
+template <int NT>
+__device__ __forceinline__ NewFac stage_new(const AcaArgs<float>& A, const BlockSh<float>& S, const Cx<float>* Un,
+                                            const Cx<float>* Vn, int rn, unsigned char* arena) {
+    NewFac f;
+    f.ldu = ((S.M + 15) & ~15) + 8;
+    f.ldv = ((S.N + 15) & ~15) + 8;
+    f.su = reinterpret_cast<Cx<float>*>(arena);
+    f.sv = f.su + (size_t)rn * f.ldu;
+    f.sm = (size_t)rn * (f.ldu + f.ldv) * sizeof(Cx<float>) <= (size_t)A.arena_bytes;
+    if (f.sm) {
+        // one warp per column, all of its loads in flight together
+        const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        for (int b = wid; b < 2 * rn; b += NT / 32) {
+            const bool u = b < rn;
+            const int L = u ? S.M : S.N, ld = u ? f.ldu : f.ldv;
+            const Cx<float>* src = u ? Un + (long long)b * S.M : Vn + (long long)(b - rn) * S.N;
+            Cx<float>* dst = u ? f.su + b * f.ldu : f.sv + (b - rn) * f.ldv;
+#pragma unroll 8
+            for (int i = lane; i < ld; i += 32) dst[i] = i < L ? ldcx(src + i) : Cx<float>{0, 0};
+        }
+    }
+    return f;
+}
+
+// largest |U' V'^H| entry of a thread's 4 x 4 tiles (staged factors)
+template <int NT>
+__device__ __forceinline__ ArgMaxT<float> pivot32(const BlockSh<float>& S, const NewFac& f, int rn) {
+    ArgMaxT<float> best = amax_none<float>();
+    const int M = S.M, N = S.N, tx = (N + 3) / 4, nt = ((M + 3) / 4) * tx;
+    for (int q = threadIdx.x; q < nt; q += NT) {
+        const int ti = (q / tx) * 4, tj = (q % tx) * 4;
+        Cx<float> acc[4][4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[a][c] = Cx<float>{0, 0};
+        const Cx<float>* pu = f.su + ti;
+        const Cx<float>* pv = f.sv + tj;
+        for (int b = 0; b < rn; ++b, pu += f.ldu, pv += f.ldv) {
+            const float4 u0 = *reinterpret_cast<const float4*>(pu), u1 = *reinterpret_cast<const float4*>(pu + 2);
+            const float4 v0 = *reinterpret_cast<const float4*>(pv), v1 = *reinterpret_cast<const float4*>(pv + 2);
+            const Cx<float> uu[4] = {{u0.x, u0.y}, {u0.z, u0.w}, {u1.x, u1.y}, {u1.z, u1.w}};
+            const Cx<float> vv[4] = {{v0.x, v0.y}, {v0.z, v0.w}, {v1.x, v1.y}, {v1.z, v1.w}};
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) cfmac(acc[a][c], uu[a], vv[c]);
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (ti + a < M && tj + c < N)
+                    best = amax_better(best, ArgMaxT<float>{cabs2(acc[a][c]), (ti + a) * N + tj + c});
+    }
+    return best;
+}
+
+// ---- eq. (norm) inner products, float32 ----------------------------------------------------
+// hh[d] = <H_l, H_d>_F = sum_{a in cross d, b} (U_d^H U_l)[a][b] conj((V_d^H V_l)[a][b]),
+// hself = ||H_l||_F^2 (a over the columns of cross l), as norm_grams, on the
+// tensor cores (the three-term TF32 split): a warp takes 16 columns a of
+// [U_1 .. U_nc U_l] against 16 columns b of U_l at a time, streams its columns
+// from L2 straight into the A fragments (32-byte sectors, four k-steps of loads
+// in flight) and reads U_l from the staged copy; no barrier until the sums per
+// column are complete (the tiled version staged every column and synchronised
+// four times per 64 rows).  The k slots of a step are the rows i0 + 2t and
+// i0 + 2t + 1 of lane group t, so that both operands load 16 adjacent bytes.
+// Sums per column in float32, over crosses in float64.  colv: a value per column.
+template <int NT, bool SM>
+__device__ void norm32_t(const AcaArgs<float>& A, BlockSh<float>& S, const Cx<float>* Un, const Cx<float>* Vn, int rn,
+                         const NewFac& f, Cx<float>* colv) {
+    constexpr int NW = NT / 32;
+    const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    const int M = S.M, N = S.N, nc = S.ncross;
+    const int n0 = S.pre[nc], na = n0 + rn;
+    for (int a0 = wid * 16; a0 < na; a0 += NW * 16) {
+        // the lane's two columns (g, g + 8): U then V; absent ones repeat the last
+        const Cx<float>* pu[2];
+        const Cx<float>* pv[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int a = min(a0 + g + 8 * h, na - 1);
+            if (a < n0) {
+                int lo = 0, hi = nc - 1;   // the cross d with pre[d] <= a < pre[d + 1]
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (S.pre[mid] <= a) lo = mid;
+                    else hi = mid - 1;
+                }
+                const int tt = a - S.pre[lo];
+                pu[h] = A.pool + S.off[lo] + (long long)tt * M;
+                pv[h] = A.pool + S.off[lo] + (long long)S.r[lo] * M + (long long)tt * N;
+            } else {
+                pu[h] = Un + (long long)(a - n0) * M;
+                pv[h] = Vn + (long long)(a - n0) * N;
+            }
+        }
+        float sx[2] = {0, 0}, sy[2] = {0, 0};   // the two columns' sums over b (this lane's b)
+        for (int b0 = 0; b0 < rn; b0 += 16) {
+            float z[2][2][2][4];   // [U, V][b tile][re, im][fragment]
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {
+#pragma unroll
+                for (int bt = 0; bt < 2; ++bt)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) z[side][bt][0][q] = z[side][bt][1][q] = 0.f;
+                const int L = side == 0 ? M : N;
+                const int ldb = side == 0 ? f.ldu : f.ldv;
+                const Cx<float>* bs = side == 0 ? f.su : f.sv;
+                const Cx<float>* bg = side == 0 ? Un : Vn;
+                const Cx<float>* c0 = side == 0 ? pu[0] : pv[0];
+                const Cx<float>* c1 = side == 0 ? pu[1] : pv[1];
+                const bool two = b0 + 8 < rn;
+                for (int i0 = 0; i0 < L; i0 += 32) {
+                    Cx<float> x[4][4];   // [k-step][(g, 2t), (g + 8, 2t), (g, 2t + 1), (g + 8, 2t + 1)]
+#pragma unroll
+                    for (int st = 0; st < 4; ++st) {
+                        const int i = i0 + 8 * st + 2 * t;
+                        x[st][0] = i < L ? ldcx(c0 + i) : Cx<float>{0, 0};
+                        x[st][1] = i < L ? ldcx(c1 + i) : Cx<float>{0, 0};
+                        x[st][2] = i + 1 < L ? ldcx(c0 + i + 1) : Cx<float>{0, 0};
+                        x[st][3] = i + 1 < L ? ldcx(c1 + i + 1) : Cx<float>{0, 0};
+                    }
+#pragma unroll
+                    for (int st = 0; st < 4; ++st) {
+                        if (i0 + 8 * st >= L) break;
+                        const int i = i0 + 8 * st + 2 * t;
+                        unsigned arh[4], arl[4], aih[4], ail[4], nih[4], nil[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const Tf32Pair r = tf32_split(x[st][q].x), m = tf32_split(x[st][q].y);
+                            arh[q] = r.hi;
+                            arl[q] = r.lo;
+                            aih[q] = m.hi;
+                            ail[q] = m.lo;
+                        }
+                        tf32_neg4(aih, nih);
+                        tf32_neg4(ail, nil);
+#pragma unroll
+                        for (int bt = 0; bt < 2; ++bt) {
+                            if (bt == 1 && !two) break;
+                            const int b = b0 + 8 * bt + g;
+                            Cx<float> y[2] = {{0, 0}, {0, 0}};
+                            if (b < rn) {
+                                if constexpr (SM) {
+                                    const float4 v = *reinterpret_cast<const float4*>(bs + b * ldb + i);
+                                    y[0] = Cx<float>{v.x, v.y};
+                                    y[1] = Cx<float>{v.z, v.w};
+                                } else {
+                                    const Cx<float>* p = bg + (long long)b * L + i;
+                                    if (i < L) y[0] = ldcx(p);
+                                    if (i + 1 < L) y[1] = ldcx(p + 1);
+                                }
+                            }
+                            unsigned brh[2], brl[2], bih[2], bil[2];
+#pragma unroll
+                            for (int q = 0; q < 2; ++q) {
+                                const Tf32Pair r = tf32_split(y[q].x), m = tf32_split(y[q].y);
+                                brh[q] = r.hi;
+                                brl[q] = r.lo;
+                                bih[q] = m.hi;
+                                bil[q] = m.lo;
+                            }
+                            float* re = z[side][bt][0];
+                            float* im = z[side][bt][1];
+                            // conj(a) b: Re = ar br + ai bi, Im = ar bi - ai br
+                            mma_tf32(re, arh, brl);
+                            mma_tf32(im, arh, bil);
+                            mma_tf32(re, arl, brh);
+                            mma_tf32(im, arl, bih);
+                            mma_tf32(re, aih, bil);
+                            mma_tf32(im, nih, brl);
+                            mma_tf32(re, ail, bih);
+                            mma_tf32(im, nil, brh);
+                            mma_tf32(re, arh, brh);
+                            mma_tf32(im, arh, bih);
+                            mma_tf32(re, aih, bih);
+                            mma_tf32(im, nih, brh);
+                        }
+                    }
+                }
+            }
+            // zu conj(zv) summed over the lane's columns b (absent ones are zero)
+#pragma unroll
+            for (int bt = 0; bt < 2; ++bt)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float ux = z[0][bt][0][q], uy = z[0][bt][1][q], vx = z[1][bt][0][q], vy = z[1][bt][1][q];
+                    sx[q >> 1] += ux * vx + uy * vy;
+                    sy[q >> 1] += uy * vx - ux * vy;
+                }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+            for (int o = 1; o < 4; o <<= 1) {
+                sx[h] += __shfl_xor_sync(0xffffffffu, sx[h], o);
+                sy[h] += __shfl_xor_sync(0xffffffffu, sy[h], o);
+            }
+            const int a = a0 + g + 8 * h;
+            if (t == 0 && a < na) colv[a] = Cx<float>{sx[h], sy[h]};
+        }
+    }
+    __syncthreads();
+    for (int d = wid; d <= nc; d += NW) {
+        const int lo = S.pre[d], hi = d < nc ? S.pre[d + 1] : na;
+        float x = 0, y = 0;
+        for (int a = lo + lane; a < hi; a += 32) {
+            const Cx<float> v = colv[a];
+            x += v.x;
+            y += v.y;
+        }
+        x = warp_sum(x);
+        y = warp_sum(y);
+        if (lane == 0) {
+            if (d < nc) S.hh[d] = Cx<double>{(double)x, (double)y};
+            else S.hself = (double)x;
+        }
+    }
+    __syncthreads();
+}
+
 }  // namespace g3
