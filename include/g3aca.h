@@ -83,9 +83,9 @@ typedef enum {
 /* Arithmetic of the path. */
 typedef enum {
     G3_FP64 = 0,   /* everything in float64; factors and near field complex128       */
-    G3_MIXED = 1   /* float32 entries and face arithmetic, float64 singular entries,
-                      fiber residuals, norms, recompression and frequencies;
-                      factors and near field complex64                                */
+    G3_MIXED = 1   /* float32 entries, face arithmetic and recompression, fiber
+                      residuals in float-float, float64 singular entries, norms and
+                      frequencies; factors and near field complex64                   */
 } g3_precision;
 
 typedef enum { G3_C64 = 0, G3_C128 = 1 } g3_dtype;
@@ -207,7 +207,8 @@ typedef struct {
     int32_t blocks_run;       /* blocks compressed (n_far unless opts->max_blocks)        */
     int64_t dense_crosses;    /* kept crosses with a dense face (face_rank_sum excludes them) */
     double ms_lowrank;        /* device time of the low-rank-face launch (last attempt)   */
-    double ms_dense;          /* device time of the dense-face launch (last attempt)      */
+    double ms_dense;          /* device time from its end to that of the dense-face launch,
+                                 which overlaps it (last attempt)                       */
     int32_t spilled_blocks;   /* blocks rerun from the spill queue after the factor pool
                                  filled up (their work up to the overflow is repeated)     */
     int32_t mlp_used;         /* the predictor's uses applied (mask as opts->mlp_use)      */

@@ -12,7 +12,7 @@ namespace g3 {
     extern template int occupancy<KER, T, NT, DENSE>(size_t);
 #define G3_ACA_EXTERN_KIND(KER)              \
     G3_ACA_EXTERN(KER, float, 256, false)    \
-    G3_ACA_EXTERN(KER, float, 256, true)     \
+    G3_ACA_EXTERN(KER, float, 128, true)     \
     G3_ACA_EXTERN(KER, float, 128, false)    \
     G3_ACA_EXTERN(KER, float, 512, false)    \
     G3_ACA_EXTERN(KER, float, 384, false)    \
@@ -24,11 +24,11 @@ G3_ACA_EXTERN_KIND(G3_SEPARABLE)
 G3_ACA_EXTERN_KIND(G3_GAL_SLP)
 // linear-element operators: the 256-thread launches only
 G3_ACA_EXTERN(G3_GAL_P1D, float, 256, false)
-G3_ACA_EXTERN(G3_GAL_P1D, float, 256, true)
+G3_ACA_EXTERN(G3_GAL_P1D, float, 128, true)
 G3_ACA_EXTERN(G3_GAL_P1D, double, 256, false)
 G3_ACA_EXTERN(G3_GAL_P1D, double, 256, true)
 G3_ACA_EXTERN(G3_GAL_P1KP, float, 256, false)
-G3_ACA_EXTERN(G3_GAL_P1KP, float, 256, true)
+G3_ACA_EXTERN(G3_GAL_P1KP, float, 128, true)
 G3_ACA_EXTERN(G3_GAL_P1KP, double, 256, false)
 G3_ACA_EXTERN(G3_GAL_P1KP, double, 256, true)
 
@@ -51,7 +51,7 @@ static g3_status launch_kind(g3_ctx* ctx, int kernel, AcaArgs<T>& A, int grid, s
     if (kernel == G3_DLP) return launch_aca_t<G3_DLP, T, NT, DENSE>(ctx, A, grid, smem);
     if (kernel == G3_GAL_SLP) return launch_aca_t<G3_GAL_SLP, T, NT, DENSE>(ctx, A, grid, smem);
     if (kernel == G3_GAL_P1D || kernel == G3_GAL_P1KP) {
-        if constexpr (NT == 256)
+        if constexpr (NT == 256 || DENSE)
             return kernel == G3_GAL_P1D ? launch_aca_t<G3_GAL_P1D, T, NT, DENSE>(ctx, A, grid, smem)
                                         : launch_aca_t<G3_GAL_P1KP, T, NT, DENSE>(ctx, A, grid, smem);
         return fail(G3_EUNSUPPORTED, "aca3_compress: linear-element operators run with 256 threads per CTA");
@@ -65,7 +65,7 @@ static int occupancy_kind(int kernel, size_t smem) {
     if (kernel == G3_DLP) return occupancy<G3_DLP, T, NT, DENSE>(smem);
     if (kernel == G3_GAL_SLP) return occupancy<G3_GAL_SLP, T, NT, DENSE>(smem);
     if (kernel == G3_GAL_P1D || kernel == G3_GAL_P1KP) {
-        if constexpr (NT == 256)
+        if constexpr (NT == 256 || DENSE)
             return kernel == G3_GAL_P1D ? occupancy<G3_GAL_P1D, T, NT, DENSE>(smem)
                                         : occupancy<G3_GAL_P1KP, T, NT, DENSE>(smem);
         return 1;
@@ -378,14 +378,20 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
         else
             per_low = occupancy_kind<T, NT, false>(kernel, smem);
     }
-    const int per_dense = o.ctas_per_sm > 0 ? o.ctas_per_sm : occupancy_kind<T, NT, true>(kernel, 0);
+    // dense faces: one CTA per block, float32 of DENSE32_NT threads
+    constexpr int NTD = sizeof(T) == 4 ? DENSE32_NT : NT;
+    const int per_dense = o.ctas_per_sm > 0 ? o.ctas_per_sm : occupancy_kind<T, NTD, true>(kernel, 0);
     const int grid_low = o.unbatched ? 1 : std::max(1, std::min(n_low, ctx->n_sm * per_low));
     const int grid_dense = o.unbatched ? 1 : std::max(1, std::min(n_dense, ctx->n_sm * per_dense));
     const int grid = std::max(grid_low, grid_dense);
     const size_t drf_off = al256(ws_bytes<T>(RF, Mmax, Nmax, Cmax, Ku));
     const size_t stride = drf_off + al256((size_t)drf_elems * sizeof(Cx<T>));
+    // the dense-face launch has a workspace of its own (no face columns): the two
+    // launches overlap
+    const size_t stride_dense = sizeof(T) == 4 ? dense_ws_bytes(Cmax, Ku) : al256(ws_bytes<T>(1, 1, 1, Cmax, Ku));
+    const size_t ws_dense = n_low > 0 ? stride * grid_low : 0;
     // per-CTA workspace, kept by the context between compressions
-    G3_CUDA(ctx->aca_ws.ensure(stride * grid));
+    G3_CUDA(ctx->aca_ws.ensure(ws_dense + (n_dense > 0 ? stride_dense * grid_dense : 0)));
     DevBuf& d_ws = ctx->aca_ws;
     // outputs of all meshes (sliced per mesh at the end)
     DevBuf g_rec, g_r3, g_cyc;
@@ -514,21 +520,38 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
         A.arena_bytes = (int)smem;
         if (!graph) G3_CUDA(cudaEventRecord(e0, ctx->stream));
         g3_status st = G3_OK;
+        // the dense-face launch runs on the side stream: its CTAs fill the SMs that
+        // the persistent low-rank launch leaves, from the start where it has few
+        // blocks and at its end, when the last (largest) blocks keep single SMs
+        // busy.  Serial under graph capture and block by block.
+        const bool overlap = !graph && !o.unbatched && n_lo > 0 && n_de > 0;
+        if (overlap) {
+            G3_CUDA(cudaEventRecord(ctx->fork, ctx->stream));
+            G3_CUDA(cudaStreamWaitEvent(ctx->side, ctx->fork, 0));
+        }
         for (int cls = 0; cls < 2 && st == G3_OK; ++cls) {
             if (cls == 1 && !graph) G3_CUDA(cudaEventRecord(ctx->ev[2], ctx->stream));
             const int cnt = cls == 0 ? n_lo : n_de;
             if (cnt == 0) continue;
+            if (overlap && cls == 1) ctx->stream = ctx->side;
             AcaArgs<T> B = A;
             B.queue = d_queue.as<int>() + (cls == 0 ? 0 : n_lo);
             B.queue_head = d_head.as<int>() + cls;
             B.n_far = cnt;
+            if (cls == 1) {  // no face columns: only the size-independent parts
+                B.ws += ws_dense;
+                B.ws_stride = stride_dense;
+                B.RF = 1;
+                B.drf_max = 0;
+                B.drf_off = 0;
+            }
             const int launches = o.unbatched ? cnt : 1;
             const int g = std::min(cls == 0 ? grid_low : grid_dense, o.unbatched ? 1 : cnt);
             for (int l = 0; l < launches && st == G3_OK; ++l) {
                 if (o.unbatched) B.single = l;
-                if (cls == 1)
-                    st = launch_kind<T, NT, true>(ctx, kernel, B, g, 0);
-                else if constexpr (sizeof(T) == 4)
+                if (cls == 1) {
+                    st = launch_kind<T, NTD, true>(ctx, kernel, B, g, 0);
+                } else if constexpr (sizeof(T) == 4)
                     st = nt_low == 512   ? launch_kind<T, 512, false>(ctx, kernel, B, g, smem)
                          : nt_low == 384 ? launch_kind<T, 384, false>(ctx, kernel, B, g, smem)
                          : nt_low == 128 ? launch_kind<T, 128, false>(ctx, kernel, B, g, smem)
@@ -536,6 +559,11 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
                 else
                     st = launch_kind<T, NT, false>(ctx, kernel, B, g, smem);
             }
+        }
+        if (overlap) {
+            ctx->stream = main_stream;
+            G3_CUDA(cudaEventRecord(ctx->join, ctx->side));
+            G3_CUDA(cudaStreamWaitEvent(ctx->stream, ctx->join, 0));
         }
         if (graph) {
             cudaError_t ce = cudaStreamEndCapture(ctx->stream, &cg);

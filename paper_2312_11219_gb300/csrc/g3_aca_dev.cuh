@@ -335,6 +335,13 @@ __device__ __forceinline__ const Cx<T>* Fp(const AcaArgs<T>& A, const BlockSh<T>
     return A.pool + S.off[p] + (long long)S.r[p] * (S.M + S.N);
 }
 
+// the fiber of cross p (dense-face crosses, r = -1: after the face's M N values)
+template <class T>
+__device__ __forceinline__ const Cx<T>* f_of(const AcaArgs<T>& A, const BlockSh<T>& S, int p) {
+    const long long span = S.r[p] < 0 ? (long long)S.M * S.N : (long long)S.r[p] * (S.M + S.N);
+    return A.pool + S.off[p] + span;
+}
+
 // ---- one quadrature point of a collocation entry --------------------------------------
 template <int KER, class G, class T>
 __device__ __forceinline__ Cx<T> colloc_q(const G& g, int i, int j, int q, T sre, T sim) {
@@ -1765,7 +1772,7 @@ __device__ __forceinline__ void norm_test(const AcaArgs<T>& A, BlockSh<T>& S, in
         if (threadIdx.x == 0) {
             const double own = S.hself * S.fself;
             S.norm2 += add + own;
-            S.stop = sqrt(fmax(own, 0.0)) <= A.eps3 * sqrt(fmax(S.norm2, 0.0));
+            S.stop = fmax(own, 0.0) <= A.eps3 * A.eps3 * fmax(S.norm2, 0.0);
             S.flag = all_used(A, S);
         }
     }
@@ -1778,12 +1785,6 @@ __device__ __forceinline__ void norm_test(const AcaArgs<T>& A, BlockSh<T>& S, in
 // frequencies: rows (2s+1) M / 64, columns (2 (11 s mod 32) + 1) N / 64.
 // Returns true when ||R_samples||_F <= eps3 ||A_samples||_F; otherwise w.rk[k]
 // holds the sampled residual energy per frequency.
-
-template <class T>
-__device__ __forceinline__ const Cx<T>* f_of(const AcaArgs<T>& A, const BlockSh<T>& S, int p) {
-    const long long span = S.r[p] < 0 ? (long long)S.M * S.N : (long long)S.r[p] * (S.M + S.N);
-    return A.pool + S.off[p] + span;
-}
 
 template <int KER, class T, int NT>
 __device__ __noinline__ bool confirm_stop(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, int ncl) {
@@ -1811,27 +1812,52 @@ __device__ __noinline__ bool confirm_stop(const AcaArgs<T>& A, const Ws<T>& w, B
         S.entries += (long long)SAMPLES * Ku;
     }
     __syncthreads();
-    // items (sample, frequency), frequencies fastest; the residual energy per
-    // frequency is summed in shared memory (S.hh is not in use here)
+    // items (samples SAMPLES / SPI apart, frequency), frequencies fastest; float64
+    // one sample each (its pipe is the bound: spread it), float32 four; the residual energy per frequency is summed in shared memory (S.hh is
+    // not in use here).  Float32 squares are scaled by a power of two near the
+    // newest pivot (their range) and summed in float-float, then in float64.
     double* rk = reinterpret_cast<double*>(S.hh);
     for (int k = tid; k < Ku; k += NT) rk[k] = 0.0;
     __syncthreads();
+    constexpr bool F32 = sizeof(T) == 4;
+    constexpr int SPI = F32 ? 4 : 1;
+    const T hm = F32 ? (T)fmax(fabs((T)S.hpiv.x), fabs((T)S.hpiv.y)) : (T)1;
+    const int ex = F32 ? min(max(ilogbf((float)hm), -100), 100) : 0;
+    const T sc = F32 ? (T)scalbnf(1.f, -ex) : (T)1;
+    const double back = F32 ? (double)scalbnf(1.f, ex) : 1.0;
     double rr_t = 0.0, aa_t = 0.0;
-    for (int e = tid; e < SAMPLES * Ku; e += NT) {
-        const int sm = e / Ku, k = e - sm * Ku;
-        const int i = (2 * sm + 1) * M / (2 * SAMPLES), j = (2 * ((11 * sm) % SAMPLES) + 1) * N / (2 * SAMPLES);
-        const Cx<T> a = ent<KER, T>(A, S.rb + i, S.cb + j, k);
-        Cx<T> r = a;
+    for (int e = tid; e < (SAMPLES / SPI) * Ku; e += NT) {
+        const int q = e / Ku, k = e - q * Ku;
+        float2 rs = make_float2(0.f, 0.f), as = rs;   // float32: sums in float-float
+        double rd = 0.0, ad = 0.0;
+        for (int sm = q; sm < SAMPLES; sm += SAMPLES / SPI) {
+            const int i = (2 * sm + 1) * M / (2 * SAMPLES), j = (2 * ((11 * sm) % SAMPLES) + 1) * N / (2 * SAMPLES);
+            const Cx<T> a = ent<KER, T>(A, S.rb + i, S.cb + j, k);
+            Cx<T> r = a;
 #pragma unroll 4
-        for (int p = 0; p < ncl; ++p) {
-            const Cx<T> c = cmul(hs[sm * A.Cmax + p], ldcx(f_of(A, S, p) + k));
-            r.x -= c.x;
-            r.y -= c.y;
+            for (int p = 0; p < ncl; ++p) {
+                const Cx<T> c = cmul(hs[sm * A.Cmax + p], ldcx(f_of(A, S, p) + k));
+                r.x -= c.x;
+                r.y -= c.y;
+            }
+            if constexpr (F32) {
+                const T rx = r.x * sc, ry = r.y * sc, ax = a.x * sc, ay = a.y * sc;
+                ff_add_prod(rs, rx, rx);
+                ff_add_prod(rs, ry, ry);
+                ff_add_prod(as, ax, ax);
+                ff_add_prod(as, ay, ay);
+            } else {
+                rd += cabs2d(r);
+                ad += cabs2d(a);
+            }
         }
-        const double rr = cabs2d(r);
-        atomicAdd(&rk[k], rr);
-        rr_t += rr;
-        aa_t += cabs2d(a);
+        if constexpr (F32) {
+            rd = ((double)rs.x + (double)rs.y) * back * back;
+            ad = ((double)as.x + (double)as.y) * back * back;
+        }
+        atomicAdd(&rk[k], rd);
+        rr_t += rd;
+        aa_t += ad;
     }
     rr_t = warp_sum(rr_t);
     aa_t = warp_sum(aa_t);
@@ -1846,7 +1872,7 @@ __device__ __noinline__ bool confirm_stop(const AcaArgs<T>& A, const Ws<T>& w, B
     return ok;
 }
 
-// ---- dense-face blocks ---------------------------------------------------------------
+// ---- dense-face blocks, float64 (float32: k_dense32) ----------------------------------
 // Algorithm 1 with the exact residual face (no low-rank approximation in the
 // face, the paper's "No Lwr" variant) for blocks with M N <= dense_max.  A
 // cross is stored as H (M x N, column-major) followed by f (Ku) and recorded
@@ -1856,6 +1882,7 @@ __device__ __noinline__ bool confirm_stop(const AcaArgs<T>& A, const Ws<T>& w, B
 template <int KER, class T, int NT>
 __device__ void dense_block(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, bool& zero_block, int& computed,
                             bool& overflow, long long* ph, long long& tclk) {
+    static_assert(sizeof(T) == 8, "float32 blocks with dense faces run one warp each");
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
     const int M = S.M, N = S.N, MN = M * N, Ku = A.Ku, blk = S.blk;
     auto lap = [&](int i) {
@@ -1901,8 +1928,9 @@ __device__ void dense_block(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, 
             for (int e = tid; e < MN; e += NT) {
                 const int i = e % M, j = e / M;
                 Cx<T> v = ent<KER, T>(A, S.rb + i, S.cb + j, kk);
+#pragma unroll 4
                 for (int p = 0; p < nc; ++p) {
-                    const Cx<T> h = A.pool[S.off[p] + e];
+                    const Cx<T> h = ldcx(A.pool + S.off[p] + e);
                     const Cx<T> x = cmul(S.fk[p], h);
                     v.x -= x.x;
                     v.y -= x.y;
@@ -1935,32 +1963,31 @@ __device__ void dense_block(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, 
         ++computed;
         const int ip = am.i / N, jp = am.i % N;
         const int ep = ip + jp * M;
-        const Cx<double> hpiv = ccast<double>(Hn[ep]);
-        for (int p = tid; p < nc; p += NT) S.hp[p] = ccast<double>(A.pool[S.off[p] + ep]);
+        const Cx<double> hpiv = Hn[ep];
+        for (int p = tid; p < nc; p += NT) S.hp[p] = A.pool[S.off[p] + ep];
         __syncthreads();
         lap(3);
         // ---- fiber (float64 residual) ----
         for (int k = tid; k < Ku; k += NT) {
-            Cx<double> e = ccast<double>(ent<KER, T>(A, S.rb + ip, S.cb + jp, k));
+            Cx<double> e = ent<KER, T>(A, S.rb + ip, S.cb + jp, k);
             for (int p = 0; p < nc; ++p) {
-                Cx<double> hf = cmul(S.hp[p], ccast<double>((A.pool + S.off[p] + MN)[k]));
+                const Cx<double> hf = cmul(S.hp[p], (A.pool + S.off[p] + MN)[k]);
                 e.x -= hf.x;
                 e.y -= hf.y;
             }
-            Cx<double> fv = cdiv(e, hpiv);
+            const Cx<double> fv = cdiv(e, hpiv);
             w.fib[k] = fv;
-            Fn[k] = ccast<T>(fv);
+            Fn[k] = fv;
         }
         if (tid == 0) S.entries += Ku;
         __syncthreads();
         lap(4);
         // ---- eq. (norm) with dense faces ----
         for (int d = wid; d <= nc; d += NT / 32) {
-            Cx<double> ff{0, 0};
-            Cx<T> hh{0, 0};
+            Cx<double> ff{0, 0}, hh{0, 0};
             if (d < nc) {
                 const Cx<T>* fd = A.pool + S.off[d] + MN;
-                for (int k = lane; k < Ku; k += 32) cfmac(ff, w.fib[k], ccast<double>(fd[k]));
+                for (int k = lane; k < Ku; k += 32) cfmac(ff, w.fib[k], fd[k]);
                 const Cx<T>* Hd = A.pool + S.off[d];
                 for (int e = lane; e < MN; e += 32) cfmac(hh, Hn[e], Hd[e]);
             } else {
@@ -1969,14 +1996,15 @@ __device__ void dense_block(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, 
             }
             ff.x = warp_sum(ff.x);
             ff.y = warp_sum(ff.y);
-            const T hx = warp_sum(hh.x), hy = warp_sum(hh.y);
+            hh.x = warp_sum(hh.x);
+            hh.y = warp_sum(hh.y);
             if (lane == 0) {
                 if (d < nc) {
                     S.ff[d] = ff;
-                    S.hh[d] = Cx<double>{(double)hx, (double)hy};
+                    S.hh[d] = hh;
                 } else {
                     S.fself = ff.x;
-                    S.hself = (double)hx;
+                    S.hself = hh.x;
                 }
             }
         }
@@ -2017,7 +2045,7 @@ __device__ void dense_block(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, 
         ArgMaxT<T> nk = amax_none<T>();
         for (int k = tid; k < Ku; k += NT)
             if (!((S.used_k[k >> 5] >> (k & 31)) & 1u))
-                nk = amax_better(nk, ArgMaxT<T>{(T)(from_samples ? w.rk[k] : cabs2(w.fib[k])), k});
+                nk = amax_better(nk, ArgMaxT<T>{from_samples ? w.rk[k] : cabs2(w.fib[k]), k});
         nk = block_argmax<NT>(nk, S.am);
         if (nk.v < 0 || nk.i < 0 || nk.i >= Ku) return;
         if (tid == 0) S.k = nk.i;
@@ -2025,6 +2053,12 @@ __device__ void dense_block(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, 
         lap(6);
     }
 }
+
+}  // namespace g3
+
+#include "g3_dense32.cuh"
+
+namespace g3 {
 
 // ---- the persistent kernel ---------------------------------------------------------
 // DENSE selects the block class this launch serves (dense faces or low-rank
@@ -2044,8 +2078,9 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3(const AcaArgs<T
     __shared__ AcaArgs<T> Ash;
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
     const int RF = P.RF;
-    const Ws<T> w = ws_carve<T>(P.ws + (size_t)blockIdx.x * P.ws_stride, RF, P.Mmax, P.Nmax, P.Cmax, P.Ku,
-                                P.drf_max > 0 ? P.drf_off : 0);
+    // (dense faces: no face columns, a workspace without them)
+    const Ws<T> w = ws_carve<T>(P.ws + (size_t)blockIdx.x * P.ws_stride, RF, DENSE ? 1 : P.Mmax, DENSE ? 1 : P.Nmax,
+                                P.Cmax, P.Ku, P.drf_max > 0 ? P.drf_off : 0);
     __shared__ int s_q;
     for (int iter = 0;; ++iter) {
         if (tid == 0) {
@@ -2111,7 +2146,7 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3(const AcaArgs<T
             if (tid == 0) atomicOr(A.status, ST_BAD_INDEX);
             overflow = true;
         }
-        if (DENSE) {
+        if constexpr (DENSE) {
             if (!overflow) dense_block<KER, T, NT>(A, w, S, zero_block, computed, spilled, ph, tclk);
             overflow = true;  // the low-rank loop below is not for this launch
         }
@@ -2324,23 +2359,30 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3(const AcaArgs<T
                     cfmac(h, ldcx(U + (long long)t * M + S.ip), ldcx(V + (long long)t * N + S.jp));
                 h.x = warp_sum(h.x);
                 h.y = warp_sum(h.y);
-                if (lane == 0) S.hp[p] = ccast<double>(h);
+                if (lane == 0) {
+                    if constexpr (sizeof(T) == 4) S.fk[p] = h;
+                    else S.hp[p] = h;
+                }
             }
             __syncthreads();
             // ---------------- fiber (float64 residual) ----------------
             const int ip = S.ip, jp = S.jp, nc = S.ncross;
-            const Cx<double> hpiv = S.hpiv;
-            for (int k = tid; k < Ku; k += NT) {
-                Cx<double> e = ccast<double>(ent<KER, T>(A, S.rb + ip, S.cb + jp, k));
-                for (int p = 0; p < nc; ++p) {
-                    Cx<double> fp = ccast<double>(Fp(A, S, p)[k]);
-                    Cx<double> hf = cmul(S.hp[p], fp);
-                    e.x -= hf.x;
-                    e.y -= hf.y;
+            if constexpr (sizeof(T) == 4) {
+                fiber32<KER, NT>(A, tid, S.rb + ip, S.cb + jp, nc, S.fk, cff_inv(ccast<float>(S.hpiv)),
+                                 [&](int p) { return Fp(A, S, p); }, Fn);
+            } else {
+                const Cx<double> hpiv = S.hpiv;
+                for (int k = tid; k < Ku; k += NT) {
+                    Cx<double> e = ent<KER, T>(A, S.rb + ip, S.cb + jp, k);
+                    for (int p = 0; p < nc; ++p) {
+                        const Cx<double> hf = cmul(S.hp[p], Fp(A, S, p)[k]);
+                        e.x -= hf.x;
+                        e.y -= hf.y;
+                    }
+                    const Cx<double> fv = cdiv(e, hpiv);
+                    w.fib[k] = fv;
+                    Fn[k] = fv;
                 }
-                Cx<double> fv = cdiv(e, hpiv);
-                w.fib[k] = fv;
-                Fn[k] = ccast<T>(fv);
             }
             if (tid == 0) S.entries += Ku;
             __syncthreads();
@@ -2473,7 +2515,7 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3_face(const AcaA
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ BlockSh<T> S;
     __shared__ int s_q;
-    const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x;
     const AcaArgs<T>& A = P;
     const int RF = A.RF;
     const Ws<T> w = ws_carve<T>(A.ws + (size_t)blockIdx.x * A.ws_stride, RF, A.Mmax, A.Nmax, A.Cmax, A.Ku);
@@ -2694,9 +2736,20 @@ g3_status launch_whole_fiber_t(g3_ctx* ctx, AcaArgs<T>& A, int pb, int pi, int p
 // g3_aca_dlp.cu and g3_aca_sep.cu, so that the kinds compile in parallel)
 // ============================================================================
 
+// the kernel of a block class
+template <int KER, class T, int NT, bool DENSE>
+constexpr auto aca_kernel() {
+    if constexpr (DENSE && sizeof(T) == 4) {
+        static_assert(NT == DENSE32_NT, "float32 dense faces");
+        return k_dense32<KER>;
+    } else {
+        return k_aca3<KER, T, NT, DENSE>;
+    }
+}
+
 template <int KER, class T, int NT, bool DENSE>
 g3_status launch_aca_t(g3_ctx* ctx, AcaArgs<T>& A, int grid, size_t smem) {
-    auto kfn = k_aca3<KER, T, NT, DENSE>;
+    auto kfn = aca_kernel<KER, T, NT, DENSE>();
     G3_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     kfn<<<grid, NT, smem, ctx->stream>>>(A);
     ctx->count(KER == G3_SEPARABLE   ? (DENSE ? "k_aca3_dense_separable" : "k_aca3_separable")
@@ -2711,7 +2764,7 @@ g3_status launch_aca_t(g3_ctx* ctx, AcaArgs<T>& A, int grid, size_t smem) {
 template <int KER, class T, int NT, bool DENSE>
 int occupancy(size_t smem) {
     int nb = 0;
-    auto kfn = k_aca3<KER, T, NT, DENSE>;
+    auto kfn = aca_kernel<KER, T, NT, DENSE>();
     cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kfn, NT, smem) != cudaSuccess) nb = 1;
     return std::max(nb, 1);

@@ -15,7 +15,7 @@ G3_ACA_INST(float, 256, false)
 G3_ACA_INST(float, 128, false)
 #endif
 #if !defined(G3_ACA_PART) || G3_ACA_PART == 1
-G3_ACA_INST(float, 256, true)
+G3_ACA_INST(float, 128, true)
 G3_ACA_INST(float, 512, false)
 #endif
 #if !defined(G3_ACA_PART) || G3_ACA_PART == 2

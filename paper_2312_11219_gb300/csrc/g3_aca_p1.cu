@@ -13,11 +13,11 @@ namespace g3 {
 // compiled in four parts (G3_ACA_PART = 0, 1, 2, 3) by separate compiler processes
 #if !defined(G3_ACA_PART) || G3_ACA_PART == 0
 G3_ACA_INST(G3_GAL_P1D, float, 256, false)
-G3_ACA_INST(G3_GAL_P1D, float, 256, true)
+G3_ACA_INST(G3_GAL_P1D, float, 128, true)
 #endif
 #if !defined(G3_ACA_PART) || G3_ACA_PART == 1
 G3_ACA_INST(G3_GAL_P1KP, float, 256, false)
-G3_ACA_INST(G3_GAL_P1KP, float, 256, true)
+G3_ACA_INST(G3_GAL_P1KP, float, 128, true)
 #endif
 #if !defined(G3_ACA_PART) || G3_ACA_PART == 2
 G3_ACA_INST(G3_GAL_P1D, double, 256, false)

@@ -724,6 +724,95 @@ __device__ void form32(BlockSh<float>& S, const ColStore& c, int r, int rn, bool
     }
 }
 
+// ---- float-float helpers of the fiber ------------------------------------------------------
+// a complex number as two float-float values
+struct Cff {
+    float2 x, y;
+};
+__device__ __forceinline__ float2 ff_mul(float2 a, float2 b) {
+    const float p = a.x * b.x;
+    const float e = fmaf(a.x, b.x, -p) + (a.x * b.y + a.y * b.x);
+    const float s = p + e;
+    return make_float2(s, e - (s - p));
+}
+__device__ __forceinline__ float2 ff_neg(float2 a) { return make_float2(-a.x, -a.y); }
+// a - h f for float32 h, f: the products exact, the sum to ~2^-48
+__device__ __forceinline__ void cff_sub_prod(Cff& a, Cx<float> h, Cx<float> f) {
+    ff_add_prod(a.x, -h.x, f.x);
+    ff_add_prod(a.x, h.y, f.y);
+    ff_add_prod(a.y, -h.x, f.y);
+    ff_add_prod(a.y, -h.y, f.x);
+}
+
+// 1 / h to ~2^-46: one Newton step in float-float from the float32 reciprocal of
+// |h|^2, h scaled to magnitude ~1 by a power of two
+__device__ __forceinline__ Cff cff_inv(Cx<float> h) {
+    const int e = min(max(ilogbf(fmaxf(fabsf(h.x), fabsf(h.y))), -120), 120);
+    const float sc = scalbnf(1.f, -e);
+    const float x = h.x * sc, y = h.y * sc;
+    float2 n = make_float2(0.f, 0.f);
+    ff_add_prod(n, x, x);
+    ff_add_prod(n, y, y);
+    const float r0 = 1.f / n.x;
+    // r = r0 + r0 (1 - n r0)
+    float2 d = ff_neg(ff_mul(n, make_float2(r0, 0.f)));
+    ff_add(d, 1.f, 0.f);
+    float2 r = make_float2(r0, 0.f);
+    const float2 c = ff_mul(d, make_float2(r0, 0.f));
+    ff_add(r, c.x, c.y);
+    const float2 rx = ff_mul(r, make_float2(x, 0.f)), ry = ff_mul(r, make_float2(-y, 0.f));
+    return Cff{make_float2(rx.x * sc, rx.y * sc), make_float2(ry.x * sc, ry.y * sc)};
+}
+
+// The fiber of the new cross at the pivot (elements gi, gj), float32 blocks:
+//   f[k] = (ENTRY(gi, gj, k) - sum_p H_p f_p[k]) / H_l   (H at the pivot).
+// The residual is formed in float-float (its operands are float32, so every
+// product is exact and the sum good to ~2^-48; the same values in float64 cost
+// 19 SM cycles per warp instruction on this part's float64 pipe, which bound
+// the blocks with dense faces).  G threads share a frequency: its quadrature
+// points and its crosses.  hp[p] = H_p at the pivot, inv = 1 / H_l, fptr(p): the
+// fiber of cross p; tid of NT threads (whole warps).
+template <int KER, int NT, class FP>
+__device__ __forceinline__ void fiber32(const AcaArgs<float>& A, int tid, int gi, int gj, int nc, const Cx<float>* hp,
+                                        const Cff inv, FP fptr, Cx<float>* Fn) {
+    const int Ku = A.Ku;
+    // the gang of 1, 2 or 4 with the fewest passes per frequency
+    int G = 1, best = 4 * ((Ku + NT - 1) / NT);
+#pragma unroll
+    for (int g = 2; g <= 4; g *= 2) {
+        const int c = (4 / g) * ((Ku * g + NT - 1) / NT);
+        if (c < best) {
+            best = c;
+            G = g;
+        }
+    }
+    const int part = tid % G;
+    for (int k0 = 0; k0 < Ku; k0 += NT / G) {
+        const int k = k0 + tid / G;
+        Cff e{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        if (k < Ku) {
+            const Cx<float> a = ent_part<KER, float>(A, gi, gj, k, part, G);
+            e.x.x = a.x;
+            e.y.x = a.y;
+#pragma unroll 2
+            for (int p = part; p < nc; p += G) cff_sub_prod(e, hp[p], ldcx(fptr(p) + k));
+        }
+        for (int o = G >> 1; o > 0; o >>= 1) {
+            const float xh = __shfl_xor_sync(0xffffffffu, e.x.x, o), xl = __shfl_xor_sync(0xffffffffu, e.x.y, o);
+            const float yh = __shfl_xor_sync(0xffffffffu, e.y.x, o), yl = __shfl_xor_sync(0xffffffffu, e.y.y, o);
+            ff_add(e.x, xh, xl);
+            ff_add(e.y, yh, yl);
+        }
+        if (k < Ku && part == 0) {
+            float2 re = ff_mul(e.x, inv.x), im = ff_mul(e.x, inv.y);
+            const float2 a = ff_neg(ff_mul(e.y, inv.y)), b = ff_mul(e.y, inv.x);
+            ff_add(re, a.x, a.y);
+            ff_add(im, b.x, b.y);
+            Fn[k] = Cx<float>{re.x + re.y, im.x + im.y};
+        }
+    }
+}
+
 // ---- the new cross's factors in shared memory --------------------------------------------
 // U' and V' (just written to the pool) staged once for the pivot search and
 // eq. (norm): column b at su + b ldu (ldu is 8 modulo 16 and at least M + 8, zero
