@@ -751,64 +751,11 @@ g3_status assemble_near(g3_ctx* ctx, const g3_tree* t, const g3_freqs* f, g3_ker
             delete nf;
             return fail(G3_EINVAL, "assemble_near: element %d has no diagonal near block", p);
         }
-    // Galerkin: the pairs with a common vertex (Sauter-Schwab); they all lie
-    // in near blocks (a far block's clusters have disjoint boxes)
-    std::vector<SsPair> ss;
-    if (t->p1) {
-        // element pairs with a common vertex inside each near block; the local
-        // entries (a, b) of the pair sit at off + a + b M (frequency stride M N)
-        const int E = t->ne_elem;
-        std::vector<int> tv(3 * (size_t)E);
-        for (int p = 0; p < E; ++p)
-            for (int k = 0; k < 3; ++k) tv[3 * (size_t)p + k] = t->tris[3 * (size_t)t->perm_elem[p] + k];
-        for (size_t b = 0; b < rg.size(); ++b) {
-            const BlockRange& r = rg[b];
-            const int M = r.re - r.rb, N = r.ce - r.cb;
-            for (int je = r.cb / 3; je < r.ce / 3; ++je)
-                for (int ie = r.rb / 3; ie < r.re / 3; ++ie) {
-                    SsPair q{};
-                    q.cas = ss_classify(&tv[3 * (size_t)ie], &tv[3 * (size_t)je], ie == je, q.px, q.py);
-                    if (q.cas == SS_REGULAR) continue;
-                    q.i = ie;
-                    q.j = je;
-                    q.stride = M * N;
-                    q.ldm = M;
-                    q.off = nf->offs[b] + (long long)(3 * je - r.cb) * M + (3 * ie - r.rb);
-                    ss.push_back(q);
-                }
-        }
-        nf->n_ss = (int)ss.size();
-    } else if (scheme == G3_GALERKIN4x4) {
-        std::vector<int> tv(3 * (size_t)t->ne);
-        for (int p = 0; p < t->ne; ++p)
-            for (int k = 0; k < 3; ++k) tv[3 * (size_t)p + k] = t->tris[3 * (size_t)t->perm[p] + k];
-        for (size_t b = 0; b < rg.size(); ++b) {
-            const BlockRange& r = rg[b];
-            const int M = r.re - r.rb, N = r.ce - r.cb;
-            for (int j = r.cb; j < r.ce; ++j)
-                for (int i = r.rb; i < r.re; ++i) {
-                    SsPair q{};
-                    q.cas = ss_classify(&tv[3 * (size_t)i], &tv[3 * (size_t)j], i == j, q.px, q.py);
-                    if (q.cas == SS_REGULAR) continue;
-                    q.i = i;
-                    q.j = j;
-                    q.stride = M * N;
-                    q.off = nf->offs[b] + (long long)(j - r.cb) * M + (i - r.rb);  // [k][j][i]
-                    ss.push_back(q);
-                }
-        }
-        nf->n_ss = (int)ss.size();
-    }
     const size_t esz = prec == G3_MIXED ? 8 : 16;
     g3_status st = G3_OK;
     auto chk = [&](cudaError_t e, const char* w) {
         if (st == G3_OK && e != cudaSuccess) st = cuda_fail(e, w);
     };
-    if (!ss.empty()) {
-        chk(nf->d_ss.alloc(ss.size() * sizeof(SsPair)), "assemble_near: singular pairs");
-        if (st == G3_OK)
-            chk(cudaMemcpy(nf->d_ss.p, ss.data(), ss.size() * sizeof(SsPair), cudaMemcpyHostToDevice), "copy");
-    }
     chk(nf->data.alloc((size_t)off * esz), "assemble_near: near-field storage");
     chk(nf->d_ranges.alloc(rg.size() * sizeof(BlockRange)), "assemble_near: ranges");
     chk(nf->d_offs.alloc(nf->offs.size() * sizeof(long long)), "assemble_near: offsets");
@@ -824,6 +771,9 @@ g3_status assemble_near(g3_ctx* ctx, const g3_tree* t, const g3_freqs* f, g3_ker
         chk(cudaMemcpyAsync(nf->d_offs.p, nf->offs.data(), nf->offs.size() * sizeof(long long), cudaMemcpyHostToDevice, ctx->stream), "copy");
         chk(cudaMemcpyAsync(nf->d_row_start.p, nf->row_start.data(), nf->row_start.size() * sizeof(int), cudaMemcpyHostToDevice, ctx->stream), "copy");
     }
+    // Galerkin: the pairs with a common vertex (Sauter-Schwab); they all lie
+    // in near blocks (a far block's clusters have disjoint boxes)
+    if (st == G3_OK && scheme == G3_GALERKIN4x4) st = launch_ss_pairs(ctx, t, nf);
     if (st == G3_OK) chk(cudaEventRecord(ctx->ev[0], ctx->stream), "event");
     if (st == G3_OK) st = launch_near(ctx, t, f, nf, kernel, scheme);
     if (st == G3_OK) chk(cudaEventRecord(ctx->ev[1], ctx->stream), "event");

@@ -506,7 +506,7 @@ __device__ __forceinline__ Cx<T> p1_entry(const GeomF& gf, const GeomD& gd, int 
 // Regions: identical 6, common edge 5, common vertex 2.
 __host__ __device__ inline int ss_regions(int cas) { return cas == SS_IDENTICAL ? 6 : (cas == SS_EDGE ? 5 : 2); }
 
-__device__ inline double ss_map(int cas, int m, double xi, double e1, double e2, double e3, double xh[2],
+__host__ __device__ inline double ss_map(int cas, int m, double xi, double e1, double e2, double e3, double xh[2],
                                 double yh[2]) {
     if (cas == SS_IDENTICAL) {
         const double f = xi * xi * xi * e1 * e1 * e2;
@@ -577,6 +577,103 @@ __device__ inline void ss_point(const SsPanels& S, int cas, int m, const double 
     w = r > 0.0 ? gw * f * S.jac / r : 0.0;
 }
 
+// ---- float-float arithmetic ----------------------------------------------------------
+// a value as an unevaluated sum of two float32 (about 48 bits), by two-sum and
+// fused-multiply-add products: full-rate instructions where float64 runs at 1/73 of
+// the float32 rate
+__device__ __forceinline__ void ff_add(float2& a, float hi, float lo) {
+    const float s = a.x + hi, bb = s - a.x;
+    const float e = (a.x - (s - bb)) + (hi - bb);
+    const float l = a.y + lo + e;
+    a.x = s + l;
+    a.y = l - (a.x - s);
+}
+__device__ __forceinline__ void ff_add_prod(float2& a, float x, float y) {
+    const float p = x * y;
+    ff_add(a, p, fmaf(x, y, -p));
+}
+__device__ __forceinline__ float2 ff_mul(float2 a, float2 b) {
+    const float p = a.x * b.x;
+    const float e = fmaf(a.x, b.x, -p) + (a.x * b.y + a.y * b.x);
+    const float s = p + e;
+    return make_float2(s, e - (s - p));
+}
+__device__ __forceinline__ void ff_add_mul(float2& s, float2 a, float2 b) {
+    const float p = a.x * b.x;
+    ff_add(s, p, fmaf(a.x, b.x, -p) + (a.x * b.y + a.y * b.x));
+}
+__device__ __forceinline__ float2 ff_neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 ff_of(double v) {
+    const float h = (float)v;
+    return make_float2(h, (float)(v - (double)h));
+}
+
+// Sauter-Schwab points for the float32 near field.  The distance vector of a point
+// is a combination of the panels' edge vectors,
+//   x - y = c0 (P1 - P0) + c1 (P2 - P1) + c2 (Q1 - Q0) + c3 (Q2 - Q1),
+// with coefficients of the reference point alone (the common vertices cancel:
+// identical panels c2 = c3 = 0, a common edge c2 = 0).  The table holds, per
+// region (vertex 0-1, edge 2-6, identical 7-12) and point, the coefficients and
+// the weight as float-float and the reference coordinates, as four float4 arrays
+// [4][SS_Q]: (c0, c1), (c2, c3), (weight, x1, x2), (y1, y2, -, -).
+constexpr int SS_Q = 6 * 6 * 6 * 6;
+__host__ __device__ inline int ss_first_region(int cas) { return cas == SS_VERTEX ? 0 : (cas == SS_EDGE ? 2 : 7); }
+
+// the pair's edge vectors and n_x products in float-float, formed from float64
+struct SsEdges {
+    float2 v[4][3];   // P1 - P0, P2 - P1, Q1 - Q0, Q2 - Q1
+    float2 vn[4];     // their products with the first panel's normal
+    float2 jac;       // (2 |tau_x|)(2 |tau_y|) / (4 pi)
+};
+__device__ inline void ss_edges(const GeomD& g, const SsPair& pr, SsEdges& S) {
+    const int t = threadIdx.x;
+    if (t < 4) {
+        const int e = t < 2 ? pr.i : pr.j, b = t & 1;   // edge b: vertices b, b + 1 of the panel
+        const int8_t* px = t < 2 ? pr.px : pr.py;
+        double vn = 0.0;
+        for (int k = 0; k < 3; ++k) {
+            const double d = g.v[(px[b + 1] * 3 + k) * g.E + e] - g.v[(px[b] * 3 + k) * g.E + e];
+            vn += d * g.n[k * g.E + pr.i];
+            S.v[t][k] = ff_of(d);
+        }
+        S.vn[t] = ff_of(vn);
+    } else if (t == 4) {
+        // 2 |tau| from the first weight of the 7-point rule, (9 / 40) |tau|
+        const double f = 80.0 / 9.0;
+        S.jac = ff_of(f * g.w[pr.i] * (f * g.w[pr.j]) * G3_INV4PI);
+    }
+}
+// point q of region m: distance r, weight (region and Gauss weight) jac / r, both
+// rounded once to float32, and with ZN also z.n_x / r^2
+template <bool ZN>
+__device__ __forceinline__ void ss_point32(const SsEdges& S, const float4* __restrict__ tab, int q, float& r, float& w,
+                                           float& zn) {
+    const float4 a = tab[q], b = tab[SS_Q + q], c = tab[2 * SS_Q + q];
+    const float2 cf[4] = {{a.x, a.y}, {a.z, a.w}, {b.x, b.y}, {b.z, b.w}};
+    float2 d2 = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        float2 z = ff_mul(cf[0], S.v[0][k]);
+#pragma unroll
+        for (int m = 1; m < 4; ++m) ff_add_mul(z, cf[m], S.v[m][k]);
+        ff_add_mul(d2, z, z);
+    }
+    r = w = zn = 0.f;
+    if (!(d2.x > 0.f)) return;
+    const float y0 = rsqrtf(d2.x), r0 = d2.x * y0, p = r0 * r0;
+    const float rl = 0.5f * y0 * ((d2.x - p) + (d2.y - fmaf(r0, r0, -p)));   // r = r0 + rl
+    r = r0 + rl;
+    const float2 wj = ff_mul(make_float2(c.x, c.y), S.jac);
+    const float q0 = wj.x * y0;
+    w = q0 + (fmaf(-q0, r0, wj.x) + (wj.y - q0 * rl)) * y0;
+    if (ZN) {
+        float2 z = ff_mul(cf[0], S.vn[0]);
+#pragma unroll
+        for (int m = 1; m < 4; ++m) ff_add_mul(z, cf[m], S.vn[m]);
+        zn = (z.x + z.y) / d2.x;
+    }
+}
+
 // ---- tensor cores: TF32 products at float32 accuracy ------------------------------
 // A real product on the tensor cores as mma.sync m16n8k8 with TF32 inputs and float32
 // accumulation, in the three-term split a b ~ a_hi b_hi + a_hi b_lo + a_lo b_hi (a_hi =
@@ -610,6 +707,12 @@ __device__ __forceinline__ void mma_tf32x3(float* d, const unsigned* ah, const u
 __device__ __forceinline__ void tf32_neg4(const unsigned* a, unsigned* o) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) o[q] = a[q] ^ 0x80000000u;
+}
+// ---- prefetch of a contiguous range into L2 (whole 16-byte units inside it) --------
+__device__ __forceinline__ void l2_prefetch(const void* p, long long bytes) {
+    const unsigned long long a = ((unsigned long long)p + 15ull) & ~15ull, e = ((unsigned long long)p + bytes) & ~15ull;
+    if (e > a)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((unsigned)(e - a)) : "memory");
 }
 // ---- asynchronous copies global -> shared (8 bytes; zero-filled when !in) ---------
 __device__ __forceinline__ void cp_async8(void* smem, const void* gmem, bool in) {

@@ -38,20 +38,6 @@ __host__ __device__ inline int cs_ld(int M, int N) {
     return l + ((4 - l) & 15);   // <= M + N + CS_PAD - 1
 }
 
-// float-float accumulation (two-sum): the squared norms of the face test keep
-// about 48 bits without the float64 pipe
-__device__ __forceinline__ void ff_add(float2& a, float hi, float lo) {
-    const float s = a.x + hi, bb = s - a.x;
-    const float e = (a.x - (s - bb)) + (hi - bb);
-    const float l = a.y + lo + e;
-    a.x = s + l;
-    a.y = l - (a.x - s);
-}
-__device__ __forceinline__ void ff_add_prod(float2& a, float x, float y) {
-    const float p = x * y;
-    ff_add(a, p, fmaf(x, y, -p));
-}
-
 // four sums over a warp with six exchanges instead of twenty: the halves of
 // the warp first split the values between them, then the lanes below.
 // Lanes 0-15 get (sum a, sum b), lanes 16-31 (sum c, sum d).
@@ -729,13 +715,6 @@ __device__ void form32(BlockSh<float>& S, const ColStore& c, int r, int rn, bool
 struct Cff {
     float2 x, y;
 };
-__device__ __forceinline__ float2 ff_mul(float2 a, float2 b) {
-    const float p = a.x * b.x;
-    const float e = fmaf(a.x, b.x, -p) + (a.x * b.y + a.y * b.x);
-    const float s = p + e;
-    return make_float2(s, e - (s - p));
-}
-__device__ __forceinline__ float2 ff_neg(float2 a) { return make_float2(-a.x, -a.y); }
 // a - h f for float32 h, f: the products exact, the sum to ~2^-48
 __device__ __forceinline__ void cff_sub_prod(Cff& a, Cx<float> h, Cx<float> f) {
     ff_add_prod(a.x, -h.x, f.x);

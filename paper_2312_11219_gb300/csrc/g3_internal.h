@@ -197,6 +197,7 @@ struct g3_ctx {
     int64_t n_launch = 0;
     std::vector<std::string> names_cache;
     g3::DevBuf gl;           // Gauss-Legendre table for self terms
+    g3::DevBuf ss_tab;       // Sauter-Schwab point table (float32 Galerkin near field; 1.1 MB, built when first needed)
     g3::DevBuf scratch;      // apply scratch (cluster-order densities, partial y)
     g3::DevBuf aca_ws;       // per-CTA workspace of the compression (grown, never shrunk)
     g3::DevBuf status;       // device status word(s)
@@ -366,6 +367,7 @@ g3_status run_aca(g3_ctx* ctx, const g3_tree* t, const g3_freqs* f, g3_factors* 
 g3_status run_apply(g3_ctx* ctx, const g3_tree* t, const g3_near* nf, const g3_factors* fa, const void* W, void* Y,
                     int dtype, int mode);
 g3_status gl_table(g3_ctx* ctx);
+g3_status launch_ss_pairs(g3_ctx* ctx, const g3_tree* t, g3_near* nf);
 g3_status run_peak(g3_ctx* ctx, int kind, double* ops_per_s, double* ms);
 
 // host tree builder (bit-exact specification)

@@ -528,6 +528,62 @@ __global__ void __launch_bounds__(NT) k_near_ss(GeomD gd, SsRule gr, const SsPai
     }
 }
 
+// The same in float32, one region's points at a time: the points' distances and
+// weights are formed in float-float from the tables (ss_point32; in float64 their
+// ~85 operations per point took 25 of the 26 ms of the 5,120-triangle sphere's
+// near field, 32 frequencies, 66,000 pairs), the sums over a region added up per
+// frequency in shared memory.  Bound by the special-function unit: three results
+// per point and frequency.  That near field: 26.3 -> 9.5 ms.
+template <int NT>
+__global__ void __launch_bounds__(NT) k_near_ss32(GeomD gd, const float4* __restrict__ tab,
+                                                  const SsPair* __restrict__ pairs, const float2* __restrict__ sf,
+                                                  int Ku, Cx<float>* __restrict__ out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* rs = reinterpret_cast<float*>(smem_raw);          // [SS_Q]
+    float* ws = rs + SS_Q;                                    // [SS_Q]
+    Cx<float>* acc = reinterpret_cast<Cx<float>*>(ws + SS_Q); // [Ku]
+    __shared__ SsEdges S;
+    const SsPair pr = pairs[blockIdx.x];
+    ss_edges(gd, pr, S);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int nreg = ss_regions(pr.cas), first = ss_first_region(pr.cas);
+    __syncthreads();
+    for (int m = 0; m < nreg; ++m) {
+        const float4* tm = tab + (size_t)(first + m) * 4 * SS_Q;
+        for (int q = threadIdx.x; q < SS_Q; q += NT) {
+            float zn;
+            ss_point32<false>(S, tm, q, rs[q], ws[q], zn);
+        }
+        __syncthreads();
+        // each warp owns every (NT / 32)-th frequency
+        for (int k = wid; k < Ku; k += NT / 32) {
+            const float2 s = sf[k];
+            float ax = 0, ay = 0;
+#pragma unroll 4
+            for (int q = lane; q < SS_Q; q += 32) {
+                const float r = rs[q];
+                const float mm = ws[q] * kexp(-s.x * r);
+                float sn, cs;
+                ksincos(s.y * r, &sn, &cs);
+                ax += mm * cs;
+                ay -= mm * sn;
+            }
+            ax = warp_sum(ax);
+            ay = warp_sum(ay);
+            if (lane == 0) {
+                Cx<float> v{ax, ay};
+                if (m > 0) {
+                    v.x += acc[k].x;
+                    v.y += acc[k].y;
+                }
+                if (m == nreg - 1) out[pr.off + (long long)k * pr.stride] = v;
+                else acc[k] = v;
+            }
+        }
+        __syncthreads();  // the region's points are consumed
+    }
+}
+
 // Linear continuous elements (element-local degrees of freedom): near-field
 // entries of element pairs without a common vertex by the 4-point rule on both
 // panels, one thread per element pair: the 16 point distances and weights are
@@ -580,22 +636,39 @@ __global__ void __launch_bounds__(256) k_near_p1(GeomF gf, GeomD gd, const int* 
 // -((x - y) . n_x) / r^2); each frequency's ten sums (the plain integral and
 // the nine weighted ones) are reduced over the CTA and added into acc.
 template <int OP, class T, int NT>
-__global__ void __launch_bounds__(NT) k_near_ss_p1(GeomD gd, SsRule gr, const SsPair* __restrict__ pairs,
-                                                   const double2* __restrict__ sd, int Ku, Cx<T>* __restrict__ out) {
+__global__ void __launch_bounds__(NT) k_near_ss_p1(GeomD gd, SsRule gr, const float4* __restrict__ tab,
+                                                   const SsPair* __restrict__ pairs, const double2* __restrict__ sd,
+                                                   const FreqT<T>* __restrict__ sk, int Ku, Cx<T>* __restrict__ out) {
     constexpr int NQ = SS_N * SS_N * SS_N * SS_N;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* pt = reinterpret_cast<T*>(smem_raw);                    // [7][NQ]: x1, x2, y1, y2, r, w, g
     Cx<T>* acc = reinterpret_cast<Cx<T>*>(pt + 7 * NQ);         // [Ku][10]
     __shared__ SsPanels P;
+    __shared__ SsEdges S32;
     const SsPair pr = pairs[blockIdx.x];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (threadIdx.x == 0) ss_panels(gd, pr.i, pr.j, pr.px, pr.py, P);
+    if constexpr (sizeof(T) == 4) ss_edges(gd, pr, S32);
+    else if (threadIdx.x == 0) ss_panels(gd, pr.i, pr.j, pr.px, pr.py, P);
     for (int e = threadIdx.x; e < Ku * 10; e += NT) acc[e] = Cx<T>{0, 0};
     double n[3];
     for (int k = 0; k < 3; ++k) n[k] = gd.n[k * gd.E + pr.i];
     __syncthreads();
     const int nreg = ss_regions(pr.cas);
     for (int mreg = 0; mreg < nreg; ++mreg) {
+        if constexpr (sizeof(T) == 4) {
+            // float32: points in float-float from the tables
+            const float4* tm = tab + (size_t)(ss_first_region(pr.cas) + mreg) * 4 * SS_Q;
+            for (int q = threadIdx.x; q < NQ; q += NT) {
+                float zn;
+                ss_point32<OP == G3_GAL_P1KP>(S32, tm, q, pt[4 * NQ + q], pt[5 * NQ + q], zn);
+                const float4 c = tm[2 * SS_Q + q], d = tm[3 * SS_Q + q];
+                pt[0 * NQ + q] = c.z;
+                pt[1 * NQ + q] = c.w;
+                pt[2 * NQ + q] = d.x;
+                pt[3 * NQ + q] = d.y;
+                pt[6 * NQ + q] = -zn;
+            }
+        } else
         for (int q = threadIdx.x; q < NQ; q += NT) {
             int rem = q;
             double g4[4], gw = 1.0;
@@ -625,8 +698,8 @@ __global__ void __launch_bounds__(NT) k_near_ss_p1(GeomD gd, SsRule gr, const Ss
         __syncthreads();
         // each warp owns every (NT / 32)-th frequency (no block-wide barrier per frequency)
         for (int k = wid; k < Ku; k += NT / 32) {
-            const double2 s = sd[k];
-            const T sre = (T)s.x, sim = (T)s.y;
+            const FreqT<T> s = sk[k];
+            const T sre = s.x, sim = s.y;
             Cx<T> v[10];
 #pragma unroll
             for (int u = 0; u < 10; ++u) v[u] = Cx<T>{0, 0};
@@ -668,24 +741,142 @@ __global__ void __launch_bounds__(NT) k_near_ss_p1(GeomD gd, SsRule gr, const Ss
         }
         __syncthreads();  // the region's points are consumed before the next region overwrites them
     }
-    // local entries (Sauter-Schwab vertex order c, d = local vertices px[c], py[d])
+    // local entries (Sauter-Schwab vertex order c, d = local vertices px[c], py[d]);
+    // the float64 factors s^2, curl_a . curl_b and n_x . n_y once per CTA, in the
+    // buffer of the consumed points
+    T* s2 = pt;            // [Ku] Re, then [Ku] Im at NQ
+    T* cn = pt + 2 * NQ;   // [9] curl products by (c, d), then n_x . n_y
+    if (OP == G3_GAL_P1D) {
+        for (int k = threadIdx.x; k < Ku; k += NT) {
+            const double2 s = sd[k];
+            s2[k] = (T)(s.x * s.x - s.y * s.y);
+            s2[NQ + k] = (T)(2.0 * s.x * s.y);
+        }
+        if (threadIdx.x < 10) {
+            const int c = threadIdx.x / 3, dd = threadIdx.x % 3;
+            T v = 0;
+            for (int kk = 0; kk < 3; ++kk)
+                v += threadIdx.x < 9 ? (T)(gd.curl[(pr.px[c] * 3 + kk) * gd.E + pr.i] * gd.curl[(pr.py[dd] * 3 + kk) * gd.E + pr.j])
+                                     : (T)(gd.n[kk * gd.E + pr.i] * gd.n[kk * gd.E + pr.j]);
+            cn[threadIdx.x] = v;
+        }
+        __syncthreads();
+    }
     for (int e = threadIdx.x; e < Ku * 9; e += NT) {
         const int k = e / 9, c = (e % 9) / 3, dd = e % 3;
         const int a = pr.px[c], b = pr.py[dd];
         Cx<T> val = acc[k * 10 + c * 3 + dd];
         if (OP == G3_GAL_P1D) {
-            const double2 s = sd[k];
-            const T s2r = (T)(s.x * s.x - s.y * s.y), s2i = (T)(2.0 * s.x * s.y);
-            T cab = 0, nn = 0;
-            for (int kk = 0; kk < 3; ++kk) {
-                cab += (T)(gd.curl[(a * 3 + kk) * gd.E + pr.i] * gd.curl[(b * 3 + kk) * gd.E + pr.j]);
-                nn += (T)(gd.n[kk * gd.E + pr.i] * gd.n[kk * gd.E + pr.j]);
-            }
+            const T s2r = s2[k], s2i = s2[NQ + k], cab = cn[c * 3 + dd], nn = cn[9];
             const Cx<T> i0 = acc[k * 10 + 9];
             val = Cx<T>{cab * i0.x + nn * (s2r * val.x - s2i * val.y), cab * i0.y + nn * (s2r * val.y + s2i * val.x)};
         }
         out[pr.off + (long long)k * pr.stride + a + (long long)b * pr.ldm] = val;
     }
+}
+
+// The pairs of a near field with a common vertex: one CTA per near block classifies
+// its element pairs and appends the records (their order does not matter; one
+// counter increment per warp).  p1: blocks of linear elements (three rows per
+// element, the record's offset that of local functions (0, 0)).
+__global__ void __launch_bounds__(256) k_ss_pairs(const int* __restrict__ tv, const BlockRange* __restrict__ ranges,
+                                                  const long long* __restrict__ offs, int p1, SsPair* __restrict__ out,
+                                                  int cap, int* __restrict__ count) {
+    const int d = p1 ? 3 : 1;
+    const BlockRange br = ranges[blockIdx.x];
+    const int M = br.re - br.rb, N = br.ce - br.cb, Me = M / d, Ne = N / d;
+    const int lane = threadIdx.x & 31;
+    for (int e0 = 0; e0 < Me * Ne; e0 += blockDim.x) {
+        const int e = e0 + threadIdx.x;
+        SsPair q{};
+        q.cas = SS_REGULAR;
+        if (e < Me * Ne) {
+            q.i = br.rb / d + e % Me;
+            q.j = br.cb / d + e / Me;
+            q.cas = ss_classify(tv + 3 * (size_t)q.i, tv + 3 * (size_t)q.j, q.i == q.j, q.px, q.py);
+            q.stride = M * N;
+            q.ldm = M;
+            q.off = offs[blockIdx.x] + (long long)(d * q.j - br.cb) * M + (d * q.i - br.rb);
+        }
+        const unsigned mask = __ballot_sync(0xffffffffu, q.cas != SS_REGULAR);
+        int base = 0;
+        if (lane == 0 && mask) base = atomicAdd(count, __popc(mask));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        const int at = base + __popc(mask & ((1u << lane) - 1u));
+        if (q.cas != SS_REGULAR && at < cap) out[at] = q;
+    }
+}
+
+g3_status launch_ss_pairs(g3_ctx* ctx, const g3_tree* t, g3_near* nf) {
+    // at most one record per (element, element) of every vertex
+    std::vector<int> deg(t->nv, 0);
+    for (int32_t v : t->tris) ++deg[v];
+    long long bound = 0;
+    for (int d : deg) bound += (long long)d * d;
+    if (bound > INT32_MAX) return fail(G3_EUNSUPPORTED, "assemble_near: too many element pairs with a common vertex");
+    const int nb = (int)nf->order.size();
+    if (nb == 0) return G3_OK;
+    DevBuf cnt;
+    G3_CUDA(cnt.alloc(sizeof(int)));
+    G3_CUDA(cudaMemsetAsync(cnt.p, 0, sizeof(int), ctx->stream));
+    G3_CUDA(nf->d_ss.alloc((size_t)std::max<long long>(bound, 1) * sizeof(SsPair)));
+    k_ss_pairs<<<nb, 256, 0, ctx->stream>>>(t->d_tv.as<int>(), nf->d_ranges.as<BlockRange>(),
+                                            nf->d_offs.as<long long>(), t->p1 ? 1 : 0, nf->d_ss.as<SsPair>(),
+                                            (int)bound, cnt.as<int>());
+    ctx->count("k_ss_pairs");
+    G3_CUDA(cudaGetLastError());
+    int n = 0;
+    G3_CUDA(cudaMemcpyAsync(&n, cnt.p, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    G3_CUDA(cudaStreamSynchronize(ctx->stream));
+    if (n > bound) return fail(G3_ECUDA, "assemble_near: %d pairs with a common vertex, at most %lld expected", n, bound);
+    nf->n_ss = n;
+    return G3_OK;
+}
+
+// the Sauter-Schwab point table of the float32 kernels (SsEdges), once per context
+static g3_status ss_table(g3_ctx* ctx) {
+    if (ctx->ss_tab.p) return G3_OK;
+    double gx[SS_N], gw[SS_N];
+    gauss_legendre01(SS_N, gx, gw);
+    static_assert(SS_Q == SS_N * SS_N * SS_N * SS_N, "points per region");
+    std::vector<float> tab((size_t)13 * 4 * SS_Q * 4, 0.f);
+    auto put = [&](int reg, int arr, int q, int c, double v) { tab[(((size_t)reg * 4 + arr) * SS_Q + q) * 4 + c] = (float)v; };
+    auto put2 = [&](int reg, int arr, int q, int c, double v) {
+        const float h = (float)v;
+        put(reg, arr, q, c, h);
+        put(reg, arr, q, c + 1, v - (double)h);
+    };
+    for (int cas = SS_VERTEX; cas <= SS_IDENTICAL; ++cas)
+        for (int m = 0; m < ss_regions(cas); ++m)
+            for (int q = 0; q < SS_Q; ++q) {
+                int rem = q;
+                double g4[4], w = 1.0;
+                for (int a = 3; a >= 0; --a) {
+                    g4[a] = gx[rem % SS_N];
+                    w *= gw[rem % SS_N];
+                    rem /= SS_N;
+                }
+                double x[2], y[2];
+                const double f = ss_map(cas, m, g4[0], g4[1], g4[2], g4[3], x, y);
+                const int reg = ss_first_region(cas) + m;
+                put2(reg, 0, q, 0, cas == SS_VERTEX ? x[0] : x[0] - y[0]);
+                put2(reg, 0, q, 2, cas == SS_IDENTICAL ? x[1] - y[1] : x[1]);
+                put2(reg, 1, q, 0, cas == SS_VERTEX ? -y[0] : 0.0);
+                put2(reg, 1, q, 2, cas == SS_IDENTICAL ? 0.0 : -y[1]);
+                put2(reg, 2, q, 0, w * f);
+                put(reg, 2, q, 2, x[0]);
+                put(reg, 2, q, 3, x[1]);
+                put(reg, 3, q, 0, y[0]);
+                put(reg, 3, q, 1, y[1]);
+            }
+    DevBuf d;
+    G3_CUDA(d.alloc(tab.size() * sizeof(float)));
+    G3_CUDA(cudaMemcpy(d.p, tab.data(), tab.size() * sizeof(float), cudaMemcpyHostToDevice));
+    ctx->ss_tab.p = d.p;
+    ctx->ss_tab.bytes = d.bytes;
+    d.p = nullptr;
+    d.bytes = 0;
+    return G3_OK;
 }
 
 // the unique frequencies in the working precision
@@ -714,8 +905,13 @@ static g3_status launch_near_p1_t(g3_ctx* ctx, const g3_tree* t, const g3_freqs*
         if (smem > ctx->smem_optin)
             return fail(G3_EUNSUPPORTED, "assemble_near: %zu bytes of shared memory for the singular pairs", smem);
         G3_CUDA(cudaFuncSetAttribute(k_near_ss_p1<OP, T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_near_ss_p1<OP, T, NT><<<nf->n_ss, NT, smem, ctx->stream>>>(t->gd, gr, nf->d_ss.as<SsPair>(),
-                                                                      f->d_sd.as<double2>(), f->Ku, o);
+        if (sizeof(T) == 4) {
+            const g3_status st = ss_table(ctx);
+            if (st != G3_OK) return st;
+        }
+        k_near_ss_p1<OP, T, NT><<<nf->n_ss, NT, smem, ctx->stream>>>(t->gd, gr, ctx->ss_tab.as<float4>(),
+                                                                      nf->d_ss.as<SsPair>(), f->d_sd.as<double2>(),
+                                                                      freqs_of<T>(f), f->Ku, o);
         ctx->count("k_near_ss_p1");
         G3_CUDA(cudaGetLastError());
     }
@@ -868,13 +1064,21 @@ static g3_status launch_near_galerkin(g3_ctx* ctx, const g3_tree* t, const g3_fr
     ctx->count("k_near");
     G3_CUDA(cudaGetLastError());
     if (nf->n_ss > 0) {
-        SsRule gr;
-        gauss_legendre01(SS_N, gr.x, gr.w);
         constexpr int NT = 256;
-        const size_t smem = 2 * (size_t)SS_N * SS_N * SS_N * SS_N * 6 * sizeof(T);
-        G3_CUDA(cudaFuncSetAttribute(k_near_ss<T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_near_ss<T, NT><<<nf->n_ss, NT, smem, ctx->stream>>>(t->gd, gr, nf->d_ss.as<SsPair>(),
-                                                              f->d_sd.as<double2>(), f->Ku, o);
+        if constexpr (sizeof(T) == 4) {
+            const g3_status st = ss_table(ctx);
+            if (st != G3_OK) return st;
+            const size_t smem = 2 * SS_Q * sizeof(float) + (size_t)f->Ku * sizeof(Cx<float>);
+            k_near_ss32<NT><<<nf->n_ss, NT, smem, ctx->stream>>>(t->gd, ctx->ss_tab.as<float4>(), nf->d_ss.as<SsPair>(),
+                                                                 f->d_sf.as<float2>(), f->Ku, o);
+        } else {
+            SsRule gr;
+            gauss_legendre01(SS_N, gr.x, gr.w);
+            const size_t smem = 2 * (size_t)SS_N * SS_N * SS_N * SS_N * 6 * sizeof(T);
+            G3_CUDA(cudaFuncSetAttribute(k_near_ss<T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            k_near_ss<T, NT><<<nf->n_ss, NT, smem, ctx->stream>>>(t->gd, gr, nf->d_ss.as<SsPair>(),
+                                                                  f->d_sd.as<double2>(), f->Ku, o);
+        }
         ctx->count("k_near_ss");
         G3_CUDA(cudaGetLastError());
     }
