@@ -35,6 +35,18 @@ __device__ __forceinline__ Cx<T> ldcx(const Cx<T>* p) {
     }
 }
 
+// the same for values read once (evicted first)
+template <class T>
+__device__ __forceinline__ Cx<T> ldcx_once(const Cx<T>* p) {
+    if constexpr (sizeof(T) == 4) {
+        const float2 v = __ldcs(reinterpret_cast<const float2*>(p));
+        return {v.x, v.y};
+    } else {
+        const double2 v = __ldcs(reinterpret_cast<const double2*>(p));
+        return {v.x, v.y};
+    }
+}
+
 template <class T>
 __device__ __forceinline__ Cx<T> cmul(Cx<T> a, Cx<T> b) {
     return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
@@ -708,16 +720,15 @@ __device__ __forceinline__ void tf32_neg4(const unsigned* a, unsigned* o) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) o[q] = a[q] ^ 0x80000000u;
 }
-// ---- prefetch of a contiguous range into L2 (whole 16-byte units inside it) --------
-__device__ __forceinline__ void l2_prefetch(const void* p, long long bytes) {
-    const unsigned long long a = ((unsigned long long)p + 15ull) & ~15ull, e = ((unsigned long long)p + bytes) & ~15ull;
-    if (e > a)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((unsigned)(e - a)) : "memory");
-}
 // ---- asynchronous copies global -> shared (8 bytes; zero-filled when !in) ---------
 __device__ __forceinline__ void cp_async8(void* smem, const void* gmem, bool in) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(sa), "l"(gmem), "r"(in ? 8 : 0) : "memory");
+}
+// 16 bytes past L1 (both addresses 16-byte aligned); the last 16 - bytes zero-filled
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem, int bytes) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
