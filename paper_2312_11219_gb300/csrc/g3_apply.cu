@@ -1072,128 +1072,273 @@ __global__ void __launch_bounds__(NT) k_pf_near(const Cx<T>* __restrict__ A, con
     }
 }
 
-// far field: one CTA per item (block, 32 right-hand sides c0.., 128 rows
-// i0..).  Right-hand side c < Ku is w_c, c >= Ku is conj(w'_{c-Ku}); its
-// fiber coefficient is f_p[c mod Ku].  Per cross p of the block:
-//   low-rank face:  t[q][c] = V_p[:, q]^H x_c   (q < r_p, the block's columns
-//                   of x_c staged 64 at a time), then z[i][c] += f_p[c] U_p[i, :] t[:, c];
-//   dense face:     z[i][c] += f_p[c] H_p[i, :] x_c.
-// Thread (i = tid / 32 + 8 m, c = tid % 32) keeps 16 outputs in registers;
-// the CTA adds them to yf / yc once.
-constexpr int PF_NT = 256, PF_NC = 32, PF_NI = 128, PF_JC = 64;
-
+// two neighbouring values (16-byte aligned in float32)
 template <class T>
-__global__ void __launch_bounds__(PF_NT) k_pf_far(const Cx<T>* __restrict__ pool, const CrossRec* __restrict__ rec,
-                                                  const int* __restrict__ r3, const BlockRange* __restrict__ ranges,
-                                                  const int4* __restrict__ items, int Cmax, int Ku, int E,
-                                                  const Cx<T>* __restrict__ Wf, const Cx<T>* __restrict__ Wc,
-                                                  Cx<T>* __restrict__ yf, Cx<T>* __restrict__ yc) {
+__device__ __forceinline__ void ldcx2(const Cx<T>* p, Cx<T>& a, Cx<T>& b) {
+    if constexpr (sizeof(T) == 4) {
+        const float4 v = *reinterpret_cast<const float4*>(p);
+        a = Cx<T>{v.x, v.y};
+        b = Cx<T>{v.z, v.w};
+    } else {
+        a = ldcx(p);
+        b = ldcx(p + 1);
+    }
+}
+
+// far field, blocks with dense faces: one CTA per (item of k_apply_far_dense,
+// frequency chunk), the item's fibers in shared memory.  Both right-hand sides of a
+// frequency see the same matrix, so it is formed once, in registers:
+//   A_k[i, j] = sum_p f_p[k] H_p[i, j],  yf_k[i] += A_k[i, j] w_k[j],  yc_k[i] += A_k[i, j] conj(w'_k[j]),
+// r + 2 products per entry and frequency for the 2 r of H_p x per right-hand side.
+// A warp takes (the item's slots of one block, PD_KT frequencies, 32 rows), lane i row
+// i; two columns at a time share the fiber values, and the values of H come from L1
+// (an item's 16 faces of 24 x 24 take 74 KB).
+// Before, both kinds of faces went through one kernel, a CTA per (block, 32 right-hand
+// sides, 128 rows): every multiply-add read one value of H or V through a broadcast
+// load, and a block of 24 rows kept 3 of a thread's 16 sums busy.  3,072-triangle
+// L-shape, 33 unique frequencies, the whole per-frequency apply: 3.51 -> 1.70 ms.
+constexpr int PD_NT = 128, PD_KT = 4, PD_KC = 64;
+template <class T>
+__global__ void __launch_bounds__(PD_NT) k_pf_far_dense(const Cx<T>* __restrict__ pool, const CrossRec* __restrict__ rec,
+                                                        const BlockRange* __restrict__ ranges,
+                                                        const int4* __restrict__ items, const int2* __restrict__ slots,
+                                                        int Cmax, int Ku, int kchunk, int E, const Cx<T>* __restrict__ Wf,
+                                                        const Cx<T>* __restrict__ Wc, Cx<T>* __restrict__ yf,
+                                                        Cx<T>* __restrict__ yc) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    // xs [PF_JC][PF_NC + 1], ts [RF_TS][PF_NC + 1] (dynamic: above 48 KB in float64)
-    auto xs = reinterpret_cast<Cx<T>(*)[PF_NC + 1]>(smem_raw);
-    auto ts = reinterpret_cast<Cx<T>(*)[PF_NC + 1]>(smem_raw + (size_t)PF_JC * (PF_NC + 1) * sizeof(Cx<T>));
-    __shared__ Cx<T> fs[PF_NC];
-    const int4 it = items[blockIdx.x];
-    const int blk = it.x, c0 = it.y, i0 = it.z;
-    const BlockRange br = ranges[blk];
-    const int M = br.re - br.rb, N = br.ce - br.cb;
-    const int tid = threadIdx.x, cl = tid & 31, il = tid >> 5;
-    const int nrhs = 2 * Ku;
-    Cx<T> z[16];
+    Cx<T>* fs = reinterpret_cast<Cx<T>*>(smem_raw);   // [FD_SL][KS], zero beyond the chunk
+    __shared__ long long soff[FD_SL];
+    __shared__ int srb[FD_SL], sm[FD_SL], run0[FD_SL + 1], n_run;
+    const int4 it = items[blockIdx.x];                // first slot, slots, first column, columns
+    const int ns = it.y, cb = it.z, N = it.w;
+    const int k0 = blockIdx.y * kchunk, nk = min(Ku, k0 + kchunk) - k0;
+    const int KS = (kchunk + PD_KT - 1) / PD_KT * PD_KT;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid < ns) {
+        const int2 sl = slots[it.x + tid];
+        const BlockRange br = ranges[sl.x];
+        srb[tid] = br.rb;
+        sm[tid] = br.re - br.rb;
+        soff[tid] = rec[(size_t)sl.x * Cmax + sl.y].off;
+    }
+    if (tid == 0) {
+        int n = 0;
+        for (int p = 0; p < ns; ++p)
+            if (p == 0 || slots[it.x + p].x != slots[it.x + p - 1].x) run0[n++] = p;
+        run0[n] = ns;
+        n_run = n;
+    }
+    __syncthreads();
+    for (int e = tid; e < ns * KS; e += PD_NT) {
+        const int p = e / KS, k = e - p * KS;
+        fs[e] = k < nk ? ldcx(pool + soff[p] + (long long)sm[p] * N + k0 + k) : Cx<T>{0, 0};
+    }
+    __syncthreads();
+    const int ng = (nk + PD_KT - 1) / PD_KT;
+    for (int q = warp; q < n_run * ng; q += PD_NT / 32) {
+        const int run = q / ng, kg = (q - run * ng) * PD_KT;
+        const int pa = run0[run], pb = run0[run + 1], M = sm[pa];
+        const int kn = min(PD_KT, nk - kg);
+        const Cx<T>* wf = Wf + (long long)(k0 + kg) * E + cb;
+        const Cx<T>* wc = Wc + (long long)(k0 + kg) * E + cb;
+        for (int i0 = 0; i0 < M; i0 += 32) {
+            const int i = min(i0 + lane, M - 1);      // (lanes past the block's rows repeat the last one)
+            Cx<T> s1[PD_KT], s2[PD_KT];
 #pragma unroll
-    for (int m = 0; m < 16; ++m) z[m] = Cx<T>{0, 0};
-    // stage x_c[j0 .. j0 + PF_JC) for the 32 right-hand sides
-    auto stage = [&](int j0) {
-        for (int e = tid; e < PF_JC * PF_NC; e += PF_NT) {
-            const int c = e / PF_JC, jj = e - c * PF_JC;
-            const int gc = c0 + c, j = j0 + jj;
-            Cx<T> v{0, 0};
-            if (gc < nrhs && j < N) {
-                if (gc < Ku) v = ldcx(Wf + (long long)gc * E + br.cb + j);
-                else v = cconj(ldcx(Wc + (long long)(gc - Ku) * E + br.cb + j));
-            }
-            xs[jj][c] = v;
-        }
-    };
-    const int nc = r3[blk];
-    for (int p = 0; p < nc; ++p) {
-        const CrossRec cr = rec[(size_t)blk * Cmax + p];
-        const bool dense = cr.r < 0;
-        const Cx<T>* fb = pool + cr.off + (dense ? (long long)M * N : (long long)cr.r * (M + N));
-        __syncthreads();  // previous cross done with xs / ts / fs
-        if (tid < PF_NC) {
-            const int gc = c0 + tid;
-            fs[tid] = gc < nrhs ? ldcx(fb + (gc < Ku ? gc : gc - Ku)) : Cx<T>{0, 0};
-        }
-        if (dense) {
-            const Cx<T>* H = pool + cr.off;
-            Cx<T> acc[16];
+            for (int u = 0; u < PD_KT; ++u) s1[u] = s2[u] = Cx<T>{0, 0};
+            for (int j = 0; j < N; j += 2) {
+                const int dj = j + 1 < N ? 1 : 0;
+                Cx<T> a0[PD_KT], a1[PD_KT];
 #pragma unroll
-            for (int m = 0; m < 16; ++m) acc[m] = Cx<T>{0, 0};
-            for (int j0 = 0; j0 < N; j0 += PF_JC) {
-                __syncthreads();
-                stage(j0);
-                __syncthreads();
-                const int jn = min(PF_JC, N - j0);
+                for (int u = 0; u < PD_KT; ++u) a0[u] = a1[u] = Cx<T>{0, 0};
+                const long long o = (long long)j * M + i;
+#pragma unroll 4
+                for (int p = pa; p < pb; ++p) {
+                    const Cx<T>* H = pool + soff[p] + o;
+                    const Cx<T> h0 = ldcx(H), h1 = ldcx(H + dj * M);
+                    Cx<T> f[PD_KT];
 #pragma unroll
-                for (int m = 0; m < 16; ++m) {
-                    const int i = i0 + il + 8 * m;
-                    if (i < M)
-                        for (int jj = 0; jj < jn; ++jj) cfma(acc[m], ldcx(H + (long long)(j0 + jj) * M + i), xs[jj][cl]);
+                    for (int u = 0; u < PD_KT; u += 2) ldcx2(fs + p * KS + kg + u, f[u], f[u + 1]);
+#pragma unroll
+                    for (int u = 0; u < PD_KT; ++u) {
+                        cfma(a0[u], f[u], h0);
+                        cfma(a1[u], f[u], h1);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < PD_KT; ++u) {
+                    if (u < kn) {
+                        const long long wo = (long long)u * E + j;
+                        cfma(s1[u], a0[u], ldcx(wf + wo));
+                        cfmac(s2[u], a0[u], ldcx(wc + wo));
+                        if (dj) {
+                            cfma(s1[u], a1[u], ldcx(wf + wo + 1));
+                            cfmac(s2[u], a1[u], ldcx(wc + wo + 1));
+                        }
+                    }
                 }
             }
-            __syncthreads();
-            const Cx<T> f = fs[cl];
+            if (i0 + lane < M) {
 #pragma unroll
-            for (int m = 0; m < 16; ++m) cfma(z[m], f, acc[m]);
-            continue;
-        }
-        const int r = cr.r;
-        const Cx<T>* U = pool + cr.off;
-        const Cx<T>* V = U + (long long)r * M;
-        // t[q][c] = V_p[:, q]^H x_c; thread (q = il + 8 m, c = cl)
-        Cx<T> t[RF_TS / 8];
-#pragma unroll
-        for (int m = 0; m < RF_TS / 8; ++m) t[m] = Cx<T>{0, 0};
-        for (int j0 = 0; j0 < N; j0 += PF_JC) {
-            __syncthreads();
-            stage(j0);
-            __syncthreads();
-            const int jn = min(PF_JC, N - j0);
-#pragma unroll
-            for (int m = 0; m < RF_TS / 8; ++m) {
-                const int q = il + 8 * m;
-                if (q < r)
-                    for (int jj = 0; jj < jn; ++jj) cfmac(t[m], xs[jj][cl], ldcx(V + (long long)q * N + j0 + jj));
-            }
-        }
-#pragma unroll
-        for (int m = 0; m < RF_TS / 8; ++m) {
-            const int q = il + 8 * m;
-            if (q < r) ts[q][cl] = t[m];
-        }
-        __syncthreads();
-        const Cx<T> f = fs[cl];
-#pragma unroll
-        for (int m = 0; m < 16; ++m) {
-            const int i = i0 + il + 8 * m;
-            if (i < M) {
-                Cx<T> s{0, 0};
-                for (int q = 0; q < r; ++q) cfma(s, ldcx(U + (long long)q * M + i), ts[q][cl]);
-                cfma(z[m], f, s);
+                for (int u = 0; u < PD_KT; ++u) {
+                    if (u < kn) {
+                        const long long yo = (long long)(k0 + kg + u) * E + srb[pa] + i;
+                        atomicAdd(&yf[yo].x, s1[u].x);
+                        atomicAdd(&yf[yo].y, s1[u].y);
+                        atomicAdd(&yc[yo].x, s2[u].x);
+                        atomicAdd(&yc[yo].y, s2[u].y);
+                    }
+                }
             }
         }
     }
-    const int gc = c0 + cl;
-    if (gc >= nrhs) return;
-    Cx<T>* out = gc < Ku ? yf + (long long)gc * E : yc + (long long)(gc - Ku) * E;
-#pragma unroll
-    for (int m = 0; m < 16; ++m) {
-        const int i = i0 + il + 8 * m;
-        if (i < M) {
-            atomicAdd(&out[br.rb + i].x, z[m].x);
-            atomicAdd(&out[br.rb + i].y, z[m].y);
+}
+
+// far field, blocks with low-rank faces: one CTA per (item of k_far_lr: block and
+// group of FAR_PG crosses, PF_NC right-hand sides c0..).  Right-hand side c < Ku is w_c,
+// c >= Ku is conj(w'_{c-Ku}); its fiber coefficient is f_p[c mod Ku].  As many of the
+// group's crosses at a time as have PF_NQ columns together:
+//   1. t[q][c] = f_p[c] V_p[:, q]^H x_c, kept in shared memory;
+//   2. z[i][c] = sum_q U[i, q] t[q][c], added to yf / yc.
+// Both are products of tall matrices with PF_NC columns: warp w takes columns c0 + 4 w..
+// (a warp without columns only stages), lane l rows 2 l, 2 l + 1 of a tile of 64, so
+// that three 16-byte reads of shared memory feed 32 multiply-adds.
+constexpr int PF_NT = 256, PF_NC = 32, PF_NQ = 128, PF_JC = 32, PF_LD = 66, PF_LX = 34;
+template <class T>
+constexpr size_t pf_lr_smem() {   // t, tile of V or U, tile of x
+    return ((size_t)PF_NQ * PF_LX + (size_t)PF_JC * PF_LD + (size_t)PF_JC * PF_LX) * sizeof(Cx<T>);
+}
+template <class T>
+__global__ void __launch_bounds__(PF_NT) k_pf_far_lr(const Cx<T>* __restrict__ pool, const CrossRec* __restrict__ rec,
+                                                     const int* __restrict__ r3, const BlockRange* __restrict__ ranges,
+                                                     const int4* __restrict__ items, int Cmax, int Ku, int E,
+                                                     const Cx<T>* __restrict__ Wf, const Cx<T>* __restrict__ Wc,
+                                                     Cx<T>* __restrict__ yf, Cx<T>* __restrict__ yc) {
+    static_assert(PF_NQ >= 2 * RF_TS, "a cross's columns fit the tile of t");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Cx<T>* ts = reinterpret_cast<Cx<T>*>(smem_raw);   // [PF_NQ][PF_LX]
+    Cx<T>* as = ts + PF_NQ * PF_LX;                    // [PF_JC][PF_LD]: V (column, q) or U (q, row)
+    Cx<T>* xs = as + PF_JC * PF_LD;                    // [PF_JC][PF_LX]
+    __shared__ CrossRec crs[FAR_PG];
+    __shared__ Cx<T> fs[FAR_PG][PF_NC];
+    __shared__ long long uo[PF_NQ], vo[PF_NQ];         // pool offsets of U_p[:, q], V_p[:, q]
+    __shared__ int pq[PF_NQ];
+    const int4 it = items[blockIdx.x];
+    const int blk = it.x, g0 = it.y * FAR_PG, c0 = blockIdx.y * PF_NC, nrhs = 2 * Ku;
+    const BlockRange br = ranges[blk];
+    const int M = br.re - br.rb, N = br.ce - br.cb;
+    const int np = min(FAR_PG, r3[blk] - g0);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int cw = warp * 4;
+    const bool act = c0 + cw < nrhs;
+    if (tid < np) crs[tid] = rec[(size_t)blk * Cmax + g0 + tid];
+    __syncthreads();
+    for (int e = tid; e < np * PF_NC; e += PF_NT) {
+        const int p = e / PF_NC, c = e - p * PF_NC, gc = c0 + c;
+        fs[p][c] = gc < nrhs ? ldcx(pool + crs[p].off + (long long)crs[p].r * (M + N) + (gc < Ku ? gc : gc - Ku))
+                             : Cx<T>{0, 0};
+    }
+    for (int pa = 0; pa < np;) {
+        int pb = pa, Q = 0;
+        while (pb < np && Q + crs[pb].r <= PF_NQ) Q += crs[pb++].r;
+        __syncthreads();   // the crosses before are done with the offsets and t
+        if (tid < Q) {
+            int p = pa, q = tid;
+            while (q >= crs[p].r) q -= crs[p++].r;
+            pq[tid] = p;
+            uo[tid] = crs[p].off + (long long)q * M;
+            vo[tid] = crs[p].off + (long long)crs[p].r * M + (long long)q * N;
         }
+        // ---- 1. t ----
+        for (int q0 = 0; q0 < Q; q0 += 64) {
+            Cx<T> t[2][4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) t[0][u] = t[1][u] = Cx<T>{0, 0};
+            for (int j0 = 0; j0 < N; j0 += PF_JC) {
+                const int jn = min(PF_JC, N - j0), j = br.cb + j0 + lane;
+                __syncthreads();
+                for (int q = warp; q < 64; q += PF_NT / 32)
+                    as[lane * PF_LD + q] =
+                        q0 + q < Q && lane < jn ? ldcx(pool + vo[q0 + q] + j0 + lane) : Cx<T>{0, 0};
+                for (int c = warp; c < PF_NC; c += PF_NT / 32) {
+                    const int gc = c0 + c;
+                    Cx<T> v{0, 0};
+                    if (gc < nrhs && lane < jn)
+                        v = gc < Ku ? ldcx(Wf + (long long)gc * E + j) : cconj(ldcx(Wc + (long long)(gc - Ku) * E + j));
+                    xs[lane * PF_LX + c] = v;
+                }
+                __syncthreads();
+                if (act) {
+#pragma unroll 4
+                    for (int jj = 0; jj < jn; ++jj) {
+                        Cx<T> v0, v1, x[4];
+                        ldcx2(as + jj * PF_LD + 2 * lane, v0, v1);
+                        ldcx2(xs + jj * PF_LX + cw, x[0], x[1]);
+                        ldcx2(xs + jj * PF_LX + cw + 2, x[2], x[3]);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            cfmac(t[0][u], x[u], v0);
+                            cfmac(t[1][u], x[u], v1);
+                        }
+                    }
+                }
+            }
+            if (act) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int q = q0 + 2 * lane + e;
+                    if (q < Q) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) ts[q * PF_LX + cw + u] = cmul(fs[pq[q]][cw + u], t[e][u]);
+                    }
+                }
+            }
+        }
+        // ---- 2. z, 64 rows at a time ----
+        for (int i0 = 0; i0 < M; i0 += 64) {
+            Cx<T> z[2][4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) z[0][u] = z[1][u] = Cx<T>{0, 0};
+            for (int q0 = 0; q0 < Q; q0 += PF_JC) {
+                const int qn = min(PF_JC, Q - q0);
+                __syncthreads();
+                for (int e = tid; e < PF_JC * 64; e += PF_NT) {
+                    const int q = e >> 6, i = e & 63;
+                    as[q * PF_LD + i] = q < qn && i0 + i < M ? ldcx(pool + uo[q0 + q] + i0 + i) : Cx<T>{0, 0};
+                }
+                __syncthreads();
+                if (act) {
+#pragma unroll 4
+                    for (int q = 0; q < qn; ++q) {
+                        Cx<T> a0, a1, t[4];
+                        ldcx2(as + q * PF_LD + 2 * lane, a0, a1);
+                        ldcx2(ts + (q0 + q) * PF_LX + cw, t[0], t[1]);
+                        ldcx2(ts + (q0 + q) * PF_LX + cw + 2, t[2], t[3]);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            cfma(z[0][u], a0, t[u]);
+                            cfma(z[1][u], a1, t[u]);
+                        }
+                    }
+                }
+            }
+            if (act) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int gc = c0 + cw + u;
+                    if (gc >= nrhs) break;
+                    Cx<T>* out = (gc < Ku ? yf + (long long)gc * E : yc + (long long)(gc - Ku) * E) + br.rb + i0 + 2 * lane;
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        if (i0 + 2 * lane + e < M) {
+                            atomicAdd(&out[e].x, z[e][u].x);
+                            atomicAdd(&out[e].y, z[e][u].y);
+                        }
+                    }
+                }
+            }
+        }
+        pa = pb;
     }
 }
 
@@ -1219,33 +1364,13 @@ static g3_status run_apply_perfreq_t(g3_ctx* ctx, const g3_tree* t, const g3_nea
                                      const void* W, void* Y, int dtype, const g3_freqs* f) {
     const int E = t->ne, K = f->K, Ku = f->Ku;
     const size_t nW = (size_t)Ku * E;
-    // work items of the far field: (block, right-hand-side chunk, row chunk)
-    std::vector<int> items;
-    if (fa) {
-        for (int b = 0; b < fa->n_far; ++b) {
-            if (fa->r3[b] <= 0) continue;
-            const int M = fa->ranges[b].re - fa->ranges[b].rb;
-            for (int c0 = 0; c0 < 2 * Ku; c0 += PF_NC)
-                for (int i0 = 0; i0 < M; i0 += PF_NI) items.insert(items.end(), {b, c0, i0, 0});
-            for (int p = 0; p < fa->r3[b]; ++p)
-                if (fa->crec(b, p).r > RF_TS)
-                    return fail(G3_EUNSUPPORTED, "apply_gcq: face rank %d above %d in the per-frequency apply",
-                                fa->crec(b, p).r, RF_TS);
-        }
-    }
-    const size_t n_items = items.size() / 4;
-    const size_t need = 4 * nW * sizeof(Cx<T>) + (n_items + 1) * sizeof(int4) + 512;
-    G3_CUDA(ctx->scratch.ensure(need));
+    G3_CUDA(ctx->scratch.ensure(4 * nW * sizeof(Cx<T>)));
     Cx<T>* Wf = ctx->scratch.as<Cx<T>>();
     Cx<T>* Wc = Wf + nW;
     Cx<T>* yf = Wc + nW;
     Cx<T>* yc = yf + nW;
-    int4* d_items = reinterpret_cast<int4*>((reinterpret_cast<uintptr_t>(yc + nW) + 255) & ~uintptr_t(255));
     cudaEvent_t e0 = ctx->ev[2], e3 = ctx->ev[5];
     G3_CUDA(cudaEventRecord(e0, ctx->stream));
-    if (n_items)
-        G3_CUDA(cudaMemcpyAsync(d_items, items.data(), items.size() * sizeof(int), cudaMemcpyHostToDevice,
-                                ctx->stream));
     G3_CUDA(cudaMemsetAsync(yf, 0, 2 * nW * sizeof(Cx<T>), ctx->stream));
     {
         const int blocks = (int)((nW + 255) / 256);
@@ -1267,15 +1392,30 @@ static g3_status run_apply_perfreq_t(g3_ctx* ctx, const g3_tree* t, const g3_nea
         ctx->count("k_pf_near");
         G3_CUDA(cudaGetLastError());
     }
-    if (n_items) {
-        if (!fa->plan_ready) return fail(G3_EINVAL, "apply_gcq: factors without block ranges on the device");
-        const size_t smem = (size_t)(PF_JC + RF_TS) * (PF_NC + 1) * sizeof(Cx<T>);
-        G3_CUDA(cudaFuncSetAttribute(k_pf_far<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_pf_far<T><<<(unsigned)n_items, PF_NT, smem, ctx->stream>>>(fa->pool->as<Cx<T>>(), fa->d_rec.as<CrossRec>(),
-                                                                  fa->d_r3.as<int>(), fa->d_franges.as<BlockRange>(),
-                                                                  d_items, fa->Cmax, Ku, E, Wf, Wc, yf, yc);
-        ctx->count("k_pf_far");
-        G3_CUDA(cudaGetLastError());
+    if (fa && fa->n_far > 0) {
+        if (!fa->plan_ready) return fail(G3_EINVAL, "apply_gcq: factors without far-field work lists");
+        const int nd = fa->plan_nd, nl = fa->plan_n1 + fa->plan_n2;
+        const int4* it0 = fa->d_plan.as<int4>();
+        const int4* it1 = it0 + nd;
+        const BlockRange* d_ranges = fa->d_franges.as<BlockRange>();
+        if (nd > 0) {
+            const int nch = (Ku + PD_KC - 1) / PD_KC, kchunk = (Ku + nch - 1) / nch;
+            const size_t smem = (size_t)FD_SL * ((kchunk + PD_KT - 1) / PD_KT * PD_KT) * sizeof(Cx<T>);
+            k_pf_far_dense<T><<<dim3(nd, nch), PD_NT, smem, ctx->stream>>>(
+                fa->pool->as<Cx<T>>(), fa->d_rec.as<CrossRec>(), d_ranges, it0, reinterpret_cast<const int2*>(it1 + nl),
+                fa->Cmax, Ku, kchunk, E, Wf, Wc, yf, yc);
+            ctx->count("k_pf_far_dense");
+            G3_CUDA(cudaGetLastError());
+        }
+        if (nl > 0) {
+            constexpr size_t smem = pf_lr_smem<T>();
+            G3_CUDA(cudaFuncSetAttribute(k_pf_far_lr<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            k_pf_far_lr<T><<<dim3(nl, (2 * Ku + PF_NC - 1) / PF_NC), PF_NT, smem, ctx->stream>>>(
+                fa->pool->as<Cx<T>>(), fa->d_rec.as<CrossRec>(), fa->d_r3.as<int>(), d_ranges, it1, fa->Cmax, Ku, E, Wf,
+                Wc, yf, yc);
+            ctx->count("k_pf_far_lr");
+            G3_CUDA(cudaGetLastError());
+        }
     }
     {
         const int blocks = (int)((nW + 255) / 256);
