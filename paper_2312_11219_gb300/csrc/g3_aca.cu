@@ -123,15 +123,6 @@ static void compact_records(g3_factors* fa, const std::vector<CrossRec>& full, i
     }
 }
 
-// move a device buffer's ownership
-static void take(DevBuf& dst, DevBuf& src) {
-    dst.release();
-    dst.p = src.p;
-    dst.bytes = src.bytes;
-    src.p = nullptr;
-    src.bytes = 0;
-}
-
 // float64: four RS x RS float64 matrices, or two of them and the Gram staging
 template <class T>
 static size_t recomp_arena_bytes(int RF) {
@@ -426,8 +417,8 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
     cap = std::max(cap, (long long)1 << 16);
     // never ask for more than 85 % of the free device memory: an estimate
     // above it is served by spill rounds instead
-    size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && free_b > 0)
+    size_t free_b = 0;
+    if (dev_mem_free(&free_b) == cudaSuccess && free_b > 0)
         cap = std::min(cap, std::max((long long)1 << 16, (long long)(0.85 * (double)free_b / sizeof(Cx<T>))));
     auto pool = std::make_shared<DevBuf>();
     G3_CUDA(pool->alloc((size_t)cap * sizeof(Cx<T>)));
@@ -629,7 +620,7 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
         add = std::max(add, (long long)(ctr - std::min<unsigned long long>(ctr, (unsigned long long)cap)));
         add = std::max(add, (long long)1 << 16);
         // the enlarged pool and the copy of the old one must fit together
-        if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) {
+        if (dev_mem_free(&free_b) == cudaSuccess) {
             const long long room = (long long)(0.9 * (double)free_b / sizeof(Cx<T>)) - cap;
             if (room < (long long)1 << 16)
                 return fail(G3_ENOMEM, "aca3_compress: the factors need more than the free device memory");
@@ -639,7 +630,7 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
         G3_CUDA(grown.alloc((size_t)(cap + add) * sizeof(Cx<T>)));
         G3_CUDA(cudaMemcpyAsync(grown.p, pool->p, (size_t)cap * sizeof(Cx<T>), cudaMemcpyDeviceToDevice, ctx->stream));
         G3_CUDA(cudaStreamSynchronize(ctx->stream));
-        take(*pool, grown);
+        pool->take(grown);
         base = (unsigned long long)cap;
         cap += add;
         G3_CUDA(cudaMemcpy(d_queue.p, nq.data(), n_spill * sizeof(int), cudaMemcpyHostToDevice));
@@ -663,7 +654,7 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
             G3_CUDA(cudaMemcpyAsync(exact.p, pool->p, (size_t)ctr * sizeof(Cx<T>), cudaMemcpyDeviceToDevice,
                                     ctx->stream));
             G3_CUDA(cudaStreamSynchronize(ctx->stream));
-            take(*pool, exact);
+            pool->take(exact);
             cap = (long long)ctr;
         } else {
             cudaGetLastError();  // keep the large pool
@@ -714,9 +705,9 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
         fa->pool = pool;
         fa->pool_cap = cap;
         if (!batched) {
-            take(fa->d_rec, g_rec);
-            take(fa->d_r3, g_r3);
-            take(fa->d_cycles, g_cyc);
+            fa->d_rec.take(g_rec);
+            fa->d_r3.take(g_r3);
+            fa->d_cycles.take(g_cyc);
         } else {
             G3_CUDA(fa->d_rec.alloc((size_t)std::max(J.n, 1) * Cmax * sizeof(CrossRec)));
             G3_CUDA(fa->d_r3.alloc((size_t)std::max(J.n, 1) * sizeof(int)));
@@ -945,7 +936,7 @@ static g3_status run_aca_whole_t(g3_ctx* ctx, const g3_tree* t, const g3_freqs* 
                 DevBuf grown;
                 G3_CUDA(grown.alloc((size_t)ncap * sizeof(Cx<T>)));
                 G3_CUDA(cudaMemcpy(grown.p, pool->p, (size_t)ctr * sizeof(Cx<T>), cudaMemcpyDeviceToDevice));
-                take(*pool, grown);
+                pool->take(grown);
                 cap = ncap;
             }
             A.pool = pool->as<Cx<T>>();
@@ -1017,8 +1008,8 @@ static g3_status run_aca_whole_t(g3_ctx* ctx, const g3_tree* t, const g3_freqs* 
     G3_CUDA(cudaMemcpy(&ctr, d_ctr.p, sizeof(ctr), cudaMemcpyDeviceToHost));
     fa->pool = pool;
     fa->pool_cap = cap;
-    take(fa->d_rec, d_rec);
-    take(fa->d_r3, d_r3);
+    fa->d_rec.take(d_rec);
+    fa->d_r3.take(d_r3);
     fa->phases.assign((size_t)n_far * NPH, 0);
     fa->cycles.assign(n_far, 0);
     g3_stats& S = fa->stats;

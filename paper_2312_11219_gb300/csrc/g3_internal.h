@@ -35,26 +35,45 @@ enum : unsigned {
     ST_JACOBI_NOCONV = 1u << 4,   // Jacobi SVD hit its sweep limit
 };
 
+// ---- device memory (g3_api.cu) ------------------------------------------------
+// Freed buffers are kept per device and handed out again.
+cudaError_t dev_alloc(size_t n, void** p, size_t* bytes, int* dev);  // on the current device; bytes >= n
+void dev_free(void* p, size_t bytes, int dev);
+cudaError_t dev_mem_free(size_t* bytes);                             // free on the current device, kept buffers included
+void dev_pool_open(int dev, size_t total_bytes);                     // a context came / went
+void dev_pool_close(int dev);
+
 // ---- owned device buffer ----------------------------------------------------
 struct DevBuf {
     void* p = nullptr;
     size_t bytes = 0;
+    int dev = 0;
     DevBuf() = default;
     DevBuf(const DevBuf&) = delete;
     DevBuf& operator=(const DevBuf&) = delete;
     ~DevBuf() { release(); }
     void release() {
-        if (p) cudaFree(p);
+        if (p) dev_free(p, bytes, dev);
         p = nullptr;
         bytes = 0;
     }
     cudaError_t alloc(size_t n) {
         release();
-        if (n == 0) n = 16;
-        cudaError_t e = cudaMalloc(&p, n);
-        if (e == cudaSuccess) bytes = n;
-        else p = nullptr;
+        const cudaError_t e = dev_alloc(n, &p, &bytes, &dev);
+        if (e != cudaSuccess) {
+            p = nullptr;
+            bytes = 0;
+        }
         return e;
+    }
+    // take over another buffer's memory
+    void take(DevBuf& src) {
+        release();
+        p = src.p;
+        bytes = src.bytes;
+        dev = src.dev;
+        src.p = nullptr;
+        src.bytes = 0;
     }
     cudaError_t ensure(size_t n) { return n <= bytes ? cudaSuccess : alloc(n); }
     template <class T> T* as() const { return static_cast<T*>(p); }

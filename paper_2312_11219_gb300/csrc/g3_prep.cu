@@ -872,10 +872,7 @@ static g3_status ss_table(g3_ctx* ctx) {
     DevBuf d;
     G3_CUDA(d.alloc(tab.size() * sizeof(float)));
     G3_CUDA(cudaMemcpy(d.p, tab.data(), tab.size() * sizeof(float), cudaMemcpyHostToDevice));
-    ctx->ss_tab.p = d.p;
-    ctx->ss_tab.bytes = d.bytes;
-    d.p = nullptr;
-    d.bytes = 0;
+    ctx->ss_tab.take(d);
     return G3_OK;
 }
 
