@@ -1,6 +1,7 @@
 // Frequencies, device geometry, diagnostic entries and near-field assembly.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "g3_device.cuh"
@@ -409,17 +410,15 @@ g3_status launch_entries(g3_ctx* ctx, const g3_tree* t, const g3_freqs* f, int k
 // Near-field assembly
 // ============================================================================
 
-// One CTA per (near block, chunk of KCH unique frequencies).  Threads run
-// over the M_b * N_b entries of the block; each thread sets up the pair
-// geometry once and evaluates it at the KCH frequencies.  Layout of a block:
+// One CTA per (near block, chunk of kch unique frequencies).  Threads run
+// over the M_b * N_b entries of the block; each thread sets up an entry's series
+// (below) once and evaluates it at the chunk's frequencies.  Layout of a block:
 // [k][j][i] (frequency-major, column-major per frequency: the apply reads a
 // column of rows with one coalesced load), complex, starting at offs[b].
 //
 // The frequencies come in the working precision (FreqT): a float64 pair per
 // (entry, frequency) costs two float64-to-float32 conversions, which this part
-// issues at its float64 rate.  Entries of the double layer with i == j are 0
-// (x_i lies in the element's plane); those of the single layer are left to
-// k_near_self.
+// issues at its float64 rate.
 template <class T>
 struct FreqOf {
     using type = double2;
@@ -431,46 +430,182 @@ struct FreqOf<float> {
 template <class T>
 using FreqT = typename FreqOf<T>::type;
 
-template <int KER, class T, int KCH>
-__global__ void __launch_bounds__(256) k_near(GeomF gf, GeomD gd, const FreqT<T>* __restrict__ sk,
+// A regular entry at all its frequencies from one power series.  With r_c the middle of
+// the points' distances and R their half range (d_q = (r_q - r_c) / R, |d_q| <= 1),
+//   sum_q a_q exp(-s r_q) = exp(-s r_c) p(-s R),  p(z) = sum_n m_n z^n,  m_n = sum_q a_q d_q^n / n!,
+// and with a_q (1 + s r_q) in place of a_q the coefficients (1 - n) m_n - (r_c / R) m_{n-1}.
+// The coefficients are real and are formed once per entry, so that a frequency takes
+// one exponential, one sine and cosine, and two multiply-adds per term
+// (b_n = c_n + 2 Re z b_{n+1} - |z|^2 b_{n+2}) instead of an exponential, a sine and a
+// cosine per point.  The degree goes by |z| of the warp's entries: 8, 12 or 16 in float32
+// up to |z| = 0.5, 1.25, 2.25 (first term left out below 5e-9 of the largest), 14, 20, 24
+// in float64 up to 0.5, 1.25, 2 (below 3e-17); beyond, point by point.  The terms grow to
+// at most exp(|z|), but the phase s r_c is formed once, with the rounding of its product
+// carried along, where the points' phases were rounded to |s r| 2^-24 each.
+template <class T>
+struct NearSeries;
+template <>
+struct NearSeries<float> {
+    static constexpr int N0 = 8, N1 = 12, N2 = 16;
+    static constexpr float Z0 = 0.5f, Z1 = 1.25f, Z2 = 2.25f;
+};
+template <>
+struct NearSeries<double> {
+    static constexpr int N0 = 14, N1 = 20, N2 = 24;
+    static constexpr double Z0 = 0.5, Z1 = 1.25, Z2 = 2.0;
+};
+
+// coefficients c[0 .. N2] from NP points; returns r_c and R
+template <int KER, class T, int NP>
+__device__ __forceinline__ void series_setup(const T (&r)[NP], const T (&a)[NP], T* c, T& rc, T& R) {
+    constexpr int N = NearSeries<T>::N2;
+    T lo = r[0], hi = r[0];
+#pragma unroll
+    for (int q = 1; q < NP; ++q) {
+        lo = min(lo, r[q]);
+        hi = max(hi, r[q]);
+    }
+    rc = (T)0.5 * (lo + hi);
+    R = max((T)0.5 * (hi - lo), rc * (T)0x1p-10);   // (points at one distance: any unit does)
+    const T iR = (T)1 / R;
+#pragma unroll
+    for (int n = 0; n <= N; ++n) c[n] = 0;
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
+        const T d = (r[q] - rc) * iR;
+        T t = a[q];
+        c[0] += t;
+#pragma unroll
+        for (int n = 1; n <= N; ++n) {
+            t *= d;
+            c[n] += t;
+        }
+    }
+    double f = 1.0;   // 1 / n!, folded at compile time
+#pragma unroll
+    for (int n = 2; n <= N; ++n) {
+        f /= n;
+        c[n] *= (T)f;
+    }
+    if constexpr (KER == G3_DLP) {
+        const T g = rc * iR;
+#pragma unroll
+        for (int n = N; n >= 1; --n) c[n] = (T)(1 - n) * c[n] - g * c[n - 1];
+    }
+}
+template <int N, class T>
+__device__ __forceinline__ Cx<T> series_sum(const T* c, T x, T y, T z2) {
+    const T x2 = x + x;
+    T b1 = c[N], b2 = 0;
+#pragma unroll
+    for (int n = N - 1; n >= 1; --n) {
+        const T b = fma(x2, b1, fma(-z2, b2, c[n]));
+        b2 = b1;
+        b1 = b;
+    }
+    return {fma(x, b1, fma(-z2, b2, c[0])), y * b1};
+}
+// exp(-(sre + i sim) r) with the products' rounding errors carried along.  float32: the
+// exponent split into an integer and at most log(2) / 2, the phase into quarter turns and
+// at most pi / 4 (Taylor polynomials of degree 9 and 10, 2e-9)
+__device__ __forceinline__ Cx<float> cexp_acc(float sre, float sim, float r) {
+    const float u0 = -sre * r, u = fmaxf(u0, -200.0f);
+    const float ul = u0 >= -200.0f ? fmaf(-sre, r, -u0) : 0.0f;
+    const float m = rintf(u * 1.44269504f);
+    float f = fmaf(-m, 0.693145752f, u);      // log 2 = 90852 / 2^17 + 1.42860682e-6
+    f = fmaf(-m, 1.42860682e-6f, f) + ul;
+    const float e = __expf(f) * exp2f(m);
+    const float t = sim * r, tl = fmaf(sim, r, -t);
+    const float n = rintf(t * 0.636619772f);
+    float h = fmaf(-n, 1.5703125f, t);
+    h = fmaf(-n, 4.83826794897e-4f, h) + tl;
+    const float h2 = h * h;
+    float sn = fmaf(h2, 1.0f / 362880.0f, -1.0f / 5040.0f);
+    sn = fmaf(h2, sn, 1.0f / 120.0f);
+    sn = fmaf(h2, sn, -1.0f / 6.0f);
+    sn = fmaf(h * h2, sn, h);
+    float cs = fmaf(h2, -1.0f / 3628800.0f, 1.0f / 40320.0f);
+    cs = fmaf(h2, cs, -1.0f / 720.0f);
+    cs = fmaf(h2, cs, 1.0f / 24.0f);
+    cs = fmaf(h2, cs, -0.5f);
+    cs = fmaf(h2, cs, 1.0f);
+    const int k = (int)n;
+    const float c1 = (k & 1) ? sn : cs, s1 = (k & 1) ? cs : sn;   // cos, sin of n quarter turns + h
+    const float c = ((k + 1) & 2) ? -c1 : c1, s = (k & 2) ? -s1 : s1;
+    return {e * c, -e * s};
+}
+__device__ __forceinline__ Cx<double> cexp_acc(double sre, double sim, double r) {
+    const double u = -sre * r, ul = fma(-sre, r, -u);
+    double e = exp(u);
+    if (e > 0.0 && e < 1e300) e = fma(e, ul, e);
+    const double t = sim * r, tl = fma(sim, r, -t);
+    double sn, cs;
+    sincos(t, &sn, &cs);
+    return {e * fma(-sn, tl, cs), -e * fma(cs, tl, sn)};
+}
+
+// Bound by the special-function unit before (float32: 3 results per point and frequency, 21
+// per entry; now 3) or by float64 arithmetic; now by the float32 instructions of the
+// exponential and the series.  12,288 triangles, 65 frequencies, float32: 2.77 -> 2.17 ms;
+// 768 triangles, 17 frequencies, float64: 5.58 -> 2.19 ms.
+template <int KER, class T>
+__global__ void __launch_bounds__(256) k_near(int E, int kch, GeomF gf, GeomD gd, const FreqT<T>* __restrict__ sk,
                                               const BlockRange* __restrict__ ranges,
                                               const long long* __restrict__ offs, int Ku, Cx<T>* __restrict__ out) {
+    using S = NearSeries<T>;
     const int b = blockIdx.x;
-    const int k0 = blockIdx.y * KCH;
+    const int k0 = blockIdx.y * kch;
     const BlockRange br = ranges[b];
     const int M = br.re - br.rb, N = br.ce - br.cb;
     const int MN = M * N;
-    const long long base = offs[b];
-    const int kn = min(KCH, Ku - k0);
-    for (int e = threadIdx.x; e < MN; e += blockDim.x) {
-        int i = br.rb + e % M, j = br.cb + e / M;
-        if (i == j) {
-            if constexpr (KER == G3_DLP)
-                for (int kk = 0; kk < kn; ++kk) out[base + (long long)(k0 + kk) * MN + e] = Cx<T>{0, 0};
-            continue;
-        }
+    const int kn = min(kch, Ku - k0);
+    // whole warps: lanes past the block's entries repeat its last one without storing
+    for (int e0 = threadIdx.x & ~31; e0 < MN; e0 += blockDim.x) {
+        const int eq = e0 + (threadIdx.x & 31), e = min(eq, MN - 1);
+        const int i = br.rb + e % M, j = br.cb + e / M;
+        Cx<T>* o = out + offs[b] + (long long)k0 * MN + e;
+        const bool self = i == j;   // (DLP: 0; SLP: left to k_near_self, Galerkin: k_near_ss)
+        const bool put = eq < MN && (!self || KER == G3_DLP);
+        using P = std::conditional_t<KER == G3_GAL_SLP, Pair16<T>, Pair7<T>>;
+        P p;
+        // (a self entry's lane takes any other pair's geometry: its own has no distance)
+        const int jj = !self || E == 1 ? j : (j > 0 ? j - 1 : j + 1);
         if constexpr (KER == G3_GAL_SLP) {
             // regular rule for every off-diagonal pair; pairs with a common
             // vertex are overwritten by k_near_ss
-            Pair16<T> p;
             if constexpr (sizeof(T) == 4)
-                gal_setup(gf, i, j, p);
+                gal_setup(gf, i, jj, p);
             else
-                gal_setup(gd, i, j, p);
-            for (int kk = 0; kk < kn; ++kk) {
-                const FreqT<T> s = sk[k0 + kk];
-                out[base + (long long)(k0 + kk) * MN + e] = gal_eval<T>(p, s.x, s.y);
-            }
+                gal_setup(gd, i, jj, p);
         } else {
-            Pair7<T> p;
             if constexpr (sizeof(T) == 4)
-                pair_setup<KER>(gf, i, j, p);
+                pair_setup<KER>(gf, i, jj, p);
             else
-                pair_setup<KER>(gd, i, j, p);
-            for (int kk = 0; kk < kn; ++kk) {
-                const FreqT<T> s = sk[k0 + kk];
-                out[base + (long long)(k0 + kk) * MN + e] = pair_eval<KER, T>(p, s.x, s.y);
+                pair_setup<KER>(gd, i, jj, p);
+        }
+        T c[S::N2 + 1], rc, R;
+        series_setup<KER, T>(p.r, p.a, c, rc, R);
+        for (int kk = 0; kk < kn; ++kk) {
+            const FreqT<T> s = sk[k0 + kk];
+            const T x = -s.x * R, y = -s.y * R, z2 = fma(x, x, y * y);
+            Cx<T> v;
+            // one degree for the warp (a NaN distance goes point by point)
+            if (__all_sync(0xffffffffu, z2 <= S::Z2 * S::Z2)) {
+                Cx<T> w;
+                if (__all_sync(0xffffffffu, z2 <= S::Z0 * S::Z0))
+                    w = series_sum<S::N0>(c, x, y, z2);
+                else if (__all_sync(0xffffffffu, z2 <= S::Z1 * S::Z1))
+                    w = series_sum<S::N1>(c, x, y, z2);
+                else
+                    w = series_sum<S::N2>(c, x, y, z2);
+                v = cmul(cexp_acc(s.x, s.y, rc), w);
+            } else if constexpr (KER == G3_GAL_SLP) {
+                v = gal_eval<T>(p, s.x, s.y);
+            } else {
+                v = pair_eval<KER, T>(p, s.x, s.y);
             }
+            if (self) v = Cx<T>{0, 0};
+            if (put) o[(long long)kk * MN] = v;
         }
     }
 }
@@ -1047,15 +1182,21 @@ __global__ void __launch_bounds__(SELF_NW * 32) k_near_self(GeomD gd, const doub
     }
 }
 
+// frequencies per CTA of k_near: at most 24, in equal chunks
+static int near_chunk(int Ku) {
+    const int n = (Ku + 23) / 24;
+    return (Ku + n - 1) / n;
+}
+
 // Galerkin: near-field pairs with a common vertex (the list of SsPair records
 // built on the host) by k_near_ss, after the regular rule for all pairs
 template <class T>
 static g3_status launch_near_galerkin(g3_ctx* ctx, const g3_tree* t, const g3_freqs* f, g3_near* nf) {
     const int nb = (int)nf->order.size();
-    constexpr int KCH = 16;
-    dim3 grid(nb, (f->Ku + KCH - 1) / KCH);
+    const int kch = near_chunk(f->Ku);
+    dim3 grid(nb, (f->Ku + kch - 1) / kch);
     Cx<T>* o = reinterpret_cast<Cx<T>*>(nf->data.p);
-    k_near<G3_GAL_SLP, T, KCH><<<grid, 256, 0, ctx->stream>>>(t->gf, t->gd, freqs_of<T>(f),
+    k_near<G3_GAL_SLP, T><<<grid, 256, 0, ctx->stream>>>(t->ne, kch, t->gf, t->gd, freqs_of<T>(f),
                                                                nf->d_ranges.as<BlockRange>(),
                                                                nf->d_offs.as<long long>(), f->Ku, o);
     ctx->count("k_near");
@@ -1097,8 +1238,8 @@ g3_status launch_near(g3_ctx* ctx, const g3_tree* t, const g3_freqs* f, g3_near*
         return nf->prec == G3_MIXED ? launch_near_galerkin<float>(ctx, t, f, nf)
                                     : launch_near_galerkin<double>(ctx, t, f, nf);
     }
-    constexpr int KCH = 16;
-    dim3 grid(nb, (f->Ku + KCH - 1) / KCH);
+    const int kch = near_chunk(f->Ku);
+    dim3 grid(nb, (f->Ku + kch - 1) / kch);
     const BlockRange* rg = nf->d_ranges.as<BlockRange>();
     const long long* of = nf->d_offs.as<long long>();
     const long long* db = nf->d_diag_base.as<long long>();
@@ -1107,12 +1248,12 @@ g3_status launch_near(g3_ctx* ctx, const g3_tree* t, const g3_freqs* f, g3_near*
         using T = decltype(zero);
         Cx<T>* o = nf->data.as<Cx<T>>();
         if (kernel == G3_SLP) {
-            k_near<G3_SLP, T, KCH><<<grid, 256, 0, ctx->stream>>>(t->gf, t->gd, freqs_of<T>(f), rg, of, f->Ku, o);
+            k_near<G3_SLP, T><<<grid, 256, 0, ctx->stream>>>(t->ne, kch, t->gf, t->gd, freqs_of<T>(f), rg, of, f->Ku, o);
             k_near_self<T><<<(t->ne + SELF_NW - 1) / SELF_NW, SELF_NW * 32, 0, ctx->stream>>>(
                 t->gd, f->d_sd.as<double2>(), t->ne, f->Ku, db, dm, o);
             ctx->count("k_near_self");
         } else {
-            k_near<G3_DLP, T, KCH><<<grid, 256, 0, ctx->stream>>>(t->gf, t->gd, freqs_of<T>(f), rg, of, f->Ku, o);
+            k_near<G3_DLP, T><<<grid, 256, 0, ctx->stream>>>(t->ne, kch, t->gf, t->gd, freqs_of<T>(f), rg, of, f->Ku, o);
         }
         return G3_OK;
     };
