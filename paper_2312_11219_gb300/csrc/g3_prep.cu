@@ -544,12 +544,16 @@ __device__ __forceinline__ Cx<double> cexp_acc(double sre, double sim, double r)
     return {e * fma(-sn, tl, cs), -e * fma(cs, tl, sn)};
 }
 
+// Four warps per CTA: a 24 x 24 block is 18 warps of entries, 90 % of five rounds (75 %
+// of three rounds of eight; 12,288 triangles 2.18 and 2.17 ms, small meshes fill the chip
+// better).
+constexpr int NEAR_NT = 128;
 // Bound by the special-function unit before (float32: 3 results per point and frequency, 21
-// per entry; now 3) or by float64 arithmetic; now by the float32 instructions of the
-// exponential and the series.  12,288 triangles, 65 frequencies, float32: 2.77 -> 2.17 ms;
+// per entry; now 3) or by float64 arithmetic; now by the instructions of the
+// exponential and the series (140 per entry and frequency, 45 % of them multiply-adds).  12,288 triangles, 65 frequencies, float32: 2.77 -> 2.17 ms;
 // 768 triangles, 17 frequencies, float64: 5.58 -> 2.19 ms.
 template <int KER, class T>
-__global__ void __launch_bounds__(256) k_near(int E, int kch, GeomF gf, GeomD gd, const FreqT<T>* __restrict__ sk,
+__global__ void __launch_bounds__(NEAR_NT) k_near(int E, int kch, GeomF gf, GeomD gd, const FreqT<T>* __restrict__ sk,
                                               const BlockRange* __restrict__ ranges,
                                               const long long* __restrict__ offs, int Ku, Cx<T>* __restrict__ out) {
     using S = NearSeries<T>;
@@ -1070,13 +1074,29 @@ static g3_status launch_near_p1_t(g3_ctx* ctx, const g3_tree* t, const g3_freqs*
 // terms exceed the sum by at most e^4, so both hold ~1e-14 relative; larger
 // |s| rh sums the points directly.
 // Bound by the float64 pipe (the moments and the series).  12,288 elements x 65
-// frequencies on a GB300: 14.0 -> 1.1 ms.
-__constant__ double SELF_INV[34] = {0.0,      1.0,      1.0 / 2,  1.0 / 3,  1.0 / 4,  1.0 / 5,  1.0 / 6,  1.0 / 7,  1.0 / 8,
-                                    1.0 / 9,  1.0 / 10, 1.0 / 11, 1.0 / 12, 1.0 / 13, 1.0 / 14, 1.0 / 15, 1.0 / 16, 1.0 / 17,
-                                    1.0 / 18, 1.0 / 19, 1.0 / 20, 1.0 / 21, 1.0 / 22, 1.0 / 23, 1.0 / 24, 1.0 / 25, 1.0 / 26,
-                                    1.0 / 27, 1.0 / 28, 1.0 / 29, 1.0 / 30, 1.0 / 31, 1.0 / 32, 1.0 / 33};
+// frequencies on a GB300: 14.0 -> 1.4 ms, and 1.1 ms with the series as Horner's rule on
+// coefficients that hold the factorials (4 operations per term for 8); beside k_near it
+// adds 0.9 ms (near field 4.72 -> 4.27 ms).
+struct SelfFact {   // 1 / n!
+    double v[34];
+    constexpr SelfFact() : v{} {
+        v[0] = 1.0;
+        for (int n = 1; n < 34; ++n) v[n] = v[n - 1] / n;
+    }
+};
+__constant__ SelfFact SELF_IFACT;
 constexpr int SELF_NM = 32;   // moments of each kind (one per lane)
 constexpr int SELF_NW = 4;    // elements (warps) per CTA
+__device__ __forceinline__ Cx<double> self_series(const double* c, double x, double y) {   // sum_n c_n (x + i y)^n
+    double ar = c[SELF_NM - 1], ai = 0.0;
+#pragma unroll 4
+    for (int n = SELF_NM - 2; n >= 0; --n) {
+        const double br = fma(x, ar, fma(-y, ai, c[n]));
+        ai = fma(x, ai, y * ar);
+        ar = br;
+    }
+    return {ar, ai};
+}
 template <class T>
 __global__ void __launch_bounds__(SELF_NW * 32) k_near_self(GeomD gd, const double2* __restrict__ sd, int E, int Ku,
                                                             const long long* __restrict__ diag_base,
@@ -1130,7 +1150,7 @@ __global__ void __launch_bounds__(SELF_NW * 32) k_near_self(GeomD gd, const doub
                     v[n] = keep + __shfl_xor_sync(0xffffffffu, send, o);
                 }
             }
-            mom[warp][kind][lane] = v[0];
+            mom[warp][kind][lane] = v[0] * SELF_IFACT.v[lane + (kind == 0 ? 1 : 0)];
         }
     }
     __syncwarp();
@@ -1141,28 +1161,11 @@ __global__ void __launch_bounds__(SELF_NW * 32) k_near_self(GeomD gd, const doub
         const double as = sqrt(s.x * s.x + s.y * s.y);
         Cx<double> v;
         if (as * rmax <= 4.0) {
-            const Cx<double> mz{-s.x * rmax, -s.y * rmax};
-            Cx<double> term{1.0, 0.0};
-            v = Cx<double>{m0[0], 0.0};
-#pragma unroll 4
-            for (int n = 1; n < SELF_NM; ++n) {
-                const double inv = SELF_INV[n + 1];
-                term = cmul(term, Cx<double>{mz.x * inv, mz.y * inv});
-                v.x = fma(term.x, m0[n], v.x);
-                v.y = fma(term.y, m0[n], v.y);
-            }
+            v = self_series(m0, -s.x * rmax, -s.y * rmax);
         } else {
             Cx<double> sum{0.0, 0.0};  // sum_q w_q exp(-s rho_q)
             if (as * rh <= 4.0) {
-                const Cx<double> mx{-s.x * rh, -s.y * rh};
-                Cx<double> term{1.0, 0.0}, acc{m1[0], 0.0};
-#pragma unroll 4
-                for (int n = 1; n < SELF_NM; ++n) {
-                    const double inv = SELF_INV[n];
-                    term = cmul(term, Cx<double>{mx.x * inv, mx.y * inv});
-                    acc.x = fma(term.x, m1[n], acc.x);
-                    acc.y = fma(term.y, m1[n], acc.y);
-                }
+                const Cx<double> acc = self_series(m1, -s.x * rh, -s.y * rh);
                 double sn, cs;
                 sincos(s.y * rc, &sn, &cs);
                 const double e = exp(-s.x * rc);
@@ -1182,9 +1185,15 @@ __global__ void __launch_bounds__(SELF_NW * 32) k_near_self(GeomD gd, const doub
     }
 }
 
-// frequencies per CTA of k_near: at most 24, in equal chunks
-static int near_chunk(int Ku) {
-    const int n = (Ku + 23) / 24;
+// frequencies per CTA of k_near, in equal chunks: at most 24, and in float32 down to 8
+// where the blocks alone leave resident CTAs (eight per SM) free.  Forming an entry's
+// series costs about as much as four of its frequencies; in float64, where the pipe is
+// full with few warps, splitting only adds to it (768 triangles, 17 frequencies: one
+// chunk 2.19 ms, two 2.50 ms; float32 on 768 triangles, two of 9: 44 us).
+template <class T>
+static int near_chunk(const g3_ctx* ctx, int nb, int Ku) {
+    int n = (Ku + 23) / 24;
+    if (sizeof(T) == 4) n = std::max(n, std::min((Ku + 7) / 8, (8 * ctx->n_sm + nb - 1) / nb));
     return (Ku + n - 1) / n;
 }
 
@@ -1193,10 +1202,10 @@ static int near_chunk(int Ku) {
 template <class T>
 static g3_status launch_near_galerkin(g3_ctx* ctx, const g3_tree* t, const g3_freqs* f, g3_near* nf) {
     const int nb = (int)nf->order.size();
-    const int kch = near_chunk(f->Ku);
+    const int kch = near_chunk<T>(ctx, nb, f->Ku);
     dim3 grid(nb, (f->Ku + kch - 1) / kch);
     Cx<T>* o = reinterpret_cast<Cx<T>*>(nf->data.p);
-    k_near<G3_GAL_SLP, T><<<grid, 256, 0, ctx->stream>>>(t->ne, kch, t->gf, t->gd, freqs_of<T>(f),
+    k_near<G3_GAL_SLP, T><<<grid, NEAR_NT, 0, ctx->stream>>>(t->ne, kch, t->gf, t->gd, freqs_of<T>(f),
                                                                nf->d_ranges.as<BlockRange>(),
                                                                nf->d_offs.as<long long>(), f->Ku, o);
     ctx->count("k_near");
@@ -1238,8 +1247,6 @@ g3_status launch_near(g3_ctx* ctx, const g3_tree* t, const g3_freqs* f, g3_near*
         return nf->prec == G3_MIXED ? launch_near_galerkin<float>(ctx, t, f, nf)
                                     : launch_near_galerkin<double>(ctx, t, f, nf);
     }
-    const int kch = near_chunk(f->Ku);
-    dim3 grid(nb, (f->Ku + kch - 1) / kch);
     const BlockRange* rg = nf->d_ranges.as<BlockRange>();
     const long long* of = nf->d_offs.as<long long>();
     const long long* db = nf->d_diag_base.as<long long>();
@@ -1247,13 +1254,21 @@ g3_status launch_near(g3_ctx* ctx, const g3_tree* t, const g3_freqs* f, g3_near*
     auto go = [&](auto zero) -> g3_status {
         using T = decltype(zero);
         Cx<T>* o = nf->data.as<Cx<T>>();
+        const int kch = near_chunk<T>(ctx, nb, f->Ku);
+        const dim3 grid(nb, (f->Ku + kch - 1) / kch);
         if (kernel == G3_SLP) {
-            k_near<G3_SLP, T><<<grid, 256, 0, ctx->stream>>>(t->ne, kch, t->gf, t->gd, freqs_of<T>(f), rg, of, f->Ku, o);
-            k_near_self<T><<<(t->ne + SELF_NW - 1) / SELF_NW, SELF_NW * 32, 0, ctx->stream>>>(
+            // the self entries (float64 pipe) run beside the regular ones (float32
+            // arithmetic, stores) on the side stream; they write other entries
+            G3_CUDA(cudaEventRecord(ctx->fork, ctx->stream));
+            G3_CUDA(cudaStreamWaitEvent(ctx->side, ctx->fork, 0));
+            k_near_self<T><<<(t->ne + SELF_NW - 1) / SELF_NW, SELF_NW * 32, 0, ctx->side>>>(
                 t->gd, f->d_sd.as<double2>(), t->ne, f->Ku, db, dm, o);
+            G3_CUDA(cudaEventRecord(ctx->join, ctx->side));
+            k_near<G3_SLP, T><<<grid, NEAR_NT, 0, ctx->stream>>>(t->ne, kch, t->gf, t->gd, freqs_of<T>(f), rg, of, f->Ku, o);
+            G3_CUDA(cudaStreamWaitEvent(ctx->stream, ctx->join, 0));
             ctx->count("k_near_self");
         } else {
-            k_near<G3_DLP, T><<<grid, 256, 0, ctx->stream>>>(t->ne, kch, t->gf, t->gd, freqs_of<T>(f), rg, of, f->Ku, o);
+            k_near<G3_DLP, T><<<grid, NEAR_NT, 0, ctx->stream>>>(t->ne, kch, t->gf, t->gd, freqs_of<T>(f), rg, of, f->Ku, o);
         }
         return G3_OK;
     };
