@@ -1075,8 +1075,8 @@ static g3_status launch_near_p1_t(g3_ctx* ctx, const g3_tree* t, const g3_freqs*
 // |s| rh sums the points directly.
 // Bound by the float64 pipe (the moments and the series).  12,288 elements x 65
 // frequencies on a GB300: 14.0 -> 1.4 ms, and 1.1 ms with the series as Horner's rule on
-// coefficients that hold the factorials (4 operations per term for 8); beside k_near it
-// adds 0.9 ms (near field 4.72 -> 4.27 ms).
+// coefficients that hold the factorials (4 operations per term for 8); both that and
+// running beside k_near: near field and its product 4.72 -> 4.27 ms.
 struct SelfFact {   // 1 / n!
     double v[34];
     constexpr SelfFact() : v{} {
