@@ -691,15 +691,20 @@ __device__ __forceinline__ void ss_point32(const SsEdges& S, const float4* __res
 // accumulation, in the three-term split a b ~ a_hi b_hi + a_hi b_lo + a_lo b_hi (a_hi =
 // a rounded to TF32, a_lo = the rounded remainder), which keeps float32 accuracy (about
 // 2^-21 relative per product instead of TF32's 2^-11).
-// (rounding to TF32, nearest with ties away from zero, in two integer operations:
-// the conversion instruction issues at the special-function rate)
+// (rounding to TF32, nearest with ties away from zero, in integer operations: the
+// conversion instruction issues at the special-function rate.  The carry wraps a NaN
+// whose fraction is all ones, the one that arithmetic produces: 0x7fffffff would
+// become -0.  So lo, the result of a subtraction, is held below that wrap and stays
+// a NaN whatever hi has become: a NaN operand gives NaN products, an infinite one
+// too (lo = inf - inf).)
 __device__ __forceinline__ unsigned tf32_rna(float x) { return (__float_as_uint(x) + 0x1000u) & 0xffffe000u; }
 struct Tf32Pair {
     unsigned hi, lo;
 };
 __device__ __forceinline__ Tf32Pair tf32_split(float x) {
     const unsigned h = tf32_rna(x);
-    return Tf32Pair{h, tf32_rna(x - __uint_as_float(h))};
+    const int l = min(__float_as_int(x - __uint_as_float(h)), 0x7fffefff);
+    return Tf32Pair{h, tf32_rna(__int_as_float(l))};
 }
 // d += a b for one 16 x 8 x 8 tile (fragment layouts of the PTX m16n8k8 .tf32 shape)
 __device__ __forceinline__ void mma_tf32(float* d, const unsigned* a, const unsigned* b) {
