@@ -288,7 +288,7 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
             if (k1_host[i] < 0 || k1_host[i] >= ku_of(i))
                 return fail(G3_EINVAL, "opts->k1[%d] = %d outside [0, %d)", i, k1_host[i], ku_of(i));
         G3_CUDA(d_k1.alloc(n_far * sizeof(int)));
-        G3_CUDA(cudaMemcpy(d_k1.p, k1_host, n_far * sizeof(int), cudaMemcpyHostToDevice));
+        G3_CUDA(upload(ctx->stream, d_k1.p, k1_host, n_far * sizeof(int)));
     }
     if (batched) {
         std::vector<GeoDesc> geos(n_jobs);
@@ -297,8 +297,8 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
                               jobs[j].f->d_sf.as<float2>(), jobs[j].Ku, jobs[j].f->k_maxabs};
         G3_CUDA(d_geos.alloc(n_jobs * sizeof(GeoDesc)));
         G3_CUDA(d_bgeo.alloc(n_far * sizeof(int)));
-        G3_CUDA(cudaMemcpy(d_geos.p, geos.data(), n_jobs * sizeof(GeoDesc), cudaMemcpyHostToDevice));
-        G3_CUDA(cudaMemcpy(d_bgeo.p, bgeo.data(), n_far * sizeof(int), cudaMemcpyHostToDevice));
+        G3_CUDA(upload(ctx->stream, d_geos.p, geos.data(), n_jobs * sizeof(GeoDesc)));
+        G3_CUDA(upload(ctx->stream, d_bgeo.p, bgeo.data(), n_far * sizeof(int)));
     }
     // separable inputs (converted to T)
     DevBuf d_sa, d_sb, d_sc;
@@ -310,7 +310,7 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
             const double* s = (const double*)src;
             for (size_t i = 0; i < 2 * n; ++i) tmp[i] = (T)s[i];
             G3_CUDA(d.alloc(tmp.size() * sizeof(T)));
-            G3_CUDA(cudaMemcpy(d.p, tmp.data(), tmp.size() * sizeof(T), cudaMemcpyHostToDevice));
+            G3_CUDA(upload(ctx->stream, d.p, tmp.data(), tmp.size() * sizeof(T)));
             return G3_OK;
         };
         g3_status st;
@@ -633,7 +633,7 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
         pool->take(grown);
         base = (unsigned long long)cap;
         cap += add;
-        G3_CUDA(cudaMemcpy(d_queue.p, nq.data(), n_spill * sizeof(int), cudaMemcpyHostToDevice));
+        G3_CUDA(upload(ctx->stream, d_queue.p, nq.data(), n_spill * sizeof(int)));
     }
     const double ms_rounds = ms_since(th1);
     const auto th2 = std::chrono::steady_clock::now();
@@ -713,12 +713,12 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
             G3_CUDA(fa->d_r3.alloc((size_t)std::max(J.n, 1) * sizeof(int)));
             G3_CUDA(fa->d_cycles.alloc((size_t)std::max(J.n, 1) * NPH * sizeof(long long)));
             if (J.n > 0) {
-                G3_CUDA(cudaMemcpy(fa->d_rec.p, g_rec.as<CrossRec>() + (size_t)J.first * Cmax,
-                                   (size_t)J.n * Cmax * sizeof(CrossRec), cudaMemcpyDeviceToDevice));
-                G3_CUDA(cudaMemcpy(fa->d_r3.p, g_r3.as<int>() + J.first, (size_t)J.n * sizeof(int),
-                                   cudaMemcpyDeviceToDevice));
-                G3_CUDA(cudaMemcpy(fa->d_cycles.p, g_cyc.as<long long>() + (size_t)J.first * NPH,
-                                   (size_t)J.n * NPH * sizeof(long long), cudaMemcpyDeviceToDevice));
+                G3_CUDA(cudaMemcpyAsync(fa->d_rec.p, g_rec.as<CrossRec>() + (size_t)J.first * Cmax,
+                                        (size_t)J.n * Cmax * sizeof(CrossRec), cudaMemcpyDeviceToDevice, ctx->stream));
+                G3_CUDA(cudaMemcpyAsync(fa->d_r3.p, g_r3.as<int>() + J.first, (size_t)J.n * sizeof(int),
+                                        cudaMemcpyDeviceToDevice, ctx->stream));
+                G3_CUDA(cudaMemcpyAsync(fa->d_cycles.p, g_cyc.as<long long>() + (size_t)J.first * NPH,
+                                        (size_t)J.n * NPH * sizeof(long long), cudaMemcpyDeviceToDevice, ctx->stream));
             }
         }
         fa->r3.assign(r3.begin() + J.first, r3.begin() + J.first + J.n);
@@ -847,12 +847,12 @@ static g3_status run_aca_whole_t(g3_ctx* ctx, const g3_tree* t, const g3_freqs* 
     G3_CUDA(d_ff.alloc((size_t)(Cmax + 1) * sizeof(Cx<double>)));
     G3_CUDA(d_scal.alloc(2 * sizeof(double)));
     G3_CUDA(d_tot.alloc(2 * sizeof(double)));
-    G3_CUDA(cudaMemcpy(d_ranges.p, ranges.data(), n_far * sizeof(BlockRange), cudaMemcpyHostToDevice));
-    G3_CUDA(cudaMemcpy(d_queue.p, queue.data(), n_far * sizeof(int), cudaMemcpyHostToDevice));
-    G3_CUDA(cudaMemset(d_counters.p, 0, 32 * sizeof(unsigned long long)));
-    G3_CUDA(cudaMemset(d_ctr.p, 0, sizeof(unsigned long long)));
-    G3_CUDA(cudaMemset(d_normb.p, 0, n_far * sizeof(double)));
-    G3_CUDA(cudaMemset(d_r3.p, 0, n_far * sizeof(int)));
+    G3_CUDA(upload(ctx->stream, d_ranges.p, ranges.data(), n_far * sizeof(BlockRange)));
+    G3_CUDA(upload(ctx->stream, d_queue.p, queue.data(), n_far * sizeof(int)));
+    G3_CUDA(cudaMemsetAsync(d_counters.p, 0, 32 * sizeof(unsigned long long), ctx->stream));
+    G3_CUDA(cudaMemsetAsync(d_ctr.p, 0, sizeof(unsigned long long), ctx->stream));
+    G3_CUDA(cudaMemsetAsync(d_normb.p, 0, n_far * sizeof(double), ctx->stream));
+    G3_CUDA(cudaMemsetAsync(d_r3.p, 0, n_far * sizeof(int), ctx->stream));
     auto pool = std::make_shared<DevBuf>();
     long long cap = 4 * worst;
     G3_CUDA(pool->alloc((size_t)cap * sizeof(Cx<T>)));
@@ -930,12 +930,13 @@ static g3_status run_aca_whole_t(g3_ctx* ctx, const g3_tree* t, const g3_freqs* 
             if (dup) continue;
             // pool room for one more cross of every block
             unsigned long long ctr = 0;
-            G3_CUDA(cudaMemcpy(&ctr, d_ctr.p, sizeof(ctr), cudaMemcpyDeviceToHost));
+            G3_CUDA(cudaMemcpyAsync(&ctr, d_ctr.p, sizeof(ctr), cudaMemcpyDeviceToHost, ctx->stream));
+            G3_CUDA(cudaStreamSynchronize(ctx->stream));
             if ((long long)ctr + worst > cap) {
                 const long long ncap = std::max((long long)ctr + 4 * worst, cap + cap / 2);
                 DevBuf grown;
                 G3_CUDA(grown.alloc((size_t)ncap * sizeof(Cx<T>)));
-                G3_CUDA(cudaMemcpy(grown.p, pool->p, (size_t)ctr * sizeof(Cx<T>), cudaMemcpyDeviceToDevice));
+                G3_CUDA(cudaMemcpyAsync(grown.p, pool->p, (size_t)ctr * sizeof(Cx<T>), cudaMemcpyDeviceToDevice, ctx->stream));
                 pool->take(grown);
                 cap = ncap;
             }
@@ -996,7 +997,7 @@ static g3_status run_aca_whole_t(g3_ctx* ctx, const g3_tree* t, const g3_freqs* 
     G3_CUDA(cudaEventElapsedTime(&ms, e0, e1));
     // every block keeps the R crosses before the dropped one
     fa->r3.assign(n_far, R);
-    G3_CUDA(cudaMemcpy(d_r3.p, fa->r3.data(), n_far * sizeof(int), cudaMemcpyHostToDevice));
+    G3_CUDA(upload(ctx->stream, d_r3.p, fa->r3.data(), n_far * sizeof(int)));
     {
         std::vector<CrossRec> full((size_t)n_far * Cmax);
         G3_CUDA(cudaMemcpy(full.data(), d_rec.p, full.size() * sizeof(CrossRec), cudaMemcpyDeviceToHost));

@@ -307,18 +307,18 @@ static g3_status finish_freqs(g3_ctx* ctx, g3_freqs* f, const std::vector<double
     // su_host: unique set as interleaved pairs [2 Ku]; f->s, f->omega: the full set
     G3_CUDA(f->d_s_all.alloc((size_t)f->K * 2 * sizeof(double)));
     G3_CUDA(f->d_w_all.alloc((size_t)f->K * 2 * sizeof(double)));
-    G3_CUDA(cudaMemcpy(f->d_s_all.p, f->s.data(), (size_t)f->K * 2 * sizeof(double), cudaMemcpyHostToDevice));
-    G3_CUDA(cudaMemcpy(f->d_w_all.p, f->omega.data(), (size_t)f->K * 2 * sizeof(double), cudaMemcpyHostToDevice));
+    G3_CUDA(upload(ctx->stream, f->d_s_all.p, f->s.data(), (size_t)f->K * 2 * sizeof(double)));
+    G3_CUDA(upload(ctx->stream, f->d_w_all.p, f->omega.data(), (size_t)f->K * 2 * sizeof(double)));
     G3_CUDA(f->d_sd.alloc((size_t)f->Ku * 2 * sizeof(double)));
     G3_CUDA(f->d_sf.alloc((size_t)f->Ku * 2 * sizeof(float)));
     std::vector<float> sf(2 * (size_t)f->Ku);
     for (size_t i = 0; i < sf.size(); ++i) sf[i] = (float)su_host[i];
-    G3_CUDA(cudaMemcpy(f->d_sd.p, su_host.data(), su_host.size() * sizeof(double), cudaMemcpyHostToDevice));
-    G3_CUDA(cudaMemcpy(f->d_sf.p, sf.data(), sf.size() * sizeof(float), cudaMemcpyHostToDevice));
+    G3_CUDA(upload(ctx->stream, f->d_sd.p, su_host.data(), su_host.size() * sizeof(double)));
+    G3_CUDA(upload(ctx->stream, f->d_sf.p, sf.data(), sf.size() * sizeof(float)));
     G3_CUDA(f->d_uniq.alloc(f->uniq.size() * sizeof(int)));
     G3_CUDA(f->d_partner.alloc(f->partner.size() * sizeof(int)));
-    G3_CUDA(cudaMemcpy(f->d_uniq.p, f->uniq.data(), f->uniq.size() * sizeof(int), cudaMemcpyHostToDevice));
-    G3_CUDA(cudaMemcpy(f->d_partner.p, f->partner.data(), f->partner.size() * sizeof(int), cudaMemcpyHostToDevice));
+    G3_CUDA(upload(ctx->stream, f->d_uniq.p, f->uniq.data(), f->uniq.size() * sizeof(int)));
+    G3_CUDA(upload(ctx->stream, f->d_partner.p, f->partner.data(), f->partner.size() * sizeof(int)));
     double best = -1;
     for (int u = 0; u < f->Ku; ++u) {
         double a = std::hypot(su_host[2 * u], su_host[2 * u + 1]);
@@ -327,7 +327,7 @@ static g3_status finish_freqs(g3_ctx* ctx, g3_freqs* f, const std::vector<double
             f->k_maxabs = u;
         }
     }
-    (void)ctx;
+    G3_CUDA(cudaStreamSynchronize(ctx->stream));  // the set may be used from another context
     return G3_OK;
 }
 
@@ -563,7 +563,7 @@ g3_status build_cluster_tree_capped(g3_ctx* ctx, const double* verts, int nv, co
         for (int p = 0; p < ne; ++p)
             for (int k = 0; k < 3; ++k) tv[3 * (size_t)p + k] = t->tris[3 * (size_t)t->perm[p] + k];
         cudaError_t e = t->d_tv.alloc(tv.size() * sizeof(int));
-        if (e == cudaSuccess) e = cudaMemcpy(t->d_tv.p, tv.data(), tv.size() * sizeof(int), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = upload(ctx->stream, t->d_tv.p, tv.data(), tv.size() * sizeof(int));
         if (e != cudaSuccess) st = cuda_fail(e, "build_cluster_tree: vertex ids");
     }
     if (st == G3_OK) st = launch_geometry(ctx, t);
@@ -603,13 +603,13 @@ g3_status g3_tree_subset(g3_ctx* ctx, const g3_tree* t, const int32_t* owner, in
     g3_status st = G3_OK;
     cudaError_t e = s->d_perm.alloc(s->ne * sizeof(int));
     if (e == cudaSuccess)
-        e = cudaMemcpy(s->d_perm.p, s->perm.data(), s->ne * sizeof(int), cudaMemcpyHostToDevice);
+        e = upload(ctx->stream, s->d_perm.p, s->perm.data(), s->ne * sizeof(int));
     if (e == cudaSuccess) {
         std::vector<int> tv(3 * (size_t)s->ne);
         for (int p = 0; p < s->ne; ++p)
             for (int k = 0; k < 3; ++k) tv[3 * (size_t)p + k] = s->tris[3 * (size_t)s->perm[p] + k];
         e = s->d_tv.alloc(tv.size() * sizeof(int));
-        if (e == cudaSuccess) e = cudaMemcpy(s->d_tv.p, tv.data(), tv.size() * sizeof(int), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = upload(ctx->stream, s->d_tv.p, tv.data(), tv.size() * sizeof(int));
     }
     if (e != cudaSuccess) st = cuda_fail(e, "g3_tree_subset: device copies");
     if (st == G3_OK) st = launch_geometry(ctx, s);
@@ -661,12 +661,12 @@ g3_status build_p1_tree(g3_ctx* ctx, const g3_tree* t, g3_tree** out) {
     };
     // element geometry (cluster order of the elements)
     chk(s->d_perm.alloc(E * sizeof(int)), "build_p1_tree: perm");
-    if (st == G3_OK) chk(cudaMemcpy(s->d_perm.p, t->perm.data(), E * sizeof(int), cudaMemcpyHostToDevice), "copy");
+    if (st == G3_OK) chk(upload(ctx->stream, s->d_perm.p, t->perm.data(), E * sizeof(int)), "copy");
     std::vector<int> tv(3 * (size_t)E);
     for (int p = 0; p < E; ++p)
         for (int k = 0; k < 3; ++k) tv[3 * (size_t)p + k] = t->tris[3 * (size_t)t->perm[p] + k];
     chk(s->d_tv.alloc(tv.size() * sizeof(int)), "build_p1_tree: vertex ids");
-    if (st == G3_OK) chk(cudaMemcpy(s->d_tv.p, tv.data(), tv.size() * sizeof(int), cudaMemcpyHostToDevice), "copy");
+    if (st == G3_OK) chk(upload(ctx->stream, s->d_tv.p, tv.data(), tv.size() * sizeof(int)), "copy");
     if (st == G3_OK) st = launch_geometry(ctx, s);
     // surface curls of the barycentric coordinates, float64 on the host:
     // curl lambda_a = n x grad lambda_a, grad lambda_a = n x (v_{a+2} - v_{a+1}) / (2 area)
@@ -699,8 +699,8 @@ g3_status build_p1_tree(g3_ctx* ctx, const g3_tree* t, g3_tree** out) {
     }
     chk(s->d_curl_d.alloc(cd.size() * sizeof(double)), "build_p1_tree: curls");
     chk(s->d_curl_f.alloc(cf.size() * sizeof(float)), "build_p1_tree: curls");
-    if (st == G3_OK) chk(cudaMemcpy(s->d_curl_d.p, cd.data(), cd.size() * sizeof(double), cudaMemcpyHostToDevice), "copy");
-    if (st == G3_OK) chk(cudaMemcpy(s->d_curl_f.p, cf.data(), cf.size() * sizeof(float), cudaMemcpyHostToDevice), "copy");
+    if (st == G3_OK) chk(upload(ctx->stream, s->d_curl_d.p, cd.data(), cd.size() * sizeof(double)), "copy");
+    if (st == G3_OK) chk(upload(ctx->stream, s->d_curl_f.p, cf.data(), cf.size() * sizeof(float)), "copy");
     // positions of the degrees of freedom: original index 3 e + a and vertex
     std::vector<int32_t> perm3(3 * (size_t)E), src(3 * (size_t)E);
     for (int p = 0; p < E; ++p)
@@ -715,9 +715,10 @@ g3_status build_p1_tree(g3_ctx* ctx, const g3_tree* t, g3_tree** out) {
         s->ne = 3 * E;
         chk(s->d_perm.alloc(perm3.size() * sizeof(int)), "build_p1_tree: perm");
         if (st == G3_OK)
-            chk(cudaMemcpy(s->d_perm.p, perm3.data(), perm3.size() * sizeof(int), cudaMemcpyHostToDevice), "copy");
+            chk(upload(ctx->stream, s->d_perm.p, perm3.data(), perm3.size() * sizeof(int)), "copy");
         chk(s->d_src.alloc(src.size() * sizeof(int)), "build_p1_tree: vertices");
-        if (st == G3_OK) chk(cudaMemcpy(s->d_src.p, src.data(), src.size() * sizeof(int), cudaMemcpyHostToDevice), "copy");
+        if (st == G3_OK) chk(upload(ctx->stream, s->d_src.p, src.data(), src.size() * sizeof(int)), "copy");
+        if (st == G3_OK) chk(cudaStreamSynchronize(ctx->stream), "build_p1_tree: copies");
     }
     if (st != G3_OK) {
         delete s;
@@ -1328,7 +1329,7 @@ static g3_status mlp_alloc(g3_ctx* ctx, const float* params, const float* mean, 
     auto up = [&](g3::DevBuf& d, const void* src, size_t bytes) -> cudaError_t {
         cudaError_t e = d.alloc(bytes);
         if (e != cudaSuccess) return e;
-        return cudaMemcpy(d.p, src, bytes, cudaMemcpyHostToDevice);
+        return g3::upload(ctx->stream, d.p, src, bytes);
     };
     const long long t0 = 0;
     cudaError_t e;
@@ -1338,6 +1339,11 @@ static g3_status mlp_alloc(g3_ctx* ctx, const float* params, const float* mean, 
         (e = up(m->d_t, &t0, sizeof(t0))) != cudaSuccess ||
         (e = up(m->d_mean, m->mean, sizeof(float) * G3_MLP_NF)) != cudaSuccess ||
         (e = up(m->d_inv_std, m->inv_std, sizeof(float) * G3_MLP_NF)) != cudaSuccess) {
+        delete m;
+        return cuda_fail(e, "g3_mlp_create: upload");
+    }
+    e = cudaStreamSynchronize(ctx->stream);  // the predictor may be used from another context
+    if (e != cudaSuccess) {
         delete m;
         return cuda_fail(e, "g3_mlp_create: upload");
     }
@@ -1375,12 +1381,12 @@ static g3_status train_cfg(const g3_train_opts* o, TrainCfg& c) {
     return G3_OK;
 }
 
-static g3_status upload_samples(const float* feats, const float* labels, int n, g3::DevBuf& dx, g3::DevBuf& dy) {
+static g3_status upload_samples(g3_ctx* ctx, const float* feats, const float* labels, int n, g3::DevBuf& dx, g3::DevBuf& dy) {
     G3_CUDA(dx.alloc((size_t)n * G3_MLP_NF * sizeof(float)));
-    G3_CUDA(cudaMemcpy(dx.p, feats, (size_t)n * G3_MLP_NF * sizeof(float), cudaMemcpyHostToDevice));
+    G3_CUDA(g3::upload(ctx->stream, dx.p, feats, (size_t)n * G3_MLP_NF * sizeof(float)));
     if (labels) {
         G3_CUDA(dy.alloc((size_t)n * 2 * sizeof(float)));
-        G3_CUDA(cudaMemcpy(dy.p, labels, (size_t)n * 2 * sizeof(float), cudaMemcpyHostToDevice));
+        G3_CUDA(g3::upload(ctx->stream, dy.p, labels, (size_t)n * 2 * sizeof(float)));
     }
     return G3_OK;
 }
@@ -1388,7 +1394,7 @@ static g3_status upload_samples(const float* feats, const float* labels, int n, 
 static g3_status fit(g3_ctx* ctx, g3_mlp* m, const float* feats, const float* labels, int n, const TrainCfg& c,
                      float* losses) {
     g3::DevBuf dx, dy, dl;
-    G3_TRY(upload_samples(feats, labels, n, dx, dy));
+    G3_TRY(upload_samples(ctx, feats, labels, n, dx, dy));
     const long long nb = ((long long)n + c.batch - 1) / c.batch;
     G3_CUDA(dl.alloc((size_t)c.epochs * nb * sizeof(float)));
     G3_TRY(mlp_fit_dev(ctx, m, dx.as<float>(), dy.as<float>(), n, c.epochs, c.batch, c.lr, c.b1, c.b2, c.eps, c.graph,
@@ -1447,7 +1453,7 @@ g3_status g3_mlp_grad(g3_ctx* ctx, const g3_mlp* m, const float* feats, const fl
     G3_CHECK(n >= 1, "g3_mlp_grad: n = %d", n);
     G3_TRY(use_device(ctx));
     g3::DevBuf dx, dy, dg, dl;
-    G3_TRY(upload_samples(feats, labels, n, dx, dy));
+    G3_TRY(upload_samples(ctx, feats, labels, n, dx, dy));
     G3_CUDA(dg.alloc(G3_MLP_NP * sizeof(float)));
     G3_CUDA(dl.alloc(sizeof(float)));
     G3_TRY(mlp_grad_dev(ctx, m, dx.as<float>(), dy.as<float>(), n, dg.as<float>(), dl.as<float>()));
@@ -1462,7 +1468,7 @@ g3_status g3_mlp_predict(g3_ctx* ctx, const g3_mlp* m, const float* feats, int n
     if (n == 0) return G3_OK;
     G3_TRY(use_device(ctx));
     g3::DevBuf dx, dy, dout;
-    G3_TRY(upload_samples(feats, nullptr, n, dx, dy));
+    G3_TRY(upload_samples(ctx, feats, nullptr, n, dx, dy));
     G3_CUDA(dout.alloc((size_t)n * 2 * sizeof(float)));
     G3_TRY(mlp_forward_dev(ctx, m, dx.as<float>(), n, dout.as<float>()));
     G3_CUDA(cudaMemcpyAsync(out, dout.p, (size_t)n * 2 * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1514,7 +1520,7 @@ g3_status g3_factors_labels(g3_ctx* ctx, const g3_factors* fa, float* out) {
     G3_TRY(use_device(ctx));
     g3::DevBuf dr, d;
     G3_CUDA(dr.alloc(fa->ranges.size() * sizeof(BlockRange)));
-    G3_CUDA(cudaMemcpy(dr.p, fa->ranges.data(), fa->ranges.size() * sizeof(BlockRange), cudaMemcpyHostToDevice));
+    G3_CUDA(upload(ctx->stream, dr.p, fa->ranges.data(), fa->ranges.size() * sizeof(BlockRange)));
     G3_CUDA(d.alloc((size_t)fa->n_far * 2 * sizeof(float)));
     G3_TRY(mlp_labels_dev(ctx, fa, dr.as<BlockRange>(), d.as<float>()));
     G3_CUDA(cudaMemcpyAsync(out, d.p, (size_t)fa->n_far * 2 * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));

@@ -856,11 +856,11 @@ g3_status far_plan_build(g3_factors* fa) {
     for (const Item& it : wide) L.insert(L.end(), {it.b, it.g, 0, 0});
     L.insert(L.end(), slots.begin(), slots.end());
     G3_CUDA(fa->d_plan.alloc(std::max<size_t>(1, L.size()) * sizeof(int)));
-    if (!L.empty()) G3_CUDA(cudaMemcpy(fa->d_plan.p, L.data(), L.size() * sizeof(int), cudaMemcpyHostToDevice));
+    const cudaStream_t stream = fa->ctx->stream;
+    G3_CUDA(upload(stream, fa->d_plan.p, L.data(), L.size() * sizeof(int)));
     G3_CUDA(fa->d_franges.alloc(std::max<size_t>(1, fa->ranges.size()) * sizeof(BlockRange)));
-    if (!fa->ranges.empty())
-        G3_CUDA(cudaMemcpy(fa->d_franges.p, fa->ranges.data(), fa->ranges.size() * sizeof(BlockRange),
-                           cudaMemcpyHostToDevice));
+    G3_CUDA(upload(stream, fa->d_franges.p, fa->ranges.data(), fa->ranges.size() * sizeof(BlockRange)));
+    G3_CUDA(cudaStreamSynchronize(stream));  // the factors may be applied from another context
     fa->plan_ready = true;
     return G3_OK;
 }

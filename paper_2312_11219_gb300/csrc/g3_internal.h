@@ -43,6 +43,16 @@ cudaError_t dev_mem_free(size_t* bytes);                             // free on 
 void dev_pool_open(int dev, size_t total_bytes);                     // a context came / went
 void dev_pool_close(int dev);
 
+// Copies to device memory go through the context's stream, never through the legacy
+// stream: a context on a non-blocking stream has no ordering with that one, and
+// freeing a buffer orders nothing (the pool keeps it).  bytes of pageable host memory
+// at src may be reused on return (they are staged by then); the device sees the copy in
+// stream order, and a call that hands out a handle waits for the stream, since the
+// handle may be used from another context's.
+inline cudaError_t upload(cudaStream_t stream, void* dst, const void* src, size_t bytes) {
+    return bytes ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, stream) : cudaSuccess;
+}
+
 // ---- owned device buffer ----------------------------------------------------
 struct DevBuf {
     void* p = nullptr;

@@ -437,7 +437,7 @@ g3_status mlp_features_dev(g3_ctx* ctx, const g3_tree* t, const g3_freqs* f, int
     }
     DevBuf d_far;
     G3_CUDA(d_far.alloc(n_far * sizeof(BlockRange)));
-    G3_CUDA(cudaMemcpy(d_far.p, rg.data(), n_far * sizeof(BlockRange), cudaMemcpyHostToDevice));
+    G3_CUDA(upload(ctx->stream, d_far.p, rg.data(), n_far * sizeof(BlockRange)));
     const int grid = (n_far + 7) / 8;
     k_mlp_features<<<grid, 256, 0, ctx->stream>>>(t->gd, d_far.as<BlockRange>(), n_far, f->d_sd.as<double2>(),
                                                    f->Ku, kernel, eps3, d_out);

@@ -309,7 +309,8 @@ g3_status gl_table(g3_ctx* ctx) {
         tab[n + i] = 2.0 / ((1.0 - x * x) * dp * dp);
     }
     G3_CUDA(ctx->gl.alloc(2 * n * sizeof(double)));
-    G3_CUDA(cudaMemcpy(ctx->gl.p, tab.data(), 2 * n * sizeof(double), cudaMemcpyHostToDevice));
+    G3_CUDA(upload(ctx->stream, ctx->gl.p, tab.data(), 2 * n * sizeof(double)));
+    G3_CUDA(cudaStreamSynchronize(ctx->stream));  // (the context may change its stream)
     return G3_OK;
 }
 
@@ -1010,7 +1011,8 @@ static g3_status ss_table(g3_ctx* ctx) {
             }
     DevBuf d;
     G3_CUDA(d.alloc(tab.size() * sizeof(float)));
-    G3_CUDA(cudaMemcpy(d.p, tab.data(), tab.size() * sizeof(float), cudaMemcpyHostToDevice));
+    G3_CUDA(upload(ctx->stream, d.p, tab.data(), tab.size() * sizeof(float)));
+    G3_CUDA(cudaStreamSynchronize(ctx->stream));  // (the context may change its stream)
     ctx->ss_tab.take(d);
     return G3_OK;
 }
