@@ -9,7 +9,10 @@
 // there are few blocks, by that chain: so every reduction takes one barrier,
 // the fiber's residual is float-float (not float64), the earlier faces' entries
 // are loaded before the entry is evaluated, and eq. (norm) takes four earlier
-// crosses per pass.  12,288-triangle single layer, 17,554 blocks: 13.1 ms (256
+// crosses per pass: face inner products in float32; those of the fibers, the sum
+// over the crosses, ||C^(l)||^2 and the stopping test in float64 (in float32 they
+// would overflow from entries of 1e16 on, and the fibers reach the ratio of the
+// largest entry to the pivot).  12,288-triangle single layer, 17,554 blocks: 13.1 ms (256
 // threads, float64 fiber) -> 5.0 ms after the low-rank launch, which it
 // overlaps.  1, 2, 4 and 8 warps per block: 80.8, 81.0, 80.7 and 82.6 ms for the
 // whole set-up there, 1.79, 1.60, 1.49 and 1.46 ms for the step on the
@@ -27,11 +30,31 @@ struct DenseSh {
     Cx<float> hk[KU_MAX];    // f_p[k] during the face, H_p[i_l, j_l] during the fiber
     unsigned used[KU_MAX / 32];
     // the warps' parts of a reduction (two buffers), a broadcast value
-    float4 part[2][W][4];
+    float2 part[2][W][4];    // <H_l, H_d> of four crosses
+    double fpart[2][W][8];   // Re, Im of their <f_l, f_d>
+    double norm2;            // ||C^(l)||^2
+    int stop;
     uint2 key[2][W];
     float4 rel[W];
     long long bc;
 };
+
+// eight sums over a warp, the exchanges halving the values a lane carries.  Returns
+// value (lane >> 2) (the four lanes of a group).
+__device__ __forceinline__ double warp_sum8(double* v) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int n = 4, o = 16; n >= 1; n >>= 1, o >>= 1) {
+        const bool hi = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const double send = hi ? v[i] : v[i + n], keep = hi ? v[i + n] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
 
 // largest candidate over the block's warps; buf alternates between calls
 template <int W>
@@ -65,8 +88,10 @@ __device__ __noinline__ bool confirm_dense(DenseSh<W>& sh, const BlockRange br, 
     }
     for (int k = tid; k < Ku; k += NT) rk[k] = 0.0;
     __syncthreads();
-    // squares scaled by a power of two near the newest pivot, float-float sums
-    const int ex = min(max(ilogbf(fmaxf(fabsf(hpiv.x), fabsf(hpiv.y))), -100), 100);
+    // squares scaled by a power of two near ||C^(l)||, which the entries do not exceed
+    // by much (near the newest pivot, they could exceed it by all of float32's range),
+    // float-float sums
+    const int ex = min(max(sh.norm2 > 0.0 ? ilogb(sh.norm2) / 2 : ilogbf(fmaxf(fabsf(hpiv.x), fabsf(hpiv.y))), -100), 100);
     const float sc = scalbnf(1.f, -ex);
     const double back = (double)scalbnf(1.f, ex);
     float2 rt = make_float2(0.f, 0.f), at = rt;
@@ -109,8 +134,7 @@ __device__ __noinline__ bool confirm_dense(DenseSh<W>& sh, const BlockRange br, 
         ff_add(at, v.z, v.w);
     }
     __syncthreads();
-    const float e3 = (float)A.eps3;
-    return rt.x <= e3 * e3 * at.x;
+    return (double)rt.x + (double)rt.y <= A.eps3 * A.eps3 * ((double)at.x + (double)at.y);
 }
 
 __host__ __device__ inline size_t dense_ws_bytes(int Cmax, int Ku) {
@@ -165,6 +189,7 @@ __global__ void __launch_bounds__(DENSE32_NT, 4) k_dense32(const AcaArgs<float> 
             }
         }
         if (tid < KU_MAX / 32) sh.used[tid] = 0u;
+        if (tid == 0) sh.norm2 = 0.0;
         __syncthreads();
         const BlockRange br = A.ranges[blk];
         const int M = br.re - br.rb, N = br.ce - br.cb, MN = M * N, Ku = A.Ku;
@@ -178,7 +203,6 @@ __global__ void __launch_bounds__(DENSE32_NT, 4) k_dense32(const AcaArgs<float> 
         };
         int k_l = A.k1 ? A.k1[blk] : 0, nc = 0, computed = 0;
         long long entries = 0;
-        float2 norm2 = make_float2(0.f, 0.f);   // ||C^(l)||^2, float-float, the same in every thread
         bool zero_block = false, spilled = false;
         auto is_used = [&](int k) { return ((sh.used[k >> 5] >> (k & 31)) & 1u) != 0; };
         for (;;) {
@@ -273,15 +297,15 @@ __global__ void __launch_bounds__(DENSE32_NT, 4) k_dense32(const AcaArgs<float> 
             __syncthreads();
             lap(4);
             // ---- eq. (norm): four earlier crosses (the last: the new one) at a time ----
-            // (products of float32 faces and of fibers normalised by their pivot:
-            // float32 sums per thread and over the block, as for low-rank faces)
-            float2 add = make_float2(0.f, 0.f), own = add;
+            double add = 0.0, own = 0.0;   // (warp 0: lane q of each pass holds cross d0 + q)
             for (int d0 = 0; d0 <= nc; d0 += 4) {
-                Cx<float> h[4], f[4];
+                Cx<float> h[4];
+                double f[8];   // Re, Im
                 const Cx<float>* Hd[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    h[q] = f[q] = Cx<float>{0, 0};
+                    h[q] = Cx<float>{0, 0};
+                    f[2 * q] = f[2 * q + 1] = 0.0;
                     Hd[q] = d0 + q < nc ? A.pool + sh.off[d0 + q] : Hn;
                 }
 #pragma unroll 4
@@ -291,50 +315,54 @@ __global__ void __launch_bounds__(DENSE32_NT, 4) k_dense32(const AcaArgs<float> 
                     for (int q = 0; q < 4; ++q) cfmac(h[q], a, ldcx(Hd[q] + e));
                 }
                 for (int k = tid; k < Ku; k += NT) {
-                    const Cx<float> a = ldcx(Fn + k);
+                    const Cx<double> a = ccast<double>(ldcx(Fn + k));
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) cfmac(f[q], a, ldcx(Hd[q] + MN + k));
+                    for (int q = 0; q < 4; ++q) {   // a conj(b)
+                        const Cx<double> b = ccast<double>(ldcx(Hd[q] + MN + k));
+                        f[2 * q] = fma(a.x, b.x, fma(a.y, b.y, f[2 * q]));
+                        f[2 * q + 1] = fma(a.y, b.x, fma(-a.x, b.y, f[2 * q + 1]));
+                    }
                 }
                 warp_sum_pair(h[0], h[1]);
                 warp_sum_pair(h[2], h[3]);
-                warp_sum_pair(f[0], f[1]);
-                warp_sum_pair(f[2], f[3]);
+                const double fs = warp_sum8(f);
+                if ((lane & 3) == 0) sh.fpart[pbuf][wid][lane >> 2] = fs;
                 if (lane == 0) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) sh.part[pbuf][wid][q] = make_float4(h[q].x, h[q].y, f[q].x, f[q].y);
+                    for (int q = 0; q < 4; ++q) sh.part[pbuf][wid][q] = make_float2(h[q].x, h[q].y);
                 }
                 __syncthreads();
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    h[q] = f[q] = Cx<float>{0, 0};
-                    for (int w = 0; w < W; ++w) {
-                        const float4 v = sh.part[pbuf][w][q];
-                        h[q].x += v.x;
-                        h[q].y += v.y;
-                        f[q].x += v.z;
-                        f[q].y += v.w;
+                if (wid == 0 && lane < 4 && d0 + lane <= nc) {
+                    float2 hs2 = sh.part[pbuf][0][lane];
+                    double fx = sh.fpart[pbuf][0][2 * lane], fy = sh.fpart[pbuf][0][2 * lane + 1];
+                    for (int w = 1; w < W; ++w) {
+                        const float2 v = sh.part[pbuf][w][lane];
+                        hs2.x += v.x;
+                        hs2.y += v.y;
+                        fx += sh.fpart[pbuf][w][2 * lane];
+                        fy += sh.fpart[pbuf][w][2 * lane + 1];
                     }
+                    const double re = (double)hs2.x * fx;
+                    if (d0 + lane < nc) add += 2.0 * (re - (double)hs2.y * fy);
+                    else own = re;
                 }
                 pbuf ^= 1;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (d0 + q < nc) {
-                        ff_add_prod(add, 2.f * h[q].x, f[q].x);
-                        ff_add_prod(add, -2.f * h[q].y, f[q].y);
-                    } else if (d0 + q == nc) {
-                        ff_add_prod(own, h[q].x, f[q].x);
-                    }
+            }
+            if (wid == 0) {
+                add = warp_sum(add);
+                own = warp_sum(own);   // (one lane holds it)
+                if (lane == 0) {
+                    const double n2 = sh.norm2 + (add + own);
+                    sh.norm2 = n2;
+                    sh.stop = fmax(own, 0.0) <= A.eps3 * A.eps3 * fmax(n2, 0.0);
+                    sh.off[nc] = off;  // staged for the stop check
                 }
             }
-            ff_add(add, own.x, own.y);
-            ff_add(norm2, add.x, add.y);
-            const float e3 = (float)A.eps3;
-            const bool stop = fmaxf(own.x, 0.f) <= e3 * e3 * fmaxf(norm2.x, 0.f);
             int nu = 0;
             for (int u = 0; u < KU_MAX / 32; ++u) nu += __popc(sh.used[u]);
             const bool all = nu >= Ku;
-            if (tid == 0) sh.off[nc] = off;  // staged for the stop check
             __syncthreads();
+            const bool stop = sh.stop != 0;
             bool from_samples = false;
             if (stop && A.sample_check && !all) {
                 from_samples = !confirm_dense<KER, W>(sh, br, nc + 1, hpiv, hs, rk);
