@@ -199,6 +199,13 @@ __device__ inline Ws<T> ws_carve(char* base, int RF, int Mmax, int Nmax, int Cma
     return w;
 }
 
+// bound of a float32 face's test on ||u||^2 ||v||^2, as float-float scaled by the power
+// of two `scale` (the squares' range is twice float32's)
+struct FaceThr {
+    float2 v;
+    float scale;
+};
+
 // shared state of the block being processed
 template <class T>
 struct BlockSh {
@@ -220,12 +227,14 @@ struct BlockSh {
     double rdU[RF_MAX], rdV[RF_MAX];  // 1 / diagonal of the Cholesky factors
     T cnV[RF_MAX];                    // column norms of V' (pivot of eq. (index))
     // float32 faces: warp candidates of the row and column argmax; the warps'
-    // parts of ||u_m||^2 and ||v_m||^2 (of ||D||_F^2 before the first step) and of
-    // the recursive norm's cross terms (float-float)
+    // parts of ||u_m||^2 and ||v_m||^2, and of ||D||_F^2 (before the first step) or of
+    // the recursive norm's cross terms
     uint2 key[2][32];
     unsigned usedm[USED_W];  // rows taken by the face ACA
     float2 nrm[32];
-    float2 crs[32];
+    double crs[32];
+    FaceThr thr;             // the face test's bound
+    float rms;               // ||C^(l-1)||_F / sqrt(Ku)
     // float32 recompression: squared norms, norms and their reciprocals of the
     // orthogonalised V columns; squared norms of W's columns (double-buffered);
     // norms of the pivot columns
@@ -667,7 +676,7 @@ __device__ void face_samples(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S,
 // and columns from D and sums only the current face's crosses.  The partial-pivot
 // ACA takes the same rows and columns as with on-demand lines; only the order of
 // the float32 sums over the earlier crosses differs.  The warps' parts of
-// ||D||_F^2 are left in S.nrm.  Tiles of 64 x (NT / 4)
+// ||D||_F^2 are left in S.crs.  Tiles of 64 x (NT / 4)
 // outputs; the earlier crosses' columns (scaled by f_p[kf]) staged DRF_KC at a
 // time in shared memory.  The sum over them is a dense complex product, on the
 // tensor cores at 256 threads (the TF32 three-term split, float32 accuracy),
@@ -1029,8 +1038,8 @@ __device__ __noinline__ void face_dense_residual(const AcaArgs<T>& A, Cx<T>* __r
         }
     }
     }
-    dn = warp_sum(dn);
-    if ((tid & 31) == 0) S.nrm[tid >> 5] = make_float2(dn, 0.f);
+    const double dw = warp_sum((double)dn);
+    if ((tid & 31) == 0) S.crs[tid >> 5] = dw;
     if (tid == 0) atomicAdd(&A.counters[7], (unsigned long long)M * N);
     __syncthreads();
 }
@@ -1772,6 +1781,7 @@ __device__ __forceinline__ void norm_test(const AcaArgs<T>& A, BlockSh<T>& S, in
         if (threadIdx.x == 0) {
             const double own = S.hself * S.fself;
             S.norm2 += add + own;
+            if constexpr (sizeof(T) == 4) S.rms = (float)sqrt(fmax(S.norm2, 0.0) / (double)A.Ku);
             S.stop = fmax(own, 0.0) <= A.eps3 * A.eps3 * fmax(S.norm2, 0.0);
             S.flag = all_used(A, S);
         }
@@ -1813,16 +1823,17 @@ __device__ __noinline__ bool confirm_stop(const AcaArgs<T>& A, const Ws<T>& w, B
     }
     __syncthreads();
     // items (samples SAMPLES / SPI apart, frequency), frequencies fastest; float64
-    // one sample each (its pipe is the bound: spread it), float32 four; the residual energy per frequency is summed in shared memory (S.hh is
-    // not in use here).  Float32 squares are scaled by a power of two near the
-    // newest pivot (their range) and summed in float-float, then in float64.
+    // one sample each (its pipe is the bound: spread it), float32 four; the residual
+    // energy per frequency is summed in shared memory (S.hh is not in use here).
+    // Float32 squares are scaled by a power of two near ||C^(l)||, which the entries do
+    // not exceed by much (near the newest pivot, they could exceed it by all of
+    // float32's range), and summed in float-float, then in float64.
     double* rk = reinterpret_cast<double*>(S.hh);
     for (int k = tid; k < Ku; k += NT) rk[k] = 0.0;
     __syncthreads();
     constexpr bool F32 = sizeof(T) == 4;
     constexpr int SPI = F32 ? 4 : 1;
-    const T hm = F32 ? (T)fmax(fabs((T)S.hpiv.x), fabs((T)S.hpiv.y)) : (T)1;
-    const int ex = F32 ? min(max(ilogbf((float)hm), -100), 100) : 0;
+    const int ex = F32 ? min(max(S.norm2 > 0.0 ? ilogb(S.norm2) / 2 : ilogb(fmax(fabs(S.hpiv.x), fabs(S.hpiv.y))), -100), 100) : 0;
     const T sc = F32 ? (T)scalbnf(1.f, -ex) : (T)1;
     const double back = F32 ? (double)scalbnf(1.f, ex) : 1.0;
     double rr_t = 0.0, aa_t = 0.0;
@@ -2120,6 +2131,7 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3(const AcaArgs<T
             S.ncross = 0;
             S.pre[0] = 0;
             S.norm2 = 0.0;
+            S.rms = 0.f;
             S.entries = 0;
             S.raw = 0;
             for (int i = 0; i < NSUB; ++i) S.sub[i] = 0;
@@ -2545,6 +2557,7 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3_face(const AcaA
                 S.pre[p + 1] = S.pre[p] + cr.r;
             }
             S.norm2 = normb[blk];
+            S.rms = (float)sqrt(fmax(S.norm2, 0.0) / (double)A.Ku);
             S.entries = 0;
             S.raw = 0;
             for (int i = 0; i < NSUB; ++i) S.sub[i] = 0;

@@ -198,6 +198,22 @@ __device__ void samples32(const AcaArgs<float>& A, BlockSh<float>& S, const Face
     __syncthreads();
 }
 
+// max(eps_face^2 ||S_m||_F^2, floor^2)
+__device__ __forceinline__ double face_bound2(const AcaArgs<float>& A, const BlockSh<float>& S) {
+    return fmax(A.eps_face * A.eps_face * fmax(S.fsn2, 0.0), A.face_floor * A.face_floor * S.norm2 / (double)A.Ku);
+}
+__device__ __forceinline__ FaceThr face_thr(double b) {
+    const int e = b > 0.0 ? min(max(ilogb(b), -120), 120) : 0;
+    b = fmin(ldexp(b, -e), 3e38);
+    const float h = (float)b;
+    return FaceThr{make_float2(h, (float)(b - (double)h)), scalbnf(1.f, -e)};
+}
+// nu2 nv2 <= bound (an overflowing left side exceeds it, a vanishing one does not)
+__device__ __forceinline__ bool face_passes(const FaceThr& t, float nu2, float nv2) {
+    const float a = nu2 * t.scale, p = a * nv2;
+    return (p - t.v.x) + (fmaf(a, nv2, -p) - t.v.y) <= 0.f;
+}
+
 // Partial-pivot ACA of the residual face at frequency kf.  Returns the rank m;
 // c holds the crosses.  Rows, columns and tests as in the float64 face_aca:
 //   ||u_m|| ||v_m|| <= eps_face ||S_m||_F  (or the absolute floor), confirmed on
@@ -208,7 +224,11 @@ __device__ void samples32(const AcaArgs<float>& A, BlockSh<float>& S, const Face
 // eps_face where the test can pass, and D's norm is a by-product of forming it.
 // Without D, ||S_m||_F is the recursive
 //   ||S_m||^2 = ||S_{m-1}||^2 + 2 Re sum_t (u_t^H u_m)(v_m^H v_t) + ||u_m||^2 ||v_m||^2
-// (a third barrier; the sum over t took a third of the step's instructions).
+// (two more barriers; the sum over t took a third of the step's instructions).
+// The sums over a vector are float32; their products and what is summed of them are
+// float64 in one warp, as in face_aca, and with D the test is taken in float-float on a
+// scaled bound that one warp forms per face (float64 in every warp would hold each
+// step for its pipe, and float32 products of squares overflow from entries of 1e12).
 template <int KER, int NT>
 __device__ int face32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float>& S, int kf, unsigned char* arena,
                       ColStore& c) {
@@ -248,16 +268,17 @@ __device__ int face32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float
     c.ncs = min(c.ncs, A.RF);
     int m = 0, irow = 0;
     bool converged = false;
-    // ||S_m||_F^2 (the same in every thread)
-    float2 fsn2 = make_float2(0.f, 0.f);
-    if (D) {
-        for (int q = 0; q < NW; ++q) ff_add(fsn2, S.nrm[q].x, 0.f);
-        __syncthreads();   // S.nrm is rewritten by the first step
+    // own <= max(eps^2 ||S||^2, floor^2); S.fsn2: ||S_m||_F^2
+    if (wid == 0) {
+        double n2 = D && lane < NW ? S.crs[lane] : 0.0;
+        n2 = warp_sum(n2);
+        if (lane == 0) {
+            S.fsn2 = n2;
+            S.thr = face_thr(face_bound2(A, S));
+        }
     }
-    // own <= max(eps^2 ||S||^2, floor^2), divided by eps^2 (eps^2 alone can take
-    // the norms of strongly damped faces below the float32 range)
-    const float e1 = (float)A.eps_face, inv_e2 = 1.f / (e1 * e1);
-    const float fl = (float)A.face_floor / e1, floor_s = fl * fl * ((float)S.norm2 / (float)A.Ku);
+    __syncthreads();
+    const FaceThr thr = S.thr;   // (with D)
     while (m < cap) {
         // ---- the residual row ----
         if (F.ncol > 0) {
@@ -332,8 +353,8 @@ __device__ int face32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float
         }
         sublap(S, 7, tf);
         if (!D) {
-            // the recursive norm's cross terms, in float-float
-            float2 part = make_float2(0.f, 0.f);
+            // the recursive norm's cross terms
+            double part = 0.0;
             for (int t = wid; t < m; t += NW) {
                 const Cx<float>* ut = cs_u<false>(c, t);
                 const Cx<float>* vt = ut + M;
@@ -344,18 +365,25 @@ __device__ int face32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float
                 for (int i = lane; i < N; i += 32) cfmac(gv, ldcx(vt + i), ldcx(vm + i));  // conj(v_m) v_t
                 // lanes 0-15: Re gu, Re gv; lanes 16-31: Im gu, Im gv
                 const float2 g = warp_sum4(gu.x, gv.x, gu.y, gv.y);
-                ff_add_prod(part, (lane & 16) ? -2.f * g.x : 2.f * g.x, g.y);
+                part = fma((lane & 16) ? -2.0 * (double)g.x : 2.0 * (double)g.x, (double)g.y, part);
             }
-            const float px = __shfl_xor_sync(0xffffffffu, part.x, 16), py = __shfl_xor_sync(0xffffffffu, part.y, 16);
-            ff_add(part, px, py);
+            part += __shfl_xor_sync(0xffffffffu, part, 16);
             if (lane == 0) S.crs[wid] = part;
             __syncthreads();
-            for (int q = 0; q < NW; ++q) ff_add(fsn2, S.crs[q].x, S.crs[q].y);
-            ff_add_prod(fsn2, nu2, nv2);
+            if (wid == 0) {
+                double add = lane < NW ? S.crs[lane] : 0.0;
+                add = warp_sum(add);
+                if (lane == 0) {
+                    const double own = (double)nu2 * (double)nv2;
+                    S.fsn2 += add + own;
+                    S.fconv = own <= face_bound2(A, S);
+                }
+            }
+            __syncthreads();
             sublap(S, 8, tf);
         }
         ++m;
-        if (nu2 * nv2 * inv_e2 <= fmaxf(fmaxf(fsn2.x, 0.f), floor_s)) {
+        if (D ? face_passes(thr, nu2, nv2) : S.fconv != 0) {
             if (!A.sample_check) {
                 converged = true;
                 break;
@@ -370,10 +398,7 @@ __device__ int face32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float
                 ArgMaxT<float> b{(float)sv, lane};
                 b = warp_argmax(b);
                 if (lane == 0) {
-                    const double e2 = A.eps_face * A.eps_face;
-                    S.fconv = (double)M * (double)N / SAMPLES * tot <=
-                              fmax(e2 * fmax((double)fsn2.x + (double)fsn2.y, 0.0),
-                                   A.face_floor * A.face_floor * S.norm2 / (double)A.Ku);
+                    S.fconv = (double)M * (double)N / SAMPLES * tot <= face_bound2(A, S);
                     S.fbs = b.i;
                 }
             }
@@ -548,7 +573,7 @@ __device__ int recompress32_t(const AcaArgs<float>& A, BlockSh<float>& S, const 
         if (lane == 0) S.cn[0][j] = s2;
     }
     __syncthreads();
-    const float sfloor = (float)A.trunc_floor * sqrtf((float)S.norm2 / (float)A.Ku);
+    const float sfloor = (float)A.trunc_floor * S.rms;
     float r00 = 0.f;
     int k = 0;
     for (; k < r; ++k) {
