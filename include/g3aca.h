@@ -203,7 +203,9 @@ typedef struct {
     int64_t phase_cycles[7];  /* SM cycles summed over CTAs: face ACA, recompression,
                                  factor formation, pivot search, fiber, eq. (norm), next k  */
     int32_t ctas;             /* persistent CTAs launched                                 */
-    int32_t recompress_fallbacks; /* faces kept unrecompressed (Cholesky breakdown)       */
+    int32_t recompress_fallbacks; /* faces whose recompression broke down (status bit 4):
+                                 G3_FP64 kept unrecompressed (Cholesky), G3_MIXED cut off
+                                 where their values stop being finite                     */
     int32_t blocks_run;       /* blocks compressed (n_far unless opts->max_blocks)        */
     int64_t dense_crosses;    /* kept crosses with a dense face (face_rank_sum excludes them) */
     double ms_lowrank;        /* device time of the low-rank-face launch (last attempt)   */

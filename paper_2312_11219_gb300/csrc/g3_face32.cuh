@@ -451,7 +451,10 @@ __device__ int face32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float
 // cycles (12,288-triangle single layer, 192 x 192 blocks: 310,000 -> see
 // k_aca3's table).
 // RT [r][ldr]: conj(R) transposed; JT [r][ldr].  Returns the kept rank;
-// S.sel, S.rk32: pivot columns and their norms.
+// S.sel, S.rk32: pivot columns and their norms.  A face that breaks down (values that
+// are not finite, or no column left of a face with crosses) is reported in the status
+// and counted: the columns are overwritten by then, so what was found up to there is
+// kept.
 template <int NT, bool SM>
 __device__ int recompress32_t(const AcaArgs<float>& A, BlockSh<float>& S, const ColStore& c, int r, Cx<float>* RT,
                               Cx<float>* JT, int ldr) {
@@ -647,6 +650,15 @@ __device__ int recompress32_t(const AcaArgs<float>& A, BlockSh<float>& S, const 
         __syncthreads();
     }
     __syncthreads();
+    if (wid == 0) {
+        const float* cn = S.cn[k & 1];
+        bool bad = k == 0;
+        for (int q = lane; q < r; q += 32) bad |= !isfinite(cn[q]);
+        if (__any_sync(0xffffffffu, bad) && lane == 0) {
+            atomicOr(A.status, ST_CHOL_FALLBACK);
+            atomicAdd(&A.counters[4], 1ull);
+        }
+    }
     sublap(S, 3, tc);
     // fold Q's normalisation into J
     for (int e = tid; e < r * ldr; e += NT) {
