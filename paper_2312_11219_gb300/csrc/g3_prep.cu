@@ -5,6 +5,7 @@
 #include <vector>
 
 #include "g3_device.cuh"
+#include "g3_series.cuh"
 
 namespace g3 {
 
@@ -431,81 +432,6 @@ struct FreqOf<float> {
 template <class T>
 using FreqT = typename FreqOf<T>::type;
 
-// A regular entry at all its frequencies from one power series.  With r_c the middle of
-// the points' distances and R their half range (d_q = (r_q - r_c) / R, |d_q| <= 1),
-//   sum_q a_q exp(-s r_q) = exp(-s r_c) p(-s R),  p(z) = sum_n m_n z^n,  m_n = sum_q a_q d_q^n / n!,
-// and with a_q (1 + s r_q) in place of a_q the coefficients (1 - n) m_n - (r_c / R) m_{n-1}.
-// The coefficients are real and are formed once per entry, so that a frequency takes
-// one exponential, one sine and cosine, and two multiply-adds per term
-// (b_n = c_n + 2 Re z b_{n+1} - |z|^2 b_{n+2}) instead of an exponential, a sine and a
-// cosine per point.  The degree goes by |z| of the warp's entries: 8, 12 or 16 in float32
-// up to |z| = 0.5, 1.25, 2.25 (first term left out below 5e-9 of the largest), 14, 20, 24
-// in float64 up to 0.5, 1.25, 2 (below 3e-17); beyond, point by point.  The terms grow to
-// at most exp(|z|), but the phase s r_c is formed once, with the rounding of its product
-// carried along, where the points' phases were rounded to |s r| 2^-24 each.
-template <class T>
-struct NearSeries;
-template <>
-struct NearSeries<float> {
-    static constexpr int N0 = 8, N1 = 12, N2 = 16;
-    static constexpr float Z0 = 0.5f, Z1 = 1.25f, Z2 = 2.25f;
-};
-template <>
-struct NearSeries<double> {
-    static constexpr int N0 = 14, N1 = 20, N2 = 24;
-    static constexpr double Z0 = 0.5, Z1 = 1.25, Z2 = 2.0;
-};
-
-// coefficients c[0 .. N2] from NP points; returns r_c and R
-template <int KER, class T, int NP>
-__device__ __forceinline__ void series_setup(const T (&r)[NP], const T (&a)[NP], T* c, T& rc, T& R) {
-    constexpr int N = NearSeries<T>::N2;
-    T lo = r[0], hi = r[0];
-#pragma unroll
-    for (int q = 1; q < NP; ++q) {
-        lo = min(lo, r[q]);
-        hi = max(hi, r[q]);
-    }
-    rc = (T)0.5 * (lo + hi);
-    R = max((T)0.5 * (hi - lo), rc * (T)0x1p-10);   // (points at one distance: any unit does)
-    const T iR = (T)1 / R;
-#pragma unroll
-    for (int n = 0; n <= N; ++n) c[n] = 0;
-#pragma unroll
-    for (int q = 0; q < NP; ++q) {
-        const T d = (r[q] - rc) * iR;
-        T t = a[q];
-        c[0] += t;
-#pragma unroll
-        for (int n = 1; n <= N; ++n) {
-            t *= d;
-            c[n] += t;
-        }
-    }
-    double f = 1.0;   // 1 / n!, folded at compile time
-#pragma unroll
-    for (int n = 2; n <= N; ++n) {
-        f /= n;
-        c[n] *= (T)f;
-    }
-    if constexpr (KER == G3_DLP) {
-        const T g = rc * iR;
-#pragma unroll
-        for (int n = N; n >= 1; --n) c[n] = (T)(1 - n) * c[n] - g * c[n - 1];
-    }
-}
-template <int N, class T>
-__device__ __forceinline__ Cx<T> series_sum(const T* c, T x, T y, T z2) {
-    const T x2 = x + x;
-    T b1 = c[N], b2 = 0;
-#pragma unroll
-    for (int n = N - 1; n >= 1; --n) {
-        const T b = fma(x2, b1, fma(-z2, b2, c[n]));
-        b2 = b1;
-        b1 = b;
-    }
-    return {fma(x, b1, fma(-z2, b2, c[0])), y * b1};
-}
 // exp(-(sre + i sim) r) with the products' rounding errors carried along.  float32: the
 // exponent split into an integer and at most log(2) / 2, the phase into quarter turns and
 // at most pi / 4 (Taylor polynomials of degree 9 and 10, 2e-9)
@@ -588,8 +514,9 @@ __global__ void __launch_bounds__(NEAR_NT) k_near(int E, int kch, GeomF gf, Geom
             else
                 pair_setup<KER>(gd, i, jj, p);
         }
-        T c[S::N2 + 1], rc, R;
-        series_setup<KER, T>(p.r, p.a, c, rc, R);
+        constexpr int X = SERIES_MORE<KER>;
+        T c[S::N2 + X + 1], rc, R;
+        series_setup<KER, S::N2 + X, T>(p.r, p.a, c, rc, R);
         for (int kk = 0; kk < kn; ++kk) {
             const FreqT<T> s = sk[k0 + kk];
             const T x = -s.x * R, y = -s.y * R, z2 = fma(x, x, y * y);
@@ -598,11 +525,11 @@ __global__ void __launch_bounds__(NEAR_NT) k_near(int E, int kch, GeomF gf, Geom
             if (__all_sync(0xffffffffu, z2 <= S::Z2 * S::Z2)) {
                 Cx<T> w;
                 if (__all_sync(0xffffffffu, z2 <= S::Z0 * S::Z0))
-                    w = series_sum<S::N0>(c, x, y, z2);
+                    w = series_sum<S::N0 + X>(c, x, y, z2);
                 else if (__all_sync(0xffffffffu, z2 <= S::Z1 * S::Z1))
-                    w = series_sum<S::N1>(c, x, y, z2);
+                    w = series_sum<S::N1 + X>(c, x, y, z2);
                 else
-                    w = series_sum<S::N2>(c, x, y, z2);
+                    w = series_sum<S::N2 + X>(c, x, y, z2);
                 v = cmul(cexp_acc(s.x, s.y, rc), w);
             } else if constexpr (KER == G3_GAL_SLP) {
                 v = gal_eval<T>(p, s.x, s.y);
