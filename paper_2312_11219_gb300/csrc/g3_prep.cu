@@ -983,7 +983,7 @@ static g3_status launch_near_p1_t(g3_ctx* ctx, const g3_tree* t, const g3_freqs*
     return G3_OK;
 }
 
-// Self entries of the single layer in the near field, float64: one warp per
+// Self entries of the single layer in the near field, in float64: one warp per
 // element p; the entry (p, p) of the diagonal leaf block sits at diag_base[p] +
 // k * diag_mn[p] (diag_base[p] < 0: not in this tree's blocks).
 //
@@ -999,9 +999,13 @@ static g3_status launch_near_p1_t(g3_ctx* ctx, const g3_tree* t, const g3_freqs*
 // for n < 32, and every lane (one frequency each) sums one of
 //   |s| rmax <= 4:  V = (1/4 pi) sum_n (-z)^n / (n+1)! m0_n,            z = s rmax
 //   |s| rh <= 4:    V = (1/4 pi s) (m1_0 - e^{-s rc} sum_n (-x)^n / n! m1_n),  x = s rh
-// whose first omitted terms are below 4^32 / 32! = 7e-17 and whose largest
-// terms exceed the sum by at most e^4, so both hold ~1e-14 relative; larger
-// |s| rh sums the points directly.
+// whose first omitted terms are below 4^32 / 32! = 7e-17; larger |s| rh sums the
+// points directly.  The terms exceed the sum by up to e^4.  Measured in float64 over
+// triangles from right-angled to slivers and all directions of s, against the points
+// summed one by one (mean 2.0e-16, largest 1e-15): the first series 2.0e-16 and 7.7e-16
+// up to |z| = 3.5, then 2.3e-16 and 8.8e-16; the second up to 4.3e-16 and 5.9e-15.
+// Entries that are rounded to float32 take both; float64 entries the first one up to
+// 3.5 and the points beyond (of the multistep frequencies none: |z| <= 3.3).
 // Bound by the float64 pipe (the moments and the series).  12,288 elements x 65
 // frequencies on a GB300: 14.0 -> 1.4 ms, and 1.1 ms with the series as Horner's rule on
 // coefficients that hold the factorials (4 operations per term for 8); both that and
@@ -1054,7 +1058,7 @@ __global__ void __launch_bounds__(SELF_NW * 32) k_near_self(GeomD gd, const doub
         // lane = point (up to three per lane), running powers; 32 moments of a
         // kind are summed over the warp by halving exchanges, which leave
         // moment n in lane n
-        for (int kind = 0; kind < 2; ++kind) {
+        for (int kind = 0; kind < (sizeof(T) == 4 ? 2 : 1); ++kind) {
             double b[3], t[3], v[SELF_NM];
 #pragma unroll
             for (int u = 0; u < 3; ++u) {
@@ -1089,8 +1093,15 @@ __global__ void __launch_bounds__(SELF_NW * 32) k_near_self(GeomD gd, const doub
         const double2 s = sd[k];
         const double as = sqrt(s.x * s.x + s.y * s.y);
         Cx<double> v;
-        if (as * rmax <= 4.0) {
+        if (as * rmax <= (sizeof(T) == 4 ? 4.0 : 3.5)) {
             v = self_series(m0, -s.x * rmax, -s.y * rmax);
+        } else if constexpr (sizeof(T) == 8) {
+            v = Cx<double>{0.0, 0.0};
+            for (int q = 0; q < 72; ++q) {
+                const Cx<double> g = g_expm1_over(Cx<double>{s.x * rho[q], s.y * rho[q]});
+                v.x += wq[q] * rho[q] * g.x;
+                v.y += wq[q] * rho[q] * g.y;
+            }
         } else {
             Cx<double> sum{0.0, 0.0};  // sum_q w_q exp(-s rho_q)
             if (as * rh <= 4.0) {
