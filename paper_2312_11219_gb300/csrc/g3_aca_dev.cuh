@@ -146,7 +146,7 @@ struct Ws {
     long long* colV;
     short* colP;
     Cx<double>* hs;       // [SAMPLES][Cmax] H_p at the stop-check samples
-    double* rk;           // [Ku] sampled residual per frequency
+    double* rk;           // [SAMPLES][Ku] sampled residual energies, then [Ku] per frequency
     Cx<T>* dres;          // [drf_max] dense residual working face (row-major, ld N), or null
 };
 
@@ -167,7 +167,7 @@ __host__ __device__ inline size_t ws_bytes(int RF, int Mmax, int Nmax, int Cmax,
     add((size_t)Cmax * RF * sizeof(long long));
     add((size_t)Cmax * RF * sizeof(short));
     add((size_t)32 * Cmax * sizeof(Cx<double>));
-    add((size_t)Ku * sizeof(double));
+    add((size_t)SAMPLES * Ku * sizeof(double));
     return b;
 }
 
@@ -195,7 +195,7 @@ __device__ inline Ws<T> ws_carve(char* base, int RF, int Mmax, int Nmax, int Cma
     w.colV = (long long*)take((size_t)Cmax * RF * sizeof(long long));
     w.colP = (short*)take((size_t)Cmax * RF * sizeof(short));
     w.hs = (Cx<double>*)take((size_t)32 * Cmax * sizeof(Cx<double>));
-    w.rk = (double*)take((size_t)Ku * sizeof(double));
+    w.rk = (double*)take((size_t)SAMPLES * Ku * sizeof(double));
     return w;
 }
 
@@ -1796,6 +1796,21 @@ __device__ __forceinline__ void norm_test(const AcaArgs<T>& A, BlockSh<T>& S, in
 // Returns true when ||R_samples||_F <= eps3 ||A_samples||_F; otherwise w.rk[k]
 // holds the sampled residual energy per frequency.
 
+// rk [n][Ku] -> its sums over n in rk[0 .. Ku), eight lanes to a sum, in one order
+// (visible to the other threads after the next barrier)
+template <int NT>
+__device__ __forceinline__ void sum_items(double* rk, int n, int Ku) {
+    const int part = threadIdx.x & 7;
+    for (int k0 = 0; k0 < Ku; k0 += NT / 8) {
+        const int k = k0 + threadIdx.x / 8;
+        double s = 0.0;
+        if (k < Ku)
+            for (int q = part; q < n; q += 8) s += rk[q * Ku + k];
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (part == 0 && k < Ku) rk[k] = s;
+    }
+}
+
 template <int KER, class T, int NT>
 __device__ __noinline__ bool confirm_stop(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, int ncl) {
     const int tid = threadIdx.x, Ku = A.Ku;
@@ -1824,13 +1839,12 @@ __device__ __noinline__ bool confirm_stop(const AcaArgs<T>& A, const Ws<T>& w, B
     __syncthreads();
     // items (samples SAMPLES / SPI apart, frequency), frequencies fastest; float64
     // one sample each (its pipe is the bound: spread it), float32 four; the residual
-    // energy per frequency is summed in shared memory (S.hh is not in use here).
+    // energies are kept per item and summed in one order, since the largest of the
+    // sums picks the next frequency.
     // Float32 squares are scaled by a power of two near ||C^(l)||, which the entries do
     // not exceed by much (near the newest pivot, they could exceed it by all of
     // float32's range), and summed in float-float, then in float64.
-    double* rk = reinterpret_cast<double*>(S.hh);
-    for (int k = tid; k < Ku; k += NT) rk[k] = 0.0;
-    __syncthreads();
+    double* rk = w.rk;   // [SAMPLES / SPI][Ku]
     constexpr bool F32 = sizeof(T) == 4;
     constexpr int SPI = F32 ? 4 : 1;
     const int ex = F32 ? min(max(S.norm2 > 0.0 ? ilogb(S.norm2) / 2 : ilogb(fmax(fabs(S.hpiv.x), fabs(S.hpiv.y))), -100), 100) : 0;
@@ -1866,7 +1880,7 @@ __device__ __noinline__ bool confirm_stop(const AcaArgs<T>& A, const Ws<T>& w, B
             rd = ((double)rs.x + (double)rs.y) * back * back;
             ad = ((double)as.x + (double)as.y) * back * back;
         }
-        atomicAdd(&rk[k], rd);
+        rk[e] = rd;
         rr_t += rd;
         aa_t += ad;
     }
@@ -1877,7 +1891,7 @@ __device__ __noinline__ bool confirm_stop(const AcaArgs<T>& A, const Ws<T>& w, B
         atomicAdd(&S.red2[1], aa_t);
     }
     __syncthreads();
-    for (int k = tid; k < Ku; k += NT) w.rk[k] = rk[k];
+    sum_items<NT>(rk, SAMPLES / SPI, Ku);
     const bool ok = S.red2[0] <= A.eps3 * A.eps3 * S.red2[1];
     __syncthreads();
     return ok;

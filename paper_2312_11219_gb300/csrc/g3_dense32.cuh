@@ -72,8 +72,9 @@ __device__ __forceinline__ uint2 dkey(DenseSh<W>& sh, ArgMaxT<float> a, int& buf
 }
 
 // The sampled residual of the approximant with ncl crosses at the 32 fixed
-// samples over all frequencies (as confirm_stop); rk[k]: residual energy per
-// frequency.  hs [SAMPLES][ncl]: H_p at the samples.
+// samples over all frequencies (as confirm_stop); rk [SAMPLES / 4][Ku]: residual
+// energies, on return [Ku] per frequency, summed in one order.  hs [SAMPLES][ncl]: H_p
+// at the samples.
 template <int KER, int W>
 __device__ __noinline__ bool confirm_dense(DenseSh<W>& sh, const BlockRange br, int ncl, Cx<float> hpiv, Cx<float>* hs,
                                            double* rk) {
@@ -86,7 +87,6 @@ __device__ __noinline__ bool confirm_dense(DenseSh<W>& sh, const BlockRange br, 
         const int i = (2 * sm + 1) * M / (2 * SAMPLES), j = (2 * ((11 * sm) % SAMPLES) + 1) * N / (2 * SAMPLES);
         hs[e] = ldcx(A.pool + sh.off[p] + i + (long long)j * M);
     }
-    for (int k = tid; k < Ku; k += NT) rk[k] = 0.0;
     __syncthreads();
     // squares scaled by a power of two near ||C^(l)||, which the entries do not exceed
     // by much (near the newest pivot, they could exceed it by all of float32's range),
@@ -116,7 +116,7 @@ __device__ __noinline__ bool confirm_dense(DenseSh<W>& sh, const BlockRange br, 
             ff_add_prod(at, ay, ay);
         }
         ff_add(rt, rs.x, rs.y);
-        atomicAdd(&rk[k], ((double)rs.x + (double)rs.y) * back * back);
+        rk[e] = ((double)rs.x + (double)rs.y) * back * back;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -133,13 +133,14 @@ __device__ __noinline__ bool confirm_dense(DenseSh<W>& sh, const BlockRange br, 
         ff_add(rt, v.x, v.y);
         ff_add(at, v.z, v.w);
     }
+    sum_items<NT>(rk, SAMPLES / 4, Ku);
     __syncthreads();
     return (double)rt.x + (double)rt.y <= A.eps3 * A.eps3 * ((double)at.x + (double)at.y);
 }
 
 __host__ __device__ inline size_t dense_ws_bytes(int Cmax, int Ku) {
     return (((size_t)SAMPLES * (Cmax + 1) * sizeof(Cx<float>) + 255) & ~size_t(255)) +
-           (((size_t)Ku * sizeof(double) + 255) & ~size_t(255));
+           (((size_t)(SAMPLES / 4) * Ku * sizeof(double) + 255) & ~size_t(255));
 }
 
 // Algorithm 1 with the exact residual face (no low-rank approximation in the
@@ -380,7 +381,7 @@ __global__ void __launch_bounds__(DENSE32_NT, 4) k_dense32(const AcaArgs<float> 
             // ---- next frequency: argmax over unused k of |f_l[k]| ----
             ArgMaxT<float> nk = amax_none<float>();
             for (int k = tid; k < Ku; k += NT)
-                if (!is_used(k)) nk = amax_better(nk, ArgMaxT<float>{from_samples ? (float)__ldcg(rk + k) : cabs2(ldcx(Fn + k)), k});
+                if (!is_used(k)) nk = amax_better(nk, ArgMaxT<float>{from_samples ? (float)rk[k] : cabs2(ldcx(Fn + k)), k});
             const uint2 key = dkey<W>(sh, nk, kbuf);
             lap(6);
             if (key.x == 0u || (int)key.y >= Ku) break;  // no finite candidate left
