@@ -239,6 +239,12 @@ typedef struct {
  * work on it. */
 g3_status g3_create(int device, void* cuda_stream, g3_ctx** out);
 g3_status g3_set_stream(g3_ctx* ctx, void* cuda_stream);
+/* Device memory that handles and calls free is kept for the next ones, per device and
+ * shared by all contexts: at most 1/32 of the device's memory, and no buffer above
+ * 128 MB while less than an eighth of the device is free.  It goes back when an
+ * allocation of the library fails, when the device's last context is destroyed, and
+ * here: call this before another allocator of the process needs it. */
+g3_status g3_trim(g3_ctx* ctx);
 /* Where the float32 (complex64) apply forms the far-field vectors
  * x_p = sum_k f_p[k] w_k of eq. (product): on = 1 (default) on the tensor cores
  * (mma.sync m16n8k8 TF32 in a three-term split, float32 accumulation, about

@@ -76,6 +76,7 @@ def _sig(name, res, *args):
 _ci = C.c_int
 _sig("g3_create", _ci, _ci, _p, _pp)
 _sig("g3_set_stream", _ci, _p, _p)
+_sig("g3_trim", _ci, _p)
 _sig("g3_set_apply_tensor_cores", _ci, _p, _ci)
 _sig("g3_destroy", _ci, _p)
 _sig("g3_last_error", C.c_char_p)
@@ -129,7 +130,7 @@ _sig("g3_mlp_free", _ci, _p)
 _sig("g3_block_features", _ci, _p, _p, _p, _ci, C.c_double, _fp)
 _sig("g3_factors_labels", _ci, _p, _p, _fp)
 
-EXPORTED = ["g3_create", "g3_set_stream", "g3_set_apply_tensor_cores", "g3_destroy", "g3_last_error", "g3_version", "g3_launch_count",
+EXPORTED = ["g3_create", "g3_set_stream", "g3_trim", "g3_set_apply_tensor_cores", "g3_destroy", "g3_last_error", "g3_version", "g3_launch_count",
             "g3_kernel_name", "g3_freqs_bdf2", "g3_freqs_gcq", "g3_freqs_from_array", "g3_freqs_info", "g3_freqs_get", "g3_freqs_free",
             "build_cluster_tree", "build_cluster_tree_capped", "build_p1_tree", "g3_shard_rows", "g3_tree_partition_host", "g3_tree_subset", "g3_tree_info", "g3_tree_get", "g3_tree_free", "g3_entries", "assemble_near",
             "g3_near_info", "g3_near_get_block", "g3_near_free", "aca3_compress", "aca3_compress_batch", "g3_autotune", "aca3_compress_separable",
@@ -194,6 +195,10 @@ class Context(_Handle):
 
     def set_stream(self, stream) -> None:
         _check(_lib.g3_set_stream(self.h, C.c_void_p(stream)), "g3_set_stream")
+
+    def trim(self) -> None:
+        """Return the device memory that the library keeps for reuse."""
+        _check(_lib.g3_trim(self.h), "g3_trim")
 
     def set_apply_tensor_cores(self, on: bool) -> None:
         """Far-field x formation of float32 applies on the tensor cores (default) or the CUDA cores."""

@@ -48,12 +48,18 @@ g3_status cuda_fail(cudaError_t e, const char* what) {
 // L-shape 7.9 -> 5.3 ms, its set-up 81.0 -> 75.6 ms.
 // Any stream, thread or context may have used the buffer before, and its work may be
 // pending.  So kept buffers freed since the last wait are handed out only after the
-// device has been waited for, by the cudaFree of a small buffer: what freeing the buffer
-// itself did (it waits for all work on the device, also where a stream elsewhere is
-// capturing and a device synchronisation would be an error).
+// device has been waited for, by the cudaFree of a small buffer, as the free of the
+// buffer itself did.  That cudaFree waits for the other streams is how it behaves, not
+// what its description promises (the tests hold a reader on another stream against it);
+// cudaDeviceSynchronize promises it, but returns cudaErrorStreamCaptureUnsupported and
+// invalidates the capture while any other thread captures, also in thread-local and
+// relaxed mode, where cudaMalloc and cudaFree work and leave the capture alone.
 // Bounds: at most 1/32 of the device's memory is kept per device (the oldest buffers go
-// first, larger ones are never kept); a failing allocation frees all of it and is tried
-// again; so does the end of the device's last context.
+// first, larger ones are never kept), and no buffer above 128 MB while less than an
+// eighth of the device is free: the memory may be wanted elsewhere in the process, and
+// goes back at once, with all that was kept (asking takes about 15 us).  A failing
+// allocation frees all of it and is tried again; so do g3_trim and the end of the
+// device's last context.
 struct DevPool {
     struct Block {
         void* p;
@@ -81,6 +87,16 @@ struct DevPool {
     void trim() {
         for (int i = 0; i < n; ++i) cudaFree(kept[i].p);
         remove(0, n);
+    }
+    // room for keeping a buffer (device `dev`)
+    static bool room(size_t bytes, int dev) {
+        if (bytes <= (128 << 20)) return true;
+        size_t free_b = 0, total = 0;
+        int cur = -1;
+        const bool ok = cudaGetDevice(&cur) == cudaSuccess && cur == dev &&
+                        cudaMemGetInfo(&free_b, &total) == cudaSuccess;
+        if (!ok) cudaGetLastError();
+        return ok && free_b >= total / 8;
     }
 };
 static DevPool* dev_pool(int dev) {
@@ -131,7 +147,9 @@ void dev_free(void* p, size_t bytes, int dev) {
     DevPool* const P = dev_pool(dev);
     if (P) {
         std::lock_guard<std::mutex> lock(P->m);
-        if (P->contexts > 0 && bytes <= P->cap) {
+        if (P->contexts > 0 && bytes <= P->cap && !P->room(bytes, dev)) {
+            P->trim();
+        } else if (P->contexts > 0 && bytes <= P->cap) {
             int drop = 0;
             size_t left = P->held;
             for (; drop < P->n && (left + bytes > P->cap || P->n - drop == DevPool::MAX); ++drop) {
@@ -165,6 +183,13 @@ void dev_pool_open(int dev, size_t total_bytes) {
         std::lock_guard<std::mutex> lock(P->m);
         ++P->contexts;
         P->cap = total_bytes / 32;
+    }
+}
+
+void dev_pool_trim(int dev) {
+    if (DevPool* const P = dev_pool(dev)) {
+        std::lock_guard<std::mutex> lock(P->m);
+        P->trim();
     }
 }
 
@@ -263,6 +288,13 @@ g3_status g3_create(int device, void* cuda_stream, g3_ctx** out) {
 g3_status g3_set_stream(g3_ctx* ctx, void* cuda_stream) {
     G3_CHECK(ctx != nullptr, "g3_set_stream: ctx is NULL");
     ctx->stream = (cudaStream_t)cuda_stream;
+    return G3_OK;
+}
+
+g3_status g3_trim(g3_ctx* ctx) {
+    G3_CHECK(ctx != nullptr, "g3_trim: ctx is NULL");
+    G3_TRY(use_device(ctx));
+    dev_pool_trim(ctx->device);
     return G3_OK;
 }
 

@@ -42,6 +42,7 @@ void dev_free(void* p, size_t bytes, int dev);
 cudaError_t dev_mem_free(size_t* bytes);                             // free on the current device, kept buffers included
 void dev_pool_open(int dev, size_t total_bytes);                     // a context came / went
 void dev_pool_close(int dev);
+void dev_pool_trim(int dev);
 
 // Copies to device memory go through the context's stream, never through the legacy
 // stream: a context on a non-blocking stream has no ordering with that one, and
