@@ -531,50 +531,50 @@ __device__ __forceinline__ void cross_sum(const AcaArgs<T>& A, const FaceTab<T>&
                                           Cx<T>& s1, Cx<T>& s2, Cx<T>& s3) {
     const long long* col = ROW ? F.colV : F.colU;
     const int nt = F.ncol;
-                int c = part;
-                // LIF loads in flight per thread (the sums wait on memory, not on arithmetic)
-                for (; c + (LIF - 1) * G < nt; c += LIF * G) {
-                    Cx<T> x[LIF];
-    #pragma unroll
-                    for (int u = 0; u < LIF; ++u) x[u] = ldcx(A.pool + col[c + u * G] + v);
-    #pragma unroll
-                    for (int u = 0; u < LIF; ++u) {
-                        Cx<T>& acc_u = (u & 3) == 0 ? s0 : (u & 3) == 1 ? s1 : (u & 3) == 2 ? s2 : s3;
-                        if (ROW) cfmac(acc_u, F.coef[c + u * G], x[u]);
-                        else cfma(acc_u, x[u], F.coef[c + u * G]);
-                    }
-                }
-                for (; c + 7 * G < nt; c += 8 * G) {
-                    Cx<T> x[8];
-    #pragma unroll
-                    for (int u = 0; u < 8; ++u) x[u] = ldcx(A.pool + col[c + u * G] + v);
-    #pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        Cx<T>& acc_u = (u & 3) == 0 ? s0 : (u & 3) == 1 ? s1 : (u & 3) == 2 ? s2 : s3;
-                        if (ROW) cfmac(acc_u, F.coef[c + u * G], x[u]);
-                        else cfma(acc_u, x[u], F.coef[c + u * G]);
-                    }
-                }
-                for (; c + 3 * G < nt; c += 4 * G) {
-                    const Cx<T> x0 = ldcx(A.pool + col[c] + v), x1 = ldcx(A.pool + col[c + G] + v);
-                    const Cx<T> x2 = ldcx(A.pool + col[c + 2 * G] + v), x3 = ldcx(A.pool + col[c + 3 * G] + v);
-                    if (ROW) {
-                        cfmac(s0, F.coef[c], x0);
-                        cfmac(s1, F.coef[c + G], x1);
-                        cfmac(s2, F.coef[c + 2 * G], x2);
-                        cfmac(s3, F.coef[c + 3 * G], x3);
-                    } else {
-                        cfma(s0, x0, F.coef[c]);
-                        cfma(s1, x1, F.coef[c + G]);
-                        cfma(s2, x2, F.coef[c + 2 * G]);
-                        cfma(s3, x3, F.coef[c + 3 * G]);
-                    }
-                }
-                for (; c < nt; c += G) {
-                    const Cx<T> x0 = ldcx(A.pool + col[c] + v);
-                    if (ROW) cfmac(s0, F.coef[c], x0);
-                    else cfma(s0, x0, F.coef[c]);
-                }
+    int c = part;
+    // LIF loads in flight per thread (the sums wait on memory, not on arithmetic)
+    for (; c + (LIF - 1) * G < nt; c += LIF * G) {
+        Cx<T> x[LIF];
+#pragma unroll
+        for (int u = 0; u < LIF; ++u) x[u] = ldcx(A.pool + col[c + u * G] + v);
+#pragma unroll
+        for (int u = 0; u < LIF; ++u) {
+            Cx<T>& acc_u = (u & 3) == 0 ? s0 : (u & 3) == 1 ? s1 : (u & 3) == 2 ? s2 : s3;
+            if (ROW) cfmac(acc_u, F.coef[c + u * G], x[u]);
+            else cfma(acc_u, x[u], F.coef[c + u * G]);
+        }
+    }
+    for (; c + 7 * G < nt; c += 8 * G) {
+        Cx<T> x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = ldcx(A.pool + col[c + u * G] + v);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            Cx<T>& acc_u = (u & 3) == 0 ? s0 : (u & 3) == 1 ? s1 : (u & 3) == 2 ? s2 : s3;
+            if (ROW) cfmac(acc_u, F.coef[c + u * G], x[u]);
+            else cfma(acc_u, x[u], F.coef[c + u * G]);
+        }
+    }
+    for (; c + 3 * G < nt; c += 4 * G) {
+        const Cx<T> x0 = ldcx(A.pool + col[c] + v), x1 = ldcx(A.pool + col[c + G] + v);
+        const Cx<T> x2 = ldcx(A.pool + col[c + 2 * G] + v), x3 = ldcx(A.pool + col[c + 3 * G] + v);
+        if (ROW) {
+            cfmac(s0, F.coef[c], x0);
+            cfmac(s1, F.coef[c + G], x1);
+            cfmac(s2, F.coef[c + 2 * G], x2);
+            cfmac(s3, F.coef[c + 3 * G], x3);
+        } else {
+            cfma(s0, x0, F.coef[c]);
+            cfma(s1, x1, F.coef[c + G]);
+            cfma(s2, x2, F.coef[c + 2 * G]);
+            cfma(s3, x3, F.coef[c + 3 * G]);
+        }
+    }
+    for (; c < nt; c += G) {
+        const Cx<T> x0 = ldcx(A.pool + col[c] + v);
+        if (ROW) cfmac(s0, F.coef[c], x0);
+        else cfma(s0, x0, F.coef[c]);
+    }
 }
 
 // Residual of one row (ROW: fixed row `fix`, all columns) or one column (!ROW:
@@ -835,7 +835,7 @@ __device__ __noinline__ void face_dense_residual(const AcaArgs<T>& A, Cx<T>* __r
     if constexpr (NT == 256) {
         // tensor cores: per 64 x 64 tile, warp w takes rows 16 (w % 4) and columns
         // 32 (w / 4) (four 16 x 8 output tiles); sum_c u_ic conj(v_jc) as the real
-        // products Re = ur vr + ui vi, Im = ui vr - ur vi (mma_tf32x3 each)
+        // products Re = ur vr + ui vi, Im = ui vr - ur vi, in the three-term split each
         const int warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
         const int rw = (warp & 3) * 16, cw = (warp >> 2) * 32;
         constexpr int KC = DRF_KC, ST = DRF_ST;

@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(NT) k_apply_near_wide(const Cx<T>* __restrict_
 // x_p = sum_k f_p[k] w_k for 16 columns x 8 crosses at a time is the real-matrix product
 // of W_sigma^T (columns x frequencies) and F (frequencies x crosses), split into four real
 // products per complex product, each on the tensor cores in the three-term TF32 split
-// of g3_device.cuh (mma_tf32x3).
+// of g3_device.cuh.
 // row stride (floats) of the split fibers in shared memory: >= the padded frequency
 // count and 4 mod 8, so the eight rows of a B fragment fall in distinct banks
 __host__ __device__ constexpr int tc_fiber_stride(int Ku) { return (Ku + 7) / 8 * 8 + 4; }
@@ -782,7 +782,7 @@ g3_status far_plan_build(g3_factors* fa) {
         int b, g;
     };
     std::vector<Item> narrow, wide, dense;
-    int mmax = 0, nmax = 0;
+    int mmax = 0;
     for (int b = 0; b < fa->n_far; ++b) {
         const int r = fa->r3[b];
         if (r <= 0) continue;
@@ -790,7 +790,6 @@ g3_status far_plan_build(g3_factors* fa) {
             const int M = fa->ranges[b].re - fa->ranges[b].rb, N = fa->ranges[b].ce - fa->ranges[b].cb;
             dense.push_back(Item{(long long)r * M * N, b, 0});
             mmax = std::max(mmax, M);
-            nmax = std::max(nmax, N);
             continue;
         }
         const int M = fa->ranges[b].re - fa->ranges[b].rb;
@@ -847,10 +846,8 @@ g3_status far_plan_build(g3_factors* fa) {
     }
     close();
     fa->plan_nd = nd;
-    fa->plan_nmax_dense = nmax;
     fa->plan_n1 = (int)narrow.size();
     fa->plan_n2 = (int)wide.size();
-    fa->plan_ab = 0;
     fa->plan_mmax_dense = mmax;
     for (const Item& it : narrow) L.insert(L.end(), {it.b, it.g, 0, 0});
     for (const Item& it : wide) L.insert(L.end(), {it.b, it.g, 0, 0});

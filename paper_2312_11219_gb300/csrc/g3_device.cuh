@@ -713,13 +713,6 @@ __device__ __forceinline__ void mma_tf32(float* d, const unsigned* a, const unsi
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
-// d += a b in the three-term split (the small terms first)
-__device__ __forceinline__ void mma_tf32x3(float* d, const unsigned* ah, const unsigned* al, const unsigned* bh,
-                                           const unsigned* bl) {
-    mma_tf32(d, ah, bl);
-    mma_tf32(d, al, bh);
-    mma_tf32(d, ah, bh);
-}
 // sign flip of TF32 bit patterns (exact)
 __device__ __forceinline__ void tf32_neg4(const unsigned* a, unsigned* o) {
 #pragma unroll
