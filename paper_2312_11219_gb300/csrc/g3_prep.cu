@@ -432,45 +432,6 @@ struct FreqOf<float> {
 template <class T>
 using FreqT = typename FreqOf<T>::type;
 
-// exp(-(sre + i sim) r) with the products' rounding errors carried along.  float32: the
-// exponent split into an integer and at most log(2) / 2, the phase into quarter turns and
-// at most pi / 4 (Taylor polynomials of degree 9 and 10, 2e-9)
-__device__ __forceinline__ Cx<float> cexp_acc(float sre, float sim, float r) {
-    const float u0 = -sre * r, u = fmaxf(u0, -200.0f);
-    const float ul = u0 >= -200.0f ? fmaf(-sre, r, -u0) : 0.0f;
-    const float m = rintf(u * 1.44269504f);
-    float f = fmaf(-m, 0.693145752f, u);      // log 2 = 90852 / 2^17 + 1.42860682e-6
-    f = fmaf(-m, 1.42860682e-6f, f) + ul;
-    const float e = __expf(f) * exp2f(m);
-    const float t = sim * r, tl = fmaf(sim, r, -t);
-    const float n = rintf(t * 0.636619772f);
-    float h = fmaf(-n, 1.5703125f, t);
-    h = fmaf(-n, 4.83826794897e-4f, h) + tl;
-    const float h2 = h * h;
-    float sn = fmaf(h2, 1.0f / 362880.0f, -1.0f / 5040.0f);
-    sn = fmaf(h2, sn, 1.0f / 120.0f);
-    sn = fmaf(h2, sn, -1.0f / 6.0f);
-    sn = fmaf(h * h2, sn, h);
-    float cs = fmaf(h2, -1.0f / 3628800.0f, 1.0f / 40320.0f);
-    cs = fmaf(h2, cs, -1.0f / 720.0f);
-    cs = fmaf(h2, cs, 1.0f / 24.0f);
-    cs = fmaf(h2, cs, -0.5f);
-    cs = fmaf(h2, cs, 1.0f);
-    const int k = (int)n;
-    const float c1 = (k & 1) ? sn : cs, s1 = (k & 1) ? cs : sn;   // cos, sin of n quarter turns + h
-    const float c = ((k + 1) & 2) ? -c1 : c1, s = (k & 2) ? -s1 : s1;
-    return {e * c, -e * s};
-}
-__device__ __forceinline__ Cx<double> cexp_acc(double sre, double sim, double r) {
-    const double u = -sre * r, ul = fma(-sre, r, -u);
-    double e = exp(u);
-    if (e > 0.0 && e < 1e300) e = fma(e, ul, e);
-    const double t = sim * r, tl = fma(sim, r, -t);
-    double sn, cs;
-    sincos(t, &sn, &cs);
-    return {e * fma(-sn, tl, cs), -e * fma(cs, tl, sn)};
-}
-
 // Four warps per CTA: a 24 x 24 block is 18 warps of entries, 90 % of five rounds (75 %
 // of three rounds of eight; 12,288 triangles 2.18 and 2.17 ms, small meshes fill the chip
 // better).

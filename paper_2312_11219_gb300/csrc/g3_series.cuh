@@ -1,6 +1,6 @@
 #pragma once
-// The power series of the near field's regular entries.  Needs Cx (g3_device.cuh) and the
-// kernel kinds; compiles for the host, too.
+// The power series of the near field's regular entries, and its exponential.  Needs Cx
+// (g3_device.cuh) and the kernel kinds; compiles for the host, too.
 
 namespace g3 {
 
@@ -83,6 +83,49 @@ __host__ __device__ __forceinline__ Cx<T> series_sum(const T* c, T x, T y, T z2)
         b1 = b;
     }
     return {fma(x, b1, fma(-z2, b2, c[0])), y * b1};
+}
+
+// exp(-(sre + i sim) r) with the products' rounding errors carried along.  float32:
+// argument reduction with constants in two parts (Cody and Waite, Software Manual for the
+// Elementary Functions, 1980): log 2 = 2839 / 2^12 + a rest, whose first part times an
+// integer of at most 12 bits is exact, and pi / 2 = 201 / 2^7 + a rest, exact up to 16
+// bits; |s| r_c stays below 2304 here (|s| R <= 2.25, R >= r_c / 1024).  That leaves at
+// most log(2) / 2 and pi / 4, for the exponential function and for Taylor polynomials of
+// degree 9 and 10 (2e-9).  Each part is within 5 x 2^-24 of the result.
+__device__ __forceinline__ Cx<float> cexp_acc(float sre, float sim, float r) {
+    const float u0 = -sre * r, u = fmaxf(u0, -200.0f);
+    const float ul = u0 >= -200.0f ? fmaf(-sre, r, -u0) : 0.0f;
+    const float m = rintf(u * 1.44269504f);
+    float f = fmaf(-m, 2839.0f / 4096.0f, u);
+    f = fmaf(-m, 3.19461849453e-5f, f) + ul;
+    const float e = __expf(f) * exp2f(m);
+    const float t = sim * r, tl = fmaf(sim, r, -t);
+    const float n = rintf(t * 0.636619772f);
+    float h = fmaf(-n, 201.0f / 128.0f, t);
+    h = fmaf(-n, 4.83826794897e-4f, h) + tl;
+    const float h2 = h * h;
+    float sn = fmaf(h2, 1.0f / 362880.0f, -1.0f / 5040.0f);
+    sn = fmaf(h2, sn, 1.0f / 120.0f);
+    sn = fmaf(h2, sn, -1.0f / 6.0f);
+    sn = fmaf(h * h2, sn, h);
+    float cs = fmaf(h2, -1.0f / 3628800.0f, 1.0f / 40320.0f);
+    cs = fmaf(h2, cs, -1.0f / 720.0f);
+    cs = fmaf(h2, cs, 1.0f / 24.0f);
+    cs = fmaf(h2, cs, -0.5f);
+    cs = fmaf(h2, cs, 1.0f);
+    const int k = (int)n;
+    const float c1 = (k & 1) ? sn : cs, s1 = (k & 1) ? cs : sn;   // cos, sin of n quarter turns + h
+    const float c = ((k + 1) & 2) ? -c1 : c1, s = (k & 2) ? -s1 : s1;
+    return {e * c, -e * s};
+}
+__device__ __forceinline__ Cx<double> cexp_acc(double sre, double sim, double r) {
+    const double u = -sre * r, ul = fma(-sre, r, -u);
+    double e = exp(u);
+    if (e > 0.0 && e < 1e300) e = fma(e, ul, e);
+    const double t = sim * r, tl = fma(sim, r, -t);
+    double sn, cs;
+    sincos(t, &sn, &cs);
+    return {e * fma(-sn, tl, cs), -e * fma(cs, tl, sn)};
 }
 
 }  // namespace g3

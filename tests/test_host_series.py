@@ -5,6 +5,9 @@ series evaluated with more digits than the precision it serves: the degrees of f
 in float64, those of float64 in extended precision.  What is left of the difference to
 the points summed one by one is the series' end, at most |z|^(N+1) / (N+1)! of p(0)
 for the single layer and the double layer.
+
+The float32 exponential beside it, against float64: its reduction carries the products'
+roundings, so that its error does not grow with the phase.
 """
 import ctypes
 import math
@@ -24,6 +27,7 @@ SRC = r"""
 #define __device__
 #define __forceinline__ inline
 using std::min; using std::max; using std::fma;
+#define __expf(x) std::exp(x)
 namespace g3 { template <class T> struct Cx { T x, y; }; enum { G3_SLP = 0, G3_DLP = 1 }; }
 #include "g3_series.cuh"
 using namespace g3;
@@ -52,6 +56,15 @@ template <int KER, class D, class T> static double levels(int l, int n, const do
     using S = NearSeries<D>;
     return l == 0 ? run<KER, D, S::N0, T>(n, r, a, x, y) : l == 1 ? run<KER, D, S::N1, T>(n, r, a, x, y) : run<KER, D, S::N2, T>(n, r, a, x, y);
 }
+extern "C" double cexp_worst(int n, const float* sre, const float* sim, const float* r) {
+    double worst = 0;
+    for (int e = 0; e < n; ++e) {
+        const Cx<float> v = cexp_acc(sre[e], sim[e], r[e]);
+        const double m = std::exp(-(double)sre[e] * r[e]), t = (double)sim[e] * r[e];
+        worst = std::max(worst, std::max(std::abs(v.x - m * std::cos(t)), std::abs(v.y + m * std::sin(t))) / m);
+    }
+    return worst;
+}
 extern "C" double worst(int ker, int f64, int l, int n, const double* r, const double* a, double x, double y) {
     if (f64) return ker ? levels<G3_DLP, double, long double>(l, n, r, a, x, y) : levels<G3_SLP, double, long double>(l, n, r, a, x, y);
     return ker ? levels<G3_DLP, float, double>(l, n, r, a, x, y) : levels<G3_SLP, float, double>(l, n, r, a, x, y);
@@ -68,9 +81,9 @@ def series(tmp_path_factory):
     so = str(d / "s.so")
     subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-Wno-unknown-pragmas", "-I",
                     os.path.join(ROOT, "paper_2312_11219_gb300", "csrc"), "-o", so, str(d / "s.cpp")], check=True)
-    f = ctypes.CDLL(so).worst
-    f.restype = ctypes.c_double
-    return f
+    lib = ctypes.CDLL(so)
+    lib.worst.restype = lib.cexp_worst.restype = ctypes.c_double
+    return lib
 
 
 @pytest.fixture(scope="module")
@@ -108,6 +121,20 @@ def test_series_end(series, pairs, ker, f64, level):
     eps = 2.0 ** (-63 if f64 else -52)
     for phase in (0.0, 0.7, 1.5):
         s = 0.9999 * z / Rmax * np.exp(1j * phase)
-        w = series(ker, f64, level, r.shape[0], r.ctypes.data_as(P), amp[ker].ctypes.data_as(P),
+        w = series.worst(ker, f64, level, r.shape[0], r.ctypes.data_as(P), amp[ker].ctypes.data_as(P),
                    ctypes.c_double(s.real), ctypes.c_double(s.imag))
         assert w <= math.exp(z) * bound + 64 * eps * math.exp(2 * z)
+
+
+@pytest.mark.parametrize("decay", [0.0, 1.0, 80.0])
+@pytest.mark.parametrize("phase", [0.5, 30.0, 2300.0])
+def test_exponential(series, decay, phase):
+    rng = np.random.default_rng(int(phase))
+    n = 200000
+    r = rng.uniform(0.3, 3.0, n).astype(np.float32)
+    sre = (decay * rng.uniform(0, 1, n) / r).astype(np.float32)
+    sim = (phase * rng.uniform(-1, 1, n) / r).astype(np.float32)
+    P = ctypes.POINTER(ctypes.c_float)
+    w = series.cexp_worst(n, sre.ctypes.data_as(P), sim.ctypes.data_as(P), r.ctypes.data_as(P))
+    # the exponential, the reduced arguments, the polynomial and the product: five roundings
+    assert w <= 5 * 2.0 ** -24
