@@ -206,6 +206,17 @@ struct FaceThr {
     float scale;
 };
 
+// the exponent of x > 0, and 2^e (|e| <= 1000): integer operations, where ilogb and ldexp
+// are calls
+__device__ __forceinline__ int exponent_of(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) - 1023; }
+__device__ __forceinline__ double pow2_of(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+// sqrt(q) as float32 for q of twice float32's range
+__device__ __forceinline__ float sqrt32(double q) {
+    if (!(q > 1e-290)) return 0.f;
+    const int e = exponent_of(q) & ~1;
+    return sqrtf((float)(q * pow2_of(-e))) * scalbnf(1.f, e / 2);
+}
+
 // shared state of the block being processed
 template <class T>
 struct BlockSh {
@@ -235,6 +246,7 @@ struct BlockSh {
     double crs[32];
     FaceThr thr;             // the face test's bound
     float rms;               // ||C^(l-1)||_F / sqrt(Ku)
+    double iku;              // 1 / Ku
     // float32 recompression: squared norms, norms and their reciprocals of the
     // orthogonalised V columns; squared norms of W's columns (double-buffered);
     // norms of the pivot columns
@@ -1781,7 +1793,7 @@ __device__ __forceinline__ void norm_test(const AcaArgs<T>& A, BlockSh<T>& S, in
         if (threadIdx.x == 0) {
             const double own = S.hself * S.fself;
             S.norm2 += add + own;
-            if constexpr (sizeof(T) == 4) S.rms = (float)sqrt(fmax(S.norm2, 0.0) / (double)A.Ku);
+            if constexpr (sizeof(T) == 4) S.rms = sqrt32(S.norm2 * S.iku);
             S.stop = fmax(own, 0.0) <= A.eps3 * A.eps3 * fmax(S.norm2, 0.0);
             S.flag = all_used(A, S);
         }
@@ -1847,7 +1859,7 @@ __device__ __noinline__ bool confirm_stop(const AcaArgs<T>& A, const Ws<T>& w, B
     double* rk = w.rk;   // [SAMPLES / SPI][Ku]
     constexpr bool F32 = sizeof(T) == 4;
     constexpr int SPI = F32 ? 4 : 1;
-    const int ex = F32 ? min(max(S.norm2 > 0.0 ? ilogb(S.norm2) / 2 : ilogb(fmax(fabs(S.hpiv.x), fabs(S.hpiv.y))), -100), 100) : 0;
+    const int ex = F32 ? min(max(S.norm2 > 0.0 ? exponent_of(S.norm2) / 2 : exponent_of(fmax(fabs(S.hpiv.x), fabs(S.hpiv.y))), -100), 100) : 0;
     const T sc = F32 ? (T)scalbnf(1.f, -ex) : (T)1;
     const double back = F32 ? (double)scalbnf(1.f, ex) : 1.0;
     double rr_t = 0.0, aa_t = 0.0;
@@ -2146,6 +2158,7 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3(const AcaArgs<T
             S.pre[0] = 0;
             S.norm2 = 0.0;
             S.rms = 0.f;
+            S.iku = 1.0 / (double)A.Ku;
             S.entries = 0;
             S.raw = 0;
             for (int i = 0; i < NSUB; ++i) S.sub[i] = 0;
@@ -2571,7 +2584,8 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3_face(const AcaA
                 S.pre[p + 1] = S.pre[p] + cr.r;
             }
             S.norm2 = normb[blk];
-            S.rms = (float)sqrt(fmax(S.norm2, 0.0) / (double)A.Ku);
+            S.iku = 1.0 / (double)A.Ku;
+            S.rms = sqrt32(S.norm2 * S.iku);
             S.entries = 0;
             S.raw = 0;
             for (int i = 0; i < NSUB; ++i) S.sub[i] = 0;

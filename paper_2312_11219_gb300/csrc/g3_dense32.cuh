@@ -91,7 +91,7 @@ __device__ __noinline__ bool confirm_dense(DenseSh<W>& sh, const BlockRange br, 
     // squares scaled by a power of two near ||C^(l)||, which the entries do not exceed
     // by much (near the newest pivot, they could exceed it by all of float32's range),
     // float-float sums
-    const int ex = min(max(sh.norm2 > 0.0 ? ilogb(sh.norm2) / 2 : ilogbf(fmaxf(fabsf(hpiv.x), fabsf(hpiv.y))), -100), 100);
+    const int ex = min(max(sh.norm2 > 0.0 ? exponent_of(sh.norm2) / 2 : ilogbf(fmaxf(fabsf(hpiv.x), fabsf(hpiv.y))), -100), 100);
     const float sc = scalbnf(1.f, -ex);
     const double back = (double)scalbnf(1.f, ex);
     float2 rt = make_float2(0.f, 0.f), at = rt;
@@ -350,8 +350,9 @@ __global__ void __launch_bounds__(DENSE32_NT, 4) k_dense32(const AcaArgs<float> 
                 pbuf ^= 1;
             }
             if (wid == 0) {
-                add = warp_sum(add);
-                own = warp_sum(own);   // (one lane holds it)
+                add += __shfl_xor_sync(0xffffffffu, add, 2);   // (lanes 0 to 3 hold them)
+                add += __shfl_xor_sync(0xffffffffu, add, 1);
+                own = __shfl_sync(0xffffffffu, own, nc & 3);
                 if (lane == 0) {
                     const double n2 = sh.norm2 + (add + own);
                     sh.norm2 = n2;

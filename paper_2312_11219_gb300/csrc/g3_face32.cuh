@@ -200,11 +200,11 @@ __device__ void samples32(const AcaArgs<float>& A, BlockSh<float>& S, const Face
 
 // max(eps_face^2 ||S_m||_F^2, floor^2)
 __device__ __forceinline__ double face_bound2(const AcaArgs<float>& A, const BlockSh<float>& S) {
-    return fmax(A.eps_face * A.eps_face * fmax(S.fsn2, 0.0), A.face_floor * A.face_floor * S.norm2 / (double)A.Ku);
+    return fmax(A.eps_face * A.eps_face * fmax(S.fsn2, 0.0), A.face_floor * A.face_floor * (S.norm2 * S.iku));
 }
 __device__ __forceinline__ FaceThr face_thr(double b) {
-    const int e = b > 0.0 ? min(max(ilogb(b), -120), 120) : 0;
-    b = fmin(ldexp(b, -e), 3e38);
+    const int e = b > 0.0 ? min(max(exponent_of(b), -120), 120) : 0;
+    b = fmin(b * pow2_of(-e), 3e38);
     const float h = (float)b;
     return FaceThr{make_float2(h, (float)(b - (double)h)), scalbnf(1.f, -e)};
 }
