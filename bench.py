@@ -39,14 +39,15 @@ METRIC = "3-way ACA entries/s & apply GB/s (1 GB300); learned+batched vs plain a
 # each one rsqrt, one ex2, one sin and one cos (Galerkin: 16 points)
 # DRAM bytes (read + write) per low-rank k_aca3 launch of the 12,288-triangle
 # L-shape, mean of the single and double layer, from one ncu capture of each
-# operator's launch (dram__bytes_read.sum + dram__bytes_write.sum: 36.8 GB and
-# 41.8 GB) of the current kernel; other workloads have no capture (null)
-ACA_TRAFFIC_BYTES = {"lshape12288": 0.5 * (19234748160 + 17581539072 + 23269448960 + 18566676224)}
+# operator's launch (dram__bytes_read.sum + dram__bytes_write.sum: 34.6 GB and
+# 40.8 GB; profiles/k_aca3_lshape12288_counters.md); other workloads have no capture
+# (null), and a change of the kernels asks for a new one
+ACA_TRAFFIC_BYTES = {"lshape12288": 0.5 * (17968108800 + 16599058176 + 22869738496 + 17924917248)}
 # DRAM bytes (read + write) of one apply of each operator of the same workload
-# (every kernel of apply_gcq, from one ncu capture per operator: 7,131.4 MB
-# single layer, 6,899.9 MB double layer); the bench's steady-state apply bytes
-# are the same sum over both operators
-APPLY_TRAFFIC_BYTES = {"lshape12288": 7131350656 + 6899897472}
+# (every kernel of apply_gcq, from one ncu capture per operator: 7,128.4 MB
+# single layer, 6,857.6 MB double layer; profiles/k_apply_lshape12288_traffic.md);
+# the bench's steady-state apply bytes are the same sum over both operators
+APPLY_TRAFFIC_BYTES = {"lshape12288": 7128394112 + 6857601536}
 MUFU_PER_ENTRY = 28
 MUFU_PER_ENTRY_GALERKIN = 64
 # special-function-unit results per clock per SM for rsqrt / sin / cos

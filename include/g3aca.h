@@ -83,9 +83,11 @@ typedef enum {
 /* Arithmetic of the path. */
 typedef enum {
     G3_FP64 = 0,   /* everything in float64; factors and near field complex128       */
-    G3_MIXED = 1   /* float32 entries, face arithmetic and recompression, fiber
-                      residuals in float-float, float64 singular entries, norms and
-                      frequencies; factors and near field complex64                   */
+    G3_MIXED = 1   /* float32 entries, face arithmetic and recompression; fiber
+                      residuals, sampled residuals and the points of Galerkin pairs
+                      with a common vertex in float-float (about 48 bits); float64
+                      collocation self entries, norms over crosses, stopping tests
+                      and frequencies; factors and near field complex64               */
 } g3_precision;
 
 typedef enum { G3_C64 = 0, G3_C128 = 1 } g3_dtype;

@@ -18,7 +18,7 @@
 //           row of eq. (index) from the factors and the largest entry of
 //           that row;
 //   fiber   f_l[k] = (ENTRY(i_l, j_l, k) - sum_p H_p[i_l, j_l] f_p[k]) / H_l[i_l, j_l]
-//           with the residual in float64;
+//           with the residual in float64 (T = float: float-float, about 48 bits);
 //   norm    eq. (norm): ||C^(l)||^2 += 2 Re sum_d <H_l, H_d><f_l, f_d> + ||H_l||^2 ||f_l||^2,
 //           face inner products through Gram products (U_d^H U_l)(V_l^H V_d);
 //   stop    ||H_l|| ||f_l|| <= eps3 ||C^(l)|| -> rank l - 1; all frequencies
@@ -28,10 +28,10 @@
 //
 // Precision: T = float (mixed) evaluates entries and face arithmetic in
 // float32 and stores complex64 factors; T = double does everything in float64.
-// In both, the fiber residuals, the sums over crosses of eq. (norm) and
-// ||C^(l)|| are float64; with T = float the recompression is float32
-// throughout (it forms no Gram matrices) and the face test's sum over crosses
-// float-float.
+// In both, the sums over crosses of eq. (norm), ||C^(l)||, the stopping test and
+// what the face test sums over its crosses are float64.  With T = float the
+// recompression is float32 throughout (it forms no Gram matrices), the fiber
+// residual float-float, and so are the sampled residuals' squares, scaled.
 //
 // No CTA waits on another: the only inter-CTA communication is the atomic
 // queue counter and the atomic pool allocator.
@@ -1919,7 +1919,7 @@ __device__ __noinline__ bool confirm_stop(const AcaArgs<T>& A, const Ws<T>& w, B
 template <int KER, class T, int NT>
 __device__ void dense_block(const AcaArgs<T>& A, const Ws<T>& w, BlockSh<T>& S, bool& zero_block, int& computed,
                             bool& overflow, long long* ph, long long& tclk) {
-    static_assert(sizeof(T) == 8, "float32 blocks with dense faces run one warp each");
+    static_assert(sizeof(T) == 8, "float32 blocks with dense faces: k_dense32");
     const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
     const int M = S.M, N = S.N, MN = M * N, Ku = A.Ku, blk = S.blk;
     auto lap = [&](int i) {
@@ -2404,7 +2404,7 @@ __global__ void __launch_bounds__(NT, aca_min_ctas<NT>()) k_aca3(const AcaArgs<T
                 }
             }
             __syncthreads();
-            // ---------------- fiber (float64 residual) ----------------
+            // ---------------- fiber (residual in float64, float32 blocks in float-float) ----------------
             const int ip = S.ip, jp = S.jp, nc = S.ncross;
             if constexpr (sizeof(T) == 4) {
                 fiber32<KER, NT>(A, tid, S.rb + ip, S.cb + jp, nc, S.fk, cff_inv(ccast<float>(S.hpiv)),

@@ -22,8 +22,8 @@ struct Cx {
 // or 128-bit (double) access.  Cx<T> has the alignment of T, so a plain
 // dereference becomes two accesses; every device buffer of complex values
 // here (factor pool, workspace, apply scratch, near field) starts at a
-// cudaMalloc'd base and is indexed in whole elements, so its elements are
-// aligned to their size.
+// multiple of 256 bytes in an allocation (dev_alloc hands out whole ones) and is
+// indexed in whole elements, so its elements are aligned to their size.
 template <class T>
 __device__ __forceinline__ Cx<T> ldcx(const Cx<T>* p) {
     if constexpr (sizeof(T) == 4) {

@@ -659,8 +659,9 @@ __global__ void __launch_bounds__(256) k_near_p1(GeomF gf, GeomD gd, const int* 
 // identical panels: the Sauter-Schwab maps (as k_near_ss) with the products
 // lambda_a(x) lambda_b(y) of the local functions in the integrand; one CTA per
 // element pair writes its 3 x 3 local entries at every frequency.  The points
-// of one region (SS_N^4) are set up in float64 and kept in shared memory (their
-// reference coordinates, distance and weight, and for the adjoint double layer
+// of one region (SS_N^4) are set up in float64 (T = float: in float-float from the
+// tables) and kept in shared memory (their reference coordinates, distance and
+// weight, and for the adjoint double layer
 // -((x - y) . n_x) / r^2); each frequency's ten sums (the plain integral and
 // the nine weighted ones) are reduced over the CTA and added into acc.
 template <int OP, class T, int NT>
@@ -1098,8 +1099,8 @@ static int near_chunk(const g3_ctx* ctx, int nb, int Ku) {
     return (Ku + n - 1) / n;
 }
 
-// Galerkin: near-field pairs with a common vertex (the list of SsPair records
-// built on the host) by k_near_ss, after the regular rule for all pairs
+// Galerkin: near-field pairs with a common vertex (the SsPair records of k_ss_pairs) by
+// k_near_ss32 or k_near_ss, after the regular rule for all pairs
 template <class T>
 static g3_status launch_near_galerkin(g3_ctx* ctx, const g3_tree* t, const g3_freqs* f, g3_near* nf) {
     const int nb = (int)nf->order.size();
