@@ -614,9 +614,11 @@ static g3_status run_aca_t(g3_ctx* ctx, std::vector<AcaJob>& jobs, int kernel, d
         for (int b : sp) n_lo += !is_dense(ranges[b]);
         n_de = n_spill - n_lo;
         // enlarged pool: the used part [0, cap) is kept at the same offsets
-        // at least 1.5 times the spilled blocks' plain estimate (which
-        // over-reserves): one round, even after the learned scale has shrunk
-        long long add = (long long)(1.5 * std::max(scale, 1.0) * est2);
+        // at least 1.5 times the spilled blocks' plain estimate (which mostly
+        // over-reserves): one round, even after the learned scale has shrunk.  A
+        // rerun block starts over, and large blocks at high frequencies need three
+        // times their estimate, so each further round adds twice as much
+        long long add = (long long)(1.5 * std::ldexp(std::max(scale, 1.0), regrows - 1) * est2);
         add = std::max(add, (long long)(ctr - std::min<unsigned long long>(ctr, (unsigned long long)cap)));
         add = std::max(add, (long long)1 << 16);
         // the enlarged pool and the copy of the old one must fit together
