@@ -2,6 +2,7 @@
 // host<->device staging.  All compute runs in the kernels of g3_prep.cu,
 // g3_aca.cu and g3_apply.cu.
 #include <algorithm>
+#include <chrono>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -57,9 +58,9 @@ g3_status cuda_fail(cudaError_t e, const char* what) {
 // Bounds: at most 1/32 of the device's memory is kept per device (the oldest buffers go
 // first, larger ones are never kept), and no buffer above 128 MB while less than an
 // eighth of the device is free: the memory may be wanted elsewhere in the process, and
-// goes back at once, with all that was kept (asking takes about 15 us).  A failing
-// allocation frees all of it and is tried again; so do g3_trim and the end of the
-// device's last context.
+// goes back at once, with all that was kept (asking takes 15 to 30 us, so an answer
+// stands for 5 ms).  A failing allocation frees all of it and is tried again; so do
+// g3_trim and the end of the device's last context.
 struct DevPool {
     struct Block {
         void* p;
@@ -88,15 +89,20 @@ struct DevPool {
         for (int i = 0; i < n; ++i) cudaFree(kept[i].p);
         remove(0, n);
     }
-    // room for keeping a buffer (device `dev`)
-    static bool room(size_t bytes, int dev) {
+    // room for keeping a buffer (device `dev`): the answer of at most 5 ms ago
+    std::chrono::steady_clock::time_point asked{};
+    bool plenty = false;
+    bool room(size_t bytes, int dev) {
         if (bytes <= (128 << 20)) return true;
+        const auto now = std::chrono::steady_clock::now();
+        if (plenty && now - asked < std::chrono::milliseconds(5)) return true;
         size_t free_b = 0, total = 0;
         int cur = -1;
-        const bool ok = cudaGetDevice(&cur) == cudaSuccess && cur == dev &&
-                        cudaMemGetInfo(&free_b, &total) == cudaSuccess;
-        if (!ok) cudaGetLastError();
-        return ok && free_b >= total / 8;
+        plenty = cudaGetDevice(&cur) == cudaSuccess && cur == dev &&
+                 cudaMemGetInfo(&free_b, &total) == cudaSuccess && free_b >= total / 8;
+        if (!plenty) cudaGetLastError();
+        asked = now;
+        return plenty;
     }
 };
 static DevPool* dev_pool(int dev) {
