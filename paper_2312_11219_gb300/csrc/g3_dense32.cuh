@@ -12,9 +12,9 @@
 // crosses per pass: face inner products in float32; those of the fibers, the sum
 // over the crosses, ||C^(l)||^2 and the stopping test in float64 (in float32 they
 // would overflow from entries of 1e16 on, and the fibers reach the ratio of the
-// largest entry to the pivot).  12,288-triangle single layer, 17,554 blocks: 13.1 ms (256
-// threads, float64 fiber) -> 5.0 ms after the low-rank launch, which it
-// overlaps.  1, 2, 4 and 8 warps per block: 80.8, 81.0, 80.7 and 82.6 ms for the
+// largest entry to the pivot).  12,288-triangle single layer, 17,450 blocks: 13.1 ms (256
+// threads, float64 fiber) -> 6.6 ms after the low-rank launch, which it
+// overlaps (the same with the sums in float32).  1, 2, 4 and 8 warps per block: 80.8, 81.0, 80.7 and 82.6 ms for the
 // whole set-up there, 1.79, 1.60, 1.49 and 1.46 ms for the step on the
 // 768-triangle cube (320 blocks).
 

@@ -227,8 +227,10 @@ __device__ __forceinline__ bool face_passes(const FaceThr& t, float nu2, float n
 // (two more barriers; the sum over t took a third of the step's instructions).
 // The sums over a vector are float32; their products and what is summed of them are
 // float64 in one warp, as in face_aca, and with D the test is taken in float-float on a
-// scaled bound that one warp forms per face (float64 in every warp would hold each
-// step for its pipe, and float32 products of squares overflow from entries of 1e12).
+// scaled bound that one warp forms per face and every step reads from shared memory
+// (float64 in every warp would hold each step for its pipe; the bound in registers
+// costs 1 % of the whole launch in spills: 12,288-triangle single layer 72.4 and
+// 71.3 ms).
 template <int KER, int NT>
 __device__ int face32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float>& S, int kf, unsigned char* arena,
                       ColStore& c) {
@@ -278,7 +280,6 @@ __device__ int face32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float
         }
     }
     __syncthreads();
-    const FaceThr thr = S.thr;   // (with D)
     while (m < cap) {
         // ---- the residual row ----
         if (F.ncol > 0) {
@@ -383,7 +384,7 @@ __device__ int face32(const AcaArgs<float>& A, const Ws<float>& w, BlockSh<float
             sublap(S, 8, tf);
         }
         ++m;
-        if (D ? face_passes(thr, nu2, nv2) : S.fconv != 0) {
+        if (D ? face_passes(S.thr, nu2, nv2) : S.fconv != 0) {
             if (!A.sample_check) {
                 converged = true;
                 break;
